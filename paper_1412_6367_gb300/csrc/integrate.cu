@@ -1257,58 +1257,73 @@ __device__ __forceinline__ const Inst &inst_of_row(const Inst &single, const Ins
     return multi[lo];
 }
 
-// The value row_sum<float> computes, formed by one thread: the 32 lanes' strided Kahan sums
-// and the same lower-lane-left merge tree, each virtual lane's sum kept in registers.  For
-// rows with few slots (2D patterns: ~1-2 segments per row) this replaces a warp per row and
-// frame by a thread; the bits are the same.
-__device__ __forceinline__ Kahan kahan_one(float v) {
-    Kahan k{0.f, 0.f};
-    kahan_add(k, 1.f, v);
-    return k;
+// The value row_sum computes, formed by one thread: the 32 lanes' strided sums (virtual lane l
+// sums slots l, l + 32, ...) merged by the same tree, depth first, so that a few sums are live.
+template <class AT, int M>
+__device__ __forceinline__ Acc<AT> row_tree(const AT *p, int n, int l) {
+    Acc<AT> x;
+    if constexpr (M == 32) {
+        x.zero();
+        for (int s = l; s < n; s += 32) x.add(AT(1), p[s]);
+    } else {
+        x = row_tree<AT, 2 * M>(p, n, l);
+        // a merge with an empty lane's {+0, +0} changes no bit
+        if (l + M < n) x.merge(row_tree<AT, 2 * M>(p, n, l + M));
+    }
+    return x;
 }
 
-__device__ __forceinline__ float row_sum_thread(const float *p, int a, int b) {
-    // Up to four slots: the tree's only non-trivial merges (a merge with an empty lane's
-    // {+0, +0} changes no bit), in the tree's order.
-    const int n = b - a;
-    if (n <= 0) return 0.f;
-    if (n == 1) return kahan_value(kahan_one(p[a]));
-    if (n <= 4) {
-        Kahan x0 = kahan_one(p[a]), x1 = kahan_one(p[a + 1]);
-        if (n == 2) {
-            kahan_merge(x0, x1);
-            return kahan_value(x0);
-        }
-        kahan_merge(x0, kahan_one(p[a + 2]));       // lanes 0 and 2 at the pairs-of-two level
-        if (n == 4) kahan_merge(x1, kahan_one(p[a + 3]));
-        kahan_merge(x0, x1);
-        return kahan_value(x0);
-    }
-    Kahan v[32];
-#pragma unroll
-    for (int l = 0; l < 32; ++l) {
-        v[l].s = 0.f;
-        v[l].nc = 0.f;
-        for (int s = a + l; s < b; s += 32) kahan_add(v[l], 1.f, p[s]);
-    }
-#pragma unroll
-    for (int m = 16; m > 0; m >>= 1)
-#pragma unroll
-        for (int l = 0; l < m; ++l) kahan_merge(v[l], v[l + m]);
-    return kahan_value(v[0]);
+template <class AT>
+__device__ __forceinline__ AT row_sum_thread(const AT *p, int a, int b) {
+    return row_tree<AT, 1>(p + a, b - a, 0).value();
 }
 
-// Frames-mode phase 2 with one thread per (row, frame), for rows of few slots.
-__global__ void phase2_frames_thread_kernel(const __grid_constant__ Inst d, int64_t n_jobs) {
-    for (int64_t job = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; job < n_jobs;
-         job += (int64_t)gridDim.x * blockDim.x) {
-        const int f = (int)(job / d.nrows), r = (int)(job - (int64_t)f * d.nrows);
-        const int a = d.row_slot_ptr[r], b = d.row_slot_ptr[r + 1];
-        const float S = row_sum_thread(static_cast<const float *>(d.partial) + (size_t)f * d.nseg, a, b);
+// Phase 2 for rows of few slots (2D patterns have one or two): a thread per row, which in
+// frames mode takes kThreadFrames frames (blockIdx.y) so that the row's slot range and N are read
+// once for them and the frames' loads are independent.  Bound by memory traffic: a slot's sum is
+// read and four (frames: two) outputs written per row, consecutive threads on consecutive rows
+// and slots.  A warp per row left 31 lanes idle on one slot and spent five rounds of shuffles:
+// 66.6 us for one frame of a 500 x 360 pattern (180 000 rows, S and N) against 12.8 us here,
+// 32.8 against 6.0 us in norm mode; in frames mode a thread per (row, frame), which divided 64-bit
+// job numbers and read the row's range for every frame, took 50.3 us for 16 frames against 37.2.
+constexpr int kThreadFrames = 4;
+constexpr int kThreadRows = 4096;
+
+template <class AT, int MODE>
+__global__ void __launch_bounds__(256, 4) phase2_thread_kernel(const __grid_constant__ Inst d, int n_frames) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= d.nrows) return;
+    const int a = d.row_slot_ptr[r], b = d.row_slot_ptr[r + 1];
+    const AT *P = static_cast<const AT *>(d.partial);
+    if (MODE == MODE_FRAMES) {
         const float N = d.norm[r];
-        const size_t o = (size_t)(d.frame_out0 + f) * d.nrows + r;
-        if (d.oS) static_cast<float *>(d.oS)[o] = S;
-        if (d.oI) static_cast<float *>(d.oI)[o] = N != 0.f ? __fdiv_rn(S, N) : 0.f;
+        const int f0 = blockIdx.y * kThreadFrames;
+#pragma unroll
+        for (int i = 0; i < kThreadFrames; ++i) {
+            const int f = f0 + i;
+            if (f >= n_frames) break;
+            const float S = (float)row_sum_thread<AT>(P + (size_t)f * d.nseg, a, b);
+            const size_t o = (size_t)(d.frame_out0 + f) * d.nrows + r;
+            if (d.oS) static_cast<float *>(d.oS)[o] = S;
+            if (d.oI) static_cast<float *>(d.oI)[o] = N != 0.f ? __fdiv_rn(S, N) : 0.f;
+        }
+    } else if (MODE == MODE_SINGLE) {
+        const AT S = row_sum_thread<AT>(P, a, b);
+        const AT N = d.single_nc == 2 ? (AT)d.norm[d.nrows + r] : row_sum_thread<AT>(P + d.nseg, a, b);
+        const AT C = d.single_nc ? (AT)d.norm[d.nrows + r] : row_sum_thread<AT>(P + 2 * (size_t)d.nseg, a, b);
+        if (d.oI) static_cast<AT *>(d.oI)[r] = N != AT(0) ? S / N : AT(0);
+        if (d.oS) static_cast<AT *>(d.oS)[r] = S;
+        if (d.oN) static_cast<AT *>(d.oN)[r] = N;
+        if (d.oC) static_cast<AT *>(d.oC)[r] = C;
+    } else {
+        const AT N = row_sum_thread<AT>(P, a, b);
+        d.norm[r] = (float)N;
+        if (d.oN) static_cast<float *>(d.oN)[r] = (float)N;
+        if (d.norm_rows == 2) {
+            const AT C = row_sum_thread<AT>(P + d.nseg, a, b);
+            d.norm[d.nrows + r] = (float)C;
+            if (d.oC) static_cast<float *>(d.oC)[r] = (float)C;
+        }
     }
 }
 
@@ -1457,11 +1472,13 @@ template <class AT, int MODE>
 int run_phase2(const Inst &single, const Inst *multi, int n_inst, int64_t n_jobs, int n_frames,
                cudaStream_t s, Profiler *prof = nullptr) {
     if (n_jobs <= 0) return AZ_OK;
-    if (MODE == MODE_FRAMES && sizeof(AT) == 4 && !multi && (int64_t)single.nseg <= 8 * (int64_t)single.nrows) {
-        // few slots per row: a thread per (row, frame)
-        const int64_t blocks = std::min<int64_t>((n_jobs + 255) / 256, (int64_t)num_sms() * 16);
+    // Rows of few slots on average: a thread per row, if the rows fill the GPU (4096 rows are 16
+    // blocks; below that a warp per row has more loads in flight).  A 2D pattern has 1 to 2 slots
+    // per row, a 1D one 100 and more: the line at 8 lies between.
+    if (!multi && (int64_t)single.nseg <= 8 * (int64_t)single.nrows && single.nrows >= kThreadRows) {
+        const int fy = MODE == MODE_FRAMES ? (n_frames + kThreadFrames - 1) / kThreadFrames : 1;
         ProfScope ps(prof, 3, s);
-        phase2_frames_thread_kernel<<<(unsigned)blocks, 256, 0, s>>>(single, n_jobs);
+        phase2_thread_kernel<AT, MODE><<<dim3((unsigned)((single.nrows + 255) / 256), (unsigned)fy), 256, 0, s>>>(single, n_frames);
         AZ_CUDA(cudaGetLastError());
         return AZ_OK;
     }
@@ -1871,7 +1888,9 @@ int preload_single_pass() {
     AZ_TRY((preload_single_dt<float, AZ_DTYPE_U32>()));
     AZ_TRY((preload_single_dt<float, AZ_DTYPE_I32>()));
     AZ_TRY(preload_kernel(phase2_kernel<double, MODE_SINGLE>));
-    return preload_kernel(phase2_kernel<float, MODE_SINGLE>);
+    AZ_TRY(preload_kernel(phase2_kernel<float, MODE_SINGLE>));
+    AZ_TRY((preload_kernel(phase2_thread_kernel<double, MODE_SINGLE>)));
+    return preload_kernel(phase2_thread_kernel<float, MODE_SINGLE>);
 }
 
 int forward_single_into(const az_integrator *h, const void *image, int dtype, const float *dark,
