@@ -40,13 +40,34 @@ int alloc_scratch(az_integrator *h) {
 }
 
 int finish_build(az_integrator *h, cudaStream_t s) {
-    // defaults measured on the Pilatus-6M workload (1D) and the 2048 x 2048 cake (2D, whose
-    // bins are compact in both directions); az_autotune refines them per matrix
-    int th = h->npt_azim > 0 ? 32 : 8, tw = h->npt_azim > 0 ? 64 : 224;
+    // Default tiles; az_autotune refines them per matrix.  1D: 8 x 120, or 16 x 64 from 2.1 entries
+    // per pixel on -- taller tiles make fewer, longer segments, which pays where the entries set
+    // the time, wider rows make fewer pieces of a copy, which pays where the pixels do.  Frames
+    // kernel, 8 x 120 against 16 x 64: 683 and 777 us (128 frames of 2527 x 2463 pixels, 1.7
+    // entries per pixel), 273 and 244 us (37 frames of 2167 x 2070, 2.6), 45 and 40 us (24 variances
+    // of 1043 x 981, 2.8).  2D: 48 x 40 (500 x 360 bins of 2048 x 2048 pixels, 16 frames and one:
+    // 91 and 29 us; 32 x 64, where only four frames fit a stage: 109 and 28 us; 24 x 56: 80 and 37).
+    int th = 48, tw = 40;
+    if (h->npt_azim == 0) {
+        const bool dense = (double)h->nnz >= 2.1 * (double)h->n_unmasked;
+        th = dense ? 16 : 8;
+        tw = dense ? 64 : 120;
+    }
     if (build_tiled_layout(h, th, tw, s) != AZ_OK) {  // a denser matrix: smaller tiles
         th = 8;
         tw = 64;
         AZ_TRY(build_tiled_layout(h, th, tw, s));
+    }
+    // The allocation-free entry point takes integrators whose FP64 partial sums fit its fixed
+    // array, or whose FP32 ones do (twice the segments).  A matrix past either limit gets larger
+    // tiles if they bring it below.
+    const int64_t most = (int64_t)AZ_NOALLOC_SCRATCH_BYTES / (3 * (int64_t)sizeof(double));
+    if (h->tl.nseg > most) {
+        const int bh = h->npt_azim > 0 ? 32 : 8, bw = h->npt_azim > 0 ? 64 : 224;
+        int64_t runs = 0;
+        AZ_TRY(count_runs(h, bh, bw, s, &runs));
+        if (runs >= 0 && (runs <= most || (h->tl.nseg > 2 * most && runs <= 2 * most)))
+            AZ_TRY(build_tiled_layout(h, bh, bw, s));
     }
     h->frames_per_pass = 8;
     h->rows_per_warp = 32 / h->frames_per_pass;
@@ -230,11 +251,11 @@ extern "C" int az_integrator_info(const az_integrator *h, az_info *out) {
     const DevBuf *bufs[] = {&h->csr_ptr, &h->csr_idx, &h->csr_w64, &h->csc_ptr, &h->csc_row,
                             &h->csc_w64, &h->csc_w32, &h->tl.tile_seg_ptr, &h->tl.tile_ent_ptr,
                             &h->tl.active_tiles, &h->tl.seg_ent_ptr, &h->tl.seg_slot,
-                            &h->tl.row_slot_ptr, &h->tl.ent_loc, &h->tl.ent_loc_p, &h->tl.ent_w32, &h->tl.ent_w64,
+                            &h->tl.row_slot_ptr, &h->tl.ent_loc, &h->tl.f_desc, &h->tl.f_rec, &h->tl.f_loc, &h->tl.f_w32, &h->tl.f_pix, &h->tl.ent_w32, &h->tl.ent_w64,
                             &h->partial, &h->norm, &h->adj, &h->status, &h->host_stage,
                             &h->tl.tile_desc, &h->tl.tile_rec, &h->tl.ent_pix, &h->tl.ent_dark,
                             &h->tl.norm_frames, &h->tl.ent_wnorm, &h->lut32, &h->lut64,
-                            &h->lut_vals, &h->lut_part, &h->one_planes, &h->bound_ent_dark,
+                            &h->lut_vals, &h->lut_part, &h->one_planes, &h->bound_ent_dark, &h->bound_dark_f,
                             &h->bound_norm};
     int64_t tot = 0;
     for (const DevBuf *b : bufs) tot += (int64_t)b->bytes;
@@ -678,7 +699,7 @@ extern "C" int az_autotune(az_integrator *h, int n_trial_frames, az_stream_t str
     cudaEvent_t e0, e1;
     AZ_CUDA(cudaEventCreate(&e0));
     AZ_CUDA(cudaEventCreate(&e1));
-    const int tiles[][2] = {{8, 224}, {8, 192}, {16, 64}, {16, 96}, {8, 128}, {16, 128}, {32, 64}, {8, 64}};
+    const int tiles[][2] = {{8, 224}, {8, 120}, {16, 64}, {16, 96}, {16, 56}, {48, 40}, {32, 64}, {24, 56}};
     const int fpps[] = {4, 8, 16};
     const int engines[] = {AZ_COPY_TMA, AZ_COPY_ASYNC};
     double best = 1e30;

@@ -92,17 +92,26 @@ struct TiledLayout {
     DevBuf seg_slot;        // int32 [nseg]        (position of the segment in row order)
     DevBuf row_slot_ptr;    // int32 [nrows + 1]
     DevBuf ent_loc;         // uint16 [padded_nnz] (shared-memory word offset in the tile)
-    // Frame-pair layout of the batched frames kernel (srow_p == 0: none for this tile shape).
-    // Frames F and F + 4 of a stage share a region of pw_p words: F's row-class slots at
-    // sl * ss_p, F + 4's slot_p words (16 mod 32: other banks) later, rows at pitch srow_p.
-    int srow_p = 0, ss_p = 0, slot_p = 0, pw_p = 0;
-    DevBuf ent_loc_p;       // uint16 [padded_nnz] (word offset in the frame-pair layout)
+    // Plane layout of the frames kernel: a block of fslots planes (0: none fits) is four class
+    // stretches of fslots * fslot_words words, plane i's rows of a class fslot_words * i words into
+    // it at pitch srow_f.
+    int srow_f = 0, fslot_words = 0, fslots = 0;
+    // The frames kernel's entries: per work item, its segments in units of eight, each unit's
+    // entries step by step, 32 to a step in lane order (lane 4 k + j: entry 4 t + j of segment k at
+    // step t; past a segment's end, weight 0 and its last pixel).  Per item a descriptor {tile,
+    // record offset (words), record words, entry offset, entries, units, 0, 0} and a record of
+    // units {first step, steps, slot[8] (-1: no segment)}.
+    int64_t f_entries = 0;
+    int f_max_entries = 0, f_max_rec = 0;
+    DevBuf f_desc, f_rec;   // int32 [n_active][8], int32 [sum of record words]
+    DevBuf f_loc, f_w32, f_pix;  // uint16, float, int32 [f_entries]
     DevBuf ent_w32;         // float  [padded_nnz]
     DevBuf ent_w64;         // double [padded_nnz]
     DevBuf ent_pix;         // int32  [padded_nnz] (pixel of the entry; -1 for padding)
-    DevBuf ent_dark;        // float  [padded_nnz] (dark of the entry's pixel, per batch call)
+    DevBuf ent_dark;        // float, per batch call: dark of the entry's pixel, in the order of the
+                            // kernel that reads it
     DevBuf norm_frames;     // float  [2][ny][nx]: flat * solid angle * polarisation, then ones
-    DevBuf ent_wnorm;       // float  [padded_nnz]: weight / (flat * solid angle * polarisation)
+    DevBuf ent_wnorm;       // float  [f_entries]: weight / (flat * solid angle * polarisation)
     // Per active tile: a 32-byte descriptor {tile, record offset (words), record words,
     // entry offset, padded entry count, segment count, 0, 0} and a 16-byte aligned record
     // {tile, ns, entry offset, entry count, slot[ns], uint16 start[ns + 1]} that the forward
@@ -190,7 +199,8 @@ struct az_integrator {
     int layout = AZ_LAYOUT_TILED;  // what az_integrate1d/2d use
     // corrections bound by az_set_corrections: per-entry darks, N and C of the current layout
     bool corr_bound = false, corr_dark = false;
-    azint::DevBuf bound_ent_dark;  // float [padded_nnz]
+    azint::DevBuf bound_ent_dark;  // float [padded_nnz], entry order of the general kernel
+    azint::DevBuf bound_dark_f;    // float [f_entries], of the frames kernel
     azint::DevBuf bound_norm;      // float [2][nrows]: N, C
     // host copies for the end-to-end path
     azint::DevBuf host_stage;  // device frames buffer for az_integrate_batch_host
@@ -212,6 +222,8 @@ int build_integrator(int ny, int nx, const double *rad, const double *chi, int n
                      int npt_azim, int unit, int split, const uint8_t *mask, cudaStream_t s,
                      az_integrator *h);
 int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s);
+// (tile, row) pairs that hold entries under th x tw tiles; -1 if not counted (too much scratch)
+int count_runs(const az_integrator *h, int th, int tw, cudaStream_t s, int64_t *out);
 int import_csr(az_integrator *h, const int32_t *indptr, const int32_t *indices, const double *data,
                cudaStream_t s);
 
@@ -254,7 +266,7 @@ int batch_norm(az_integrator *h, const float *flat, const float *sa, const float
                float *oC, cudaStream_t s);
 int batch_frames(az_integrator *h, const void *frames, int n, int dtype, const float *dark,
                  float *oI, float *oS, int frame_out0, cudaStream_t s,
-                 const float *ent_dark_given = nullptr, const float *norm = nullptr);
+                 bool bound_dark = false, const float *norm = nullptr);
 int bind_corrections(az_integrator *h, const float *dark, const float *flat, const float *sa,
                      const float *pol, cudaStream_t s);
 int forward_batch_bound(az_integrator *h, const void *frames, int n, int dtype, float *oI, float *oS,
@@ -292,6 +304,10 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
     uint64_t st;
     asm volatile("mbarrier.arrive.shared::cta.b64 %0, [%1];" : "=l"(st) : "r"(smem_addr(bar)) : "memory");
     (void)st;
+}
+
+__device__ __forceinline__ void mbar_arrive_n(uint64_t *bar, uint32_t count) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {

@@ -21,6 +21,8 @@ namespace {
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 constexpr int kScanTile = kScanThreads * kScanItems;
+constexpr int kSegEntries = 96;      // longest segment (entries)
+constexpr int32_t kSegFew = 300000;  // segments up to which long runs are cut
 constexpr double kKeep2D = 1e-12;  // relative area below which a 2D candidate is dropped
 
 int blocks_for(int64_t n, int per_block) { return (int)((n + per_block - 1) / per_block); }
@@ -662,15 +664,40 @@ __device__ __forceinline__ int tile_loc(const TileGeom &T, int32_t p) {
     return sl * T.ss + cs + jj * T.srow + lx;
 }
 
-// Offsets of the padded entries in the frame-pair layout (geometry Tp): the same formula at
-// the pair layout's row pitch and slot stride; padding entries read the zero band at 4 ss.
-__global__ void pair_loc_kernel(TileGeom Tp, const int32_t *__restrict__ pix, int64_t n,
-                                uint16_t *__restrict__ loc) {
+// First entry of every segment (and the entry count after the last) from the start flags.
+__global__ void seg_first_kernel(const int32_t *__restrict__ flag, const int32_t *__restrict__ segid, int64_t n,
+                                 int32_t *__restrict__ first) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e <= n;
+         e += (int64_t)gridDim.x * blockDim.x)
+        if (e == n || flag[e]) first[segid[e]] = (int32_t)e;
+}
+
+// Start flags with the runs longer than `cap` entries cut into pieces of nearly equal length, a
+// multiple of 4 entries.
+__global__ void split_flags_kernel(const int32_t *__restrict__ seg, const int32_t *__restrict__ first, int64_t n,
+                                   int cap, int32_t *__restrict__ flag) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
          e += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t p = pix[e];
-        loc[e] = (uint16_t)(p >= 0 ? tile_loc(Tp, p) : 4 * Tp.ss);
+        const int s = seg[e], a = first[s], len = first[s + 1] - a, pos = (int)e - a;
+        const int k = (len + cap - 1) / cap;
+        const int piece = ((len + k - 1) / k + 3) & ~3;
+        flag[e] = pos % piece == 0;
     }
+}
+
+// Longest segment, and the segment of every matrix entry (in the order of the matrix).
+__global__ void seg_of_kernel(const int32_t *__restrict__ seg, const int32_t *__restrict__ perm,
+                              const int32_t *__restrict__ first, int64_t n, int32_t *__restrict__ seg_of,
+                              int32_t *__restrict__ longest) {
+    int m = 0;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int s = seg[e];
+        seg_of[perm[e]] = s;
+        m = max(m, first[s + 1] - first[s]);
+    }
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(longest, m);
 }
 
 __global__ void tile_keys_kernel(TileGeom T, const int32_t *__restrict__ idx, int64_t n,
@@ -749,11 +776,11 @@ __global__ void seg_index_kernel(const int32_t *__restrict__ flag, const int32_t
 }
 
 // Sort key putting the longer segments of a tile first: max_len - length of the segment.
-__global__ void seg_len_key_kernel(const int32_t *__restrict__ seg, const int32_t *__restrict__ len,
+__global__ void seg_len_key_kernel(const int32_t *__restrict__ seg, const int32_t *__restrict__ first,
                                    int32_t max_len, int64_t n, uint32_t *__restrict__ key) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
          e += (int64_t)gridDim.x * blockDim.x)
-        key[e] = (uint32_t)(max_len - len[seg[e]]);
+        key[e] = (uint32_t)(max_len - (first[seg[e] + 1] - first[seg[e]]));
 }
 
 
@@ -795,11 +822,34 @@ __global__ void tiled_fill_kernel(TiledFillArgs A) {
     }
 }
 
+// Start flags in the final order: where the segment of the matrix entry changes.
+__global__ void seg_change_kernel(const int32_t *__restrict__ seg_of, const int32_t *__restrict__ perm, int64_t n,
+                                  int32_t *__restrict__ flag) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
+         e += (int64_t)gridDim.x * blockDim.x)
+        flag[e] = e == 0 || seg_of[perm[e]] != seg_of[perm[e - 1]];
+}
+
 __global__ void scatter_slots_kernel(const int32_t *__restrict__ perm, int nseg,
                                      int32_t *__restrict__ slot) {
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < nseg;
          s += (int64_t)gridDim.x * blockDim.x)
         slot[perm[s]] = (int32_t)s;
+}
+
+// One bit per (row, tile) that has entries, and their number.
+__global__ void mark_runs_kernel(TileGeom T, const int32_t *__restrict__ ptr, const int32_t *__restrict__ idx,
+                                 int nrows, int64_t words, uint32_t *__restrict__ bits,
+                                 unsigned long long *__restrict__ count) {
+    int n = 0;
+    for (int r = blockIdx.x; r < nrows; r += gridDim.x)
+        for (int e = ptr[r] + threadIdx.x; e < ptr[r + 1]; e += blockDim.x) {
+            const int t = tile_of(T, idx[e]);
+            const uint32_t m = 1u << (t & 31);
+            n += !(atomicOr(&bits[(int64_t)r * words + (t >> 5)], m) & m);
+        }
+    for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(count, (unsigned long long)n);
 }
 
 __global__ void max_kernel(const int32_t *a, int n, int32_t *out) {
@@ -822,9 +872,10 @@ __global__ void diff_kernel(const int32_t *ptr, int n, int32_t *out) {
 }
 
 // Work items: a tile's segments (longest first) cut into runs whose entries, counted from
-// the run's first entry rounded down to a multiple of 8, stay within `cap` (a single longer
-// segment makes an item of its own).  One thread per tile; `fill` = 0 counts the items,
-// 1 writes (tile, first segment, end segment) for each.
+// the run's first entry rounded down to a multiple of 8, stay within `cap`, and so do those of
+// its units of eight segments (32 entries a step, as many steps as the unit's longest segment has
+// quads); a single longer segment makes an item of its own.  One thread per tile; `fill` = 0
+// counts the items, 1 writes (tile, first segment, end segment) for each.
 __global__ void chunk_kernel(const int32_t *__restrict__ tile_seg_ptr, const int32_t *__restrict__ seg_start,
                              const int32_t *__restrict__ seg_end, int ntiles, int cap, int fill,
                              int32_t *__restrict__ count, const int32_t *__restrict__ offs,
@@ -835,8 +886,13 @@ __global__ void chunk_kernel(const int32_t *__restrict__ tile_seg_ptr, const int
         int n = 0, i = s0;
         while (i < s1) {
             const int e0 = seg_start[i] & ~7;
+            int padded = 8 * (seg_end[i] - seg_start[i]);
             int j = i + 1;
-            while (j < s1 && seg_end[j] - e0 <= cap) ++j;
+            for (; j < s1; ++j) {
+                const int b = seg_end[j], more = ((j - i) & 7) == 0 ? 8 * (b - seg_start[j]) : 0;
+                if (b - e0 > cap || padded + more > cap) break;
+                padded += more;
+            }
             if (fill) {
                 int32_t *c = chunks + 3 * (size_t)(offs[t] + n);
                 c[0] = (int32_t)t; c[1] = i; c[2] = j;
@@ -845,6 +901,79 @@ __global__ void chunk_kernel(const int32_t *__restrict__ tile_seg_ptr, const int
             i = j;
         }
         if (!fill) count[t] = n;
+    }
+}
+
+// Units of every item: steps (most quads of the unit's eight segments), and per item the steps
+// and the record's words.
+__global__ void unit_steps_kernel(const int32_t *__restrict__ chunks, int n_items,
+                                  const int32_t *__restrict__ seg_start, const int32_t *__restrict__ seg_end,
+                                  int32_t *__restrict__ steps, int32_t *__restrict__ words) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; a < n_items;
+         a += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const int s0 = chunks[3 * a + 1], s1 = chunks[3 * a + 2];
+        int tot = 0;
+        for (int b = s0; b < s1; b += 32) {
+            int q = b + lane < s1 ? (seg_end[b + lane] - seg_start[b + lane]) >> 2 : 0;
+            for (int o = 4; o > 0; o >>= 1) q = max(q, __shfl_xor_sync(0xffffffffu, q, o));
+            for (int o = 16; o > 4; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+            tot += q;
+        }
+        if (lane == 0) {
+            steps[a] = tot;
+            words[a] = ((s1 - s0 + 7) / 8 * 10 + 3) & ~3;
+        }
+    }
+}
+
+struct UnitFillArgs {
+    TileGeom Tf;
+    const int32_t *chunks, *seg_start, *seg_end, *seg_slot, *step_off, *rec_off, *pix_in;
+    const float *w_in;
+    int32_t *rec, *desc, *pix;
+    uint16_t *loc;
+    float *w;
+    int n_items;
+};
+
+// Records, descriptors and entries of the items' units, one warp per item.
+__global__ void unit_fill_kernel(UnitFillArgs A) {
+    const int lane = threadIdx.x & 31, k = lane >> 2, j = lane & 3;
+    for (int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; a < A.n_items;
+         a += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const int t = A.chunks[3 * a], s0 = A.chunks[3 * a + 1], ns = A.chunks[3 * a + 2] - s0;
+        const int64_t base = 32 * (int64_t)A.step_off[a];
+        const int off = A.rec_off[a], words = A.rec_off[a + 1] - off, nu = (ns + 7) / 8;
+        int32_t *rec = A.rec + off;
+        int step = 0;
+        for (int u = 0; u < nu; ++u) {
+            const int s = s0 + 8 * u + k;
+            const bool on = 8 * u + k < ns;
+            const int e0 = on ? A.seg_start[s] : 0, len = on ? A.seg_end[s] - e0 : 0;
+            int n = len >> 2;
+            for (int o = 16; o > 2; o >>= 1) n = max(n, __shfl_xor_sync(0xffffffffu, n, o));
+            if (lane == 0) { rec[10 * u] = step; rec[10 * u + 1] = n; }
+            if (j == 0) rec[10 * u + 2 + k] = on ? A.seg_slot[s] : -1;
+            int last = 0;  // the segment's last pixel
+            for (int b = 1; b <= 4 && on; ++b) {
+                const int p = A.pix_in[e0 + len - b];
+                if (p >= 0) { last = (int)tile_loc(A.Tf, p); break; }
+            }
+            for (int q = 0; q < n; ++q) {
+                const int64_t o = base + 32 * (int64_t)(step + q) + lane;
+                const int p = 4 * q < len ? A.pix_in[e0 + 4 * q + j] : -1;
+                A.pix[o] = p;
+                A.w[o] = p >= 0 ? A.w_in[e0 + 4 * q + j] : 0.f;
+                A.loc[o] = (uint16_t)(p >= 0 ? tile_loc(A.Tf, p) : last);
+            }
+            step += n;
+        }
+        for (int i = 10 * nu + lane; i < words; i += 32) rec[i] = 0;
+        if (lane < 8) {
+            const int v[8] = {t, off, words, (int)base, 32 * step, nu, 0, 0};
+            A.desc[8 * a + lane] = v[lane];
+        }
     }
 }
 
@@ -1070,6 +1199,29 @@ int import_csr(az_integrator *h, const int32_t *indptr, const int32_t *indices, 
     return AZ_OK;
 }
 
+int count_runs(const az_integrator *h, int th, int tw, cudaStream_t s, int64_t *out) {
+    *out = -1;
+    TileGeom T{};
+    T.nx = h->nx; T.th = th; T.tw = tw; T.ntx = (h->nx + tw - 1) / tw;
+    const int64_t words = ((int64_t)T.ntx * ((h->ny + th - 1) / th) + 31) / 32;
+    const size_t bytes = sizeof(uint32_t) * (size_t)words * (size_t)h->nrows;
+    if (bytes > ((size_t)1 << 30)) return AZ_OK;
+    DevBuf bits, count;
+    AZ_TRY(bits.alloc(bytes));
+    AZ_TRY(count.alloc(sizeof(unsigned long long)));
+    AZ_CUDA(cudaMemsetAsync(bits.p, 0, bytes, s));
+    AZ_CUDA(cudaMemsetAsync(count.p, 0, count.bytes, s));
+    mark_runs_kernel<<<std::min(h->nrows, num_sms() * 16), 256, 0, s>>>(T, h->csr_ptr.as<int32_t>(), h->csr_idx.as<int32_t>(),
+                                                                      h->nrows, words, bits.as<uint32_t>(),
+                                                                      count.as<unsigned long long>());
+    AZ_CUDA(cudaGetLastError());
+    unsigned long long n = 0;
+    AZ_CUDA(cudaMemcpyAsync(&n, count.p, sizeof(n), cudaMemcpyDeviceToHost, s));
+    AZ_CUDA(cudaStreamSynchronize(s));
+    *out = (int64_t)n;
+    return AZ_OK;
+}
+
 int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     TiledLayout &L = h->tl;
     h->count_ready = false;  // the accumulation order of C depends on the layout
@@ -1086,7 +1238,7 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     if ((int64_t)4 * T.ss + 32 > 65535) return fail(AZ_EINVAL, "tile %dx%d too large", th, tw);
 
     // row of each CSR entry, tile key of each CSR entry, stable sort by tile
-    DevBuf csr_row, tkey, perm;
+    DevBuf csr_row, tkey, perm, seg_of;
     AZ_TRY(csr_row.alloc(sizeof(int32_t) * nnz));
     AZ_TRY(tkey.alloc(sizeof(uint32_t) * nnz));
     AZ_TRY(perm.alloc(sizeof(int32_t) * nnz));
@@ -1099,29 +1251,48 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
         // Within a tile, order the segments (runs of one row) by decreasing length, rows in
         // increasing order among equal lengths; the entries of a segment keep pixel order.
         // Warps that take consecutive segments then get runs of similar length.
-        DevBuf f0, id0, seg0, len0, mx0, key2;
+        // Runs of more than kSegEntries entries are first cut into pieces, so that no segment keeps
+        // the units of its tile waiting (a tile above or below the beam centre has few, long runs:
+        // up to 59 quads in a 16 x 64 tile of the 6-Mpixel detector, 15 on average); where that
+        // makes more than kSegFew segments the pieces are made longer, because the partial sums
+        // of a frame (24 bytes a segment in FP64) have to fit the allocation-free entry point.
+        DevBuf f0, id0, seg0, first0, mx0, key2;
         AZ_TRY(f0.alloc(sizeof(int32_t) * nnz));
         AZ_TRY(id0.alloc(sizeof(int32_t) * (nnz + 1)));
         AZ_TRY(seg0.alloc(sizeof(int32_t) * nnz));
+        AZ_TRY(seg_of.alloc(sizeof(int32_t) * nnz));
+        AZ_TRY(mx0.alloc(sizeof(int32_t)));
         AZ_TRY(launch_gs(seg_flags_kernel, nnz, s, tkey.as<uint32_t>(), perm.as<int32_t>(),
                          csr_row.as<int32_t>(), nnz, f0.as<int32_t>()));
-        AZ_TRY(exclusive_scan_i32(f0.as<int32_t>(), id0.as<int32_t>(), nnz, s));
-        int32_t nseg0 = 0;
-        AZ_CUDA(cudaMemcpyAsync(&nseg0, id0.as<int32_t>() + nnz, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        AZ_CUDA(cudaStreamSynchronize(s));
-        AZ_TRY(launch_gs(seg_index_kernel, nnz, s, f0.as<int32_t>(), id0.as<int32_t>(), nnz,
-                         seg0.as<int32_t>()));
-        AZ_TRY(len0.alloc(sizeof(int32_t) * std::max(nseg0, 1)));
-        AZ_CUDA(cudaMemsetAsync(len0.p, 0, sizeof(int32_t) * std::max(nseg0, 1), s));
-        AZ_TRY(launch_gs(count_keys_kernel, nnz, s, seg0.as<int32_t>(), nnz, len0.as<int32_t>()));
-        AZ_TRY(mx0.alloc(sizeof(int32_t)));
-        max_kernel<<<1, 1024, 0, s>>>(len0.as<int32_t>(), nseg0, mx0.as<int32_t>());
-        AZ_CUDA(cudaGetLastError());
+        auto number = [&](int32_t &count) -> int {  // segments of the flags: their ids and firsts
+            AZ_TRY(exclusive_scan_i32(f0.as<int32_t>(), id0.as<int32_t>(), nnz, s));
+            AZ_CUDA(cudaMemcpyAsync(&count, id0.as<int32_t>() + nnz, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+            AZ_CUDA(cudaStreamSynchronize(s));
+            AZ_TRY(launch_gs(seg_index_kernel, nnz, s, f0.as<int32_t>(), id0.as<int32_t>(), nnz,
+                             seg0.as<int32_t>()));
+            AZ_TRY(first0.alloc(sizeof(int32_t) * (count + 1)));
+            return launch_gs(seg_first_kernel, nnz + 1, s, f0.as<int32_t>(), id0.as<int32_t>(), nnz,
+                             first0.as<int32_t>());
+        };
+        int32_t whole = 0, pieces = 0;
+        AZ_TRY(number(whole));
+        for (int cap = kSegEntries;; cap *= 2) {
+            AZ_TRY(launch_gs(split_flags_kernel, nnz, s, seg0.as<int32_t>(), first0.as<int32_t>(), nnz, cap,
+                             f0.as<int32_t>()));
+            AZ_TRY(number(pieces));
+            if (pieces <= std::max(whole, kSegFew) || cap > (1 << 20)) break;
+            AZ_TRY(launch_gs(seg_flags_kernel, nnz, s, tkey.as<uint32_t>(), perm.as<int32_t>(),
+                             csr_row.as<int32_t>(), nnz, f0.as<int32_t>()));
+            AZ_TRY(number(whole));
+        }
+        AZ_CUDA(cudaMemsetAsync(mx0.p, 0, sizeof(int32_t), s));
+        AZ_TRY(launch_gs(seg_of_kernel, nnz, s, seg0.as<int32_t>(), perm.as<int32_t>(), first0.as<int32_t>(), nnz,
+                         seg_of.as<int32_t>(), mx0.as<int32_t>()));
         int32_t max_len = 0;
         AZ_CUDA(cudaMemcpyAsync(&max_len, mx0.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
         AZ_CUDA(cudaStreamSynchronize(s));
         AZ_TRY(key2.alloc(sizeof(uint32_t) * nnz));
-        AZ_TRY(launch_gs(seg_len_key_kernel, nnz, s, seg0.as<int32_t>(), len0.as<int32_t>(), max_len,
+        AZ_TRY(launch_gs(seg_len_key_kernel, nnz, s, seg0.as<int32_t>(), first0.as<int32_t>(), max_len,
                          nnz, key2.as<uint32_t>()));
         AZ_TRY(stable_sort_pairs(key2.as<uint32_t>(), perm.as<int32_t>(), nnz, bits_for(max_len), s));
         AZ_TRY(launch_gs(tile_keys_perm_kernel, nnz, s, T, h->csr_idx.as<int32_t>(), perm.as<int32_t>(),
@@ -1136,8 +1307,7 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     AZ_TRY(flag.alloc(sizeof(int32_t) * nnz));
     AZ_TRY(segid.alloc(sizeof(int32_t) * (nnz + 1)));
     AZ_TRY(segx.alloc(sizeof(int32_t) * nnz));
-    AZ_TRY(launch_gs(seg_flags_kernel, nnz, s, tkey.as<uint32_t>(), perm.as<int32_t>(),
-                     csr_row.as<int32_t>(), nnz, flag.as<int32_t>()));
+    AZ_TRY(launch_gs(seg_change_kernel, nnz, s, seg_of.as<int32_t>(), perm.as<int32_t>(), nnz, flag.as<int32_t>()));
     AZ_TRY(exclusive_scan_i32(flag.as<int32_t>(), segid.as<int32_t>(), nnz, s));
     int32_t nseg = 0;
     AZ_CUDA(cudaMemcpyAsync(&nseg, segid.as<int32_t>() + nnz, sizeof(int32_t),
@@ -1202,32 +1372,22 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     A.pix = L.ent_pix.as<int32_t>(); A.n = nnz;
     AZ_TRY(launch_gs(tiled_fill_kernel, nnz, s, A));
 
-    // Frame-pair layout: a 3D copy of one row class of frames F and F + 4 writes the two
-    // frames' boxes (th / 4 rows of srow_p words each) back to back, so F + 4 sits slot_p =
-    // (th / 4) srow_p words after F.  slot_p = 16 mod 32 puts the two frames on different
-    // banks; slots of 2 slot_p words keep F's slots 128-byte aligned; boxes are at most 256
-    // words wide.  Tile shapes without such a pitch use the plain layout only.
-    int srow_p = 0, ss_p = 0, slot_p = 0, pw_p = 0;
-    for (int sr = T.srow; sr <= 256 && !srow_p; sr += 4)
-        if (((th / 4) * sr) % 32 == 16) srow_p = sr;
-    if (srow_p) {
-        slot_p = (th / 4) * srow_p;
-        ss_p = 2 * slot_p;
-        pw_p = (4 * ss_p + slot_p + 32 + 31) & ~31;
-        if (pw_p > 65535) srow_p = 0;
+    // Plane layout of the frames kernel: one copy of a row class of D frames writes D times the
+    // tile's th / 4 rows of that class back to back.  A row holds tw pixels after at most 3 + 3
+    // words of phase (the row class's and the frame's); fslot_words is a multiple of 32 words, so
+    // that every plane of a class starts 128-byte aligned; boxes are at most 256 words wide.
+    int srow_f = 0, fslot_words = 0, fslots = 0;
+    for (int sr = tw + 8; sr <= 256 && !srow_f; sr += 4)
+        if (((th / 4) * sr) % 32 == 0) srow_f = sr;
+    if (srow_f && th / 4 <= 256) {
+        fslot_words = (th / 4) * srow_f;
+        // planes per block: eight, fewer when a block of eight takes most of the shared memory
+        for (fslots = 8; fslots > 1; fslots >>= 1)
+            if (4 * (int64_t)fslots * fslot_words <= 65535 &&
+                16 * (int64_t)fslots * fslot_words <= (int64_t)max_smem_per_block() - 2 * 24 * 1024)
+                break;
+        if (4 * (int64_t)fslot_words > 65535) fslots = 0;
     }
-    L.ent_loc_p.release();
-    if (srow_p) {
-        TileGeom Tp = T;
-        Tp.srow = srow_p;
-        Tp.ss = ss_p;
-        AZ_TRY(L.ent_loc_p.alloc(sizeof(uint16_t) * (size_t)padded));
-        AZ_TRY(launch_gs(pair_loc_kernel, padded, s, Tp, L.ent_pix.as<int32_t>(), (int64_t)padded,
-                         L.ent_loc_p.as<uint16_t>()));
-    } else {
-        ss_p = slot_p = pw_p = 0;
-    }
-
     // slots: segments in row order (stable sort of segment ids by row)
     DevBuf skey, sperm, rcnt;
     AZ_TRY(skey.alloc(sizeof(uint32_t) * nseg));
@@ -1245,14 +1405,25 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
 
     // Work items: a tile whose entries would not fit, twice, beside two stages of four frame
     // planes in shared memory is cut at segment boundaries (about 11.5 bytes of shared memory
-    // per entry: location, weight, dark and its share of the record).
+    // per entry: location, weight, dark and its share of the record).  Where the cut still leaves
+    // the average tile whole (with the units' padding, a quarter), it is made for more of the
+    // frames kernel's blocks of planes: the tiles around a beam centre in 2D, whose pixels reach
+    // hundreds of azimuthal bins, would else take the room of every other tile's planes.
     const int64_t plane_bytes = 4 * ((int64_t)4 * T.ss + 32);
-    const int64_t budget = ((int64_t)max_smem_per_block() - 1024 - 2 * (4 * plane_bytes + 256)) / 2;
+    const int64_t room = (int64_t)max_smem_per_block() - 2048;
+    int64_t budget = (room - 2 * (4 * plane_bytes + 256)) / 2;
+    for (int blocks = 4; blocks >= 1 && fslots; --blocks) {
+        const int64_t b = (room - (int64_t)blocks * 16 * fslots * fslot_words) / 2;
+        if (b * 2 / 23 >= (int64_t)padded * 3 / 2 / std::max(ntiles, 1)) {
+            budget = std::min(budget, b);
+            break;
+        }
+    }
     const int kItemEntries = (int)std::max<int64_t>(1024, std::min<int64_t>(60000, budget * 2 / 23) & ~7);
     DevBuf icnt, ioff, chunks, mx;
     AZ_TRY(icnt.alloc(sizeof(int32_t) * ntiles));
     AZ_TRY(ioff.alloc(sizeof(int32_t) * (ntiles + 1)));
-    AZ_TRY(mx.alloc(sizeof(int32_t) * 3));
+    AZ_TRY(mx.alloc(sizeof(int32_t) * 5));
     AZ_TRY(launch_gs(chunk_kernel, ntiles, s, L.tile_seg_ptr.as<int32_t>(), L.seg_ent_ptr.as<int32_t>(),
                      L.seg_ent_ptr.as<int32_t>() + nseg, ntiles, kItemEntries, 0, icnt.as<int32_t>(),
                      (const int32_t *)nullptr, (int32_t *)nullptr));
@@ -1283,13 +1454,56 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
                      L.seg_ent_ptr.as<int32_t>(), L.seg_ent_ptr.as<int32_t>() + nseg,
                      L.seg_slot.as<int32_t>(), roff.as<int32_t>(), L.tile_rec.as<int32_t>(),
                      L.tile_desc.as<int32_t>(), ient.as<int32_t>(), iseg.as<int32_t>()));
+    // the same items in units for the frames kernel
+    DevBuf usteps, uwords, uoff, uroff;
+    int32_t f_steps = 0, f_words = 0;
+    if (fslots) {
+        TileGeom Tf = T;
+        Tf.srow = srow_f;
+        Tf.ss = fslots * fslot_words;
+        AZ_TRY(usteps.alloc(sizeof(int32_t) * std::max(n_items, 1)));
+        AZ_TRY(uwords.alloc(sizeof(int32_t) * std::max(n_items, 1)));
+        AZ_TRY(uoff.alloc(sizeof(int32_t) * (n_items + 1)));
+        AZ_TRY(uroff.alloc(sizeof(int32_t) * (n_items + 1)));
+        AZ_TRY(launch_gs(unit_steps_kernel, 32 * (int64_t)n_items, s, chunks.as<int32_t>(), n_items,
+                         L.seg_ent_ptr.as<int32_t>(), L.seg_ent_ptr.as<int32_t>() + nseg, usteps.as<int32_t>(),
+                         uwords.as<int32_t>()));
+        AZ_TRY(exclusive_scan_i32(usteps.as<int32_t>(), uoff.as<int32_t>(), n_items, s));
+        AZ_TRY(exclusive_scan_i32(uwords.as<int32_t>(), uroff.as<int32_t>(), n_items, s));
+        AZ_CUDA(cudaMemcpyAsync(&f_steps, uoff.as<int32_t>() + n_items, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+        AZ_CUDA(cudaMemcpyAsync(&f_words, uroff.as<int32_t>() + n_items, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+        AZ_CUDA(cudaStreamSynchronize(s));
+        if ((int64_t)f_steps * 32 > INT32_MAX) fslots = 0;
+    }
+    L.f_entries = fslots ? 32 * (int64_t)f_steps : 0;
+    L.f_desc.release(); L.f_rec.release(); L.f_loc.release(); L.f_w32.release(); L.f_pix.release();
+    if (fslots) {
+        AZ_TRY(L.f_desc.alloc(sizeof(int32_t) * 8 * (size_t)std::max(n_items, 1)));
+        AZ_TRY(L.f_rec.alloc(sizeof(int32_t) * (size_t)std::max(f_words, 4)));
+        AZ_TRY(L.f_loc.alloc(sizeof(uint16_t) * (size_t)L.f_entries));
+        AZ_TRY(L.f_w32.alloc(sizeof(float) * (size_t)L.f_entries));
+        AZ_TRY(L.f_pix.alloc(sizeof(int32_t) * (size_t)L.f_entries));
+        UnitFillArgs U;
+        U.Tf = T; U.Tf.srow = srow_f; U.Tf.ss = fslots * fslot_words;
+        U.chunks = chunks.as<int32_t>(); U.seg_start = L.seg_ent_ptr.as<int32_t>();
+        U.seg_end = L.seg_ent_ptr.as<int32_t>() + nseg; U.seg_slot = L.seg_slot.as<int32_t>();
+        U.step_off = uoff.as<int32_t>(); U.rec_off = uroff.as<int32_t>(); U.pix_in = L.ent_pix.as<int32_t>();
+        U.w_in = L.ent_w32.as<float>(); U.rec = L.f_rec.as<int32_t>(); U.desc = L.f_desc.as<int32_t>();
+        U.pix = L.f_pix.as<int32_t>(); U.loc = L.f_loc.as<uint16_t>(); U.w = L.f_w32.as<float>();
+        U.n_items = n_items;
+        AZ_TRY(launch_gs(unit_fill_kernel, 32 * (int64_t)n_items, s, U));
+        max_kernel<<<1, 1024, 0, s>>>(usteps.as<int32_t>(), n_items, mx.as<int32_t>() + 3);
+        AZ_CUDA(cudaGetLastError());
+        max_kernel<<<1, 1024, 0, s>>>(uwords.as<int32_t>(), n_items, mx.as<int32_t>() + 4);
+        AZ_CUDA(cudaGetLastError());
+    }
     max_kernel<<<1, 1024, 0, s>>>(ient.as<int32_t>(), n_items, mx.as<int32_t>());
     AZ_CUDA(cudaGetLastError());
     max_kernel<<<1, 1024, 0, s>>>(iseg.as<int32_t>(), n_items, mx.as<int32_t>() + 1);
     AZ_CUDA(cudaGetLastError());
     max_kernel<<<1, 1024, 0, s>>>(rwords.as<int32_t>(), n_items, mx.as<int32_t>() + 2);
     AZ_CUDA(cudaGetLastError());
-    int32_t maxes[3];
+    int32_t maxes[5] = {};
     AZ_CUDA(cudaMemcpyAsync(maxes, mx.p, sizeof(maxes), cudaMemcpyDeviceToHost, s));
     AZ_CUDA(cudaStreamSynchronize(s));
     if (maxes[0] > 65535)
@@ -1305,10 +1519,12 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     const int32_t max_rec = maxes[2];
 
     L.th = th; L.tw = tw; L.srow = T.srow; L.ss = T.ss; L.ntx = T.ntx; L.nty = nty; L.ntiles = ntiles;
-    L.srow_p = srow_p; L.ss_p = ss_p; L.slot_p = slot_p; L.pw_p = pw_p;
+    L.srow_f = srow_f; L.fslot_words = fslot_words; L.fslots = fslots;
     L.n_active = n_active; L.nseg = nseg; L.padded_nnz = padded;
     L.max_tile_entries = maxes[0]; L.max_tile_segments = maxes[1];
     L.max_rec_words = max_rec;
+    L.f_max_entries = fslots ? 32 * maxes[3] : 0;
+    L.f_max_rec = fslots ? maxes[4] : 0;
     return AZ_OK;
 }
 

@@ -3,10 +3,11 @@
 //
 //   frames_kernel (persistent, one CTA per SM): a work item is a pixel tile (or a piece of
 //     a heavy one) for every frame of the launch.  One producer warp copies the item's
-//     record and entries (location, weight, per-entry dark) once into a ring of entry
+//     units and entries (location, weight, per-entry dark) once into a ring of entry
 //     buffers and streams the tile's pixels, G frames at a time, into a ring of plane stages
-//     (bulk and tensor TMA, mbarrier-tracked, every wait bounded); 15 consumer warps give
-//     lanes (segment, frame) pairs and write one partial sum per (segment, frame).  It serves
+//     (bulk and tensor TMA, mbarrier-tracked, every wait bounded); 15 consumer warps take
+//     units of eight segments, four lanes a segment and G frames a lane, and write one partial
+//     sum per (segment, frame).  It serves
 //     batches, the frame-independent sums N and C, the propagated variance, the per-pixel-
 //     corrected form and single FP32 frames (after single_planes_kernel forms the corrected
 //     frame and its normalisation per pixel).
@@ -140,27 +141,10 @@ __device__ __forceinline__ TileDesc load_desc(const Inst &d, int64_t local) {
 constexpr uint32_t kZeroBand = 32;
 __host__ __device__ __forceinline__ uint32_t plane_stride(int ss) { return 4u * (uint32_t)ss + kZeroBand; }
 
-// Zero words band_from .. pw - 1 of every plane of every stage (never written by the copies):
-// the band after a plane, or in the frame-pair layout the tail of a region that holds both
-// frames' bands.
-__device__ __forceinline__ void zero_bands(unsigned char *first_plane, uint32_t stage_bytes, int nstages,
-                                           int planes, uint32_t pw, uint32_t band_from) {
-    const int band = (int)(pw - band_from);
-    const int per_stage = planes * band;
-    for (int i = threadIdx.x; i < nstages * per_stage; i += blockDim.x) {
-        const int st = i / per_stage, r = i - st * per_stage;
-        const int pl = r / band, w = r - pl * band;
-        reinterpret_cast<uint32_t *>(first_plane + (size_t)st * stage_bytes)[(size_t)pl * pw + band_from + w] = 0u;
-    }
-}
-
 // Four 2D tensor maps per staged array, one per tile-row class (rows of equal index mod 4,
 // 16 * nx bytes apart).  Index: 0 image, 1 dark, 2 flat, 3 solid angle, 4 polarisation.
-// pair: the image's four class maps in three dimensions (x, class row, period of four
-// frames) for the frame-pair layout of the frames kernel.
 struct TmaSet {
     CUtensorMap m[5][4];
-    CUtensorMap pair[4];
 };
 
 // Stage layout: [header 256 B][tile record][planes][entry locs][entry weights].
@@ -722,36 +706,59 @@ phase1_kernel(const __grid_constant__ Inst single, const Inst *__restrict__ mult
 // ------------------------------------------------------------------------------------
 // frames pass with tile-resident entries
 // ------------------------------------------------------------------------------------
-// The batched frames pass spends most of its bytes on pixels, so a work item is one pixel
-// tile for every frame of the launch: the tile's record and entries (location, weight,
-// dark) are copied once into one of two entry buffers and stay there while the tile's
-// pixels stream through a ring of plane stages, G frames per stage.  One producer warp
-// issues every copy (bulk and tensor TMA); 15 consumer warps reduce (16 warps in all, four
-// per scheduler: with 16 consumers the 64-frame Pilatus pass took 2.5% longer, with 20 or
-// 24 longer still).  The consumer
-// arithmetic is exactly that of the frames mode of phase1_kernel: the same entry order,
-// accumulator assignment and merge, so results do not depend on the kernel that made them.
+// The batched frames pass spends most of its bytes on pixels, so a work item is one pixel tile (or a
+// piece of a heavy one) for every frame of the launch: the item's units and entries (location,
+// weight, dark) are copied once into one of two or more entry buffers and stay there while the
+// tile's pixels stream through a ring of plane stages, G frames per stage.  One producer warp
+// issues every copy (bulk and tensor TMA); 15 consumer warps reduce.
+//
+// What bounds it (64 frames of 2527 x 2463 pixels, 9.63 M entries): staging alone runs at the
+// copy peak (246 us a launch), the consumers alone take 320 us, both together 340 us; the kernel
+// before this one took 468 us.  The consumers are held by shared memory (38 wavefronts per 256
+// products, half of them bank conflicts of the gathers) and by the FP32 pipe, which a packed
+// f32x2 instruction occupies for two cycles (1.45 us of pipe time per frame).  Why this form:
+//   - a lane sums one accumulator of one segment for all frames of a stage, so a unit of eight
+//     segments reads each entry once for eight frames: 7 words of metadata and 16 gathers per 256
+//     products.  One lane per (segment, frame) read 40 bytes of metadata per quad and frame group
+//     (18 wavefronts per 128 products); four frames per lane measured 12% slower than eight.
+//   - a box of depth D moves one row class of D frames: four copies per 8-frame stage instead of
+//     sixteen, which takes the issue of the copies off the critical path.
+//   - consumers take units from one counter across stages and items instead of passing every
+//     stage together, so nobody waits for the slowest warp of a stage (11 to 15 consumer warps
+//     are within 2%, 23 are 5% slower).
+//   - f32x2 has no subtraction: sub.rn.f32x2 costs two more instructions, a multiply-add by -1
+//     does not.
 constexpr int kFrConsumers = 15;
 constexpr int kFrThreads = 32 * (1 + kFrConsumers);
-constexpr int kFrMaxStages = 8;
+constexpr int kFrMaxStages = 16;
 constexpr int kFrMaxEbufs = 6;
+constexpr int kUnitWords = 10;           // a unit in the item's record: first step, steps, 8 slots
+constexpr uint32_t kFrUnits = 1u << 19;  // arrivals that complete a stage's release barrier
 // What the frames kernel sums per entry: w (img), w (img - dark), or w^2 max(img, 0) (the
 // propagated Poisson variance of the signal sum).
 enum ValueMode { VM_PLAIN = 0, VM_DARK = 1, VM_VAR = 2 };
-constexpr uint32_t kFrStageHeader = 128;  // per plane stage: nimg, group, G plane offsets
+
+// Three-dimensional maps of the frames: [q][c] covers the rows of equal index c mod 4 of the
+// frames f = q mod 4, in (x, class row, frame / 4).  Rows of a class are 16 nx bytes apart and
+// frames four apart 16 npix bytes, so any width and height meets the 16-byte stride rule, and a
+// box of depth D copies one class of a tile's rows from D frames.
+struct FrMaps {
+    CUtensorMap m[4][4];
+};
 
 struct FrArgs {
-    const char *img;                      // first frame of this launch
-    int n_frames, n_groups, n_tiles;      // frames in the launch, groups of G, active tiles
-    const int32_t *tile_desc, *tile_rec;  // per active tile: descriptor [8] and record
+    int n_frames, n_groups, n_tiles;      // frames in the launch, stages per item, items
+    int nq, ld, nd;                       // a stage: nq values of q, D = 2^ld frames of each; nd
+                                          // stages cover the frames of one q
+    const int32_t *desc, *rec;            // per item: descriptor [8] and its units
     const uint16_t *ent_loc;
     const float *ent_w, *ent_dark;        // ent_dark: NULL without a dark
     float *partial;                       // [n_frames][nseg]
-    int nseg, ny, nx, th, tw, srow, ss, ntx;
+    int nseg, ny, nx, th, tw, ntx;
+    int slot, cstride;                    // words: rows of a class, class stride
+    int beta, fphase;                     // word phase of frame 0, and npix mod 4 (a frame's step)
     int *status;
     int var;                              // sum w^2 max(img, 0) instead of w img
-    int pair;                             // frame-pair layout (8 frames per stage, whole stages)
-    int slot;                             // its offset of frame F + 4 from frame F (words)
 };
 
 struct FrGeom {
@@ -759,15 +766,14 @@ struct FrGeom {
     uint32_t ent_cap;       // entry capacity (multiple of 8)
     uint32_t ebuf_bytes;    // one entry buffer (multiple of 128)
     int nebufs;             // entry buffers in the ring (2 .. kFrMaxEbufs)
-    uint32_t plane_words;   // words per plane (frame-pair layout: per region of two frames)
-    uint32_t band_from;     // first word of a plane's zero band
-    uint32_t pstage_bytes;  // one plane stage: G planes (G / 2 regions)
-    int nstages;            // plane stages
+    uint32_t block_bytes;   // plane ring block: fslots planes
+    int spb;                // stages per block (fslots / G)
+    int nblocks, nstages;   // blocks and plane stages of the ring
     int dk;                 // entries carry a dark
 };
 
 __device__ __forceinline__ TileDesc fr_desc(const FrArgs &a, int item) {
-    const int4 *p = reinterpret_cast<const int4 *>(a.tile_desc) + 2 * (size_t)item;
+    const int4 *p = reinterpret_cast<const int4 *>(a.desc) + 2 * (size_t)item;
     const int4 x = __ldg(p), y = __ldg(p + 1);
     return TileDesc{x.x, x.y, x.z, x.w, y.x, y.y};
 }
@@ -779,7 +785,7 @@ __device__ __forceinline__ void fr_stage_entries(const FrArgs &a, const FrGeom &
     const uint32_t bytes = (uint32_t)td.rec_words * 4u + ne * (fg.dk ? 10u : 6u);
     fence_proxy_async_smem();
     mbar_arrive_expect_tx(bar, bytes);
-    bulk_g2s(eb, a.tile_rec + td.rec_off, (uint32_t)td.rec_words * 4u, bar);
+    bulk_g2s(eb, a.rec + td.rec_off, (uint32_t)td.rec_words * 4u, bar);
     if (ne) {
         unsigned char *el = eb + fg.rec_cap;
         unsigned char *ew = el + fg.ent_cap * 2u;
@@ -789,163 +795,44 @@ __device__ __forceinline__ void fr_stage_entries(const FrArgs &a, const FrGeom &
     }
 }
 
-// The producer warp in the frame-pair layout (a whole stage of 8 frames): frames q and q + 4
-// (q < 4) share region q of the stage, and one 3D tensor copy per (q, row class) moves that
-// class of both frames -- periods m and m + 1 of the pair maps, m = (f0 + q) / 4 -- so a
-// stage takes 16 copies.  Frame q's box starts 4 s_q words early as in fr_stage_planes (s_q =
-// (q / P) mod 4 for the phase period P of the first four frames); frame q + 4, whose rows are
-// 4 ny rows later, has frame q's word phase and shift, and its plane is a.slot words after
-// frame q's.  Lane 0 then publishes the stage header and resets the stage's claim counter.
-__device__ __forceinline__ void fr_stage_pairs(const FrArgs &a, const TmaSet &tm, const TileDesc &td, int g,
-                                               uint32_t *planes, int *hdr, const FrGeom &fg, uint64_t *bar,
-                                               int *ctr) {
+// The producer warp: stage g of an item into the planes at `dst`.  Stage g holds, for nq values
+// of q from q0 on, the D frames q + 4 (D db + d), d < D; lane (qi, c) copies row class c of the D
+// frames of q0 + qi with one 3D tensor copy (frames after the last are filled with zeros, and
+// never reduced).  Plane i = qi D + d sits i a.slot words into each class's stretch of a.cstride
+// words.  Class c's box starts at the 16-byte aligned column that puts pixel (ly, c0 + lx) at
+// word c_s + phi + lx of its row for every class, c_s = (nx c) mod 4 (part of the entries'
+// locations) and phi the word phase of the frame.
+__device__ __forceinline__ void fr_stage_planes(const FrArgs &a, const FrMaps &fm, const TileDesc &td, int g,
+                                                uint32_t dst, uint64_t *bar) {
     const int lane = threadIdx.x & 31;
-    const int f0 = g * 8;
-    if (a.n_frames - f0 < 8) {
-        // a partial stage (the host launches whole stages only): no frames, an error status
-        if (lane == 0) {
-            atomicExch(a.status, AZ_EINVAL);
-            hdr[0] = 0;
-            hdr[1] = g;
-            *ctr = 0;
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar);
-        return;
-    }
     const int ti = td.t / a.ntx, tj = td.t - ti * a.ntx;
-    const int r0 = ti * a.th, c0 = tj * a.tw;
-    const int nu = a.nx & 3;
-    const int rows4 = a.th >> 2;
-    const uint32_t pw = fg.plane_words;
-    const int beta = (int)((reinterpret_cast<uintptr_t>(a.img) >> 2) & 3u);
-    const int c = (nu * (a.ny & 3)) & 3;
-    const int lp = c == 0 ? 0 : (c == 2 ? 1 : 2);  // log2 of the phase period P
-    const int q = (lane >> 2) & 3, k = lane & 3;     // lanes 0..15: (frame q, class k)
-    const int phi_row = (int)(((int64_t)(f0 + q) * a.ny + r0) & 3);
-    const int phi = (beta + nu * phi_row) & 3;
-    const int sq = (q >> lp) & 3;
+    const int c0 = tj * a.tw;
+    const int qg = g / a.nd, db = g - qg * a.nd;
+    const int qi = lane >> 2, c = lane & 3, q = qg * a.nq + qi;
+    const int d0 = db << a.ld;                       // first frame of q in this stage: q + 4 d0
+    const bool on = qi < a.nq && q + 4 * d0 < a.n_frames && c < a.ny;
+    const uint32_t box = (uint32_t)(a.slot << a.ld) * 4u;
+    const uint32_t n = (uint32_t)__popc(__ballot_sync(0xffffffffu, on));
     fence_proxy_async_smem();
-    if (lane == 0)
-        asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)),
-                     "r"((uint32_t)(16 * a.srow * rows4 * 2 * 4))
-                     : "memory");
+    if (lane == 0) mbar_arrive_expect_tx(bar, n * box);
     __syncwarp();
-    if (lane < 16) {
-        const int sl = (k - phi_row) & 3;
-        const int offk = (beta + k * nu) & 3;
-        const int flag = (((nu * sl) & 3) + phi - offk) >> 2;
-        const int x = c0 - 4 * (flag + sq);
-        const int y = (q * a.ny + r0 + sl - k) >> 2;  // class row within the period (exact)
-        const int m = (f0 + q) >> 2;
+    if (on) {
+        const int phi = (a.beta + q * a.fphase) & 3, cs = ((a.nx & 3) * c) & 3;
+        const int x = c0 - ((phi + cs) & 4);
+        const uint32_t to = dst + (uint32_t)(c * a.cstride + (qi << a.ld) * a.slot) * 4u;
         asm volatile(
             "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-            " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_addr(planes + (size_t)q * pw + (size_t)sl * a.ss)),
-            "l"(reinterpret_cast<uint64_t>(&tm.pair[k])), "r"(x), "r"(y), "r"(m), "r"(smem_addr(bar))
+            " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(to),
+            "l"(reinterpret_cast<uint64_t>(&fm.m[q][c])), "r"(x), "r"(ti * (a.th >> 2)), "r"(d0), "r"(smem_addr(bar))
             : "memory");
     }
-    if (lane < 8) {
-        const int qa = lane & 3;
-        const int pha = (beta + nu * (int)(((int64_t)(f0 + qa) * a.ny + r0) & 3)) & 3;
-        hdr[2 + lane] = (int)(qa * pw) + (lane >> 2) * a.slot + pha + 4 * ((qa >> lp) & 3);
-    }
-    if (lane == 0) {
-        hdr[0] = 8;
-        hdr[1] = g;
-        *ctr = 0;
-    }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(bar);  // publishes the header and the counter
-}
-
-// The producer warp: frames f0 .. f0 + nimg - 1 of the tile into plane stage `planes`, one
-// tensor copy per (frame, row class), as in produce(); G <= 16, so a lane has at most two
-// copies.  Frame q's box starts 4 * s_q words early, s_q = (number of earlier frames of the
-// group whose rows have the same word phase) mod 4, so that the frames of a group fall on
-// different shared-memory banks for as many frames as the phases and shifts allow.  Lane 0
-// then publishes the stage header and resets the stage's claim counter.
-template <int G>
-__device__ __forceinline__ void fr_stage_planes(const FrArgs &a, const TmaSet &tm, const TileDesc &td,
-                                                int g, uint32_t *planes, int *hdr, const FrGeom &fg,
-                                                uint64_t *bar, int *ctr) {
-    static_assert(G >= 1 && G <= 16, "a plane stage holds at most 16 frames");
-    if constexpr (G == 8) {
-        if (a.pair) {
-            fr_stage_pairs(a, tm, td, g, planes, hdr, fg, bar, ctr);
-            return;
-        }
-    }
-    const int lane = threadIdx.x & 31;
-    const int ti = td.t / a.ntx, tj = td.t - ti * a.ntx;
-    const int r0 = ti * a.th, c0 = tj * a.tw;
-    const int f0 = g * G;
-    const int nimg = min(G, a.n_frames - f0);
-    const int nu = a.nx & 3;
-    const int rows4 = a.th >> 2;
-    const int64_t rows_total = (int64_t)a.n_frames * a.ny;
-    const uint32_t pw = fg.plane_words;
-    const int beta = (int)((reinterpret_cast<uintptr_t>(a.img) >> 2) & 3u);
-    // lane q < nimg: word phase of frame q's tile rows and its shift (earlier frames of the
-    // group with the same phase, mod 4)
-    const int64_t gl = (int64_t)(f0 + lane) * a.ny + r0;
-    const int ph = (beta + nu * (int)(gl & 3)) & 3;
-    const unsigned same = __match_any_sync(0xffffffffu, lane < nimg ? ph : 4 + lane);
-    const int sh = __popc(same & ((1u << lane) - 1u)) & 3;
-    // a lane's jobs are (frame, class) = (lane / 4, lane % 4) and (8 + lane / 4, lane % 4)
-    const int shj[2] = {__shfl_sync(0xffffffffu, sh, lane >> 2), __shfl_sync(0xffffffffu, sh, 8 + (lane >> 2))};
-    uint32_t mine = 0;
-#pragma unroll
-    for (int h2 = 0; h2 < 2; ++h2) {
-        const int job = lane + 32 * h2;
-        if (job >= 4 * nimg) break;
-        const int q = job >> 2, k = job & 3;
-        const int64_t g0 = (int64_t)(f0 + q) * a.ny + r0;
-        const int sl = (k - (int)(g0 & 3)) & 3;
-        if (g0 + sl < rows_total) mine += (uint32_t)(a.srow * rows4 * 4);
-    }
-    fence_proxy_async_smem();
-    if (mine)
-        asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)),
-                     "r"(mine)
-                     : "memory");
-#pragma unroll
-    for (int h2 = 0; h2 < 2; ++h2) {
-        const int job = lane + 32 * h2;
-        if (job >= 4 * nimg) break;
-        const int q = job >> 2, k = job & 3;
-        const int64_t g0 = (int64_t)(f0 + q) * a.ny + r0;
-        const int phi_row = (int)(g0 & 3);
-        const int sl = (k - phi_row) & 3;
-        if (g0 + sl >= rows_total) continue;
-        const int phi = (beta + nu * phi_row) & 3;
-        const int offk = (beta + k * nu) & 3;
-        const int cs = (nu * sl) & 3;
-        const int flag = (cs + phi - offk) >> 2;
-        const int x = c0 - 4 * (flag + shj[h2]);
-        uint32_t *dst = planes + (size_t)q * pw + (size_t)sl * a.ss;
-        const int y = (int)((g0 + sl - k) >> 2);
-        const CUtensorMap *map = &tm.m[0][k];
-        asm volatile(
-            "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-            " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_addr(dst)),
-            "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_addr(bar))
-            : "memory");
-    }
-    if (lane < nimg) hdr[2 + lane] = (int)(lane * pw) + ph + 4 * sh;
-    if (lane == 0) {
-        hdr[0] = nimg;
-        hdr[1] = g;
-        *ctr = 0;
-    }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(bar);  // publishes the header and the counter
 }
 
 // Load of a 4-byte word of shared memory at a 32-bit shared-window address (the gathers of
 // the consumers index the staged planes with 32-bit arithmetic).
 __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
     uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
     return v;
 }
 
@@ -965,20 +852,14 @@ __device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
-__device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 __device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
     f32x2 r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
+}
+// a - b as b (-1) + a: the same single rounding of the same exact value.
+__device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b) {
+    return f2_fma(b, 0xbf800000bf800000ull, a);
 }
 // Two Kahan accumulators stepped together: the same operations as kahan_add on each half.
 __device__ __forceinline__ void kahan2_add(f32x2 &s, f32x2 &nc, f32x2 w, f32x2 v) {
@@ -987,248 +868,315 @@ __device__ __forceinline__ void kahan2_add(f32x2 &s, f32x2 &nc, f32x2 w, f32x2 v
     nc = f2_sub(y, f2_sub(t, s));
     s = t;
 }
-
-// Consumer warps: lane (sub, q) reduces segment b + sub for frame q of the stage, with the
-// entry stream of the tile's entry buffer, exactly as consume_serial does in frames mode (same
-// entry order, accumulator assignment and merge); accumulators (0, 1) and (2, 3) are stepped
-// as packed f32x2 pairs.
-template <int G, int DT, int VM>
-__device__ __forceinline__ void fr_consume(const FrArgs &a, const FrGeom &fg, const unsigned char *eb,
-                                           const uint32_t *planes, const int *hdr, int *ctr) {
-    constexpr int R = 32 / G;
-    const int lane = threadIdx.x & 31;
-    const int sub = lane / G, q = lane % G;
-    const int *rec = reinterpret_cast<const int *>(eb);
-    const int ns = rec[1];
-    const int *slots = rec + 4;
-    const uint16_t *starts = reinterpret_cast<const uint16_t *>(slots + ns);
-    const uint16_t *L = reinterpret_cast<const uint16_t *>(eb + fg.rec_cap);
-    const float *W = reinterpret_cast<const float *>(eb + fg.rec_cap + fg.ent_cap * 2u);
-    const float *D = W + fg.ent_cap;
-    const int nimg = hdr[0], g = hdr[1];
-    const bool active = q < nimg;
-    const uint32_t P = smem_addr(planes + hdr[2 + (active ? q : 0)]);
-    float *out = a.partial + (size_t)(g * G + q) * (size_t)a.nseg;
-    while (true) {
-        int b = 0;
-        if (lane == 0) b = atomicAdd(ctr, R);
-        b = __shfl_sync(0xffffffffu, b, 0);
-        if (b >= ns) break;
-        const int sl = b + sub;
-        int e0 = 0, e1 = 0, slot = 0;
-        if (sl < ns) {
-            e0 = starts[sl];
-            e1 = starts[sl + 1];
-            slot = slots[sl];
-        }
-        if (!active) e1 = e0;
-        // Segments start on a quad and hold whole quads (padding entries add w = 0 times 0).
-        f32x2 s01 = 0ull, n01 = 0ull, s23 = 0ull, n23 = 0ull;
-        for (int qd = e0; qd < e1; qd += 4) {
-            const uint2 l2 = *reinterpret_cast<const uint2 *>(L + qd);
-            const float4 w4 = *reinterpret_cast<const float4 *>(W + qd);
-            float v[4];
-            v[0] = img_f32<DT>(lds_u32(P + ((l2.x & 0xffffu) << 2)));
-            v[1] = img_f32<DT>(lds_u32(P + ((l2.x >> 16) << 2)));
-            v[2] = img_f32<DT>(lds_u32(P + ((l2.y & 0xffffu) << 2)));
-            v[3] = img_f32<DT>(lds_u32(P + ((l2.y >> 16) << 2)));
-            if (VM == VM_VAR) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) v[j] = fmaxf(v[j], 0.f);
-            }
-            f32x2 v01 = f2_pack(v[0], v[1]), v23 = f2_pack(v[2], v[3]);
-            if (VM == VM_DARK) {
-                const float4 d4 = *reinterpret_cast<const float4 *>(D + qd);
-                v01 = f2_sub(v01, f2_pack(d4.x, d4.y));
-                v23 = f2_sub(v23, f2_pack(d4.z, d4.w));
-            }
-            f32x2 w01 = f2_pack(w4.x, w4.y), w23 = f2_pack(w4.z, w4.w);
-            if (VM == VM_VAR) {
-                w01 = f2_mul(w01, w01);
-                w23 = f2_mul(w23, w23);
-            }
-            kahan2_add(s01, n01, w01, v01);
-            kahan2_add(s23, n23, w23, v23);
-        }
-        Kahan k[4];
-        f2_unpack(s01, k[0].s, k[1].s);
-        f2_unpack(n01, k[0].nc, k[1].nc);
-        f2_unpack(s23, k[2].s, k[3].s);
-        f2_unpack(n23, k[2].nc, k[3].nc);
-        kahan_merge(k[0], k[1]);
-        kahan_merge(k[2], k[3]);
-        kahan_merge(k[0], k[2]);
-        if (sl < ns && active) out[slot] = kahan_value(k[0]);
-    }
+// ... and merged: kahan_merge on each half.
+__device__ __forceinline__ void kahan2_merge(f32x2 &as, f32x2 &an, f32x2 bs, f32x2 bn) {
+    const f32x2 t = f2_add(as, bs);
+    const f32x2 z = f2_sub(t, as);
+    const f32x2 e = f2_add(f2_sub(as, f2_sub(t, z)), f2_sub(bs, z));
+    an = f2_add(f2_add(an, bn), e);
+    as = t;
 }
 
-// One or two frames per stage: a warp would take 32 or 16 segments at once and run each
-// segment's whole entry stream on one lane, while a tile has only some tens of segments.  Here
-// four lanes share a (segment, frame): lane j keeps accumulator j (the entries e = j mod 4 of
-// every quad, in order, exactly as one lane of fr_consume steps its accumulator j), and the
-// four are merged by shuffles as ((a0 + a1) + (a2 + a3)), the merge of fr_consume.  Same
-// operations on the same values, so the same bits, with a quarter of the chain per lane and
-// 8 / G segments per claim.
+// One unit of work of a consumer warp: eight segments of the tile for the G frames of a stage.
+// Four lanes share a segment: lane j keeps accumulator j, i.e. the entries e = j mod 4 in order,
+// for all G frames at once (stepped as packed f32x2 pairs), so that an entry's location, weight
+// and dark are read from shared memory once for G frames.  The unit's entries are stored step by
+// step, 32 to a step in lane order (a lane whose segment has ended gets weight 0 and the
+// segment's last pixel), so these reads touch no bank twice and the loop has no branches.  The
+// four accumulators are then merged as ((a0 + a1) + (a2 + a3)) by exchanges that halve the frames
+// a lane keeps (a merge gives the same bits in either order: its rounding error is formed
+// exactly).  Each value is formed by the operations of consume_serial in the same order, so a
+// frame's sums do not depend on the kernel or on the frames it shares a stage with.
+// unit: first step, steps, the segments' eight slots (-1: none).
+// tab: of the stage's frames, the offset (bytes) of plane i from the stage's first word, and
+// the frame's row of the partial sums (-1: past the last frame).
 template <int G, int DT, int VM>
-__device__ __forceinline__ void fr_consume_split(const FrArgs &a, const FrGeom &fg, const unsigned char *eb,
-                                                 const uint32_t *planes, const int *hdr, int *ctr) {
-    static_assert(G == 1 || G == 2, "split consumer is for one or two frames per stage");
-    constexpr int R = 8 / G;
+__device__ __forceinline__ void fr_unit(const FrArgs &a, const FrGeom &fg, const unsigned char *eb, uint32_t planes,
+                                        const int2 *tab, int u) {
+    static_assert(G == 1 || G == 2 || G == 4 || G == 8, "frames per stage");
+    constexpr int H = G > 1 ? G / 2 : 1;
     const int lane = threadIdx.x & 31;
-    const int j = lane & 3, q = (lane >> 2) % G, sub = lane / (4 * G);
-    const int *rec = reinterpret_cast<const int *>(eb);
-    const int ns = rec[1];
-    const int *slots = rec + 4;
-    const uint16_t *starts = reinterpret_cast<const uint16_t *>(slots + ns);
-    const uint16_t *L = reinterpret_cast<const uint16_t *>(eb + fg.rec_cap);
-    const float *W = reinterpret_cast<const float *>(eb + fg.rec_cap + fg.ent_cap * 2u);
+    const int j = lane & 3;
+    const int *unit = reinterpret_cast<const int *>(eb) + kUnitWords * u;
+    const int n = unit[1], slot = unit[2 + (lane >> 2)];
+    const int e0 = unit[0] * 32 + lane;
+    const uint16_t *L = reinterpret_cast<const uint16_t *>(eb + fg.rec_cap) + e0;
+    const float *W = reinterpret_cast<const float *>(eb + fg.rec_cap + fg.ent_cap * 2u) + e0;
     const float *D = W + fg.ent_cap;
-    const int nimg = hdr[0], g = hdr[1];
-    const bool active = q < nimg;
-    const uint32_t P = smem_addr(planes + hdr[2 + (active ? q : 0)]);
-    float *out = a.partial + (size_t)(g * G + q) * (size_t)a.nseg;
-    while (true) {
-        int b = 0;
-        if (lane == 0) b = atomicAdd(ctr, R);
-        b = __shfl_sync(0xffffffffu, b, 0);
-        if (b >= ns) break;
-        const int sl = b + sub;
-        int e0 = 0, e1 = 0, slot = 0;
-        if (sl < ns) {
-            e0 = starts[sl];
-            e1 = starts[sl + 1];
-            slot = slots[sl];
+    uint32_t P[G];
+#pragma unroll
+    for (int i = 0; i < G; ++i) P[i] = planes + (uint32_t)tab[i].x;
+    f32x2 s[H], c[H];
+    Kahan k0{0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < H; ++i) s[i] = c[i] = 0ull;
+#pragma unroll 4
+    for (int t = 0; t < n; ++t) {
+        const uint32_t o = (uint32_t)L[32 * t] << 2;
+        float w = W[32 * t];
+        float d = 0.f;
+        if (VM == VM_DARK) d = D[32 * t];
+        if (VM == VM_VAR) w = __fmul_rn(w, w);
+        float v[G];
+#pragma unroll
+        for (int i = 0; i < G; ++i) v[i] = img_f32<DT>(lds_u32(P[i] + o));
+        if (VM == VM_VAR) {
+#pragma unroll
+            for (int i = 0; i < G; ++i) v[i] = fmaxf(v[i], 0.f);
         }
-        if (!active) e1 = e0;
-        Kahan k{0.f, 0.f};
-        for (int e = e0 + j; e < e1; e += 4) {
-            float v = img_f32<DT>(lds_u32(P + ((uint32_t)L[e] << 2)));
-            float w = W[e];
-            if (VM == VM_VAR) {
-                v = fmaxf(v, 0.f);
-                w = __fmul_rn(w, w);
+        if constexpr (G == 1) {
+            if (VM == VM_DARK) v[0] = __fsub_rn(v[0], d);
+            kahan_add(k0, w, v[0]);
+        } else {
+            const f32x2 w2 = f2_pack(w, w), d2 = f2_pack(d, d);
+#pragma unroll
+            for (int i = 0; i < H; ++i) {
+                f32x2 x = f2_pack(v[2 * i], v[2 * i + 1]);
+                if (VM == VM_DARK) x = f2_sub(x, d2);
+                kahan2_add(s[i], c[i], w2, x);
             }
-            if (VM == VM_DARK) v = __fsub_rn(v, D[e]);
-            kahan_add(k, w, v);
         }
-        // lanes j = 0, 2 take (a0 + a1), (a2 + a3); lane 0 then adds the second to the first
-        Kahan o = shfl_xor(k, 1);
-        kahan_merge(k, o);
-        o = shfl_xor(k, 2);
-        kahan_merge(k, o);
-        if (j == 0 && sl < ns && active) out[slot] = kahan_value(k);
+    }
+    // lanes j, j ^ 1 form a0 + a1 and a2 + a3, lanes j, j ^ 2 the sum of the two
+    auto put = [&](int i, const Kahan &k) {
+        const int f = tab[i].y;
+        if (slot >= 0 && f >= 0) a.partial[(size_t)f * (size_t)a.nseg + slot] = kahan_value(k);
+    };
+    if constexpr (G == 1) {
+        kahan_merge(k0, shfl_xor(k0, 1));
+        kahan_merge(k0, shfl_xor(k0, 2));
+        if (j == 0) put(0, k0);
+    } else if constexpr (G == 2) {
+        Kahan x0, x1;
+        f2_unpack(s[0], x0.s, x1.s);
+        f2_unpack(c[0], x0.nc, x1.nc);
+        Kahan k = (j & 1) ? x1 : x0;
+        kahan_merge(k, shfl_xor((j & 1) ? x0 : x1, 1));
+        kahan_merge(k, shfl_xor(k, 2));
+        if (j < 2) put(j, k);
+    } else {
+        constexpr int K = H / 2;  // pairs a lane keeps after the first exchange
+        f32x2 ks[K], kn[K];
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            const f32x2 os = (j & 1) ? s[i] : s[K + i], on = (j & 1) ? c[i] : c[K + i];
+            ks[i] = (j & 1) ? s[K + i] : s[i];
+            kn[i] = (j & 1) ? c[K + i] : c[i];
+            kahan2_merge(ks[i], kn[i], __shfl_xor_sync(0xffffffffu, os, 1), __shfl_xor_sync(0xffffffffu, on, 1));
+        }
+        Kahan x0, x1;
+        if constexpr (G == 4) {
+            f2_unpack(ks[0], x0.s, x1.s);
+            f2_unpack(kn[0], x0.nc, x1.nc);
+            Kahan k = (j & 2) ? x1 : x0;
+            kahan_merge(k, shfl_xor((j & 2) ? x0 : x1, 2));
+            put(2 * (j & 1) + (j >> 1), k);
+        } else {
+            f32x2 fs = (j & 2) ? ks[1] : ks[0], fn = (j & 2) ? kn[1] : kn[0];
+            const f32x2 os = (j & 2) ? ks[0] : ks[1], on = (j & 2) ? kn[0] : kn[1];
+            kahan2_merge(fs, fn, __shfl_xor_sync(0xffffffffu, os, 2), __shfl_xor_sync(0xffffffffu, on, 2));
+            f2_unpack(fs, x0.s, x1.s);
+            f2_unpack(fn, x0.nc, x1.nc);
+            put(4 * (j & 1) + (j & 2), x0);
+            put(4 * (j & 1) + (j & 2) + 1, x1);
+        }
     }
 }
 
 // Bounded grace wait for copies this CTA issued before giving up (every wait is bounded).
 __device__ __forceinline__ void fr_drain(uint64_t *bar, uint32_t parity) { (void)mbar_wait_bounded(bar, parity); }
 
+// Consumer warps take units (8 segments of a stage) from one counter of the CTA: item after
+// item, stage after stage, longest segments first, so that a warp that finishes early goes on
+// with the next stage (or item) that has landed.  A stage is released by its units: the
+// producer first makes up the difference to the barrier's fixed count.  The entry buffer of an
+// item is free when its last stage is, which the producer learns by waiting for that stage.
 template <int G, int DT, int VM>
 __global__ void __launch_bounds__(kFrThreads, 1)
-frames_kernel(const __grid_constant__ FrArgs a, FrGeom fg, const __grid_constant__ TmaSet tm) {
+frames_kernel(const __grid_constant__ FrArgs a, FrGeom fg, const __grid_constant__ FrMaps fm) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 127u) & ~static_cast<uintptr_t>(127u));
     const int S = fg.nstages;
-    unsigned char *ebuf0 = smem;
     const int NE = fg.nebufs;
-    unsigned char *pst = smem + (size_t)NE * fg.ebuf_bytes;
-    int *hdrs = reinterpret_cast<int *>(pst + (size_t)S * fg.pstage_bytes);
-    uint64_t *efull = reinterpret_cast<uint64_t *>(reinterpret_cast<unsigned char *>(hdrs) +
-                                                   (size_t)S * kFrStageHeader);
-    uint64_t *eempty = efull + NE;
-    uint64_t *pfull = eempty + NE;
+    unsigned char *ebuf0 = smem;
+    unsigned char *ring = smem + (size_t)NE * fg.ebuf_bytes;
+    uint64_t *efull = reinterpret_cast<uint64_t *>(ring + (size_t)fg.nblocks * fg.block_bytes);
+    uint64_t *pfull = efull + NE;
     uint64_t *pempty = pfull + S;
-    int *ctr = reinterpret_cast<int *>(pempty + S);
-    volatile int *abort_flag = ctr + S;
+    int2 *ftab = reinterpret_cast<int2 *>(pempty + S);            // [n_groups][G]
+    uint32_t *sbase = reinterpret_cast<uint32_t *>(ftab + a.n_groups * G);  // [S] stages' first word
+    int *ctr = reinterpret_cast<int *>(sbase + S);
+    volatile int *abort_flag = ctr + 1;
+    volatile int *issued = ctr + 2;  // plane stages and items' entries the producer has issued
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int i = 0; i < NE; ++i) {
-            mbar_init(&efull[i], 1);
-            mbar_init(&eempty[i], kFrConsumers);
-        }
+        for (int i = 0; i < NE; ++i) mbar_init(&efull[i], 1);
         for (int i = 0; i < S; ++i) {
             mbar_init(&pfull[i], 1);
-            mbar_init(&pempty[i], kFrConsumers);
+            mbar_init(&pempty[i], kFrUnits);
         }
+        *ctr = 0;
         *abort_flag = 0;
+        issued[0] = issued[1] = 0;
         fence_barrier_init();
     }
-    zero_bands(pst, fg.pstage_bytes, S, (int)(fg.pstage_bytes / (fg.plane_words * 4u)), fg.plane_words,
-               fg.band_from);
+    for (int t = threadIdx.x; t < a.n_groups * G; t += kFrThreads) {
+        const int g = t / G, i = t - g * G;
+        const int qg = g / a.nd, db = g - qg * a.nd;
+        const int q = qg * a.nq + (i >> a.ld), f = q + 4 * ((db << a.ld) + (i & ((1 << a.ld) - 1)));
+        ftab[t] = make_int2(4 * (i * a.slot + ((a.beta + q * a.fphase) & 3)), f < a.n_frames ? f : -1);
+    }
+    // blocks of fslots planes (interleaved by row class), spb stages of G planes in each
+    for (int t = threadIdx.x; t < S; t += kFrThreads)
+        sbase[t] = smem_addr(ring) + (uint32_t)(t / fg.spb) * fg.block_bytes + (uint32_t)((t % fg.spb) * G * a.slot) * 4u;
     __syncthreads();
+    const int step = (int)gridDim.x;
     if (warp == 0) {
-        int k = 0, issued = 0;  // items seen, items whose entries were issued
-        uint32_t j = 0;         // plane stages issued
+        // entries: ke items issued; a buffer is free again when the last stage of the item NE
+        // before is, i.e. once `free_items` items are known to be done
+        int ke = 0, free_items = NE;
+        uint32_t j = 0;  // plane stages issued
         bool stop = false;
-        // descriptors are read two items ahead: with one or two frame groups per item the
-        // producer would otherwise wait for a descriptor from DRAM on every item
+        // descriptors are read ahead, for the entries and for the planes: the producer would
+        // otherwise wait for a descriptor from DRAM on every item
+        int64_t e_item = blockIdx.x;
+        TileDesc e_next = fr_desc(a, (int)e_item);
+        auto issue_entries = [&]() {
+            while (ke < free_items && e_item < a.n_tiles) {
+                const TileDesc td = e_next;
+                e_item += step;
+                if (e_item < a.n_tiles) e_next = fr_desc(a, (int)e_item);
+                if (lane == 0)
+                    fr_stage_entries(a, fg, td, ebuf0 + (size_t)(ke % NE) * fg.ebuf_bytes, &efull[ke % NE]);
+                ++ke;
+                if (lane == 0) {
+                    __threadfence_block();
+                    issued[1] = ke;
+                }
+            }
+        };
+        issue_entries();
         TileDesc ahead[2] = {};
         for (int u = 0; u < 2; ++u)
-            if (blockIdx.x + u * gridDim.x < (unsigned)a.n_tiles) ahead[u] = fr_desc(a, blockIdx.x + u * gridDim.x);
-        for (int item = blockIdx.x; item < a.n_tiles && !stop; item += gridDim.x, ++k) {
+            if ((int)blockIdx.x + u * step < a.n_tiles) ahead[u] = fr_desc(a, (int)blockIdx.x + u * step);
+        int s = 0;          // stage in the ring, and the parity of the ring's turn
+        uint32_t turn = 0;
+        int seen_g = 0;  // stages known to be done, within the item free_items - NE
+        for (int item = blockIdx.x; item < a.n_tiles && !stop; item += step) {
             const TileDesc td = ahead[0];
             ahead[0] = ahead[1];
-            const int64_t far = (int64_t)item + 2 * (int64_t)gridDim.x;
+            const int64_t far = (int64_t)item + 2 * (int64_t)step;
             if (far < a.n_tiles) ahead[1] = fr_desc(a, (int)far);
-            const int eb = k % NE;
-            bool ok = true;
-            if (k >= NE) ok = mbar_wait_bounded(&eempty[eb], (uint32_t)(((k / NE) - 1) & 1));
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok || *abort_flag != 0) { stop = true; if (!ok && lane == 0) atomicExch(a.status, AZ_ETIMEOUT); break; }
-            if (lane == 0) fr_stage_entries(a, fg, td, ebuf0 + (size_t)eb * fg.ebuf_bytes, &efull[eb]);
-            issued = k + 1;
-            for (int g = 0; g < a.n_groups; ++g, ++j) {
-                const int s = (int)(j % (uint32_t)S);
-                ok = true;
-                if (j >= (uint32_t)S) ok = mbar_wait_bounded(&pempty[s], ((j / S) - 1) & 1);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok || *abort_flag != 0) { stop = true; if (!ok && lane == 0) atomicExch(a.status, AZ_ETIMEOUT); break; }
-                fr_stage_planes<G>(a, tm, td, g, reinterpret_cast<uint32_t *>(pst + (size_t)s * fg.pstage_bytes),
-                                   hdrs + s * (kFrStageHeader / 4), fg, &pfull[s], &ctr[s]);
+            const uint32_t units = (uint32_t)td.ns;
+            for (int g = 0; g < a.n_groups; ++g, ++j, s = s + 1 == S ? 0 : s + 1, turn ^= (s == 0)) {
+                if (j >= (uint32_t)S) {
+                    bool ok = mbar_wait_bounded(&pempty[s], turn ^ 1u);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok || *abort_flag != 0) {
+                        stop = true;
+                        if (!ok && lane == 0) atomicExch(a.status, AZ_ETIMEOUT);
+                        break;
+                    }
+                    if (++seen_g == a.n_groups) {
+                        seen_g = 0;
+                        ++free_items;
+                        issue_entries();
+                    }
+                }
+                if (lane == 0) mbar_arrive_n(&pempty[s], kFrUnits - units);
+                fr_stage_planes(a, fm, td, g, sbase[s], &pfull[s]);
+                if (lane == 0) {
+                    __threadfence_block();
+                    issued[0] = (int)j + 1;
+                }
             }
         }
         if (stop && lane == 0) {
             *abort_flag = 1;
             // grace for this CTA's own copies still in flight
             for (uint32_t jj = j > (uint32_t)S ? j - S : 0; jj < j; ++jj) fr_drain(&pfull[jj % S], (jj / S) & 1);
-            for (int kk = issued > NE ? issued - NE : 0; kk < issued; ++kk)
-                fr_drain(&efull[kk % NE], (uint32_t)((kk / NE) & 1));
+            for (int kk = ke > NE ? ke - NE : 0; kk < ke; ++kk) fr_drain(&efull[kk % NE], (uint32_t)((kk / NE) & 1));
         }
-    } else {
-        int k = 0;
-        uint32_t j = 0;
-        bool stop = false;
-        for (int item = blockIdx.x; item < a.n_tiles && !stop; item += gridDim.x, ++k) {
-            const int eb = k % NE;
-            bool ok = mbar_wait_bounded(&efull[eb], (uint32_t)((k / NE) & 1));
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok || *abort_flag != 0) {
-                if (!ok && lane == 0) { atomicExch(a.status, AZ_ETIMEOUT); *abort_flag = 1; }
-                break;
+        return;
+    }
+    // consumers
+    auto give_up = [&]() {
+        if (lane == 0) { atomicExch(a.status, AZ_ETIMEOUT); *abort_flag = 1; }
+        return false;
+    };
+    // The phase `parity` of `bar`, once the producer has issued more than n of what `count`
+    // counts: a unit may lie more than a turn of the ring ahead, where the parity alone would be
+    // taken for the turn before.
+    auto wait = [&](int which, int &known, int n, uint64_t *bar, uint32_t parity) -> bool {
+        if (known <= n) {
+            known = __shfl_sync(0xffffffffu, issued[which], 0);
+            const long long t0 = clock64();
+            while (known <= n) {
+                __nanosleep(64);
+                const bool late = clock64() - t0 > kWaitLimitCycles;
+                if (__any_sync(0xffffffffu, late)) return give_up();
+                if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+                known = __shfl_sync(0xffffffffu, issued[which], 0);
             }
-            const unsigned char *ebp = ebuf0 + (size_t)eb * fg.ebuf_bytes;
-            for (int g = 0; g < a.n_groups; ++g, ++j) {
-                const int s = (int)(j % (uint32_t)S);
-                ok = mbar_wait_bounded(&pfull[s], (j / S) & 1);
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok || *abort_flag != 0) {
-                    if (!ok && lane == 0) { atomicExch(a.status, AZ_ETIMEOUT); *abort_flag = 1; }
-                    stop = true;
-                    break;
-                }
-                const uint32_t *pl = reinterpret_cast<const uint32_t *>(pst + (size_t)s * fg.pstage_bytes);
-                if constexpr (G <= 2)
-                    fr_consume_split<G, DT, VM>(a, fg, ebp, pl, hdrs + s * (kFrStageHeader / 4), &ctr[s]);
-                else
-                    fr_consume<G, DT, VM>(a, fg, ebp, pl, hdrs + s * (kFrStageHeader / 4), &ctr[s]);
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&pempty[s]);
-            }
-            if (stop) break;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&eempty[eb]);
         }
+        bool ok = mbar_try_wait(bar, parity);
+        if (!__all_sync(0xffffffffu, ok)) {
+            ok = mbar_wait_bounded(bar, parity);
+            if (!__all_sync(0xffffffffu, ok)) return give_up();
+            if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+        }
+        return true;
+    };
+    int stages_known = 0, entries_known = 0;
+    // An item's units per stage are read from its descriptor in global memory, an item ahead: a warp may pass over an item that the others have finished, whose entry
+    // buffer holds another item by then.
+    auto unit_count = [&](int64_t it) -> int {
+        return it < a.n_tiles ? __ldg(a.desc + 8 * it + 5) : 0;
+    };
+    int64_t item = blockIdx.x;
+    int k = 0;                        // this CTA's item number
+    int per = unit_count(item), per_next = unit_count(item + step);  // units per stage
+    int first = 0, units = per * a.n_groups;  // the item's first unit and its units
+    float inv = 1.f / (float)per;
+    int j0 = 0;                       // its first stage
+    int jc = 0, s = 0;                // the last unit's stage: its number, place in the ring and
+    uint32_t turn = 0;                // the parity of the ring's turn
+    int eb = 0;                       // the item's entry buffer and its parity
+    uint32_t eturn = 0;
+    bool landed = false;              // its entries have been waited for
+    int next = 0;
+    if (lane == 0) next = atomicAdd(ctr, 1);
+    while (true) {
+        const int u = __shfl_sync(0xffffffffu, next, 0);
+        while (u >= first + units) {
+            j0 += a.n_groups;
+            first += units;
+            item += step;
+            ++k;
+            if (++eb == NE) { eb = 0; eturn ^= 1u; }
+            landed = false;
+            if (item >= a.n_tiles) return;
+            per = per_next;
+            inv = 1.f / (float)per;
+            units = per * a.n_groups;
+            per_next = unit_count(item + step);
+        }
+        if (lane == 0) next = atomicAdd(ctr, 1);
+        // stage of the item and unit of the stage: u - first and per are far below 2^20, so the
+        // product's error cannot reach the half that keeps it off the integers
+        const int x = u - first;
+        const int g = (int)(((float)x + 0.5f) * inv);
+        const int j = j0 + g;
+        s += j - jc;
+        jc = j;
+        while (s >= S) { s -= S; turn ^= 1u; }
+        if (!landed && !wait(1, entries_known, k, &efull[eb], eturn)) return;
+        landed = true;
+        if (!wait(0, stages_known, j, &pfull[s], turn)) return;
+        fr_unit<G, DT, VM>(a, fg, ebuf0 + (size_t)eb * fg.ebuf_bytes, sbase[s], ftab + g * G, x - g * per);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&pempty[s]);
     }
 }
 
@@ -1595,75 +1543,78 @@ uint32_t plane_words_of(const az_integrator *h) { return plane_stride(h->tl.ss);
 uint32_t rec_words_of(const az_integrator *h) { return (uint32_t)h->tl.max_rec_words; }
 
 // ---- frames kernel with tile-resident entries -----------------------------------------
-constexpr uint32_t kFrFixedBytes = 128 + 384;  // alignment slack; barriers, counters, flag
+// alignment slack; barriers, stage addresses, counters; the stages' frames (up to 64 + 3 * 8)
+constexpr uint32_t kFrFixedBytes = 128 + 512 + 8 * 96;
 
-// The image's row-class maps for the frame-pair layout, in three dimensions: x, the ny class
-// rows of a period of four frames (class k holds rows k, k + 4, ... of the stacked frames, so
-// a period is 4 ny rows = ny class rows), and the period (16 npix bytes, a multiple of 16).
-// Class k of frames F and F + 4 are the same class rows of consecutive periods, so a box of
-// depth 2 copies both.  Only the nf / 4 whole periods of the nf frames are mapped.
-int encode_pair_maps(const void *img, int nf, int ny, int nx, int box_w, int box_h, CUtensorMap out[4]) {
+// The frames' maps (FrMaps) over nf frames starting at img: map [q][c] starts at the 16-byte
+// aligned address just before row c of frame q, so its element (x, y, m) is column
+// x - off of row 4 y + c of frame q + 4 m, off = the word phase of that row.  Reads outside the
+// rows of the class or after the last frame return zeros.
+int encode_frame_maps(const void *img, int nf, int ny, int nx, int box_w, int box_h, int depth, FrMaps &out) {
     AZ_TRY(get_encoder());
+    memset(&out, 0, sizeof(out));
     const uintptr_t base = reinterpret_cast<uintptr_t>(img);
-    const int beta = (int)((base >> 2) & 3u), nu = nx & 3;
-    for (int k = 0; k < 4; ++k) {
-        const int offk = (beta + k * nu) & 3;
-        void *basek = reinterpret_cast<void *>(base + 4u * (uintptr_t)k * (uintptr_t)nx - 4u * (uintptr_t)offk);
-        cuuint64_t dims[3] = {(cuuint64_t)(nx + offk), (cuuint64_t)ny, (cuuint64_t)(nf / 4)};
-        cuuint64_t strides[2] = {(cuuint64_t)16 * (cuuint64_t)nx, (cuuint64_t)16 * (cuuint64_t)nx * (cuuint64_t)ny};
-        cuuint32_t box[3] = {(cuuint32_t)box_w, (cuuint32_t)box_h, 2};
-        cuuint32_t estr[3] = {1, 1, 1};
-        CUresult r = g_encode(&out[k], CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, basek, dims, strides, box, estr,
-                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return fail(AZ_ECUDA, "cuTensorMapEncodeTiled (pairs) failed (%d)", (int)r);
-    }
+    for (int q = 0; q < 4 && q < nf; ++q)
+        for (int c = 0; c < 4 && c < ny; ++c) {
+            const uintptr_t row = base + 4u * ((uintptr_t)q * (uintptr_t)ny + (uintptr_t)c) * (uintptr_t)nx;
+            const int off = (int)((row >> 2) & 3u);
+            cuuint64_t dims[3] = {(cuuint64_t)(nx + off), (cuuint64_t)((ny - c + 3) / 4), (cuuint64_t)((nf - q + 3) / 4)};
+            cuuint64_t strides[2] = {(cuuint64_t)16 * (cuuint64_t)nx, (cuuint64_t)16 * (cuuint64_t)nx * (cuuint64_t)ny};
+            cuuint32_t box[3] = {(cuuint32_t)box_w, (cuuint32_t)box_h, (cuuint32_t)depth};
+            cuuint32_t estr[3] = {1, 1, 1};
+            CUresult r = g_encode(&out.m[q][c], CU_TENSOR_MAP_DATA_TYPE_UINT32, 3,
+                                  reinterpret_cast<void *>(row - 4u * (uintptr_t)off), dims, strides, box, estr,
+                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+            if (r != CUDA_SUCCESS) return fail(AZ_ECUDA, "cuTensorMapEncodeTiled (frames) failed (%d)", (int)r);
+        }
     return AZ_OK;
 }
 
-// Sizes for G frames per plane stage (pair: the frame-pair layout, G / 2 regions of two
-// frames); false unless two entry buffers and two plane stages fit.
-bool fr_geom(const az_integrator *h, int G, int dk, int n_groups, FrGeom &fg, bool pair = false) {
-    fg.rec_cap = (rec_words_of(h) * 4u + 127u) & ~127u;
-    fg.ent_cap = ((uint32_t)h->tl.max_tile_entries + 7u) & ~7u;
+// Sizes for G frames per plane stage; false unless two entry buffers and two stages fit.
+bool fr_geom(const az_integrator *h, int G, int dk, int n_groups, FrGeom &fg) {
+    const TiledLayout &L = h->tl;
+    if (L.fslots < G) return false;
+    fg.rec_cap = ((uint32_t)L.f_max_rec * 4u + 127u) & ~127u;
+    fg.ent_cap = (uint32_t)L.f_max_entries;
     fg.dk = dk;
     fg.ebuf_bytes = (fg.rec_cap + fg.ent_cap * (dk ? 10u : 6u) + 127u) & ~127u;
-    if (pair) {
-        fg.plane_words = (uint32_t)h->tl.pw_p;
-        fg.band_from = 4u * (uint32_t)h->tl.ss_p;
-        fg.pstage_bytes = (uint32_t)(G / 2) * fg.plane_words * 4u;
-    } else {
-        fg.plane_words = plane_words_of(h);
-        fg.band_from = fg.plane_words - kZeroBand;
-        fg.pstage_bytes = (uint32_t)G * fg.plane_words * 4u;
-    }
-    // two entry buffers and as many plane stages as fit; then, when a work item has few
-    // frame groups (the entries dominate its copies), more entry buffers in what is left
-    const int64_t per = (int64_t)fg.pstage_bytes + kFrStageHeader;
-    const int64_t avail = (int64_t)max_smem_per_block() - 2 * (int64_t)fg.ebuf_bytes - kFrFixedBytes;
-    fg.nstages = (int)std::min<int64_t>(kFrMaxStages, avail > 0 ? avail / per : 0);
+    fg.block_bytes = 4u * (uint32_t)L.fslots * (uint32_t)L.fslot_words * 4u;
+    fg.spb = L.fslots / G;
+    auto need = [&](int e, int blocks) {
+        return (int64_t)e * fg.ebuf_bytes + (int64_t)blocks * fg.block_bytes + kFrFixedBytes;
+    };
+    const int64_t smem = max_smem_per_block();
+    // two entry buffers and as many plane stages as fit; when a work item has few stages (the
+    // entries dominate its copies), more entry buffers too: both rings grow together, so that as
+    // many items are in flight for their planes as for their entries
     fg.nebufs = 2;
+    fg.nblocks = 0;
+    while ((fg.nblocks + 1) * fg.spb <= std::max(kFrMaxStages, fg.spb) && need(2, fg.nblocks + 1) <= smem) ++fg.nblocks;
+    fg.nstages = fg.nblocks * fg.spb;
     if (n_groups <= 2 && fg.nstages >= 2) {
-        // every item takes n_groups plane stages: grow both rings together, so that as many
-        // items are in flight for their planes as for their entries
         for (int e = 2; e <= kFrMaxEbufs; ++e) {
             const int ns = std::min(kFrMaxStages, std::max(2, n_groups * e));
-            const int64_t need = (int64_t)e * fg.ebuf_bytes + (int64_t)ns * per + kFrFixedBytes;
-            if (need > (int64_t)max_smem_per_block()) break;
+            const int blocks = (ns + fg.spb - 1) / fg.spb;
+            if (need(e, blocks) > smem) break;
             fg.nebufs = e;
+            fg.nblocks = blocks;
             fg.nstages = ns;
         }
     }
+    // The producer sees a stage's release when it issues the stage nstages later, and an item's
+    // entries follow the release of the item nebufs before: more stages than nebufs items have
+    // would leave the last items' entries unissued.
+    fg.nstages = std::min(fg.nstages, fg.nebufs * n_groups);
     return fg.nstages >= 2;
 }
 
 uint32_t fr_smem(const FrGeom &fg) {
-    return (uint32_t)fg.nebufs * fg.ebuf_bytes + (uint32_t)fg.nstages * (fg.pstage_bytes + kFrStageHeader) +
-           kFrFixedBytes;
+    return (uint32_t)fg.nebufs * fg.ebuf_bytes + (uint32_t)fg.nblocks * fg.block_bytes + kFrFixedBytes;
 }
 
 template <int G, int DT, int VM>
-int fr_launch(const FrArgs &a, const FrGeom &fg, const TmaSet &tm, cudaStream_t s, Profiler *prof,
+int fr_launch(const FrArgs &a, const FrGeom &fg, const FrMaps &fm, cudaStream_t s, Profiler *prof,
               int prof_kind) {
     if (a.n_tiles <= 0) return AZ_OK;
     const uint32_t smem = fr_smem(fg);
@@ -1672,14 +1623,14 @@ int fr_launch(const FrArgs &a, const FrGeom &fg, const TmaSet &tm, cudaStream_t 
     const int grid = std::min(a.n_tiles, num_sms());
     {
         ProfScope ps(prof, prof_kind, s);
-        kern<<<grid, kFrThreads, smem, s>>>(a, fg, tm);
+        kern<<<grid, kFrThreads, smem, s>>>(a, fg, fm);
     }
     AZ_CUDA(cudaGetLastError());
     return AZ_OK;
 }
 
 template <int G>
-int fr_launch_dt(int dtype, const FrArgs &a, const FrGeom &fg, const TmaSet &tm, cudaStream_t s,
+int fr_launch_dt(int dtype, const FrArgs &a, const FrGeom &fg, const FrMaps &tm, cudaStream_t s,
                  Profiler *prof, int kind) {
     const int vm = a.var ? VM_VAR : (a.ent_dark != nullptr ? VM_DARK : VM_PLAIN);
     switch (dtype) {
@@ -1698,70 +1649,60 @@ int fr_launch_dt(int dtype, const FrArgs &a, const FrGeom &fg, const TmaSet &tm,
     }
 }
 
-// Frames kernel over `nf` frames starting at `img` (nf <= the partial buffer's frames from
-// frame0 on): per-segment partials [nf][nseg] in h->partial from frame frame0.  With 8 frames
-// per stage, whole stages go through the frame-pair layout when the tile shape has one and
-// its stages fit; the frames of a last partial stage then go through the plain layout in a
-// second launch (a frame's sums do not depend on the layout it is read through: the entry
-// order is the same).  Returns AZ_EUNSUPPORTED (without error text) when the TMA engine or
-// the shared memory it needs is not available.
-int frames_v3(az_integrator *h, const void *img, int nf, int dtype, const float *ent_dark,
-              int prof_kind, cudaStream_t s, bool var = false, const float *ent_weights = nullptr,
-              int frame0 = 0, bool allow_pair = true) {
-    if (engine_for(h) != AZ_COPY_TMA) return AZ_EUNSUPPORTED;
-    int G = h->frames_per_pass >= 16 ? 16 : (h->frames_per_pass >= 8 ? 8 : 4);
-    FrGeom fg;
-    // one frame (any image type, with or without a dark), or two frames of float values
-    // without a dark (the norm pass): one lane per segment and frame
-    const bool small = nf == 1 || (nf == 2 && dtype == AZ_DTYPE_F32 && ent_dark == nullptr && !var);
-    if (small) G = nf;
-    else if (nf < G) G = nf <= 4 ? 4 : (nf <= 8 ? 8 : G);
-    bool fits = fr_geom(h, G, ent_dark != nullptr, (nf + G - 1) / G, fg);
-    while (!fits && G > 4 && !small) {
-        G >>= 1;
-        fits = fr_geom(h, G, ent_dark != nullptr, (nf + G - 1) / G, fg);
+// How a launch of nf frames is cut into stages (a) and laid out in shared memory (fg): frames
+// per stage as tuned (8 by default, 4 below that), no more than the launch has; a stage covers nq
+// of the four frame classes q and D frames of each, chosen for the fewest stages and then for the
+// deepest copies.  False when the TMA engine or the shared memory it needs is not available.
+bool fr_plan(const az_integrator *h, int nf, int dk, FrArgs &a, FrGeom &fg, int &G) {
+    if (engine_for(h) != AZ_COPY_TMA || h->tl.fslots < 1) return false;
+    G = h->frames_per_pass >= 8 ? 8 : 4;
+    while (G > 1 && G / 2 >= nf) G >>= 1;
+    for (; G >= 1; G >>= 1) {
+        a.n_groups = 0;
+        for (int ld = 0; (1 << ld) <= G; ++ld) {
+            const int nq = G >> ld;
+            if (nq > 4 || (nq > 1 && nq / 2 >= nf)) continue;
+            const int nd = ((nf + 3) / 4 + (1 << ld) - 1) >> ld;
+            const int groups = ((std::min(nf, 4) + nq - 1) / nq) * nd;
+            if (a.n_groups == 0 || groups <= a.n_groups) {
+                a.n_groups = groups; a.nq = nq; a.ld = ld; a.nd = nd;
+            }
+        }
+        if (a.n_groups > 0 && fr_geom(h, G, dk, a.n_groups, fg)) return true;
     }
-    if (!fits) return AZ_EUNSUPPORTED;
-    const TiledLayout &L = h->tl;
-    const int nf8 = nf & ~7;
-    FrGeom fp;
-    const bool pair = allow_pair && G == 8 && !small && L.srow_p > 0 && nf8 > 0 &&
-                      fr_geom(h, 8, ent_dark != nullptr, nf8 / 8, fp, true);
-    if (pair) fg = fp;
-    const int nrun = pair ? nf8 : nf;
+    return false;
+}
+
+// Frames kernel over `nf` frames starting at `img` (nf <= the partial buffer's frames): per-
+// segment partials [nf][nseg] in h->partial.  ent_dark and ent_weights (NULL: the matrix's) are in
+// the order of the layout's f_pix.  Returns AZ_EUNSUPPORTED (without error text) when fr_plan
+// finds no form.
+int frames_v3(az_integrator *h, const void *img, int nf, int dtype, const float *ent_dark,
+              int prof_kind, cudaStream_t s, bool var = false, const float *ent_weights = nullptr) {
+    FrGeom fg;
     FrArgs a{};
-    a.img = static_cast<const char *>(img);
-    a.n_frames = nrun; a.n_groups = (nrun + G - 1) / G; a.n_tiles = L.n_active;
-    a.tile_desc = L.tile_desc.as<int32_t>(); a.tile_rec = L.tile_rec.as<int32_t>();
-    a.ent_loc = pair ? L.ent_loc_p.as<uint16_t>() : L.ent_loc.as<uint16_t>();
-    a.ent_w = ent_weights ? ent_weights : L.ent_w32.as<float>();
+    int G = 0;
+    if (!fr_plan(h, nf, ent_dark != nullptr, a, fg, G)) return AZ_EUNSUPPORTED;
+    const TiledLayout &L = h->tl;
+    a.n_frames = nf; a.n_tiles = L.n_active;
+    a.desc = L.f_desc.as<int32_t>(); a.rec = L.f_rec.as<int32_t>();
+    a.ent_loc = L.f_loc.as<uint16_t>();
+    a.ent_w = ent_weights ? ent_weights : L.f_w32.as<float>();
     a.ent_dark = ent_dark;
     a.var = var ? 1 : 0;
-    a.partial = h->partial.as<float>() + (size_t)frame0 * (size_t)L.nseg;
-    a.nseg = L.nseg; a.ny = h->ny; a.nx = h->nx; a.th = L.th; a.tw = L.tw;
-    a.srow = pair ? L.srow_p : L.srow;
-    a.ss = pair ? L.ss_p : L.ss;
-    a.ntx = L.ntx;
-    a.pair = pair ? 1 : 0;
-    a.slot = L.slot_p;
+    a.partial = h->partial.as<float>();
+    a.nseg = L.nseg; a.ny = h->ny; a.nx = h->nx; a.th = L.th; a.tw = L.tw; a.ntx = L.ntx;
+    a.slot = L.fslot_words; a.cstride = L.fslots * L.fslot_words;
+    a.beta = (int)((reinterpret_cast<uintptr_t>(img) >> 2) & 3u);
+    a.fphase = (int)(((int64_t)h->ny * h->nx) & 3);
     a.status = h->status.as<int>();
-    TmaSet tm;
-    if (pair) {
-        memset(&tm, 0, sizeof(tm));
-        AZ_TRY(encode_pair_maps(img, nrun, h->ny, h->nx, L.srow_p, L.th / 4, tm.pair));
-        AZ_TRY(fr_launch_dt<8>(dtype, a, fg, tm, s, &h->prof, prof_kind));
-        if (nrun == nf) return AZ_OK;
-        return frames_v3(h, static_cast<const char *>(img) + (size_t)nrun * (size_t)h->ny * (size_t)h->nx * 4u,
-                         nf - nrun, dtype, ent_dark, prof_kind, s, var, ent_weights, frame0 + nrun, false);
-    }
-    AZ_TRY(make_maps(h, AZ_COPY_TMA, img, (int64_t)nf * h->ny, nullptr, nullptr, nullptr, nullptr, tm));
-    if (small)
-        return G == 1 ? fr_launch_dt<1>(dtype, a, fg, tm, s, &h->prof, prof_kind)
-                      : fr_launch<2, AZ_DTYPE_F32, VM_PLAIN>(a, fg, tm, s, &h->prof, prof_kind);
+    FrMaps fm;
+    AZ_TRY(encode_frame_maps(img, nf, h->ny, h->nx, L.srow_f, L.th / 4, 1 << a.ld, fm));
     switch (G) {
-        case 4: return fr_launch_dt<4>(dtype, a, fg, tm, s, &h->prof, prof_kind);
-        case 8: return fr_launch_dt<8>(dtype, a, fg, tm, s, &h->prof, prof_kind);
-        default: return fr_launch_dt<16>(dtype, a, fg, tm, s, &h->prof, prof_kind);
+        case 1: return fr_launch_dt<1>(dtype, a, fg, fm, s, &h->prof, prof_kind);
+        case 2: return fr_launch_dt<2>(dtype, a, fg, fm, s, &h->prof, prof_kind);
+        case 4: return fr_launch_dt<4>(dtype, a, fg, fm, s, &h->prof, prof_kind);
+        default: return fr_launch_dt<8>(dtype, a, fg, fm, s, &h->prof, prof_kind);
     }
 }
 
@@ -1972,24 +1913,54 @@ int batch_norm(az_integrator *h, const float *flat, const float *sa, const float
     return AZ_OK;
 }
 
+// The dark of every entry: in the order of the frames kernel's entries (f) or of the general
+// kernel's.
+int gather_darks(az_integrator *h, const float *dark, bool f, DevBuf &out, cudaStream_t s) {
+    TiledLayout &L = h->tl;
+    const int64_t n = f ? L.f_entries : L.padded_nnz;
+    if (out.bytes < sizeof(float) * (size_t)n) AZ_TRY(out.alloc(sizeof(float) * (size_t)n));
+    const int64_t blocks = std::min<int64_t>((n + 255) / 256, (int64_t)num_sms() * 8);
+    ProfScope ps(&h->prof, 4, s);
+    gather_dark_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), 256, 0, s>>>(
+        (f ? L.f_pix : L.ent_pix).as<int32_t>(), dark, n, out.as<float>());
+    AZ_CUDA(cudaGetLastError());
+    return AZ_OK;
+}
+
 int batch_frames(az_integrator *h, const void *frames, int n, int dtype, const float *dark,
-                 float *oI, float *oS, int frame_out0, cudaStream_t s, const float *ent_dark_given,
-                 const float *norm) {
+                 float *oI, float *oS, int frame_out0, cudaStream_t s, bool bound_dark, const float *norm) {
     // the dark of every entry, in entry order, so that the frames pass reads it with the
-    // weights instead of staging a dark plane with every group of frames (given: bound once
-    // by az_set_corrections)
-    const int ent_dk = dark != nullptr || ent_dark_given != nullptr;
-    if (dark && !ent_dark_given) {
-        TiledLayout &L = h->tl;
-        if (L.ent_dark.bytes < sizeof(float) * (size_t)L.padded_nnz)
-            AZ_TRY(L.ent_dark.alloc(sizeof(float) * (size_t)L.padded_nnz));
-        const int64_t blocks = std::min<int64_t>((L.padded_nnz + 255) / 256, (int64_t)num_sms() * 8);
-        ProfScope ps(&h->prof, 4, s);
-        gather_dark_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), 256, 0, s>>>(
-            L.ent_pix.as<int32_t>(), dark, L.padded_nnz, L.ent_dark.as<float>());
-        AZ_CUDA(cudaGetLastError());
+    // weights instead of staging a dark plane with every group of frames (bound_dark: gathered
+    // once by az_set_corrections)
+    const int ent_dk = dark != nullptr || bound_dark;
+    const int64_t cap = (int64_t)(h->partial_bytes / (sizeof(float) * (size_t)std::max(h->tl.nseg, 1)));
+    const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(cap, kMaxFramesPerLaunch));
+    {
+        // tile-resident entries (frames_kernel), up to kMaxFramesPerLaunch frames per launch
+        FrArgs fa{};
+        FrGeom fgeo;
+        int G = 0;
+        if (n > 0 && fr_plan(h, std::min(chunk, n), ent_dk, fa, fgeo, G)) {
+            if (dark && !bound_dark) AZ_TRY(gather_darks(h, dark, true, h->tl.ent_dark, s));
+            const float *ent_dark = !ent_dk ? nullptr : (bound_dark ? h->bound_dark_f : h->tl.ent_dark).as<float>();
+            for (int f0 = 0; f0 < n; f0 += chunk) {
+                const int nf = std::min(chunk, n - f0);
+                Inst d = make_inst(h, false);
+                d.img = static_cast<const char *>(frames) + (size_t)f0 * (size_t)d.npix * 4u;
+                const int rc = frames_v3(h, d.img, nf, dtype, ent_dark, 0, s);
+                if (rc == AZ_EUNSUPPORTED)
+                    return fail(AZ_EUNSUPPORTED, "batch of %d frames: the tiles do not fit in shared memory", nf);
+                AZ_TRY(rc);
+                if (norm) d.norm = const_cast<float *>(norm);
+                d.n_frames = nf;
+                d.oI = oI; d.oS = oS; d.frame_out0 = frame_out0 + f0;
+                AZ_TRY((run_phase2<float, MODE_FRAMES>(d, nullptr, 1, (int64_t)nf * h->nrows, nf, s, &h->prof)));
+            }
+            return AZ_OK;
+        }
     }
-    const float *ent_dark = ent_dark_given ? ent_dark_given : h->tl.ent_dark.as<float>();
+    if (dark && !bound_dark) AZ_TRY(gather_darks(h, dark, false, h->tl.ent_dark, s));
+    const float *ent_dark = (bound_dark ? h->bound_ent_dark : h->tl.ent_dark).as<float>();
     // frames per pass as tuned, halved while two stages of that many frame planes do not fit,
     // or while the tile's entries would not fit beside them (down to 4 frames per pass)
     int fpi = h->frames_per_pass;
@@ -2000,30 +1971,12 @@ int batch_frames(az_integrator *h, const void *frames, int n, int dtype, const f
         if ((int)smem_for(g) <= max_smem_per_block() && (se || fpi <= 4)) break;
         fpi >>= 1;
     }
-    const int64_t cap = (int64_t)(h->partial_bytes / (sizeof(float) * (size_t)std::max(h->tl.nseg, 1)));
     const int chunk_max = (int)std::max<int64_t>(fpi, (cap / fpi) * fpi);
     const int planes = fpi;
     int stage_e = 0;
     StageGeom sg = choose_stage(plane_words_of(h), planes, (uint32_t)h->tl.max_tile_entries, 4,
                                 rec_words_of(h), stage_e, ent_dk);
     const int eng = engine_for(h);
-    if (eng == AZ_COPY_TMA) {
-        // tile-resident entries (frames_kernel), up to kMaxFramesPerLaunch frames per launch
-        const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(cap, kMaxFramesPerLaunch));
-        for (int f0 = 0; f0 < n; f0 += chunk) {
-            const int nf = std::min(chunk, n - f0);
-            Inst d = make_inst(h, false);
-            d.img = static_cast<const char *>(frames) + (size_t)f0 * (size_t)d.npix * 4u;
-            const int rc = frames_v3(h, d.img, nf, dtype, ent_dk ? ent_dark : nullptr, 0, s);
-            if (rc == AZ_EUNSUPPORTED && f0 == 0) break;  // the general kernel below
-            AZ_TRY(rc);
-            if (norm) d.norm = const_cast<float *>(norm);
-            d.n_frames = nf;
-            d.oI = oI; d.oS = oS; d.frame_out0 = frame_out0 + f0;
-            AZ_TRY((run_phase2<float, MODE_FRAMES>(d, nullptr, 1, (int64_t)nf * h->nrows, nf, s, &h->prof)));
-            if (f0 + nf >= n) return AZ_OK;
-        }
-    }
     for (int f0 = 0; f0 < n; f0 += chunk_max) {
         const int nf = std::min(chunk_max, n - f0);
         Inst d = make_inst(h, false);
@@ -2057,7 +2010,7 @@ int batch_frames(az_integrator *h, const void *frames, int n, int dtype, const f
 int batch_pixelnorm(az_integrator *h, const void *frames, int n, int dtype, const float *dark,
                     const float *flat, const float *sa, const float *pol, float *oI, float *oU,
                     float *oC, cudaStream_t s) {
-    if (engine_for(h) != AZ_COPY_TMA || h->partial_bytes < 2 * sizeof(float) * (size_t)h->tl.nseg)
+    if (engine_for(h) != AZ_COPY_TMA || h->tl.fslots < 1 || h->partial_bytes < 2 * sizeof(float) * (size_t)h->tl.nseg)
         return fail(AZ_EUNSUPPORTED, "az_integrate_batch_pixelnorm: needs the tensor-copy engine (tiles up to 236 pixels wide)");
     TiledLayout &L = h->tl;
     const int64_t npix = (int64_t)h->ny * h->nx;
@@ -2069,30 +2022,25 @@ int batch_pixelnorm(az_integrator *h, const void *frames, int n, int dtype, cons
     if (n == 0) return AZ_OK;
     // per-pixel normalisation, per-entry corrected weights and darks
     const int64_t pblocks = std::min<int64_t>((npix + 255) / 256, (int64_t)num_sms() * 8);
-    const int64_t eblocks = std::max<int64_t>(1, std::min<int64_t>((L.padded_nnz + 255) / 256, (int64_t)num_sms() * 8));
+    const int64_t eblocks = std::max<int64_t>(1, std::min<int64_t>((L.f_entries + 255) / 256, (int64_t)num_sms() * 8));
     if (L.norm_frames.bytes < 2 * sizeof(float) * (size_t)npix) {
         AZ_TRY(L.norm_frames.alloc(2 * sizeof(float) * (size_t)npix));
         fill_f32_kernel<<<(unsigned)pblocks, 256, 0, s>>>(L.norm_frames.as<float>() + npix, npix, 1.f);
         AZ_CUDA(cudaGetLastError());
     }
-    if (L.ent_wnorm.bytes < sizeof(float) * (size_t)L.padded_nnz)
-        AZ_TRY(L.ent_wnorm.alloc(sizeof(float) * (size_t)L.padded_nnz));
+    if (L.ent_wnorm.bytes < sizeof(float) * (size_t)L.f_entries)
+        AZ_TRY(L.ent_wnorm.alloc(sizeof(float) * (size_t)L.f_entries));
     {
         ProfScope ps(&h->prof, 4, s);
         norm_pixels_kernel<<<(unsigned)pblocks, 256, 0, s>>>(flat, sa, pol, npix, L.norm_frames.as<float>());
-        gather_wnorm_kernel<<<(unsigned)eblocks, 256, 0, s>>>(L.ent_pix.as<int32_t>(), L.ent_w32.as<float>(),
-                                                              L.norm_frames.as<float>(), L.padded_nnz,
+        gather_wnorm_kernel<<<(unsigned)eblocks, 256, 0, s>>>(L.f_pix.as<int32_t>(), L.f_w32.as<float>(),
+                                                              L.norm_frames.as<float>(), L.f_entries,
                                                               L.ent_wnorm.as<float>());
         AZ_CUDA(cudaGetLastError());
     }
     const float *ent_dk = nullptr;
     if (dark) {
-        if (L.ent_dark.bytes < sizeof(float) * (size_t)L.padded_nnz)
-            AZ_TRY(L.ent_dark.alloc(sizeof(float) * (size_t)L.padded_nnz));
-        ProfScope ps(&h->prof, 4, s);
-        gather_dark_kernel<<<(unsigned)eblocks, 256, 0, s>>>(L.ent_pix.as<int32_t>(), dark, L.padded_nnz,
-                                                             L.ent_dark.as<float>());
-        AZ_CUDA(cudaGetLastError());
+        AZ_TRY(gather_darks(h, dark, true, L.ent_dark, s));
         ent_dk = L.ent_dark.as<float>();
     }
     const int64_t cap = (int64_t)(h->partial_bytes / (sizeof(float) * (size_t)std::max(L.nseg, 1)));
@@ -2184,17 +2132,12 @@ int forward_batch(az_integrator *h, const void *frames, int n, int dtype, const 
 // az_integrate_batch do not touch.  The caller's arrays are not read again.
 int bind_corrections(az_integrator *h, const float *dark, const float *flat, const float *sa,
                      const float *pol, cudaStream_t s) {
-    TiledLayout &L = h->tl;
     h->corr_bound = false;
     h->corr_dark = dark != nullptr;
     if (dark) {
-        if (h->bound_ent_dark.bytes < sizeof(float) * (size_t)L.padded_nnz)
-            AZ_TRY(h->bound_ent_dark.alloc(sizeof(float) * (size_t)L.padded_nnz));
-        const int64_t blocks = std::min<int64_t>((L.padded_nnz + 255) / 256, (int64_t)num_sms() * 8);
-        ProfScope ps(&h->prof, 4, s);
-        gather_dark_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), 256, 0, s>>>(
-            L.ent_pix.as<int32_t>(), dark, L.padded_nnz, h->bound_ent_dark.as<float>());
-        AZ_CUDA(cudaGetLastError());
+        // for both kernels: which one a batch takes depends on the copy engine of the time
+        AZ_TRY(gather_darks(h, dark, false, h->bound_ent_dark, s));
+        if (h->tl.fslots) AZ_TRY(gather_darks(h, dark, true, h->bound_dark_f, s));
     }
     if (h->bound_norm.bytes < 2 * sizeof(float) * (size_t)h->nrows)
         AZ_TRY(h->bound_norm.alloc(2 * sizeof(float) * (size_t)h->nrows));
@@ -2216,8 +2159,7 @@ int forward_batch_bound(az_integrator *h, const void *frames, int n, int dtype, 
     if (oN) AZ_CUDA(cudaMemcpyAsync(oN, bN, rb, cudaMemcpyDeviceToDevice, s));
     if (oC) AZ_CUDA(cudaMemcpyAsync(oC, bN + h->nrows, rb, cudaMemcpyDeviceToDevice, s));
     if (n == 0) return AZ_OK;
-    return batch_frames(h, frames, n, dtype, nullptr, oI, oS, 0, s,
-                        h->corr_dark ? h->bound_ent_dark.as<float>() : nullptr, bN);
+    return batch_frames(h, frames, n, dtype, nullptr, oI, oS, 0, s, h->corr_dark, bN);
 }
 
 // ------------------------------------------------------------------------------------
