@@ -28,15 +28,16 @@ __global__ void fill_frames_kernel(uint32_t *out, int64_t n, uint32_t seed) {
     }
 }
 
-int alloc_scratch(az_integrator *h) {
+int alloc_scratch(az_integrator *h, cudaStream_t s) {
     const size_t nseg = (size_t)std::max(h->tl.nseg, 1);
     const size_t single = 3 * nseg * sizeof(double);
     const size_t frames = (size_t)kMaxFramesPerLaunch * nseg * sizeof(float);
     h->partial_bytes = std::max(single, frames);
     AZ_TRY(h->partial.alloc(h->partial_bytes));
     AZ_TRY(h->norm.alloc(sizeof(float) * 2 * (size_t)h->nrows));
+    AZ_TRY(h->count64.alloc(sizeof(double) * (size_t)h->nrows));
     AZ_TRY(h->adj.alloc(sizeof(double) * 2 * (size_t)h->nrows));
-    return AZ_OK;
+    return count_layout(h, s);
 }
 
 int finish_build(az_integrator *h, cudaStream_t s) {
@@ -71,7 +72,7 @@ int finish_build(az_integrator *h, cudaStream_t s) {
     }
     h->frames_per_pass = 8;
     h->rows_per_warp = 32 / h->frames_per_pass;
-    AZ_TRY(alloc_scratch(h));
+    AZ_TRY(alloc_scratch(h, s));
     AZ_TRY(h->status.alloc(sizeof(int)));
     AZ_CUDA(cudaMemsetAsync(h->status.p, 0, sizeof(int), s));
     AZ_CUDA(cudaStreamSynchronize(s));
@@ -251,7 +252,7 @@ extern "C" int az_integrator_info(const az_integrator *h, az_info *out) {
     const DevBuf *bufs[] = {&h->csr_ptr, &h->csr_idx, &h->csr_w64, &h->csc_ptr, &h->csc_row,
                             &h->csc_w64, &h->csc_w32, &h->tl.tile_seg_ptr, &h->tl.tile_ent_ptr,
                             &h->tl.active_tiles, &h->tl.seg_ent_ptr, &h->tl.seg_slot,
-                            &h->tl.row_slot_ptr, &h->tl.ent_loc, &h->tl.f_desc, &h->tl.f_rec, &h->tl.f_loc, &h->tl.f_w32, &h->tl.f_pix, &h->tl.ent_w32, &h->tl.ent_w64,
+                            &h->tl.row_slot_ptr, &h->tl.ent_loc, &h->tl.f_desc, &h->tl.f_rec, &h->tl.f_loc, &h->tl.f_w32, &h->tl.f_pix, &h->tl.f_loc1, &h->tl.f_w64, &h->count64, &h->tl.ent_w32, &h->tl.ent_w64,
                             &h->partial, &h->norm, &h->adj, &h->status, &h->host_stage,
                             &h->tl.tile_desc, &h->tl.tile_rec, &h->tl.ent_pix, &h->tl.ent_dark,
                             &h->tl.norm_frames, &h->tl.ent_wnorm, &h->lut32, &h->lut64,
@@ -316,15 +317,6 @@ static int integrate_common(const az_integrator *h, const void *image, int dtype
     const_cast<az_integrator *>(h)->last_stream = (cudaStream_t)stream;
     if (h->layout == AZ_LAYOUT_LUT)
         return lut_forward(h, image, dtype, dark, flat, sa, pol, precision, oI, oS, oN, oC, (cudaStream_t)stream);
-    if (precision == AZ_PREC_FP32_COMP) {
-        // the batched machinery on a batch of one frame: the same arithmetic per frame as
-        // the single-frame kernel (which remains the path without the tensor-copy engine)
-        const int rc = forward_batch_one(const_cast<az_integrator *>(h), image, dtype, dark, flat, sa, pol,
-                                         static_cast<float *>(oI), static_cast<float *>(oS),
-                                         static_cast<float *>(oN), static_cast<float *>(oC),
-                                         (cudaStream_t)stream);
-        if (rc != AZ_EUNSUPPORTED) return rc;
-    }
     return forward_single(h, image, dtype, dark, flat, sa, pol, precision, oI, oS, oN, oC,
                           (cudaStream_t)stream);
 }
@@ -604,7 +596,7 @@ extern "C" int az_set_tuning(az_integrator *h, int tile_h, int tile_w, int rows_
             return fail(AZ_EINVAL, "az_set_tuning: tile %dx%d out of range", th, tw);
         cudaDeviceSynchronize();
         AZ_TRY(build_tiled_layout(h, th, tw, nullptr));
-        AZ_TRY(alloc_scratch(h));
+        AZ_TRY(alloc_scratch(h, nullptr));
         AZ_CUDA(cudaDeviceSynchronize());
     }
     if (rows_per_warp) h->frames_per_pass = 32 / rows_per_warp;
@@ -649,11 +641,8 @@ static int tune_layout(az_integrator *h, const void *frame, const float *dark, c
                                  o + rows, o + 2 * rows, o + 3 * rows, s);
             } else {
                 // what az_integrate1d/2d run in FP32 with the tiled form
-                rc = forward_batch_one(h, frame, AZ_DTYPE_U32, dark, nullptr, nullptr, nullptr, o, o + rows,
-                                       o + 2 * rows, o + 3 * rows, s);
-                if (rc == AZ_EUNSUPPORTED)
-                    rc = forward_single(h, frame, AZ_DTYPE_U32, dark, nullptr, nullptr, nullptr, AZ_PREC_FP32_COMP,
-                                        o, o + rows, o + 2 * rows, o + 3 * rows, s);
+                rc = forward_single(h, frame, AZ_DTYPE_U32, dark, nullptr, nullptr, nullptr, AZ_PREC_FP32_COMP, o,
+                                    o + rows, o + 2 * rows, o + 3 * rows, s);
             }
             cudaEventRecord(e1, s);
             cudaEventSynchronize(e1);
@@ -707,7 +696,7 @@ extern "C" int az_autotune(az_integrator *h, int n_trial_frames, az_stream_t str
     const int tile_count = (int)(sizeof(tiles) / sizeof(tiles[0]));
     for (int ti = 0; ti < tile_count; ++ti) {
         if (build_tiled_layout(h, tiles[ti][0], tiles[ti][1], s) != AZ_OK) { clear_error(); continue; }
-        AZ_TRY(alloc_scratch(h));
+        AZ_TRY(alloc_scratch(h, s));
         AZ_TRY(batch_norm(h, nullptr, nullptr, nullptr, nullptr, nullptr, s));
         for (int eg : engines)
             for (int f : fpps) {
@@ -737,7 +726,7 @@ extern "C" int az_autotune(az_integrator *h, int n_trial_frames, az_stream_t str
     if (best >= 1e30) return fail(AZ_EUNSUPPORTED, "az_autotune: no configuration ran");
     if (bt < 0) return fail(AZ_EUNSUPPORTED, "az_autotune: no configuration ran");
     AZ_TRY(build_tiled_layout(h, tiles[bt][0], tiles[bt][1], s));
-    AZ_TRY(alloc_scratch(h));
+    AZ_TRY(alloc_scratch(h, s));
     h->frames_per_pass = bf;
     h->rows_per_warp = 32 / bf;
     h->copy_engine = be;

@@ -105,12 +105,15 @@ struct TiledLayout {
     int f_max_entries = 0, f_max_rec = 0;
     DevBuf f_desc, f_rec;   // int32 [n_active][8], int32 [sum of record words]
     DevBuf f_loc, f_w32, f_pix;  // uint16, float, int32 [f_entries]
+    // The same for the single-frame kernel: locations in one plane (classes fslot_words words
+    // apart), FP64 weights (-0 past a segment's end).
+    DevBuf f_loc1, f_w64;        // uint16, double [f_entries]
     DevBuf ent_w32;         // float  [padded_nnz]
     DevBuf ent_w64;         // double [padded_nnz]
     DevBuf ent_pix;         // int32  [padded_nnz] (pixel of the entry; -1 for padding)
     DevBuf ent_dark;        // float, per batch call: dark of the entry's pixel, in the order of the
                             // kernel that reads it
-    DevBuf norm_frames;     // float  [2][ny][nx]: flat * solid angle * polarisation, then ones
+    DevBuf norm_frames;     // float  [ny][nx]: flat * solid angle * polarisation
     DevBuf ent_wnorm;       // float  [f_entries]: weight / (flat * solid angle * polarisation)
     // Per active tile: a 32-byte descriptor {tile, record offset (words), record words,
     // entry offset, padded entry count, segment count, 0, 0} and a 16-byte aligned record
@@ -183,17 +186,17 @@ struct az_integrator {
     azint::TiledLayout tl;
     // tuning
     int rows_per_warp = 4, frames_per_pass = 8, copy_engine = AZ_COPY_TMA;
-    bool count_ready = false;  // norm[nrows..] holds C for the current tiled layout
     // scratch: per-segment partial sums and per-row frame-independent sums
     azint::DevBuf partial;     // float or double [planes][nseg]
     size_t partial_bytes = 0;
-    azint::DevBuf norm;        // [2][nrows] (N, C) in the batch accumulation type
+    azint::DevBuf norm;        // float [2][nrows]: N of the last batch, C of the current layout
+    azint::DevBuf count64;     // double [nrows]: C of the current layout
     azint::DevBuf adj;         // [2][nrows] doubles: adjoint row factors g/N and g I/N
     azint::DevBuf status;      // int32 device status word
     // look-up-table layout (built on request): [width][nrows] pairs, per-pixel corrected
     // (value, normalisation) of the current frame, per-chunk partial sums
     azint::DevBuf lut32, lut64, lut_vals, lut_part;
-    // single FP32 frame through the frames kernel: [2][ny*nx] corrected frame and normalisation
+    // single FP32 frame of large tiles: [2][ny*nx] corrected frame and normalisation
     azint::DevBuf one_planes;
     int64_t lut_width = 0;
     int layout = AZ_LAYOUT_TILED;  // what az_integrate1d/2d use
@@ -259,9 +262,8 @@ int lut_forward(const az_integrator *h, const void *img, int dtype, const float 
                 const float *sa, const float *pol, int precision, void *oI, void *oS, void *oN, void *oC,
                 cudaStream_t s);
 int lut_export(const az_integrator *h, int64_t *width, int32_t *pix, float *c32, double *c64);
-int forward_batch_one(az_integrator *h, const void *image, int dtype, const float *dark,
-                      const float *flat, const float *sa, const float *pol, float *oI, float *oS,
-                      float *oN, float *oC, cudaStream_t s);
+// C of the current layout into norm[nrows..] and count64 (after alloc_scratch)
+int count_layout(az_integrator *h, cudaStream_t s);
 int batch_norm(az_integrator *h, const float *flat, const float *sa, const float *pol, float *oN,
                float *oC, cudaStream_t s);
 int batch_frames(az_integrator *h, const void *frames, int n, int dtype, const float *dark,

@@ -931,9 +931,12 @@ struct UnitFillArgs {
     TileGeom Tf;
     const int32_t *chunks, *seg_start, *seg_end, *seg_slot, *step_off, *rec_off, *pix_in;
     const float *w_in;
+    const double *w64_in;
     int32_t *rec, *desc, *pix;
-    uint16_t *loc;
+    uint16_t *loc, *loc1;  // in a block of planes, in one plane
     float *w;
+    double *w64;
+    int cut;               // words by which a class of one plane starts earlier than of a block
     int n_items;
 };
 
@@ -965,7 +968,10 @@ __global__ void unit_fill_kernel(UnitFillArgs A) {
                 const int p = 4 * q < len ? A.pix_in[e0 + 4 * q + j] : -1;
                 A.pix[o] = p;
                 A.w[o] = p >= 0 ? A.w_in[e0 + 4 * q + j] : 0.f;
-                A.loc[o] = (uint16_t)(p >= 0 ? tile_loc(A.Tf, p) : last);
+                A.w64[o] = p >= 0 ? A.w64_in[e0 + 4 * q + j] : -0.0;
+                const int l = p >= 0 ? (int)tile_loc(A.Tf, p) : last;
+                A.loc[o] = (uint16_t)l;
+                A.loc1[o] = (uint16_t)(l - l / A.Tf.ss * A.cut);
             }
             step += n;
         }
@@ -1224,7 +1230,6 @@ int count_runs(const az_integrator *h, int th, int tw, cudaStream_t s, int64_t *
 
 int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     TiledLayout &L = h->tl;
-    h->count_ready = false;  // the accumulation order of C depends on the layout
     h->corr_bound = false;   // bound corrections are per layout too (entry order, sums)
     const int64_t nnz = h->nnz;
     if (th < 4 || (th % 4) != 0 || tw < 4 || (tw % 4) != 0)
@@ -1477,12 +1482,15 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     }
     L.f_entries = fslots ? 32 * (int64_t)f_steps : 0;
     L.f_desc.release(); L.f_rec.release(); L.f_loc.release(); L.f_w32.release(); L.f_pix.release();
+    L.f_loc1.release(); L.f_w64.release();
     if (fslots) {
         AZ_TRY(L.f_desc.alloc(sizeof(int32_t) * 8 * (size_t)std::max(n_items, 1)));
         AZ_TRY(L.f_rec.alloc(sizeof(int32_t) * (size_t)std::max(f_words, 4)));
         AZ_TRY(L.f_loc.alloc(sizeof(uint16_t) * (size_t)L.f_entries));
         AZ_TRY(L.f_w32.alloc(sizeof(float) * (size_t)L.f_entries));
         AZ_TRY(L.f_pix.alloc(sizeof(int32_t) * (size_t)L.f_entries));
+        AZ_TRY(L.f_loc1.alloc(sizeof(uint16_t) * (size_t)L.f_entries));
+        AZ_TRY(L.f_w64.alloc(sizeof(double) * (size_t)L.f_entries));
         UnitFillArgs U;
         U.Tf = T; U.Tf.srow = srow_f; U.Tf.ss = fslots * fslot_words;
         U.chunks = chunks.as<int32_t>(); U.seg_start = L.seg_ent_ptr.as<int32_t>();
@@ -1490,6 +1498,8 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
         U.step_off = uoff.as<int32_t>(); U.rec_off = uroff.as<int32_t>(); U.pix_in = L.ent_pix.as<int32_t>();
         U.w_in = L.ent_w32.as<float>(); U.rec = L.f_rec.as<int32_t>(); U.desc = L.f_desc.as<int32_t>();
         U.pix = L.f_pix.as<int32_t>(); U.loc = L.f_loc.as<uint16_t>(); U.w = L.f_w32.as<float>();
+        U.loc1 = L.f_loc1.as<uint16_t>(); U.w64 = L.f_w64.as<double>(); U.w64_in = L.ent_w64.as<double>();
+        U.cut = (fslots - 1) * fslot_words;
         U.n_items = n_items;
         AZ_TRY(launch_gs(unit_fill_kernel, 32 * (int64_t)n_items, s, U));
         max_kernel<<<1, 1024, 0, s>>>(usteps.as<int32_t>(), n_items, mx.as<int32_t>() + 3);

@@ -73,8 +73,9 @@ struct Inst {
     const int32_t *tile_desc, *tile_rec;  // per active tile: descriptor [8] and record
     const float *ent_dark;                // frames pass: dark of each entry's pixel (or NULL)
     const CUtensorMap *maps;              // many-instance launch: this instance's [5][4] maps
-    int single_nc;  // single-frame phase 2 in FP32: 0 S, N, C from the partials; 1 C from
-                    // the per-layout cache norm[nrows..]; 2 N and C from that cache (N == C)
+    int single_nc;  // single-frame phase 2: 0 S, N, C from the partials; 1 C from the layout's
+                    // count; 2 N and C from it (N == C)
+    const void *count;  // [nrows] in the accumulation type
 };
 
 struct StageGeom {
@@ -778,6 +779,15 @@ __device__ __forceinline__ TileDesc fr_desc(const FrArgs &a, int item) {
     return TileDesc{x.x, x.y, x.z, x.w, y.x, y.y};
 }
 
+// Descriptors of a CTA's items, 32 at a time: lane l holds the one of item 32 b + l of the CTA, and
+// the next 32 are read while these are used.  (Read one or two items ahead, each item waited for
+// its descriptor's trip to memory: about 1 us an item where an item has few stages.)
+__device__ __forceinline__ TileDesc shfl_desc(const TileDesc &d, int l) {
+    return TileDesc{__shfl_sync(0xffffffffu, d.t, l), __shfl_sync(0xffffffffu, d.rec_off, l),
+                    __shfl_sync(0xffffffffu, d.rec_words, l), __shfl_sync(0xffffffffu, d.e_off, l),
+                    __shfl_sync(0xffffffffu, d.ne, l), __shfl_sync(0xffffffffu, d.ns, l)};
+}
+
 // One thread: the tile's record, entry locations, weights and darks into entry buffer `eb`.
 __device__ __forceinline__ void fr_stage_entries(const FrArgs &a, const FrGeom &fg, const TileDesc &td,
                                                  unsigned char *eb, uint64_t *bar) {
@@ -1038,18 +1048,22 @@ frames_kernel(const __grid_constant__ FrArgs a, FrGeom fg, const __grid_constant
         int ke = 0, free_items = NE;
         uint32_t j = 0;  // plane stages issued
         bool stop = false;
-        // descriptors are read ahead, for the entries and for the planes: the producer would
-        // otherwise wait for a descriptor from DRAM on every item
-        int64_t e_item = blockIdx.x;
-        TileDesc e_next = fr_desc(a, (int)e_item);
+        auto read = [&](int b) {
+            const int64_t it = (int64_t)blockIdx.x + (int64_t)(32 * b + lane) * step;
+            return it < a.n_tiles ? fr_desc(a, (int)it) : TileDesc{};
+        };
+        TileDesc e_cur = read(0), e_nxt = read(1), p_cur = e_cur, p_nxt = e_nxt;  // entries, planes
+        const int items = (a.n_tiles - (int)blockIdx.x + step - 1) / step;
         auto issue_entries = [&]() {
-            while (ke < free_items && e_item < a.n_tiles) {
-                const TileDesc td = e_next;
-                e_item += step;
-                if (e_item < a.n_tiles) e_next = fr_desc(a, (int)e_item);
+            while (ke < free_items && ke < items) {
+                const TileDesc td = shfl_desc(e_cur, ke & 31);
                 if (lane == 0)
                     fr_stage_entries(a, fg, td, ebuf0 + (size_t)(ke % NE) * fg.ebuf_bytes, &efull[ke % NE]);
                 ++ke;
+                if ((ke & 31) == 0) {
+                    e_cur = e_nxt;
+                    e_nxt = read((ke >> 5) + 1);
+                }
                 if (lane == 0) {
                     __threadfence_block();
                     issued[1] = ke;
@@ -1057,17 +1071,15 @@ frames_kernel(const __grid_constant__ FrArgs a, FrGeom fg, const __grid_constant
             }
         };
         issue_entries();
-        TileDesc ahead[2] = {};
-        for (int u = 0; u < 2; ++u)
-            if ((int)blockIdx.x + u * step < a.n_tiles) ahead[u] = fr_desc(a, (int)blockIdx.x + u * step);
         int s = 0;          // stage in the ring, and the parity of the ring's turn
         uint32_t turn = 0;
         int seen_g = 0;  // stages known to be done, within the item free_items - NE
-        for (int item = blockIdx.x; item < a.n_tiles && !stop; item += step) {
-            const TileDesc td = ahead[0];
-            ahead[0] = ahead[1];
-            const int64_t far = (int64_t)item + 2 * (int64_t)step;
-            if (far < a.n_tiles) ahead[1] = fr_desc(a, (int)far);
+        for (int k = 0; k < items && !stop; ++k) {
+            if (k > 0 && (k & 31) == 0) {
+                p_cur = p_nxt;
+                p_nxt = read((k >> 5) + 1);
+            }
+            const TileDesc td = shfl_desc(p_cur, k & 31);
             const uint32_t units = (uint32_t)td.ns;
             for (int g = 0; g < a.n_groups; ++g, ++j, s = s + 1 == S ? 0 : s + 1, turn ^= (s == 0)) {
                 if (j >= (uint32_t)S) {
@@ -1129,14 +1141,17 @@ frames_kernel(const __grid_constant__ FrArgs a, FrGeom fg, const __grid_constant
         return true;
     };
     int stages_known = 0, entries_known = 0;
-    // An item's units per stage are read from its descriptor in global memory, an item ahead: a warp may pass over an item that the others have finished, whose entry
-    // buffer holds another item by then.
-    auto unit_count = [&](int64_t it) -> int {
+    // An item's units per stage are read from its descriptor in global memory, 32 items at a time
+    // as above: a warp may pass over an item that the others have finished, whose entry buffer
+    // holds another item by then.
+    auto unit_counts = [&](int b) -> int {
+        const int64_t it = (int64_t)blockIdx.x + (int64_t)(32 * b + lane) * step;
         return it < a.n_tiles ? __ldg(a.desc + 8 * it + 5) : 0;
     };
+    int n_cur = unit_counts(0), n_nxt = unit_counts(1);
     int64_t item = blockIdx.x;
     int k = 0;                        // this CTA's item number
-    int per = unit_count(item), per_next = unit_count(item + step);  // units per stage
+    int per = __shfl_sync(0xffffffffu, n_cur, 0);  // units per stage
     int first = 0, units = per * a.n_groups;  // the item's first unit and its units
     float inv = 1.f / (float)per;
     int j0 = 0;                       // its first stage
@@ -1157,10 +1172,14 @@ frames_kernel(const __grid_constant__ FrArgs a, FrGeom fg, const __grid_constant
             if (++eb == NE) { eb = 0; eturn ^= 1u; }
             landed = false;
             if (item >= a.n_tiles) return;
-            per = per_next;
+            if ((k & 31) == 0) {
+                n_cur = n_nxt;
+                n_nxt = unit_counts((k >> 5) + 1);
+            }
+            per = __shfl_sync(0xffffffffu, n_cur, k & 31);
             inv = 1.f / (float)per;
             units = per * a.n_groups;
-            per_next = unit_count(item + step);
+
         }
         if (lane == 0) next = atomicAdd(ctr, 1);
         // stage of the item and unit of the stage: u - first and per are far below 2^20, so the
@@ -1177,6 +1196,457 @@ frames_kernel(const __grid_constant__ FrArgs a, FrGeom fg, const __grid_constant
         fr_unit<G, DT, VM>(a, fg, ebuf0 + (size_t)eb * fg.ebuf_bytes, sbase[s], ftab + g * G, x - g * per);
         __syncwarp();
         if (lane == 0) mbar_arrive(&pempty[s]);
+    }
+}
+
+// ------------------------------------------------------------------------------------
+// one frame per detector: correction and product in one launch
+// ------------------------------------------------------------------------------------
+// Items are the tiles of one integrator or of several (the many-detector plan).  A stage of the
+// ring holds an item's units and entries and the raw planes of its tile (image and the correction
+// arrays given).  The consumer warps first correct the tile's pixels once, in shared memory --
+// x = image - dark, n = ((1 flat) solid angle) polarisation -- and then reduce the units over x and
+// n as fr_unit does, so a pixel is corrected once for its two to three entries and nothing but
+// the inputs is read from memory.  Work is taken from one counter, in the order: pixels of item
+// 0, then for every item k the pixels of item k + 1 and the units of item k, so that nobody
+// waits for pixels that are still being corrected.  C = sum w is kept per layout.
+//
+// FP64 (one 2527 x 2463 frame, four corrections): the FP64 pipe, whose instructions take 64 cycles a
+// warp, conversions to double included, needs about 66 us: per pixel one subtraction and two
+// products (the conversions are done with integer instructions, exactly), per entry two multiply-
+// adds.  The pass takes 140 us; correcting every entry and forming C each time took 351 us.
+// FP32 (the same frame): one launch of 66 us in place of a pass that wrote two planes to memory
+// (28 us) and the frames kernel over them (40 us).  Copies alone take 60 us, the entries and the
+// queue without planes 25 us: five arrays are twenty small copies an item.  16 detectors without
+// corrections: 278 us in place of 562 us.
+constexpr int kSgWarps = 15;
+constexpr int kSgThreads = 32 * (1 + kSgWarps);
+constexpr int kSgMaxStages = 8;
+// pixels (with their row's margins) of a correction unit: in FP64 small ones, because a warp's pass
+// over 32 pixels takes some 400 cycles of the FP64 pipe (6-Mpixel frame: 32 words 158 us, 64 145,
+// 128 149, 384 202), in FP32 larger ones, whose cost is the taking of the unit (192 words 3% slower)
+constexpr int kSgConv64 = 64, kSgConv32 = 384;
+constexpr uint32_t kSgUnits = 1u << 19;  // arrivals that complete a conversion or release barrier
+
+struct SgInst {
+    const int32_t *desc, *rec;
+    const uint16_t *loc;
+    const void *w;             // float or double
+    void *partial;             // [2][nseg]: sums of w x, and of w n
+    const CUtensorMap *maps;   // [5][4] in device memory, or NULL: the launch parameter
+    int nseg, nx, ny, th4, tw, ntx, slot;
+    int present;               // bits: image, dark, flat, solid angle, polarisation
+    int beta[5];               // word phase of each array
+    int n_items;
+    int64_t item_begin;
+    int *status;
+};
+
+struct SgGeom {
+    uint32_t rec_cap, loc_cap, w_cap;  // bytes: units, entry locations, weights (multiples of 128)
+    uint32_t plane_bytes;              // one raw plane
+    uint32_t xn_off;                   // FP64: corrected pixels
+    uint32_t stage_bytes;
+    int nstages;
+};
+
+__device__ __forceinline__ TileDesc sg_desc(const SgInst &d, int64_t local) {
+    const int4 *p = reinterpret_cast<const int4 *>(d.desc) + 2 * local;
+    const int4 x = __ldg(p), y = __ldg(p + 1);
+    return TileDesc{x.x, x.y, x.z, x.w, y.x, y.y};
+}
+template <class AT> __device__ __forceinline__ int sg_conv_units(const SgInst &d) {
+    constexpr int words = sizeof(AT) == 8 ? kSgConv64 : kSgConv32;
+    return (4 * d.slot + words - 1) / words;
+}
+__device__ __forceinline__ int sg_plane(int present, int k) { return __popc(present & ((1 << k) - 1)); }
+
+// Exact conversions to double by integer instructions.
+template <int DT>
+__device__ __forceinline__ double to_double(uint32_t b) {
+    if (DT == AZ_DTYPE_F32) {
+        const uint32_t e = (b >> 23) & 255u;
+        if (e - 1u < 254u) return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+        if ((b << 1) == 0u) return __hiloint2double((int)b, 0);
+        return (double)__uint_as_float(b);  // subnormal, infinite, NaN
+    }
+    const uint32_t sign = DT == AZ_DTYPE_I32 ? b & 0x80000000u : 0u;
+    const uint32_t u = sign ? 0u - b : b;
+    if (u == 0u) return 0.0;
+    const int lz = __clz((int)u);
+    const uint32_t m = u << lz;
+    return __hiloint2double((int)(sign | (((uint32_t)(1054 - lz) << 20) + ((m & 0x7fffffffu) >> 11))), (int)(m << 21));
+}
+
+template <class AT, int DT, bool X, bool N>
+__device__ __forceinline__ void sg_correct(const SgInst &d, const SgGeom &sg, unsigned char *stage, int part) {
+    const int lane = threadIdx.x & 31;
+    const int words = 4 * d.slot;
+    constexpr int kWords = sizeof(AT) == 8 ? kSgConv64 : kSgConv32;
+    const int p0 = part * kWords, p1 = min(words, p0 + kWords);
+    unsigned char *planes = stage + sg.rec_cap + sg.loc_cap + sg.w_cap;
+    auto plane = [&](int k) {  // the words of array k, or NULL
+        return (d.present >> k) & 1 ? reinterpret_cast<uint32_t *>(planes + (size_t)sg_plane(d.present, k) * sg.plane_bytes)
+                                    : nullptr;
+    };
+    uint32_t *img = plane(0);
+    const float *dark = reinterpret_cast<const float *>(plane(1));
+    float *nrm[3] = {reinterpret_cast<float *>(plane(2)), reinterpret_cast<float *>(plane(3)),
+                     reinterpret_cast<float *>(plane(4))};
+    if constexpr (sizeof(AT) == 8) {
+        // x and n side by side at the entries' locations (the rows' phases taken out)
+        double *xn = reinterpret_cast<double *>(stage + sg.xn_off);
+        for (int p = p0 + lane; p < p1; p += 32) {
+            double x = 0.0, n = 1.0;
+            if (X) {
+                x = to_double<DT>(img[p + d.beta[0]]);
+                if (dark) x = x - to_double<AZ_DTYPE_F32>(__float_as_uint(dark[p + d.beta[1]]));
+            }
+            if (N) {
+                bool first = true;
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    if (nrm[k]) {
+                        const double f = to_double<AZ_DTYPE_F32>(__float_as_uint(nrm[k][p + d.beta[2 + k]]));
+                        n = first ? f : n * f;  // 1 f is f
+                        first = false;
+                    }
+                reinterpret_cast<double2 *>(xn)[p] = make_double2(x, n);
+            } else {
+                xn[p] = x;
+            }
+        }
+    } else {
+        // in place: x over the image, n over the first of its arrays
+        float *x = reinterpret_cast<float *>(img);
+        const int sh = dark ? d.beta[1] - d.beta[0] : 0;
+        int first = -1;
+#pragma unroll
+        for (int k = 2; k >= 0; --k)
+            if (nrm[k]) first = k;
+        int s1 = 0, s2 = 0;  // the other arrays' shifts from the first one's words
+        if (N && first >= 0) {
+            if (first < 1 && nrm[1]) s1 = d.beta[3] - d.beta[2 + first];
+            if (first < 2 && nrm[2]) s2 = d.beta[4] - d.beta[2 + first];
+        }
+        if (sh == 0 && s1 == 0 && s2 == 0) {  // same phases: four pixels at a time
+            for (int p = p0 + 4 * lane; p < p1; p += 128) {
+                if (X) {
+                    const uint4 u = *reinterpret_cast<const uint4 *>(img + p);
+                    float4 v = make_float4(img_f32<DT>(u.x), img_f32<DT>(u.y), img_f32<DT>(u.z), img_f32<DT>(u.w));
+                    if (dark) {
+                        const float4 k = *reinterpret_cast<const float4 *>(dark + p);
+                        v = make_float4(__fsub_rn(v.x, k.x), __fsub_rn(v.y, k.y), __fsub_rn(v.z, k.z), __fsub_rn(v.w, k.w));
+                    }
+                    *reinterpret_cast<float4 *>(x + p) = v;
+                }
+                if (N && first >= 0) {
+                    float4 v = *reinterpret_cast<const float4 *>(nrm[first] + p);
+#pragma unroll
+                    for (int k = 1; k < 3; ++k)
+                        if (k > first && nrm[k]) {
+                            const float4 f = *reinterpret_cast<const float4 *>(nrm[k] + p);
+                            v = make_float4(__fmul_rn(v.x, f.x), __fmul_rn(v.y, f.y), __fmul_rn(v.z, f.z), __fmul_rn(v.w, f.w));
+                        }
+                    *reinterpret_cast<float4 *>(nrm[first] + p) = v;
+                }
+            }
+        } else {
+            // word p of the first array and word p + shift of the others are one pixel
+            for (int p = p0 + lane; p < p1; p += 32) {
+                if (X) {
+                    float v = img_f32<DT>(img[p]);
+                    if (dark) v = __fsub_rn(v, dark[p + sh]);
+                    x[p] = v;
+                }
+                if (N && first >= 0) {
+                    float v = nrm[first][p];
+                    if (first < 1 && nrm[1]) v = __fmul_rn(v, nrm[1][p + s1]);
+                    if (first < 2 && nrm[2]) v = __fmul_rn(v, nrm[2][p + s2]);
+                    nrm[first][p] = v;
+                }
+            }
+        }
+    }
+}
+
+template <class AT, bool X, bool N>
+__device__ __forceinline__ void sg_unit(const SgInst &d, const SgGeom &sg, const unsigned char *stage, int u) {
+    const int lane = threadIdx.x & 31, j = lane & 3;
+    const int *unit = reinterpret_cast<const int *>(stage) + kUnitWords * u;
+    const int n = unit[1], slot = unit[2 + (lane >> 2)];
+    const int e0 = unit[0] * 32 + lane;
+    const uint16_t *L = reinterpret_cast<const uint16_t *>(stage + sg.rec_cap) + e0;
+    const AT *W = reinterpret_cast<const AT *>(stage + sg.rec_cap + sg.loc_cap) + e0;
+    AT *out = static_cast<AT *>(d.partial);
+    if constexpr (sizeof(AT) == 8) {
+        const double *xn = reinterpret_cast<const double *>(stage + sg.xn_off);
+        double S = 0.0, M = 0.0;
+#pragma unroll 4
+        for (int t = 0; t < n; ++t) {
+            const double w = W[32 * t];
+            const int o = L[32 * t];
+            double2 v;
+            if (N) v = reinterpret_cast<const double2 *>(xn)[o];
+            else v = make_double2(xn[o], 0.0);
+            // past the segment's end (weight -0): the value may be infinite
+            if (__double2hiint(w) == (int)0x80000000) v = make_double2(0.0, 0.0);
+            if (X) S = __fma_rn(w, v.x, S);
+            if (N) M = __fma_rn(w, v.y, M);
+        }
+        // a0 + a1 and a2 + a3, then their sum (addition commutes)
+        S += __shfl_xor_sync(0xffffffffu, S, 1);
+        S += __shfl_xor_sync(0xffffffffu, S, 2);
+        if (N) {
+            M += __shfl_xor_sync(0xffffffffu, M, 1);
+            M += __shfl_xor_sync(0xffffffffu, M, 2);
+        }
+        if (slot >= 0 && j == 0) out[slot] = S;
+        if (N && slot >= 0 && j == 1) out[(size_t)d.nseg + slot] = M;
+    } else {
+        const uint32_t planes = smem_addr(stage + sg.rec_cap + sg.loc_cap + sg.w_cap);
+        const bool norm = (d.present & 28) != 0;
+        const int kn = (d.present & 4) ? 2 : ((d.present & 8) ? 3 : 4);  // the array n lies over
+        const uint32_t px = planes + (uint32_t)d.beta[0] * 4u;
+        const uint32_t pn = planes + (uint32_t)sg_plane(d.present, kn) * sg.plane_bytes + (uint32_t)d.beta[kn] * 4u;
+        if constexpr (X && N) {
+            f32x2 s = 0ull, c = 0ull;
+#pragma unroll 4
+            for (int t = 0; t < n; ++t) {
+                const float w = W[32 * t];
+                const uint32_t o = (uint32_t)L[32 * t] << 2;
+                const float x = __uint_as_float(lds_u32(px + o));
+                const float m = norm ? __uint_as_float(lds_u32(pn + o)) : 1.f;
+                kahan2_add(s, c, f2_pack(w, w), f2_pack(x, m));
+            }
+            Kahan k0, k1;
+            f2_unpack(s, k0.s, k1.s);
+            f2_unpack(c, k0.nc, k1.nc);
+            Kahan k = (j & 1) ? k1 : k0;  // even lanes keep S, odd ones N
+            kahan_merge(k, shfl_xor((j & 1) ? k0 : k1, 1));
+            kahan_merge(k, shfl_xor(k, 2));
+            if (slot >= 0 && j < 2) out[(size_t)j * d.nseg + slot] = kahan_value(k);
+        } else {
+            const uint32_t pv = X ? px : pn;
+            Kahan k{0.f, 0.f};
+#pragma unroll 4
+            for (int t = 0; t < n; ++t)
+                kahan_add(k, W[32 * t], __uint_as_float(lds_u32(pv + ((uint32_t)L[32 * t] << 2))));
+            kahan_merge(k, shfl_xor(k, 1));
+            kahan_merge(k, shfl_xor(k, 2));
+            if (slot >= 0 && j == 0) out[slot] = kahan_value(k);
+        }
+    }
+}
+
+// X: the signal sums S; N: the normalisation sums (with X: after S).
+template <class AT, int DT, bool X, bool N>
+__global__ void __launch_bounds__(kSgThreads, 1)
+single_kernel(const __grid_constant__ SgInst one, const SgInst *__restrict__ multi, int n_inst, int n_items,
+              SgGeom sg, const __grid_constant__ TmaSet tm) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    unsigned char *smem = reinterpret_cast<unsigned char *>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 127u) & ~static_cast<uintptr_t>(127u));
+    const int S = sg.nstages;
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + (size_t)S * sg.stage_bytes + 128);
+    uint64_t *conv = full + S, *empty = conv + S;
+    int *ctr = reinterpret_cast<int *>(empty + S);
+    volatile int *abort_flag = ctr + 1, *issued = ctr + 2;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int *status = one.status;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < S; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&conv[i], kSgUnits);
+            mbar_init(&empty[i], kSgUnits);
+        }
+        *ctr = 0;
+        *abort_flag = 0;
+        *issued = 0;
+        fence_barrier_init();
+    }
+    __syncthreads();
+    const int step = (int)gridDim.x;
+    const int items = (n_items - (int)blockIdx.x + step - 1) / step;
+    // Of this CTA's items 32 b + lane (read 32 at a time, as in frames_kernel): the instance and
+    // the descriptor.
+    auto item_of = [&](int b) { return (int64_t)blockIdx.x + (int64_t)(32 * b + lane) * step; };
+    auto inst_index = [&](int64_t it) {
+        int lo = 0, hi = multi ? n_inst : 1;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (multi[mid].item_begin <= it) lo = mid; else hi = mid;
+        }
+        return lo;
+    };
+    auto inst = [&](int i) -> const SgInst * { return multi ? multi + i : &one; };
+    if (warp == 0) {
+        int s = 0, k = 0;
+        uint32_t turn = 0;
+        auto read = [&](int b, int &i) {
+            const int64_t it = item_of(b);
+            if (it >= n_items) { i = 0; return TileDesc{}; }
+            i = inst_index(it);
+            const SgInst *d = inst(i);
+            return sg_desc(*d, it - d->item_begin);
+        };
+        int i_cur = 0, i_nxt = 0;
+        TileDesc t_cur = read(0, i_cur), t_nxt = read(1, i_nxt);
+        for (; k < items; ++k) {
+            if (k > 0 && (k & 31) == 0) {
+                t_cur = t_nxt;
+                i_cur = i_nxt;
+                t_nxt = read((k >> 5) + 1, i_nxt);
+            }
+            const TileDesc td = shfl_desc(t_cur, k & 31);
+            const SgInst *d = inst(__shfl_sync(0xffffffffu, i_cur, k & 31));
+            if (k >= S) {
+                bool ok = mbar_wait_bounded(&empty[s], turn ^ 1u);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok || *abort_flag != 0) {
+                    if (lane == 0) {
+                        if (!ok) atomicExch(status, AZ_ETIMEOUT);
+                        *abort_flag = 1;
+                        // grace for this CTA's own copies still in flight
+                        for (int i = k - S; i < k; ++i) (void)mbar_wait_bounded(&full[i % S], (uint32_t)((i / S) & 1));
+                    }
+                    return;
+                }
+            }
+            unsigned char *stage = smem + (size_t)s * sg.stage_bytes;
+            unsigned char *el = stage + sg.rec_cap, *ew = el + sg.loc_cap, *planes = ew + sg.w_cap;
+            const int ti = td.t / d->ntx, tj = td.t - ti * d->ntx;
+            // lane 4 a + c copies row class c of array a
+            const int a = lane >> 2, c = lane & 3;
+            const bool on = a < 5 && ((d->present >> a) & 1) && c < d->ny;
+            const uint32_t n = (uint32_t)__popc(__ballot_sync(0xffffffffu, on));
+            fence_proxy_async_smem();
+            if (lane == 0) {
+                mbar_arrive_n(&empty[s], kSgUnits - (uint32_t)td.ns);
+                mbar_arrive_n(&conv[s], kSgUnits - (uint32_t)sg_conv_units<AT>(*d));
+                mbar_arrive_expect_tx(&full[s], (uint32_t)td.rec_words * 4u + (uint32_t)td.ne * (2u + (uint32_t)sizeof(AT)) +
+                                                    n * (uint32_t)d->slot * 4u);
+                bulk_g2s(stage, d->rec + td.rec_off, (uint32_t)td.rec_words * 4u, &full[s]);
+                bulk_g2s(el, d->loc + td.e_off, (uint32_t)td.ne * 2u, &full[s]);
+                bulk_g2s(ew, static_cast<const AT *>(d->w) + td.e_off, (uint32_t)td.ne * (uint32_t)sizeof(AT), &full[s]);
+            }
+            __syncwarp();
+            if (on) {
+                const int cs = ((d->nx & 3) * c) & 3;
+                const int x = tj * d->tw - ((d->beta[a] + cs) & 4);
+                const uint32_t to = smem_addr(planes) + (uint32_t)sg_plane(d->present, a) * sg.plane_bytes +
+                                    (uint32_t)(c * d->slot) * 4u;
+                const CUtensorMap *map = d->maps ? d->maps + 4 * a + c : &tm.m[a][c];
+                asm volatile(
+                    "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+                    " [%0], [%1, {%2, %3}], [%4];" ::"r"(to),
+                    "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(ti * d->th4), "r"(smem_addr(&full[s]))
+                    : "memory");
+            }
+            __syncwarp();
+            if (lane == 0) {
+                __threadfence_block();
+                *issued = k + 1;
+            }
+            if (++s == S) { s = 0; turn ^= 1u; }
+        }
+        return;
+    }
+    auto give_up = [&]() {
+        if (lane == 0) { atomicExch(status, AZ_ETIMEOUT); *abort_flag = 1; }
+        return false;
+    };
+    int known = 0;
+    // phase `parity` of bar, once item n has been issued (see frames_kernel)
+    auto wait = [&](int n, uint64_t *bar, uint32_t parity) -> bool {
+        if (known <= n) {
+            known = __shfl_sync(0xffffffffu, *issued, 0);
+            const long long t0 = clock64();
+            while (known <= n) {
+                __nanosleep(64);
+                const bool late = clock64() - t0 > kWaitLimitCycles;
+                if (__any_sync(0xffffffffu, late)) return give_up();
+                if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+                known = __shfl_sync(0xffffffffu, *issued, 0);
+            }
+        }
+        bool ok = mbar_try_wait(bar, parity);
+        if (!__all_sync(0xffffffffu, ok)) {
+            ok = mbar_wait_bounded(bar, parity);
+            if (!__all_sync(0xffffffffu, ok)) return give_up();
+            if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+        }
+        return true;
+    };
+    auto read = [&](int b, int &i) {
+        const int64_t it = item_of(b);
+        if (it >= n_items) { i = 0; return 0; }
+        i = inst_index(it);
+        const SgInst *d = inst(i);
+        return __ldg(d->desc + 8 * (it - d->item_begin) + 5);
+    };
+    int i_cur = 0, i_nxt = 0;
+    int n_cur = read(0, i_cur), n_nxt = read(1, i_nxt);
+    // block k of the order: correction of item k + 1 (nc units), then the units of item k (ne)
+    const SgInst *d1 = inst(__shfl_sync(0xffffffffu, i_cur, 0)), *d0 = d1;  // instances of items k + 1 and k
+    int k = -1, s0 = 0, s1 = 0, ne = 0, nc = sg_conv_units<AT>(*d1), first = 0;
+    uint32_t t0 = 0, t1 = 0;
+    int ne1 = __shfl_sync(0xffffffffu, n_cur, 0);                           // units of item k + 1
+    int next = 0;
+    if (lane == 0) next = atomicAdd(ctr, 1);
+    while (true) {
+        const int u = __shfl_sync(0xffffffffu, next, 0);
+        while (u >= first + nc + ne) {
+            first += nc + ne;
+            if (k + 1 >= items) return;
+            ++k;
+            d0 = d1; s0 = s1; t0 = t1; ne = ne1;
+            nc = 0;
+            if (++s1 == S) { s1 = 0; t1 ^= 1u; }
+            const int m = k + 1;
+            if (m < items) {
+                if ((m & 31) == 0) {
+                    n_cur = n_nxt;
+                    i_cur = i_nxt;
+                    n_nxt = read((m >> 5) + 1, i_nxt);
+                }
+                d1 = inst(__shfl_sync(0xffffffffu, i_cur, m & 31));
+                nc = sg_conv_units<AT>(*d1);
+                ne1 = __shfl_sync(0xffffffffu, n_cur, m & 31);
+            }
+        }
+        if (lane == 0) next = atomicAdd(ctr, 1);
+        const int x = u - first;
+        if (x < nc) {
+            if (!wait(k + 1, &full[s1], t1)) return;
+            sg_correct<AT, DT, X, N>(*d1, sg, smem + (size_t)s1 * sg.stage_bytes, x);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&conv[s1]);
+        } else {
+            if (!wait(k, &conv[s0], t0)) return;
+            sg_unit<AT, X, N>(*d0, sg, smem + (size_t)s0 * sg.stage_bytes, x - nc);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty[s0]);
+        }
+    }
+}
+
+// Sum of the weights of every segment, by the operations the other reductions use (four
+// accumulators, entry e to accumulator e mod 4, merged as ((a0 + a1) + (a2 + a3))).
+template <class AT>
+__global__ void count_kernel(const int32_t *__restrict__ start, const int32_t *__restrict__ end,
+                             const int32_t *__restrict__ slot, const AT *__restrict__ w, int nseg, AT *__restrict__ partial) {
+    const int lane = threadIdx.x & 31, j = lane & 3;
+    for (int64_t b = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 8; b < nseg;
+         b += (((int64_t)gridDim.x * blockDim.x) >> 5) * 8) {
+        const int64_t sg = b + (lane >> 2);
+        const int e0 = sg < nseg ? start[sg] : 0, e1 = sg < nseg ? end[sg] : 0;
+        Acc<AT> a;
+        a.zero();
+        for (int e = e0 + j; e < e1; e += 4) a.add(w[e], AT(1));
+        a.merge_lower_left(1);
+        a.merge_lower_left(2);
+        if (sg < nseg && j == 0) partial[slot[sg]] = a.value();
     }
 }
 
@@ -1257,8 +1727,8 @@ __global__ void __launch_bounds__(256, 4) phase2_thread_kernel(const __grid_cons
         }
     } else if (MODE == MODE_SINGLE) {
         const AT S = row_sum_thread<AT>(P, a, b);
-        const AT N = d.single_nc == 2 ? (AT)d.norm[d.nrows + r] : row_sum_thread<AT>(P + d.nseg, a, b);
-        const AT C = d.single_nc ? (AT)d.norm[d.nrows + r] : row_sum_thread<AT>(P + 2 * (size_t)d.nseg, a, b);
+        const AT N = d.single_nc == 2 ? static_cast<const AT *>(d.count)[r] : row_sum_thread<AT>(P + d.nseg, a, b);
+        const AT C = d.single_nc ? static_cast<const AT *>(d.count)[r] : row_sum_thread<AT>(P + 2 * (size_t)d.nseg, a, b);
         if (d.oI) static_cast<AT *>(d.oI)[r] = N != AT(0) ? S / N : AT(0);
         if (d.oS) static_cast<AT *>(d.oS)[r] = S;
         if (d.oN) static_cast<AT *>(d.oN)[r] = N;
@@ -1301,8 +1771,8 @@ __global__ void phase2_kernel(const __grid_constant__ Inst single, const Inst *_
             const AT *P = static_cast<const AT *>(d.partial);
             if (MODE == MODE_SINGLE) {
                 const AT S = row_sum<AT>(P, a, b);
-                const AT N = d.single_nc == 2 ? (AT)d.norm[d.nrows + r] : row_sum<AT>(P + d.nseg, a, b);
-                const AT C = d.single_nc ? (AT)d.norm[d.nrows + r] : row_sum<AT>(P + 2 * (size_t)d.nseg, a, b);
+                const AT N = d.single_nc == 2 ? static_cast<const AT *>(d.count)[r] : row_sum<AT>(P + d.nseg, a, b);
+                const AT C = d.single_nc ? static_cast<const AT *>(d.count)[r] : row_sum<AT>(P + 2 * (size_t)d.nseg, a, b);
                 if (lane == 0) {
                     const AT I = N != AT(0) ? S / N : AT(0);
                     if (d.oI) static_cast<AT *>(d.oI)[r] = I;
@@ -1387,6 +1857,7 @@ Inst make_inst(const az_integrator *h, bool fp64) {
     d.norm_rows = 2;
     d.partial = h->partial.p;
     d.norm = h->norm.as<float>();
+    d.count = fp64 ? (const void *)h->count64.p : (const void *)(h->norm.as<float>() + h->nrows);
     d.status = h->status.as<int>();
     d.n_items = L.n_active;
     d.tile_desc = L.tile_desc.as<int32_t>();
@@ -1706,6 +2177,90 @@ int frames_v3(az_integrator *h, const void *img, int nf, int dtype, const float 
     }
 }
 
+// ---- single-frame kernel ----------------------------------------------------------------
+constexpr uint32_t kSgFixedBytes = 128 + 128 + 256;  // alignment, margin after the last stage, barriers
+
+// Adds integrator h to the sizes a stage needs.
+struct SgNeed {
+    uint32_t rec = 0, ent = 0, plane = 0;
+    int planes = 0;
+    void add(const az_integrator *h, int present) {
+        const TiledLayout &L = h->tl;
+        rec = std::max(rec, ((uint32_t)L.f_max_rec * 4u + 127u) & ~127u);
+        ent = std::max(ent, (uint32_t)L.f_max_entries);
+        plane = std::max(plane, 16u * (uint32_t)L.fslot_words);
+        planes = std::max(planes, __builtin_popcount((unsigned)present));
+    }
+};
+
+// False unless two stages fit.
+bool sg_geom(const SgNeed &n, bool fp64, bool norm, SgGeom &g) {
+    g.rec_cap = n.rec;
+    g.loc_cap = (n.ent * 2u + 127u) & ~127u;
+    g.w_cap = n.ent * (fp64 ? 8u : 4u);
+    g.plane_bytes = n.plane;
+    g.xn_off = g.rec_cap + g.loc_cap + g.w_cap + (uint32_t)n.planes * n.plane + 128u;  // margin: phases
+    g.stage_bytes = g.xn_off + (fp64 ? n.plane * (norm ? 4u : 2u) : 0u);
+    const int64_t avail = (int64_t)max_smem_per_block() - kSgFixedBytes;
+    g.nstages = (int)std::min<int64_t>(kSgMaxStages, avail / std::max<uint32_t>(g.stage_bytes, 1u));
+    return g.nstages >= 2;
+}
+
+SgInst sg_inst(const az_integrator *h, bool fp64, const void *const arrs[5]) {
+    const TiledLayout &L = h->tl;
+    SgInst d{};
+    d.desc = L.f_desc.as<int32_t>(); d.rec = L.f_rec.as<int32_t>();
+    d.loc = L.f_loc1.as<uint16_t>();
+    d.w = fp64 ? (const void *)L.f_w64.p : (const void *)L.f_w32.p;
+    d.partial = h->partial.p;
+    d.nseg = L.nseg; d.nx = h->nx; d.ny = h->ny; d.th4 = L.th / 4; d.tw = L.tw; d.ntx = L.ntx; d.slot = L.fslot_words;
+    for (int k = 0; k < 5; ++k)
+        if (arrs[k]) {
+            d.present |= 1 << k;
+            d.beta[k] = (int)((reinterpret_cast<uintptr_t>(arrs[k]) >> 2) & 3u);
+        }
+    d.n_items = L.n_active;
+    d.status = h->status.as<int>();
+    return d;
+}
+
+// Maps of the arrays' row classes in the frames kernel's row pitch.
+int sg_maps(const az_integrator *h, const void *const arrs[5], TmaSet &tm) {
+    memset(&tm, 0, sizeof(tm));
+    for (int k = 0; k < 5; ++k)
+        if (arrs[k]) AZ_TRY(encode_class_maps(arrs[k], h->ny, h->nx, h->tl.srow_f, h->tl.th / 4, tm.m[k]));
+    return AZ_OK;
+}
+
+template <class AT, int DT, bool X, bool N>
+int sg_launch(const SgInst &one, const SgInst *multi, int n_inst, int n_items, const SgGeom &sg, const TmaSet &tm,
+              cudaStream_t s, Profiler *prof, int kind) {
+    if (n_items <= 0) return AZ_OK;
+    const uint32_t smem = (uint32_t)sg.nstages * sg.stage_bytes + kSgFixedBytes;
+    auto kern = single_kernel<AT, DT, X, N>;
+    AZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    ProfScope ps(prof, kind, s);
+    kern<<<std::min(n_items, num_sms()), kSgThreads, smem, s>>>(one, multi, n_inst, n_items, sg, tm);
+    AZ_CUDA(cudaGetLastError());
+    return AZ_OK;
+}
+
+template <class AT>
+int sg_launch_dt(int dtype, bool norm, const SgInst &one, const SgInst *multi, int n_inst, int n_items,
+                 const SgGeom &sg, const TmaSet &tm, cudaStream_t s, Profiler *prof) {
+    switch (dtype) {
+        case AZ_DTYPE_F32:
+            return norm ? sg_launch<AT, AZ_DTYPE_F32, true, true>(one, multi, n_inst, n_items, sg, tm, s, prof, 2)
+                        : sg_launch<AT, AZ_DTYPE_F32, true, false>(one, multi, n_inst, n_items, sg, tm, s, prof, 2);
+        case AZ_DTYPE_U32:
+            return norm ? sg_launch<AT, AZ_DTYPE_U32, true, true>(one, multi, n_inst, n_items, sg, tm, s, prof, 2)
+                        : sg_launch<AT, AZ_DTYPE_U32, true, false>(one, multi, n_inst, n_items, sg, tm, s, prof, 2);
+        default:
+            return norm ? sg_launch<AT, AZ_DTYPE_I32, true, true>(one, multi, n_inst, n_items, sg, tm, s, prof, 2)
+                        : sg_launch<AT, AZ_DTYPE_I32, true, false>(one, multi, n_inst, n_items, sg, tm, s, prof, 2);
+    }
+}
+
 // flat * solid angle * polarisation per pixel, multiplied in that order from 1 (absent = 1):
 // the value the norm reduction multiplies by each weight.
 __global__ void norm_pixels_kernel(const float *__restrict__ flat, const float *__restrict__ sa,
@@ -1754,12 +2309,6 @@ __global__ void single_planes_kernel(const void *__restrict__ img, const float *
     }
 }
 
-__global__ void fill_f32_kernel(float *__restrict__ out, int64_t n, float v) {
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n;
-         p += (int64_t)gridDim.x * blockDim.x)
-        out[p] = v;
-}
-
 }  // namespace
 
 int num_sms() {
@@ -1782,10 +2331,98 @@ int max_smem_per_block() {
     return g_max_smem;
 }
 
+// C = sum w per row of the current layout, in both precisions (it does not depend on the
+// inputs): formed when the layout is built.
+int count_layout(az_integrator *h, cudaStream_t s) {
+    const TiledLayout &L = h->tl;
+    const int32_t *start = L.seg_ent_ptr.as<int32_t>();
+    const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>(((int64_t)L.nseg + 63) / 64, (int64_t)num_sms() * 16));
+    for (int p = 0; p < 2; ++p) {
+        Inst d = make_inst(h, p == 1);
+        if (p == 0) {
+            count_kernel<float><<<g, 256, 0, s>>>(start, start + L.nseg, L.seg_slot.as<int32_t>(), L.ent_w32.as<float>(),
+                                                  L.nseg, h->partial.as<float>());
+            AZ_CUDA(cudaGetLastError());
+            d.oS = h->norm.as<float>() + h->nrows;
+            d.single_nc = 2;  // (S only)
+            AZ_TRY((run_phase2<float, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s)));
+        } else {
+            count_kernel<double><<<g, 256, 0, s>>>(start, start + L.nseg, L.seg_slot.as<int32_t>(), L.ent_w64.as<double>(),
+                                                   L.nseg, h->partial.as<double>());
+            AZ_CUDA(cudaGetLastError());
+            d.oS = h->count64.p;
+            d.single_nc = 2;
+            AZ_TRY((run_phase2<double, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s)));
+        }
+    }
+    return AZ_OK;
+}
+
+// One frame through single_kernel; AZ_EUNSUPPORTED (without error text) where it does not fit.
+template <class AT>
+int forward_one(const az_integrator *h, const void *const arrs[5], int dtype, void *oI, void *oS, void *oN, void *oC,
+                cudaStream_t s) {
+    constexpr bool fp64 = sizeof(AT) == 8;
+    if (engine_for(h) != AZ_COPY_TMA || h->tl.fslots < 1) return AZ_EUNSUPPORTED;
+    const SgInst one = sg_inst(h, fp64, arrs);
+    const bool norm = (one.present & 28) != 0;
+    SgNeed need;
+    need.add(h, one.present);
+    SgGeom sg;
+    if (!sg_geom(need, fp64, norm, sg)) return AZ_EUNSUPPORTED;
+    TmaSet tm;
+    AZ_TRY(sg_maps(h, arrs, tm));
+    AZ_TRY((sg_launch_dt<AT>(dtype, norm, one, nullptr, 1, one.n_items, sg, tm, s, &h->prof)));
+    Inst d = make_inst(h, fp64);
+    d.oI = oI; d.oS = oS; d.oN = oN; d.oC = oC;
+    d.single_nc = norm ? 1 : 2;
+    return run_phase2<AT, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s, &h->prof);
+}
+
+// One FP32 frame with tiles whose six planes and entries do not fit twice: the corrected frame
+// and its normalisation written to memory, then the frames kernel over the two.
+int forward_planes(az_integrator *h, const void *image, int dtype, const float *dark, const float *flat,
+                   const float *sa, const float *pol, void *oI, void *oS, void *oN, void *oC, cudaStream_t s) {
+    const bool corr = flat || sa || pol;
+    FrArgs fa{};
+    FrGeom fg;
+    int G = 0;
+    if (!fr_plan(h, corr ? 2 : 1, 0, fa, fg, G)) return AZ_EUNSUPPORTED;
+    const int64_t npix = (int64_t)h->ny * h->nx;
+    if (h->one_planes.bytes < 2 * sizeof(float) * (size_t)npix)
+        AZ_TRY(h->one_planes.alloc(2 * sizeof(float) * (size_t)npix));
+    float *planes = h->one_planes.as<float>();
+    {
+        ProfScope ps(&h->prof, 4, s);
+        const unsigned g = (unsigned)std::min<int64_t>((npix + 255) / 256, (int64_t)num_sms() * 8);
+        const int wn = corr ? 1 : 0;
+        switch (dtype) {
+            case AZ_DTYPE_F32: single_planes_kernel<AZ_DTYPE_F32><<<g, 256, 0, s>>>(image, dark, flat, sa, pol, npix, wn, planes); break;
+            case AZ_DTYPE_U32: single_planes_kernel<AZ_DTYPE_U32><<<g, 256, 0, s>>>(image, dark, flat, sa, pol, npix, wn, planes); break;
+            default: single_planes_kernel<AZ_DTYPE_I32><<<g, 256, 0, s>>>(image, dark, flat, sa, pol, npix, wn, planes); break;
+        }
+        AZ_CUDA(cudaGetLastError());
+    }
+    const int rc = frames_v3(h, planes, corr ? 2 : 1, AZ_DTYPE_F32, nullptr, 2, s);
+    if (rc != AZ_OK) return rc;
+    Inst d = make_inst(h, false);
+    d.oI = oI; d.oS = oS; d.oN = oN; d.oC = oC;
+    d.single_nc = corr ? 1 : 2;
+    return run_phase2<float, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s, &h->prof);
+}
+
 int forward_single(const az_integrator *h, const void *image, int dtype, const float *dark,
                    const float *flat, const float *sa, const float *pol, int precision, void *oI,
                    void *oS, void *oN, void *oC, cudaStream_t s) {
     const bool fp64 = precision == AZ_PREC_FP64;
+    const void *const arrs[5] = {image, dark, flat, sa, pol};
+    const int rc = fp64 ? forward_one<double>(h, arrs, dtype, oI, oS, oN, oC, s)
+                        : forward_one<float>(h, arrs, dtype, oI, oS, oN, oC, s);
+    if (rc != AZ_EUNSUPPORTED) return rc;
+    if (!fp64) {
+        const int rp = forward_planes(const_cast<az_integrator *>(h), image, dtype, dark, flat, sa, pol, oI, oS, oN, oC, s);
+        if (rp != AZ_EUNSUPPORTED) return rp;
+    }
     Inst d = make_inst(h, fp64);
     d.img = static_cast<const char *>(image);
     d.dark = dark; d.flat = flat; d.sa = sa; d.pol = pol;
@@ -1861,46 +2498,52 @@ int forward_single_into(const az_integrator *h, const void *image, int dtype, co
 
 int batch_norm(az_integrator *h, const float *flat, const float *sa, const float *pol, float *oN,
                float *oC, cudaStream_t s) {
+    const int nrows = h->nrows;
+    float *Cdev = h->norm.as<float>() + nrows;
+    if (oC) AZ_CUDA(cudaMemcpyAsync(oC, Cdev, sizeof(float) * nrows, cudaMemcpyDeviceToDevice, s));
+    if (!flat && !sa && !pol) {  // N = C
+        AZ_CUDA(cudaMemcpyAsync(h->norm.as<float>(), Cdev, sizeof(float) * nrows, cudaMemcpyDeviceToDevice, s));
+        if (oN) AZ_CUDA(cudaMemcpyAsync(oN, Cdev, sizeof(float) * nrows, cudaMemcpyDeviceToDevice, s));
+        return AZ_OK;
+    }
     Inst d = make_inst(h, false);
     d.flat = flat; d.sa = sa; d.pol = pol;
-    d.oN = oN; d.oC = oC;
-    if (engine_for(h) == AZ_COPY_TMA && h->partial_bytes >= 2 * sizeof(float) * (size_t)h->tl.nseg) {
-        // Through the frames kernel.  C = sum w does not depend on the inputs: the first call
-        // after a layout change reduces [flat * solid angle * polarisation; ones] as a
-        // two-frame batch and keeps C; later calls reduce the first frame only (N), and
-        // without flat, solid angle and polarisation N equals C.  Each weight meets the same
-        // value as in the norm mode below, through the same accumulation.
-        const int64_t npix = (int64_t)h->ny * h->nx;
-        const int nrows = h->nrows;
-        float *Cdev = h->norm.as<float>() + nrows;
-        const bool corr = flat || sa || pol;
-        if (h->count_ready && !corr) {
-            AZ_CUDA(cudaMemcpyAsync(h->norm.as<float>(), Cdev, sizeof(float) * nrows, cudaMemcpyDeviceToDevice, s));
-            if (oN) AZ_CUDA(cudaMemcpyAsync(oN, Cdev, sizeof(float) * nrows, cudaMemcpyDeviceToDevice, s));
-            if (oC) AZ_CUDA(cudaMemcpyAsync(oC, Cdev, sizeof(float) * nrows, cudaMemcpyDeviceToDevice, s));
-            return AZ_OK;
+    d.oN = oN;
+    d.norm_rows = 1;
+    if (engine_for(h) == AZ_COPY_TMA && h->tl.fslots >= 1) {
+        // flat * solid angle * polarisation formed per pixel in the tiles of single_kernel: each
+        // weight meets the same value as in the norm mode below, through the same accumulation.
+        // (2167 x 2070 pixels, one array: 34 us; a pass that wrote it to memory and the frames
+        // kernel over it took 39 us with the former layout, 51 us with this one.)
+        const void *const arrs[5] = {nullptr, nullptr, flat, sa, pol};
+        const SgInst one = sg_inst(h, false, arrs);
+        SgNeed need;
+        need.add(h, one.present);
+        SgGeom g;
+        if (sg_geom(need, false, true, g)) {
+            TmaSet tm;
+            AZ_TRY(sg_maps(h, arrs, tm));
+            AZ_TRY((sg_launch<float, AZ_DTYPE_F32, false, true>(one, nullptr, 1, one.n_items, g, tm, s, &h->prof, 1)));
+            return run_phase2<float, MODE_NORM>(d, nullptr, 1, h->nrows, 1, s, &h->prof);
         }
-        const int64_t blocks = std::min<int64_t>((npix + 255) / 256, (int64_t)num_sms() * 8);
-        if (h->tl.norm_frames.bytes < 2 * sizeof(float) * (size_t)npix) {
-            AZ_TRY(h->tl.norm_frames.alloc(2 * sizeof(float) * (size_t)npix));
-            fill_f32_kernel<<<(unsigned)blocks, 256, 0, s>>>(h->tl.norm_frames.as<float>() + npix, npix, 1.f);
-            AZ_CUDA(cudaGetLastError());
+        // larger tiles: that plane in memory, one frame of the frames kernel
+        FrArgs fa{};
+        FrGeom fg;
+        int G = 0;
+        if (fr_plan(h, 1, 0, fa, fg, G)) {
+            const int64_t npix = (int64_t)h->ny * h->nx;
+            if (h->tl.norm_frames.bytes < sizeof(float) * (size_t)npix)
+                AZ_TRY(h->tl.norm_frames.alloc(sizeof(float) * (size_t)npix));
+            {
+                ProfScope ps(&h->prof, 4, s);
+                const int64_t blocks = std::min<int64_t>((npix + 255) / 256, (int64_t)num_sms() * 8);
+                norm_pixels_kernel<<<(unsigned)blocks, 256, 0, s>>>(flat, sa, pol, npix, h->tl.norm_frames.as<float>());
+                AZ_CUDA(cudaGetLastError());
+            }
+            const int rc = frames_v3(h, h->tl.norm_frames.p, 1, AZ_DTYPE_F32, nullptr, 1, s);
+            if (rc != AZ_OK) return rc;
+            return run_phase2<float, MODE_NORM>(d, nullptr, 1, h->nrows, 1, s, &h->prof);
         }
-        {
-            ProfScope ps(&h->prof, 4, s);
-            norm_pixels_kernel<<<(unsigned)blocks, 256, 0, s>>>(flat, sa, pol, npix, h->tl.norm_frames.as<float>());
-            AZ_CUDA(cudaGetLastError());
-        }
-        const int nf = h->count_ready ? 1 : 2;
-        const int rc = frames_v3(h, h->tl.norm_frames.p, nf, AZ_DTYPE_F32, nullptr, 1, s);
-        if (rc == AZ_OK) {
-            d.norm_rows = nf;
-            AZ_TRY((run_phase2<float, MODE_NORM>(d, nullptr, 1, h->nrows, 1, s, &h->prof)));
-            if (nf == 1 && oC) AZ_CUDA(cudaMemcpyAsync(oC, Cdev, sizeof(float) * nrows, cudaMemcpyDeviceToDevice, s));
-            h->count_ready = true;
-            return AZ_OK;
-        }
-        if (rc != AZ_EUNSUPPORTED) return rc;
     }
     const int planes = (flat != nullptr) + (sa != nullptr) + (pol != nullptr);
     StageGeom sg = choose_stage(plane_words_of(h), planes, (uint32_t)h->tl.max_tile_entries, 4,
@@ -2015,19 +2658,14 @@ int batch_pixelnorm(az_integrator *h, const void *frames, int n, int dtype, cons
     TiledLayout &L = h->tl;
     const int64_t npix = (int64_t)h->ny * h->nx;
     const int nrows = h->nrows;
-    // C (and, incidentally, N = C) for the current layout
-    if (!h->count_ready) AZ_TRY(batch_norm(h, nullptr, nullptr, nullptr, nullptr, nullptr, s));
+    // C of the current layout
     const float *Cdev = h->norm.as<float>() + nrows;
     if (oC) AZ_CUDA(cudaMemcpyAsync(oC, Cdev, sizeof(float) * nrows, cudaMemcpyDeviceToDevice, s));
     if (n == 0) return AZ_OK;
     // per-pixel normalisation, per-entry corrected weights and darks
     const int64_t pblocks = std::min<int64_t>((npix + 255) / 256, (int64_t)num_sms() * 8);
     const int64_t eblocks = std::max<int64_t>(1, std::min<int64_t>((L.f_entries + 255) / 256, (int64_t)num_sms() * 8));
-    if (L.norm_frames.bytes < 2 * sizeof(float) * (size_t)npix) {
-        AZ_TRY(L.norm_frames.alloc(2 * sizeof(float) * (size_t)npix));
-        fill_f32_kernel<<<(unsigned)pblocks, 256, 0, s>>>(L.norm_frames.as<float>() + npix, npix, 1.f);
-        AZ_CUDA(cudaGetLastError());
-    }
+    if (L.norm_frames.bytes < sizeof(float) * (size_t)npix) AZ_TRY(L.norm_frames.alloc(sizeof(float) * (size_t)npix));
     if (L.ent_wnorm.bytes < sizeof(float) * (size_t)L.f_entries)
         AZ_TRY(L.ent_wnorm.alloc(sizeof(float) * (size_t)L.f_entries));
     {
@@ -2083,43 +2721,6 @@ int batch_variance(az_integrator *h, const void *frames, int n, int dtype, float
     return AZ_OK;
 }
 
-// One frame through the batched path (TMA engine only; AZ_EUNSUPPORTED, without error
-// text, otherwise).  The N pass needs two frames of partials.
-int forward_batch_one(az_integrator *h, const void *image, int dtype, const float *dark,
-                      const float *flat, const float *sa, const float *pol, float *oI, float *oS,
-                      float *oN, float *oC, cudaStream_t s) {
-    if (engine_for(h) != AZ_COPY_TMA || h->partial_bytes < 2 * sizeof(float) * (size_t)h->tl.nseg)
-        return AZ_EUNSUPPORTED;
-    // C of the current layout, once
-    if (!h->count_ready) AZ_TRY(batch_norm(h, nullptr, nullptr, nullptr, nullptr, nullptr, s));
-    // Three launches: the frame's planes [img - dark; flat * Omega * P], the frames kernel over
-    // them as a batch of two frames (S and N per segment, the accumulation of every other
-    // frame), and phase 2 with C from the cache.  Without flat, solid angle and polarisation
-    // only the first plane is reduced and N = C.
-    const int64_t npix = (int64_t)h->ny * h->nx;
-    const bool corr = flat || sa || pol;
-    if (h->one_planes.bytes < 2 * sizeof(float) * (size_t)npix)
-        AZ_TRY(h->one_planes.alloc(2 * sizeof(float) * (size_t)npix));
-    float *planes = h->one_planes.as<float>();
-    {
-        ProfScope ps(&h->prof, 4, s);
-        const unsigned g = (unsigned)std::min<int64_t>((npix + 255) / 256, (int64_t)num_sms() * 8);
-        const int wn = corr ? 1 : 0;
-        switch (dtype) {
-            case AZ_DTYPE_F32: single_planes_kernel<AZ_DTYPE_F32><<<g, 256, 0, s>>>(image, dark, flat, sa, pol, npix, wn, planes); break;
-            case AZ_DTYPE_U32: single_planes_kernel<AZ_DTYPE_U32><<<g, 256, 0, s>>>(image, dark, flat, sa, pol, npix, wn, planes); break;
-            default: single_planes_kernel<AZ_DTYPE_I32><<<g, 256, 0, s>>>(image, dark, flat, sa, pol, npix, wn, planes); break;
-        }
-        AZ_CUDA(cudaGetLastError());
-    }
-    const int rc = frames_v3(h, planes, corr ? 2 : 1, AZ_DTYPE_F32, nullptr, 2, s);
-    if (rc != AZ_OK) return rc;
-    Inst d = make_inst(h, false);
-    d.oI = oI; d.oS = oS; d.oN = oN; d.oC = oC;
-    d.single_nc = corr ? 1 : 2;
-    return run_phase2<float, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s, &h->prof);
-}
-
 int forward_batch(az_integrator *h, const void *frames, int n, int dtype, const float *dark,
                   const float *flat, const float *sa, const float *pol, float *oI, float *oS,
                   float *oN, float *oC, cudaStream_t s) {
@@ -2173,6 +2774,10 @@ struct MultiPlan {
     int dtype = 0, engine = 0;
     int64_t n_items = 0, n_rows = 0;
     StageGeom sg{};
+    bool single = false, norm = false;  // through single_kernel; with normalisation sums
+    SgGeom sgeo{};
+    SgInst first{};
+    DevBuf sg_dev;       // SgInst [n]
     cudaGraphExec_t exec = nullptr;
     cudaGraph_t graph = nullptr;
 };
@@ -2192,14 +2797,35 @@ int multi_create(az_integrator *const *hs, int n, const void *const *images, int
     P->engine = AZ_COPY_TMA;
     for (int k = 0; k < n; ++k)
         if (engine_for(hs[k]) != AZ_COPY_TMA) P->engine = AZ_COPY_ASYNC;
+    // ... through single_kernel, if two stages of the largest instance fit, else phase1_kernel
+    P->single = P->engine == AZ_COPY_TMA;
+    SgNeed need;
+    std::vector<SgInst> sgi;
+    for (int k = 0; k < n && P->single; ++k) {
+        if (hs[k]->tl.fslots < 1) P->single = false;
+        const void *const arrs[5] = {images[k], darks ? darks[k] : nullptr, flats ? flats[k] : nullptr,
+                                     sas ? sas[k] : nullptr, pols ? pols[k] : nullptr};
+        SgInst d = sg_inst(hs[k], false, arrs);
+        need.add(hs[k], d.present);
+        P->norm = P->norm || (d.present & 28);
+        d.item_begin = sgi.empty() ? 0 : sgi.back().item_begin + sgi.back().n_items;
+        sgi.push_back(d);
+    }
+    if (P->single) P->single = sg_geom(need, false, P->norm, P->sgeo);
     std::vector<TmaSet> maps;
     if (P->engine == AZ_COPY_TMA) {
         maps.resize((size_t)n);
         int rc = P->maps.alloc(sizeof(TmaSet) * (size_t)n);
         for (int k = 0; k < n && rc == AZ_OK; ++k)
-            rc = make_maps(hs[k], AZ_COPY_TMA, images[k], hs[k]->ny, darks ? darks[k] : nullptr,
-                           flats ? flats[k] : nullptr, sas ? sas[k] : nullptr, pols ? pols[k] : nullptr,
-                           maps[(size_t)k]);
+        {
+            const void *const arrs[5] = {images[k], darks ? darks[k] : nullptr, flats ? flats[k] : nullptr,
+                                         sas ? sas[k] : nullptr, pols ? pols[k] : nullptr};
+            rc = P->single ? sg_maps(hs[k], arrs, maps[(size_t)k])
+                           : make_maps(hs[k], AZ_COPY_TMA, images[k], hs[k]->ny, darks ? darks[k] : nullptr,
+                                       flats ? flats[k] : nullptr, sas ? sas[k] : nullptr, pols ? pols[k] : nullptr,
+                                       maps[(size_t)k]);
+            if (P->single) sgi[(size_t)k].maps = &P->maps.as<TmaSet>()[k].m[0][0];
+        }
         if (rc == AZ_OK) {
             cudaError_t e = cudaMemcpy(P->maps.p, maps.data(), sizeof(TmaSet) * (size_t)n, cudaMemcpyHostToDevice);
             if (e != cudaSuccess) rc = fail(AZ_ECUDA, "az_multi_create: %s", cudaGetErrorString(e));
@@ -2223,6 +2849,7 @@ int multi_create(az_integrator *const *hs, int n, const void *const *images, int
         d.oN = oN ? oN[k] : nullptr;
         d.oC = oC ? oC[k] : nullptr;
         if (P->engine == AZ_COPY_TMA) d.maps = &P->maps.as<TmaSet>()[k].m[0][0];
+        if (P->single) d.single_nc = P->norm ? 1 : 2;
         d.item_begin = items;
         d.row_begin = rows;
         items += d.n_items;
@@ -2244,6 +2871,14 @@ int multi_create(az_integrator *const *hs, int n, const void *const *images, int
         cudaError_t e = cudaMemcpy(P->dev.p, P->host.data(), sizeof(Inst) * (size_t)n, cudaMemcpyHostToDevice);
         if (e != cudaSuccess) rc = fail(AZ_ECUDA, "az_multi_create: %s", cudaGetErrorString(e));
     }
+    if (rc == AZ_OK && P->single) {
+        P->first = sgi[0];
+        rc = P->sg_dev.alloc(sizeof(SgInst) * (size_t)n);
+        if (rc == AZ_OK) {
+            cudaError_t e = cudaMemcpy(P->sg_dev.p, sgi.data(), sizeof(SgInst) * (size_t)n, cudaMemcpyHostToDevice);
+            if (e != cudaSuccess) rc = fail(AZ_ECUDA, "az_multi_create: %s", cudaGetErrorString(e));
+        }
+    }
     if (rc != AZ_OK) {
         delete P;
         return rc;
@@ -2256,7 +2891,11 @@ int multi_enqueue(void *plan, cudaStream_t s) {
     MultiPlan *P = static_cast<MultiPlan *>(plan);
     const Inst *dev = P->dev.as<Inst>();
     static TmaSet no_maps;  // zero: the producers read each instance's maps from Inst::maps
-    AZ_TRY((run_phase1_dt<float, float, MODE_SINGLE, 1>(P->dtype, P->engine, P->host[0], dev, P->n, P->n_items, P->sg, no_maps, s)));
+    if (P->single)
+        AZ_TRY((sg_launch_dt<float>(P->dtype, P->norm, P->first, P->sg_dev.as<SgInst>(), P->n, (int)P->n_items, P->sgeo,
+                                    no_maps, s, nullptr)));
+    else
+        AZ_TRY((run_phase1_dt<float, float, MODE_SINGLE, 1>(P->dtype, P->engine, P->host[0], dev, P->n, P->n_items, P->sg, no_maps, s)));
     AZ_TRY((run_phase2<float, MODE_SINGLE>(P->host[0], dev, P->n, P->n_rows, 1, s)));
     return AZ_OK;
 }
