@@ -33,10 +33,10 @@ int alloc_scratch(az_integrator *h, cudaStream_t s) {
     const size_t single = 3 * nseg * sizeof(double);
     const size_t frames = (size_t)kMaxFramesPerLaunch * nseg * sizeof(float);
     h->partial_bytes = std::max(single, frames);
-    AZ_TRY(h->partial.alloc(h->partial_bytes));
-    AZ_TRY(h->norm.alloc(sizeof(float) * 2 * (size_t)h->nrows));
-    AZ_TRY(h->count64.alloc(sizeof(double) * (size_t)h->nrows));
-    AZ_TRY(h->adj.alloc(sizeof(double) * 2 * (size_t)h->nrows));
+    AZ_TRY(alloc_parts(h->slab_scratch, {{&h->partial, h->partial_bytes},
+                                         {&h->norm, sizeof(float) * 2 * (size_t)h->nrows},
+                                         {&h->count64, sizeof(double) * (size_t)h->nrows},
+                                         {&h->adj, sizeof(double) * 2 * (size_t)h->nrows}}));
     return count_layout(h, s);
 }
 
@@ -159,7 +159,10 @@ extern "C" int az_csr_build(const az_geometry *geom, int ny, int nx, int npt_rad
     const bool corners = split != AZ_SPLIT_NONE;
     const bool need_chi = npt_azim > 0 || split == AZ_SPLIT_FULL;
     const int64_t npos = corners ? (int64_t)(ny + 1) * (nx + 1) : (int64_t)ny * nx;
-    DevBuf rad, chi;
+    // scratch of the whole build; at first positions, bin coordinates, counts and their sums
+    ScratchScope scope;
+    AZ_TRY(ScratchScope::reserve((size_t)npos * 8 * (need_chi ? 3 : 2) + (size_t)ny * nx * 16 + ((size_t)2 << 20)));
+    TmpBuf rad, chi;
     AZ_TRY(rad.alloc(sizeof(double) * npos));
     if (need_chi) AZ_TRY(chi.alloc(sizeof(double) * npos));
     AZ_TRY(launch_positions(geom->g, ny, nx, unit, corners ? AZ_WHERE_CORNERS : AZ_WHERE_CENTRES,

@@ -3,9 +3,11 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdarg>
 #include <cstdint>
 #include <cstdio>
+#include <initializer_list>
 #include <vector>
 
 #include "azint.h"
@@ -33,23 +35,21 @@ void clear_error();
         if (rc_ != AZ_OK) return rc_;                                                      \
     } while (0)
 
-// Device allocation owned by the library (freed in the destructor).
+// Device memory of the library: an allocation of its own (freed in the destructor) or a part of
+// another one (view).
 struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;
+    bool own = true;
     DevBuf() = default;
     DevBuf(const DevBuf &) = delete;
     DevBuf &operator=(const DevBuf &) = delete;
-    DevBuf(DevBuf &&o) noexcept : p(o.p), bytes(o.bytes) { o.p = nullptr; o.bytes = 0; }
-    DevBuf &operator=(DevBuf &&o) noexcept {
-        if (this != &o) { release(); p = o.p; bytes = o.bytes; o.p = nullptr; o.bytes = 0; }
-        return *this;
-    }
     ~DevBuf() { release(); }
     void release() {
-        if (p) cudaFree(p);
+        if (p && own) cudaFree(p);
         p = nullptr;
         bytes = 0;
+        own = true;
     }
     int alloc(size_t n) {
         release();
@@ -62,6 +62,108 @@ struct DevBuf {
         bytes = n;
         return AZ_OK;
     }
+    void view(void *q, size_t n) {
+        release();
+        p = q;
+        bytes = n;
+        own = false;
+    }
+    template <class T> T *as() const { return static_cast<T *>(p); }
+};
+
+// Several buffers in one allocation (each 256-byte aligned).  An allocation and its release cost
+// some 30 us each, about as much as all the kernels that fill a 1-Mpixel layout's buffer.
+struct Part {
+    DevBuf *buf;
+    size_t bytes;
+};
+inline int alloc_parts(DevBuf &slab, std::initializer_list<Part> parts) {
+    size_t total = 0;
+    for (const Part &p : parts) {
+        p.buf->release();
+        total += (std::max<size_t>(p.bytes, 16) + 255) & ~(size_t)255;
+    }
+    const int rc = slab.alloc(total);
+    if (rc != AZ_OK) return rc;
+    char *at = slab.as<char>();
+    for (const Part &p : parts) {
+        p.buf->view(at, std::max<size_t>(p.bytes, 16));
+        at += (std::max<size_t>(p.bytes, 16) + 255) & ~(size_t)255;
+    }
+    return AZ_OK;
+}
+
+// Temporary device memory of a build: a few chunks from which TmpBuf::alloc takes pieces in
+// order; a scope gives its pieces back at its end, to be used again by work queued later on the
+// same stream.  The outermost scope of a thread owns the chunks and frees them at its end (after
+// the device has finished with them: cudaFree waits), so nothing outlives a call, and threads do
+// not share chunks.
+struct ScratchScope {
+    struct Pool {
+        static constexpr int kChunks = 64;
+        struct Chunk { char *p; size_t n; } chunks[kChunks] = {};
+        int n_chunks = 0, chunk = 0;
+        size_t off = 0;
+    };
+    static Pool *&current() {
+        static thread_local Pool *pool = nullptr;
+        return pool;
+    }
+    Pool mine;
+    bool outer;
+    int chunk;
+    size_t off;
+    ScratchScope() {
+        Pool *&c = current();
+        outer = c == nullptr;
+        if (outer) c = &mine;
+        chunk = c->chunk;
+        off = c->off;
+    }
+    ~ScratchScope() {
+        Pool *&c = current();
+        c->chunk = chunk;
+        c->off = off;
+        if (outer) {
+            for (int k = 0; k < mine.n_chunks; ++k) cudaFree(mine.chunks[k].p);
+            c = nullptr;
+        }
+    }
+    ScratchScope(const ScratchScope &) = delete;
+    ScratchScope &operator=(const ScratchScope &) = delete;
+    // n bytes in one piece; `room`: how much to allocate at least if a new chunk is needed
+    static int take(size_t n, void **out, size_t room = (size_t)8 << 20) {
+        Pool *c = current();
+        n = (std::max<size_t>(n, 16) + 255) & ~(size_t)255;
+        while (c->chunk < c->n_chunks && c->off + n > c->chunks[c->chunk].n) {
+            ++c->chunk;
+            c->off = 0;
+        }
+        if (c->chunk == c->n_chunks) {
+            if (c->n_chunks == Pool::kChunks) return fail(AZ_ENOMEM, "build scratch: more than %d chunks", Pool::kChunks);
+            void *p = nullptr;
+            const size_t want = std::max(n, room);
+            cudaError_t e = cudaMalloc(&p, want);
+            if (e != cudaSuccess) return fail(AZ_ENOMEM, "cudaMalloc(%zu) failed: %s", want, cudaGetErrorString(e));
+            c->chunks[c->n_chunks++] = {static_cast<char *>(p), want};
+            c->off = 0;
+        }
+        *out = c->chunks[c->chunk].p + c->off;
+        c->off += n;
+        return AZ_OK;
+    }
+    // Room for `n` more bytes in one chunk, ahead of several pieces.
+    static int reserve(size_t n) {
+        void *p = nullptr;
+        const int rc = take(n, &p, n);
+        if (rc == AZ_OK) current()->off -= (std::max<size_t>(n, 16) + 255) & ~(size_t)255;
+        return rc;
+    }
+};
+
+struct TmpBuf {  // within a ScratchScope
+    void *p = nullptr;
+    int alloc(size_t n) { return ScratchScope::take(n, &p); }
     template <class T> T *as() const { return static_cast<T *>(p); }
 };
 
@@ -85,6 +187,7 @@ struct TiledLayout {
     int max_tile_entries = 0;          // padded entry count of the largest tile
     int max_tile_segments = 0;
     int64_t padded_nnz = 0;
+    DevBuf slab_tiles, slab_entries, slab_items;  // hold the buffers below
     DevBuf tile_seg_ptr;    // int32 [ntiles + 1]
     DevBuf tile_ent_ptr;    // int32 [ntiles + 1]  (padded start of each tile's entries)
     DevBuf active_tiles;    // int32 [n_active]
@@ -180,6 +283,7 @@ struct az_integrator {
     int64_t nnz = 0;
     double lo = 0, hi = 0, delta = 0;
     // canonical CSR (rows = bins)
+    azint::DevBuf slab_matrix, slab_scratch;  // hold the matrix, and the scratch below
     azint::DevBuf csr_ptr, csr_idx, csr_w64;
     // pixel-major CSC (columns = pixels) for the adjoint
     azint::DevBuf csc_ptr, csc_row, csc_w64, csc_w32;

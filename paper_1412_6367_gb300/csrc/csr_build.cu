@@ -19,7 +19,7 @@ namespace azint {
 namespace {
 
 constexpr int kScanThreads = 1024;
-constexpr int kScanItems = 4;
+constexpr int kScanItems = 8;
 constexpr int kScanTile = kScanThreads * kScanItems;
 constexpr int kSegEntries = 96;      // longest segment (entries)
 constexpr int32_t kSegFew = 300000;  // segments up to which long runs are cut
@@ -101,7 +101,8 @@ template <class T>
 int exclusive_scan_impl(const T *in, T *out, int64_t n, cudaStream_t s) {
     const int64_t n_out = n + 1;
     const int tiles = blocks_for(n_out, kScanTile);
-    DevBuf sums, offs;
+    ScratchScope scope;
+    TmpBuf sums, offs;
     AZ_TRY(sums.alloc(sizeof(T) * (tiles + 1)));
     AZ_TRY(offs.alloc(sizeof(T) * (tiles + 1)));
     scan_tiles_kernel<T><<<tiles, kScanThreads, 0, s>>>(in, out, n, n_out, sums.as<T>());
@@ -239,31 +240,61 @@ __global__ void range_partial_kernel(const double *__restrict__ rad,
     }
 }
 
-__global__ void range_final_kernel(const double *pmin, const double *pmax, const int *pcnt,
-                                   int nb, double *out, int *cnt_out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__global__ void __launch_bounds__(1024) range_final_kernel(const double *pmin, const double *pmax, const int *pcnt,
+                                                           int nb, double *out, int *cnt_out) {
+    __shared__ double smin[32], smax[32];
+    __shared__ int scnt[32];
     double lo = INFINITY, hi = -INFINITY;
-    long long c = 0;
-    for (int k = 0; k < nb; ++k) {
+    int c = 0;
+    for (int k = threadIdx.x; k < nb; k += blockDim.x) {
         lo = fmin(lo, pmin[k]);
         hi = fmax(hi, pmax[k]);
         c += pcnt[k];
     }
-    out[0] = lo;
-    out[1] = hi;
-    *cnt_out = (int)c;
+    auto fold = [&]() {
+        for (int o = 16; o > 0; o >>= 1) {
+            lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+            c += __shfl_xor_sync(0xffffffffu, c, o);
+        }
+    };
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    fold();
+    if (lane == 0) { smin[w] = lo; smax[w] = hi; scnt[w] = c; }
+    __syncthreads();
+    if (w != 0) return;
+    const bool on = lane < (int)(blockDim.x >> 5);
+    lo = on ? smin[lane] : INFINITY;
+    hi = on ? smax[lane] : -INFINITY;
+    c = on ? scnt[lane] : 0;
+    fold();
+    if (lane == 0) {
+        out[0] = lo;
+        out[1] = hi;
+        *cnt_out = c;
+    }
 }
 
 // ------------------------------------------------------------------------------------
 // per-pixel split (the paper's Sec. 4 rules; readings shared with the documented design)
 // ------------------------------------------------------------------------------------
 struct SplitParams {
-    const double *rad;
+    const double *f;  // (radial value - lo) / delta of every position
     const double *chi;
     const uint8_t *mask;
     int ny, nx, npt, nch, split;
-    double lo, delta, dchi;
+    double dchi;
 };
+
+// Radial bin coordinates of the positions: a division per position here, in place of four per
+// pixel in each of the two passes over the pixels (1043 x 981 pixels, bounding box: count 82 -> 28
+// us, fill 266 -> 201 us, this pass 20 us).
+__global__ void bin_position_kernel(const double *__restrict__ rad, int64_t n, double lo, double delta,
+                                    double *__restrict__ f) {
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
+         k += (int64_t)gridDim.x * blockDim.x)
+        f[k] = (rad[k] - lo) / delta;
+}
 
 __device__ __forceinline__ int bin_none(double f, int npt) {
     const int b = (int)floor(f);
@@ -381,7 +412,7 @@ __device__ __forceinline__ void corner_ids(int nx, int64_t i, int64_t j, int64_t
 template <class Emit>
 __device__ void visit_1d(const SplitParams &P, int64_t p, Emit &emit) {
     if (P.split == AZ_SPLIT_NONE) {
-        const double f = (P.rad[p] - P.lo) / P.delta;
+        const double f = P.f[p];
         emit(bin_none(f, P.npt), 1.0);
         return;
     }
@@ -390,7 +421,7 @@ __device__ void visit_1d(const SplitParams &P, int64_t p, Emit &emit) {
     corner_ids(P.nx, i, j, k);
     double f[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) f[c] = (P.rad[k[c]] - P.lo) / P.delta;
+    for (int c = 0; c < 4; ++c) f[c] = P.f[k[c]];
     double fmin = f[0], fmax = f[0];
 #pragma unroll
     for (int c = 1; c < 4; ++c) {
@@ -434,7 +465,7 @@ template <class Emit>
 __device__ void visit_2d(const SplitParams &P, int64_t p, Emit &emit) {
     const int npt = P.npt, nch = P.nch;
     if (P.split == AZ_SPLIT_NONE) {
-        const double f = (P.rad[p] - P.lo) / P.delta;
+        const double f = P.f[p];
         const double g = (P.chi[p] + 180.0) / P.dchi;
         const int kc = ((int)floor(g)) % nch;
         emit(kc * npt + bin_none(f, npt), 1.0);
@@ -446,7 +477,7 @@ __device__ void visit_2d(const SplitParams &P, int64_t p, Emit &emit) {
     double f[4], ch[4], g[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        f[c] = (P.rad[k[c]] - P.lo) / P.delta;
+        f[c] = P.f[k[c]];
         ch[c] = P.chi[k[c]];
     }
     const bool singular = unwrap_singular(ch);
@@ -598,6 +629,21 @@ __global__ void count_keys_kernel(const int32_t *__restrict__ key, int64_t n,
         atomicAdd(&cnt[key[k]], 1);
 }
 
+// ptr[r] = first position of the ascending keys with key >= r, r = 0 .. nkeys.  (Counting the
+// keys with atomics and a scan took 35 us for 2.6 M keys of 1000 values.)
+template <class K>
+__global__ void key_ptr_kernel(const K *__restrict__ key, int64_t n, int64_t nkeys, int32_t *__restrict__ ptr) {
+    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r <= nkeys;
+         r += (int64_t)gridDim.x * blockDim.x) {
+        int64_t lo = 0, hi = n;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            if ((int64_t)key[mid] < r) lo = mid + 1; else hi = mid;
+        }
+        ptr[r] = (int32_t)lo;
+    }
+}
+
 __global__ void csr_gather_kernel(const int32_t *__restrict__ perm, const int32_t *__restrict__ pix,
                                   const double *__restrict__ w, int32_t *__restrict__ idx_out,
                                   double *__restrict__ w_out, int64_t n) {
@@ -685,19 +731,12 @@ __global__ void split_flags_kernel(const int32_t *__restrict__ seg, const int32_
     }
 }
 
-// Longest segment, and the segment of every matrix entry (in the order of the matrix).
-__global__ void seg_of_kernel(const int32_t *__restrict__ seg, const int32_t *__restrict__ perm,
-                              const int32_t *__restrict__ first, int64_t n, int32_t *__restrict__ seg_of,
-                              int32_t *__restrict__ longest) {
-    int m = 0;
+// The segment of every matrix entry (in the order of the matrix).
+__global__ void seg_of_kernel(const int32_t *__restrict__ seg, const int32_t *__restrict__ perm, int64_t n,
+                              int32_t *__restrict__ seg_of) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        const int s = seg[e];
-        seg_of[perm[e]] = s;
-        m = max(m, first[s + 1] - first[s]);
-    }
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(longest, m);
+         e += (int64_t)gridDim.x * blockDim.x)
+        seg_of[perm[e]] = seg[e];
 }
 
 __global__ void tile_keys_kernel(TileGeom T, const int32_t *__restrict__ idx, int64_t n,
@@ -715,6 +754,7 @@ __global__ void seg_info_kernel(const int32_t *__restrict__ flag, const int32_t 
                                 int32_t *__restrict__ tile) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
          e += (int64_t)gridDim.x * blockDim.x) {
+        if (e == n - 1) first[segid[n]] = (int32_t)n;
         if (!flag[e]) continue;
         const int32_t s = segid[e];
         first[s] = (int32_t)e;
@@ -724,10 +764,10 @@ __global__ void seg_info_kernel(const int32_t *__restrict__ flag, const int32_t 
 }
 
 // Segment lengths rounded up to whole quads of entries.
-__global__ void quad_len_kernel(const int32_t *__restrict__ len, int64_t n, int32_t *__restrict__ plen) {
+__global__ void quad_len_kernel(const int32_t *__restrict__ first, int64_t n, int32_t *__restrict__ plen) {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
          k += (int64_t)gridDim.x * blockDim.x)
-        plen[k] = (len[k] + 3) & ~3;
+        plen[k] = (first[k + 1] - first[k] + 3) & ~3;
 }
 
 // Padded entries of a tile: its segments' quad-rounded lengths, rounded up to 8.
@@ -852,38 +892,36 @@ __global__ void mark_runs_kernel(TileGeom T, const int32_t *__restrict__ ptr, co
     if ((threadIdx.x & 31) == 0 && n) atomicAdd(count, (unsigned long long)n);
 }
 
-__global__ void max_kernel(const int32_t *a, int n, int32_t *out) {
-    __shared__ int32_t sm[32];
-    int32_t m = 0;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) m = max(m, a[k]);
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 1; k < (int)(blockDim.x >> 5); ++k) m = max(m, sm[k]);
-        *out = m;
-    }
-}
-
-__global__ void diff_kernel(const int32_t *ptr, int n, int32_t *out) {
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
-         t += (int64_t)gridDim.x * blockDim.x)
-        out[t] = ptr[t + 1] - ptr[t];
-}
-
 // Work items: a tile's segments (longest first) cut into runs whose entries, counted from
 // the run's first entry rounded down to a multiple of 8, stay within `cap`, and so do those of
 // its units of eight segments (32 entries a step, as many steps as the unit's longest segment has
-// quads); a single longer segment makes an item of its own.  One thread per tile; `fill` = 0
+// quads); a single longer segment makes an item of its own.  One warp per tile; `fill` = 0
 // counts the items, 1 writes (tile, first segment, end segment) for each.
 __global__ void chunk_kernel(const int32_t *__restrict__ tile_seg_ptr, const int32_t *__restrict__ seg_start,
                              const int32_t *__restrict__ seg_end, int ntiles, int cap, int fill,
                              int32_t *__restrict__ count, const int32_t *__restrict__ offs,
                              int32_t *__restrict__ chunks) {
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < ntiles;
-         t += (int64_t)gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; t < ntiles;
+         t += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const int s0 = tile_seg_ptr[t], s1 = tile_seg_ptr[t + 1];
         int n = 0, i = s0;
+        if (s0 < s1) {  // the whole tile, if it fits
+            int padded = 0;
+            for (int b = s0; b < s1; b += 32) {
+                int q = b + lane < s1 && (lane & 7) == 0 ? 8 * (seg_end[b + lane] - seg_start[b + lane]) : 0;
+                for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+                padded += q;
+            }
+            if (padded <= cap && seg_end[s1 - 1] - (seg_start[s0] & ~7) <= cap) {
+                if (fill && lane == 0) {
+                    int32_t *c = chunks + 3 * (size_t)offs[t];
+                    c[0] = (int32_t)t; c[1] = s0; c[2] = s1;
+                }
+                n = 1;
+                i = s1;
+            }
+        }
         while (i < s1) {
             const int e0 = seg_start[i] & ~7;
             int padded = 8 * (seg_end[i] - seg_start[i]);
@@ -893,14 +931,14 @@ __global__ void chunk_kernel(const int32_t *__restrict__ tile_seg_ptr, const int
                 if (b - e0 > cap || padded + more > cap) break;
                 padded += more;
             }
-            if (fill) {
+            if (fill && lane == 0) {
                 int32_t *c = chunks + 3 * (size_t)(offs[t] + n);
                 c[0] = (int32_t)t; c[1] = i; c[2] = j;
             }
             ++n;
             i = j;
         }
-        if (!fill) count[t] = n;
+        if (!fill && lane == 0) count[t] = n;
     }
 }
 
@@ -908,7 +946,8 @@ __global__ void chunk_kernel(const int32_t *__restrict__ tile_seg_ptr, const int
 // and the record's words.
 __global__ void unit_steps_kernel(const int32_t *__restrict__ chunks, int n_items,
                                   const int32_t *__restrict__ seg_start, const int32_t *__restrict__ seg_end,
-                                  int32_t *__restrict__ steps, int32_t *__restrict__ words) {
+                                  int32_t *__restrict__ steps, int32_t *__restrict__ words,
+                                  int32_t *__restrict__ most) {
     const int lane = threadIdx.x & 31;
     for (int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; a < n_items;
          a += ((int64_t)gridDim.x * blockDim.x) >> 5) {
@@ -923,6 +962,8 @@ __global__ void unit_steps_kernel(const int32_t *__restrict__ chunks, int n_item
         if (lane == 0) {
             steps[a] = tot;
             words[a] = ((s1 - s0 + 7) / 8 * 10 + 3) & ~3;
+            atomicMax(most, tot);
+            atomicMax(most + 1, words[a]);
         }
     }
 }
@@ -940,11 +981,14 @@ struct UnitFillArgs {
     int n_items;
 };
 
-// Records, descriptors and entries of the items' units, one warp per item.
+// Records, descriptors and entries of the items' units, four warps per item (every fourth unit
+// each): bound by the latency of a unit's steps, which are read four at a time.
 __global__ void unit_fill_kernel(UnitFillArgs A) {
     const int lane = threadIdx.x & 31, k = lane >> 2, j = lane & 3;
-    for (int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; a < A.n_items;
-         a += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    for (int64_t aw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; aw < 4 * (int64_t)A.n_items;
+         aw += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const int64_t a = aw >> 2;
+        const int part = (int)(aw & 3);
         const int t = A.chunks[3 * a], s0 = A.chunks[3 * a + 1], ns = A.chunks[3 * a + 2] - s0;
         const int64_t base = 32 * (int64_t)A.step_off[a];
         const int off = A.rec_off[a], words = A.rec_off[a + 1] - off, nu = (ns + 7) / 8;
@@ -956,15 +1000,19 @@ __global__ void unit_fill_kernel(UnitFillArgs A) {
             const int e0 = on ? A.seg_start[s] : 0, len = on ? A.seg_end[s] - e0 : 0;
             int n = len >> 2;
             for (int o = 16; o > 2; o >>= 1) n = max(n, __shfl_xor_sync(0xffffffffu, n, o));
-            if (lane == 0) { rec[10 * u] = step; rec[10 * u + 1] = n; }
+            const int at = step;
+            step += n;
+            if ((u & 3) != part) continue;
+            if (lane == 0) { rec[10 * u] = at; rec[10 * u + 1] = n; }
             if (j == 0) rec[10 * u + 2 + k] = on ? A.seg_slot[s] : -1;
             int last = 0;  // the segment's last pixel
             for (int b = 1; b <= 4 && on; ++b) {
                 const int p = A.pix_in[e0 + len - b];
                 if (p >= 0) { last = (int)tile_loc(A.Tf, p); break; }
             }
+#pragma unroll 4
             for (int q = 0; q < n; ++q) {
-                const int64_t o = base + 32 * (int64_t)(step + q) + lane;
+                const int64_t o = base + 32 * (int64_t)(at + q) + lane;
                 const int p = 4 * q < len ? A.pix_in[e0 + 4 * q + j] : -1;
                 A.pix[o] = p;
                 A.w[o] = p >= 0 ? A.w_in[e0 + 4 * q + j] : 0.f;
@@ -973,8 +1021,8 @@ __global__ void unit_fill_kernel(UnitFillArgs A) {
                 A.loc[o] = (uint16_t)l;
                 A.loc1[o] = (uint16_t)(l - l / A.Tf.ss * A.cut);
             }
-            step += n;
         }
+        if (part != 0) continue;
         for (int i = 10 * nu + lane; i < words; i += 32) rec[i] = 0;
         if (lane < 8) {
             const int v[8] = {t, off, words, (int)base, 32 * step, nu, 0, 0};
@@ -1000,26 +1048,30 @@ __global__ void rec_words_kernel(const int32_t *__restrict__ chunks, int n_items
 __global__ void rec_fill_kernel(const int32_t *__restrict__ chunks, int n_items,
                                 const int32_t *__restrict__ seg_start, const int32_t *__restrict__ seg_end,
                                 const int32_t *__restrict__ seg_slot, const int32_t *__restrict__ rec_off,
-                                int32_t *__restrict__ rec, int32_t *__restrict__ desc,
-                                int32_t *__restrict__ item_entries, int32_t *__restrict__ item_segments) {
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n_items;
-         a += (int64_t)gridDim.x * blockDim.x) {
+                                int32_t *__restrict__ rec, int32_t *__restrict__ desc, int32_t *__restrict__ most) {
+    const int lane = threadIdx.x & 31;  // one warp per item
+    for (int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; a < n_items;
+         a += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const int t = chunks[3 * a], s0 = chunks[3 * a + 1], ns = chunks[3 * a + 2] - s0;
         const int e0 = seg_start[s0] & ~7;
         const int ne = ((seg_end[s0 + ns - 1] - e0) + 7) & ~7;
         const int off = rec_off[a], words = rec_off[a + 1] - off;
         int32_t *r = rec + off;
-        r[0] = t; r[1] = ns; r[2] = e0; r[3] = ne;
-        for (int i = 0; i < ns; ++i) r[4 + i] = seg_slot[s0 + i];
         uint16_t *st = reinterpret_cast<uint16_t *>(r + 4 + ns);
-        for (int i = 0; i < ns; ++i) st[i] = (uint16_t)(seg_start[s0 + i] - e0);
-        st[ns] = (uint16_t)(seg_end[s0 + ns - 1] - e0);
-        for (int k = 4 + ns + (ns + 2) / 2; k < words; ++k) r[k] = 0;
-        int32_t *dd = desc + 8 * a;
-        dd[0] = t; dd[1] = off; dd[2] = words; dd[3] = e0;
-        dd[4] = ne; dd[5] = ns; dd[6] = 0; dd[7] = 0;
-        item_entries[a] = ne;
-        item_segments[a] = ns;
+        for (int i = lane; i < ns; i += 32) {
+            r[4 + i] = seg_slot[s0 + i];
+            st[i] = (uint16_t)(seg_start[s0 + i] - e0);
+        }
+        if (lane == 0) {
+            st[ns] = (uint16_t)(seg_end[s0 + ns - 1] - e0);
+            atomicMax(most, ne);
+            atomicMax(most + 1, ns);
+            atomicMax(most + 2, words);
+        }
+        for (int k = 4 + ns + (ns + 2) / 2 + lane; k < words; k += 32) r[k] = 0;
+        const int head[4] = {t, ns, e0, ne}, dd[8] = {t, off, words, e0, ne, ns, 0, 0};
+        if (lane < 4) r[lane] = head[lane];
+        if (lane < 8) desc[8 * a + lane] = dd[lane];
     }
 }
 
@@ -1048,7 +1100,8 @@ int exclusive_scan_i32(const int32_t *in, int32_t *out, int64_t n, cudaStream_t 
 int stable_sort_pairs(uint32_t *keys, int32_t *vals, int64_t n, int key_bits, cudaStream_t s) {
     if (n <= 1) return AZ_OK;
     const int nblocks = blocks_for(n, kRsTile);
-    DevBuf k2, v2, hist, offs;
+    ScratchScope scope;
+    TmpBuf k2, v2, hist, offs;
     AZ_TRY(k2.alloc(sizeof(uint32_t) * n));
     AZ_TRY(v2.alloc(sizeof(int32_t) * n));
     AZ_TRY(hist.alloc(sizeof(int32_t) * 256 * (size_t)nblocks));
@@ -1071,19 +1124,31 @@ int stable_sort_pairs(uint32_t *keys, int32_t *vals, int64_t n, int key_bits, cu
         AZ_CUDA(cudaMemcpyAsync(keys, ka, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
         AZ_CUDA(cudaMemcpyAsync(vals, va, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
     }
-    AZ_CUDA(cudaStreamSynchronize(s));  // k2/v2 are freed on return
     return AZ_OK;
+}
+
+// The matrix's arrays (CSR and CSC) in one allocation.
+static int alloc_matrix(az_integrator *h) {
+    const size_t npix = (size_t)h->ny * (size_t)h->nx, nnz = (size_t)h->nnz;
+    return alloc_parts(h->slab_matrix, {{&h->csc_ptr, sizeof(int32_t) * (npix + 1)},
+                                        {&h->csc_row, sizeof(int32_t) * nnz},
+                                        {&h->csc_w64, sizeof(double) * nnz},
+                                        {&h->csc_w32, sizeof(float) * nnz},
+                                        {&h->csr_ptr, sizeof(int32_t) * ((size_t)h->nrows + 1)},
+                                        {&h->csr_idx, sizeof(int32_t) * nnz},
+                                        {&h->csr_w64, sizeof(double) * nnz}});
 }
 
 int build_integrator(int ny, int nx, const double *rad, const double *chi, int npt_rad,
                      int npt_azim, int unit, int split, const uint8_t *mask, cudaStream_t s,
                      az_integrator *h) {
+    ScratchScope scope;
     const int64_t npix = (int64_t)ny * nx;
     const int corners = split != AZ_SPLIT_NONE;
 
     // 1. radial range over unmasked pixels
     const int rb = std::min<int64_t>(grid_stride_blocks(npix, 256), 1024);
-    DevBuf pmin, pmax, pcnt, rng, rcnt;
+    TmpBuf pmin, pmax, pcnt, rng, rcnt;
     AZ_TRY(pmin.alloc(sizeof(double) * rb));
     AZ_TRY(pmax.alloc(sizeof(double) * rb));
     AZ_TRY(pcnt.alloc(sizeof(int) * rb));
@@ -1092,7 +1157,7 @@ int build_integrator(int ny, int nx, const double *rad, const double *chi, int n
     range_partial_kernel<<<rb, 256, 0, s>>>(rad, mask, ny, nx, corners, pmin.as<double>(),
                                             pmax.as<double>(), pcnt.as<int>());
     AZ_CUDA(cudaGetLastError());
-    range_final_kernel<<<1, 32, 0, s>>>(pmin.as<double>(), pmax.as<double>(), pcnt.as<int>(), rb,
+    range_final_kernel<<<1, 1024, 0, s>>>(pmin.as<double>(), pmax.as<double>(), pcnt.as<int>(), rb,
                                         rng.as<double>(), rcnt.as<int>());
     AZ_CUDA(cudaGetLastError());
     double lohi[2];
@@ -1110,13 +1175,17 @@ int build_integrator(int ny, int nx, const double *rad, const double *chi, int n
     h->lo = lohi[0]; h->hi = lohi[1];
     h->delta = (h->hi - h->lo) / npt_rad;
 
+    const int64_t npos = corners ? (int64_t)(ny + 1) * (nx + 1) : npix;
+    TmpBuf f;
+    AZ_TRY(f.alloc(sizeof(double) * npos));
+    AZ_TRY(launch_gs(bin_position_kernel, npos, s, rad, npos, h->lo, h->delta, f.as<double>()));
     SplitParams P;
-    P.rad = rad; P.chi = chi; P.mask = mask; P.ny = ny; P.nx = nx; P.npt = npt_rad;
-    P.nch = npt_azim; P.split = split; P.lo = h->lo; P.delta = h->delta;
+    P.f = f.as<double>(); P.chi = chi; P.mask = mask; P.ny = ny; P.nx = nx; P.npt = npt_rad;
+    P.nch = npt_azim; P.split = split;
     P.dchi = npt_azim > 0 ? 360.0 / npt_azim : 0.0;
 
     // 2. per-pixel counts -> 3. exclusive scan
-    DevBuf cnt, ptr64;
+    TmpBuf cnt, ptr64;
     AZ_TRY(cnt.alloc(sizeof(int64_t) * npix));
     AZ_TRY(ptr64.alloc(sizeof(int64_t) * (npix + 1)));
     AZ_TRY(launch_gs(count_kernel, npix, s, P, cnt.as<int64_t>()));
@@ -1128,40 +1197,30 @@ int build_integrator(int ny, int nx, const double *rad, const double *chi, int n
     if (nnz > INT32_MAX) return fail(AZ_EOVERFLOW, "csr_build: %lld entries exceed 2^31 - 1", (long long)nnz);
     if (nnz == 0) return fail(AZ_ERANGE, "csr_build: the matrix has no entries");
     h->nnz = nnz;
-    cnt.release();
 
     // 4. pixel-major fill (the "scatter" view, kept as the CSC for the adjoint)
-    AZ_TRY(h->csc_ptr.alloc(sizeof(int32_t) * (npix + 1)));
-    AZ_TRY(h->csc_row.alloc(sizeof(int32_t) * nnz));
-    AZ_TRY(h->csc_w64.alloc(sizeof(double) * nnz));
-    AZ_TRY(h->csc_w32.alloc(sizeof(float) * nnz));
-    DevBuf pix;
+    AZ_TRY(alloc_matrix(h));
+    // the rest of the build takes about 60 bytes of scratch per entry
+    AZ_TRY(ScratchScope::reserve(72 * (size_t)nnz + ((size_t)4 << 20)));
+    TmpBuf pix;
     AZ_TRY(pix.alloc(sizeof(int32_t) * nnz));
     AZ_TRY(launch_gs(fill_kernel, npix, s, P, ptr64.as<int64_t>(), h->csc_row.as<int32_t>(),
                      h->csc_w64.as<double>(), pix.as<int32_t>()));
     AZ_TRY(launch_gs(i64_to_i32_kernel, npix + 1, s, ptr64.as<int64_t>(), h->csc_ptr.as<int32_t>(),
                      npix + 1));
     AZ_TRY(launch_gs(f64_to_f32_kernel, nnz, s, h->csc_w64.as<double>(), h->csc_w32.as<float>(), nnz));
-    ptr64.release();
 
     // 5. stable sort by row -> CSR (the "gather" view, rows ascending by pixel)
-    DevBuf keys, perm, rowcnt;
+    TmpBuf keys, perm;
     AZ_TRY(keys.alloc(sizeof(uint32_t) * nnz));
     AZ_TRY(perm.alloc(sizeof(int32_t) * nnz));
     AZ_TRY(launch_gs(to_u32_kernel, nnz, s, h->csc_row.as<int32_t>(), keys.as<uint32_t>(), nnz));
     AZ_TRY(launch_gs(iota_kernel, nnz, s, perm.as<int32_t>(), nnz));
     AZ_TRY(stable_sort_pairs(keys.as<uint32_t>(), perm.as<int32_t>(), nnz, bits_for(h->nrows - 1), s));
-    AZ_TRY(h->csr_ptr.alloc(sizeof(int32_t) * (h->nrows + 1)));
-    AZ_TRY(h->csr_idx.alloc(sizeof(int32_t) * nnz));
-    AZ_TRY(h->csr_w64.alloc(sizeof(double) * nnz));
     AZ_TRY(launch_gs(csr_gather_kernel, nnz, s, perm.as<int32_t>(), pix.as<int32_t>(),
                      h->csc_w64.as<double>(), h->csr_idx.as<int32_t>(), h->csr_w64.as<double>(), nnz));
-    AZ_TRY(rowcnt.alloc(sizeof(int32_t) * h->nrows));
-    AZ_CUDA(cudaMemsetAsync(rowcnt.p, 0, sizeof(int32_t) * h->nrows, s));
-    AZ_TRY(launch_gs(count_keys_kernel, nnz, s, h->csc_row.as<int32_t>(), nnz, rowcnt.as<int32_t>()));
-    AZ_TRY(exclusive_scan_i32(rowcnt.as<int32_t>(), h->csr_ptr.as<int32_t>(), h->nrows, s));
-    AZ_CUDA(cudaStreamSynchronize(s));
-    return AZ_OK;
+    return launch_gs(key_ptr_kernel<uint32_t>, (int64_t)h->nrows + 1, s, keys.as<uint32_t>(), nnz, (int64_t)h->nrows,
+                     h->csr_ptr.as<int32_t>());
 }
 
 // The integrator's matrix from a host CSR (already checked by the caller): the CSR copied to
@@ -1169,14 +1228,13 @@ int build_integrator(int ny, int nx, const double *rad, const double *chi, int n
 // pixel's entries keep ascending row order), and the count of pixels that have entries.
 int import_csr(az_integrator *h, const int32_t *indptr, const int32_t *indices, const double *data,
                cudaStream_t s) {
+    ScratchScope scope;
     const int64_t npix = (int64_t)h->ny * h->nx, nnz = h->nnz;
-    AZ_TRY(h->csr_ptr.alloc(sizeof(int32_t) * (h->nrows + 1)));
-    AZ_TRY(h->csr_idx.alloc(sizeof(int32_t) * nnz));
-    AZ_TRY(h->csr_w64.alloc(sizeof(double) * nnz));
+    AZ_TRY(alloc_matrix(h));
     AZ_CUDA(cudaMemcpyAsync(h->csr_ptr.p, indptr, sizeof(int32_t) * (h->nrows + 1), cudaMemcpyHostToDevice, s));
     AZ_CUDA(cudaMemcpyAsync(h->csr_idx.p, indices, sizeof(int32_t) * nnz, cudaMemcpyHostToDevice, s));
     AZ_CUDA(cudaMemcpyAsync(h->csr_w64.p, data, sizeof(double) * nnz, cudaMemcpyHostToDevice, s));
-    DevBuf rows, keys, perm, cnt, nonempty;
+    TmpBuf rows, keys, perm, nonempty;
     AZ_TRY(rows.alloc(sizeof(int32_t) * nnz));
     AZ_TRY(keys.alloc(sizeof(uint32_t) * nnz));
     AZ_TRY(perm.alloc(sizeof(int32_t) * nnz));
@@ -1184,17 +1242,10 @@ int import_csr(az_integrator *h, const int32_t *indptr, const int32_t *indices, 
     AZ_TRY(launch_gs(to_u32_kernel, nnz, s, h->csr_idx.as<int32_t>(), keys.as<uint32_t>(), nnz));
     AZ_TRY(launch_gs(iota_kernel, nnz, s, perm.as<int32_t>(), nnz));
     AZ_TRY(stable_sort_pairs(keys.as<uint32_t>(), perm.as<int32_t>(), nnz, bits_for(npix - 1), s));
-    AZ_TRY(h->csc_ptr.alloc(sizeof(int32_t) * (npix + 1)));
-    AZ_TRY(h->csc_row.alloc(sizeof(int32_t) * nnz));
-    AZ_TRY(h->csc_w64.alloc(sizeof(double) * nnz));
-    AZ_TRY(h->csc_w32.alloc(sizeof(float) * nnz));
     AZ_TRY(launch_gs(csr_gather_kernel, nnz, s, perm.as<int32_t>(), rows.as<int32_t>(), h->csr_w64.as<double>(),
                      h->csc_row.as<int32_t>(), h->csc_w64.as<double>(), nnz));
     AZ_TRY(launch_gs(f64_to_f32_kernel, nnz, s, h->csc_w64.as<double>(), h->csc_w32.as<float>(), nnz));
-    AZ_TRY(cnt.alloc(sizeof(int32_t) * npix));
-    AZ_CUDA(cudaMemsetAsync(cnt.p, 0, sizeof(int32_t) * npix, s));
-    AZ_TRY(launch_gs(count_keys_kernel, nnz, s, h->csr_idx.as<int32_t>(), nnz, cnt.as<int32_t>()));
-    AZ_TRY(exclusive_scan_i32(cnt.as<int32_t>(), h->csc_ptr.as<int32_t>(), npix, s));
+    AZ_TRY(launch_gs(key_ptr_kernel<uint32_t>, npix + 1, s, keys.as<uint32_t>(), nnz, npix, h->csc_ptr.as<int32_t>()));
     AZ_TRY(nonempty.alloc(sizeof(int)));
     AZ_CUDA(cudaMemsetAsync(nonempty.p, 0, sizeof(int), s));
     AZ_TRY(launch_gs(nonempty_kernel, npix, s, h->csc_ptr.as<int32_t>(), npix, nonempty.as<int>()));
@@ -1206,17 +1257,18 @@ int import_csr(az_integrator *h, const int32_t *indptr, const int32_t *indices, 
 }
 
 int count_runs(const az_integrator *h, int th, int tw, cudaStream_t s, int64_t *out) {
+    ScratchScope scope;
     *out = -1;
     TileGeom T{};
     T.nx = h->nx; T.th = th; T.tw = tw; T.ntx = (h->nx + tw - 1) / tw;
     const int64_t words = ((int64_t)T.ntx * ((h->ny + th - 1) / th) + 31) / 32;
     const size_t bytes = sizeof(uint32_t) * (size_t)words * (size_t)h->nrows;
     if (bytes > ((size_t)1 << 30)) return AZ_OK;
-    DevBuf bits, count;
+    TmpBuf bits, count;
     AZ_TRY(bits.alloc(bytes));
     AZ_TRY(count.alloc(sizeof(unsigned long long)));
     AZ_CUDA(cudaMemsetAsync(bits.p, 0, bytes, s));
-    AZ_CUDA(cudaMemsetAsync(count.p, 0, count.bytes, s));
+    AZ_CUDA(cudaMemsetAsync(count.p, 0, sizeof(unsigned long long), s));
     mark_runs_kernel<<<std::min(h->nrows, num_sms() * 16), 256, 0, s>>>(T, h->csr_ptr.as<int32_t>(), h->csr_idx.as<int32_t>(),
                                                                       h->nrows, words, bits.as<uint32_t>(),
                                                                       count.as<unsigned long long>());
@@ -1229,6 +1281,7 @@ int count_runs(const az_integrator *h, int th, int tw, cudaStream_t s, int64_t *
 }
 
 int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
+    ScratchScope scope;
     TiledLayout &L = h->tl;
     h->corr_bound = false;   // bound corrections are per layout too (entry order, sums)
     const int64_t nnz = h->nnz;
@@ -1240,10 +1293,13 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     T.ntx = (h->nx + tw - 1) / tw;
     const int nty = (h->ny + th - 1) / th;
     const int ntiles = T.ntx * nty;
+    AZ_TRY(ScratchScope::reserve(66 * (size_t)nnz + ((size_t)2 << 20)));
     if ((int64_t)4 * T.ss + 32 > 65535) return fail(AZ_EINVAL, "tile %dx%d too large", th, tw);
 
     // row of each CSR entry, tile key of each CSR entry, stable sort by tile
-    DevBuf csr_row, tkey, perm, seg_of;
+    int32_t nseg = 0;
+    int cap = kSegEntries;
+    TmpBuf csr_row, tkey, perm, seg_of;
     AZ_TRY(csr_row.alloc(sizeof(int32_t) * nnz));
     AZ_TRY(tkey.alloc(sizeof(uint32_t) * nnz));
     AZ_TRY(perm.alloc(sizeof(int32_t) * nnz));
@@ -1261,41 +1317,36 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
         // up to 59 quads in a 16 x 64 tile of the 6-Mpixel detector, 15 on average); where that
         // makes more than kSegFew segments the pieces are made longer, because the partial sums
         // of a frame (24 bytes a segment in FP64) have to fit the allocation-free entry point.
-        DevBuf f0, id0, seg0, first0, mx0, key2;
+        TmpBuf f0, id0, seg0, first0, key2;
         AZ_TRY(f0.alloc(sizeof(int32_t) * nnz));
         AZ_TRY(id0.alloc(sizeof(int32_t) * (nnz + 1)));
         AZ_TRY(seg0.alloc(sizeof(int32_t) * nnz));
         AZ_TRY(seg_of.alloc(sizeof(int32_t) * nnz));
-        AZ_TRY(mx0.alloc(sizeof(int32_t)));
         AZ_TRY(launch_gs(seg_flags_kernel, nnz, s, tkey.as<uint32_t>(), perm.as<int32_t>(),
                          csr_row.as<int32_t>(), nnz, f0.as<int32_t>()));
-        auto number = [&](int32_t &count) -> int {  // segments of the flags: their ids and firsts
+        AZ_TRY(first0.alloc(sizeof(int32_t) * (nnz + 1)));
+        auto number = [&]() -> int {  // segments of the flags: their ids and firsts
             AZ_TRY(exclusive_scan_i32(f0.as<int32_t>(), id0.as<int32_t>(), nnz, s));
-            AZ_CUDA(cudaMemcpyAsync(&count, id0.as<int32_t>() + nnz, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-            AZ_CUDA(cudaStreamSynchronize(s));
             AZ_TRY(launch_gs(seg_index_kernel, nnz, s, f0.as<int32_t>(), id0.as<int32_t>(), nnz,
                              seg0.as<int32_t>()));
-            AZ_TRY(first0.alloc(sizeof(int32_t) * (count + 1)));
             return launch_gs(seg_first_kernel, nnz + 1, s, f0.as<int32_t>(), id0.as<int32_t>(), nnz,
                              first0.as<int32_t>());
         };
-        int32_t whole = 0, pieces = 0;
-        AZ_TRY(number(whole));
-        for (int cap = kSegEntries;; cap *= 2) {
-            AZ_TRY(launch_gs(split_flags_kernel, nnz, s, seg0.as<int32_t>(), first0.as<int32_t>(), nnz, cap,
-                             f0.as<int32_t>()));
-            AZ_TRY(number(pieces));
-            if (pieces <= std::max(whole, kSegFew) || cap > (1 << 20)) break;
+        int32_t whole = 0;
+        for (;; cap *= 2) {
             AZ_TRY(launch_gs(seg_flags_kernel, nnz, s, tkey.as<uint32_t>(), perm.as<int32_t>(),
                              csr_row.as<int32_t>(), nnz, f0.as<int32_t>()));
-            AZ_TRY(number(whole));
+            AZ_TRY(number());
+            AZ_CUDA(cudaMemcpyAsync(&whole, id0.as<int32_t>() + nnz, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+            AZ_TRY(launch_gs(split_flags_kernel, nnz, s, seg0.as<int32_t>(), first0.as<int32_t>(), nnz, cap,
+                             f0.as<int32_t>()));
+            AZ_TRY(number());
+            AZ_CUDA(cudaMemcpyAsync(&nseg, id0.as<int32_t>() + nnz, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+            AZ_CUDA(cudaStreamSynchronize(s));
+            if (nseg <= std::max(whole, kSegFew) || cap > (1 << 20)) break;
         }
-        AZ_CUDA(cudaMemsetAsync(mx0.p, 0, sizeof(int32_t), s));
-        AZ_TRY(launch_gs(seg_of_kernel, nnz, s, seg0.as<int32_t>(), perm.as<int32_t>(), first0.as<int32_t>(), nnz,
-                         seg_of.as<int32_t>(), mx0.as<int32_t>()));
-        int32_t max_len = 0;
-        AZ_CUDA(cudaMemcpyAsync(&max_len, mx0.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        AZ_CUDA(cudaStreamSynchronize(s));
+        AZ_TRY(launch_gs(seg_of_kernel, nnz, s, seg0.as<int32_t>(), perm.as<int32_t>(), nnz, seg_of.as<int32_t>()));
+        const int32_t max_len = cap;  // no segment is longer
         AZ_TRY(key2.alloc(sizeof(uint32_t) * nnz));
         AZ_TRY(launch_gs(seg_len_key_kernel, nnz, s, seg0.as<int32_t>(), first0.as<int32_t>(), max_len,
                          nnz, key2.as<uint32_t>()));
@@ -1308,45 +1359,36 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     // Segments (runs of one row inside a tile) in the final entry order.  Each segment is
     // padded to whole quads of entries with dummy entries of weight 0 whose location is the
     // zero band after every staged plane (pixel -1), so that reductions read whole quads only.
-    DevBuf flag, segid, segx;
+    TmpBuf flag, segid, segx;
     AZ_TRY(flag.alloc(sizeof(int32_t) * nnz));
     AZ_TRY(segid.alloc(sizeof(int32_t) * (nnz + 1)));
     AZ_TRY(segx.alloc(sizeof(int32_t) * nnz));
     AZ_TRY(launch_gs(seg_change_kernel, nnz, s, seg_of.as<int32_t>(), perm.as<int32_t>(), nnz, flag.as<int32_t>()));
     AZ_TRY(exclusive_scan_i32(flag.as<int32_t>(), segid.as<int32_t>(), nnz, s));
-    int32_t nseg = 0;
-    AZ_CUDA(cudaMemcpyAsync(&nseg, segid.as<int32_t>() + nnz, sizeof(int32_t),
-                            cudaMemcpyDeviceToHost, s));
-    AZ_CUDA(cudaStreamSynchronize(s));
     AZ_TRY(launch_gs(seg_index_kernel, nnz, s, flag.as<int32_t>(), segid.as<int32_t>(), nnz,
                      segx.as<int32_t>()));
-    DevBuf seg_first, seg_row, seg_tile, seg_len, seg_plen, pstart;
-    AZ_TRY(seg_first.alloc(sizeof(int32_t) * nseg));
+    TmpBuf seg_first, seg_row, seg_tile, seg_plen, pstart;
+    AZ_TRY(seg_first.alloc(sizeof(int32_t) * (nseg + 1)));
     AZ_TRY(seg_row.alloc(sizeof(int32_t) * nseg));
     AZ_TRY(seg_tile.alloc(sizeof(int32_t) * nseg));
-    AZ_TRY(seg_len.alloc(sizeof(int32_t) * nseg));
     AZ_TRY(seg_plen.alloc(sizeof(int32_t) * nseg));
     AZ_TRY(pstart.alloc(sizeof(int32_t) * (nseg + 1)));
     AZ_TRY(launch_gs(seg_info_kernel, nnz, s, flag.as<int32_t>(), segid.as<int32_t>(), perm.as<int32_t>(),
                      csr_row.as<int32_t>(), tkey.as<uint32_t>(), nnz, seg_first.as<int32_t>(),
                      seg_row.as<int32_t>(), seg_tile.as<int32_t>()));
-    AZ_CUDA(cudaMemsetAsync(seg_len.p, 0, sizeof(int32_t) * nseg, s));
-    AZ_TRY(launch_gs(count_keys_kernel, nnz, s, segx.as<int32_t>(), nnz, seg_len.as<int32_t>()));
-    AZ_TRY(launch_gs(quad_len_kernel, nseg, s, seg_len.as<int32_t>(), (int64_t)nseg, seg_plen.as<int32_t>()));
+    AZ_TRY(launch_gs(quad_len_kernel, nseg, s, seg_first.as<int32_t>(), (int64_t)nseg, seg_plen.as<int32_t>()));
     AZ_TRY(exclusive_scan_i32(seg_plen.as<int32_t>(), pstart.as<int32_t>(), nseg, s));
 
     // segments per tile -> tile_seg_ptr; padded entries per tile (multiple of 8) -> tile_ent_ptr
-    DevBuf scnt, tpadcnt;
-    AZ_TRY(scnt.alloc(sizeof(int32_t) * ntiles));
+    TmpBuf tpadcnt;
     AZ_TRY(tpadcnt.alloc(sizeof(int32_t) * ntiles));
-    AZ_CUDA(cudaMemsetAsync(scnt.p, 0, sizeof(int32_t) * ntiles, s));
-    AZ_TRY(launch_gs(count_keys_kernel, nseg, s, seg_tile.as<int32_t>(), (int64_t)nseg, scnt.as<int32_t>()));
-    AZ_TRY(L.tile_seg_ptr.alloc(sizeof(int32_t) * (ntiles + 1)));
-    AZ_TRY(exclusive_scan_i32(scnt.as<int32_t>(), L.tile_seg_ptr.as<int32_t>(), ntiles, s));
+    AZ_TRY(alloc_parts(L.slab_tiles, {{&L.tile_seg_ptr, sizeof(int32_t) * (size_t)(ntiles + 1)},
+                                      {&L.tile_ent_ptr, sizeof(int32_t) * (size_t)(ntiles + 1)},
+                                      {&L.row_slot_ptr, sizeof(int32_t) * ((size_t)h->nrows + 1)}}));
+    AZ_TRY(launch_gs(key_ptr_kernel<int32_t>, (int64_t)ntiles + 1, s, seg_tile.as<int32_t>(), (int64_t)nseg,
+                     (int64_t)ntiles, L.tile_seg_ptr.as<int32_t>()));
     AZ_TRY(launch_gs(tile_pad_kernel, ntiles, s, L.tile_seg_ptr.as<int32_t>(), pstart.as<int32_t>(), ntiles,
                      tpadcnt.as<int32_t>()));
-    L.tile_ent_ptr.release();
-    AZ_TRY(L.tile_ent_ptr.alloc(sizeof(int32_t) * (ntiles + 1)));
     AZ_TRY(exclusive_scan_i32(tpadcnt.as<int32_t>(), L.tile_ent_ptr.as<int32_t>(), ntiles, s));
     int32_t padded = 0;
     AZ_CUDA(cudaMemcpyAsync(&padded, L.tile_ent_ptr.as<int32_t>() + ntiles, sizeof(int32_t),
@@ -1354,18 +1396,18 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     AZ_CUDA(cudaStreamSynchronize(s));
 
     // padded entry arrays
-    L.ent_loc.release(); L.ent_w32.release(); L.ent_w64.release();
-    AZ_TRY(L.ent_loc.alloc(sizeof(uint16_t) * (size_t)padded));
-    AZ_TRY(L.ent_w32.alloc(sizeof(float) * (size_t)padded));
-    AZ_TRY(L.ent_w64.alloc(sizeof(double) * (size_t)padded));
-    AZ_TRY(L.ent_pix.alloc(sizeof(int32_t) * (size_t)padded));
+    AZ_TRY(alloc_parts(L.slab_entries, {{&L.ent_loc, sizeof(uint16_t) * (size_t)padded},
+                                        {&L.ent_w32, sizeof(float) * (size_t)padded},
+                                        {&L.ent_w64, sizeof(double) * (size_t)padded},
+                                        {&L.ent_pix, sizeof(int32_t) * (size_t)padded},
+                                        {&L.seg_ent_ptr, sizeof(int32_t) * 2 * (size_t)nseg},  // [start | end]
+                                        {&L.seg_slot, sizeof(int32_t) * (size_t)nseg}}));
     L.ent_dark.release();
     AZ_TRY(launch_gs(fill_u16_kernel, padded, s, L.ent_loc.as<uint16_t>(), (int64_t)padded,
                      (uint16_t)(4 * T.ss)));  // dummies read the zero band
     AZ_CUDA(cudaMemsetAsync(L.ent_w32.p, 0, L.ent_w32.bytes, s));
     AZ_CUDA(cudaMemsetAsync(L.ent_w64.p, 0, L.ent_w64.bytes, s));
     AZ_CUDA(cudaMemsetAsync(L.ent_pix.p, 0xff, L.ent_pix.bytes, s));  // padding entries: -1
-    AZ_TRY(L.seg_ent_ptr.alloc(sizeof(int32_t) * 2 * (size_t)nseg));  // [start | end]
     AZ_TRY(launch_gs(seg_span_kernel, nseg, s, seg_tile.as<int32_t>(), pstart.as<int32_t>(),
                      seg_plen.as<int32_t>(), L.tile_seg_ptr.as<int32_t>(), L.tile_ent_ptr.as<int32_t>(),
                      nseg, L.seg_ent_ptr.as<int32_t>(), L.seg_ent_ptr.as<int32_t>() + nseg));
@@ -1394,19 +1436,15 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
         if (4 * (int64_t)fslot_words > 65535) fslots = 0;
     }
     // slots: segments in row order (stable sort of segment ids by row)
-    DevBuf skey, sperm, rcnt;
+    TmpBuf skey, sperm;
     AZ_TRY(skey.alloc(sizeof(uint32_t) * nseg));
     AZ_TRY(sperm.alloc(sizeof(int32_t) * nseg));
     AZ_TRY(launch_gs(to_u32_kernel, nseg, s, seg_row.as<int32_t>(), skey.as<uint32_t>(), (int64_t)nseg));
     AZ_TRY(launch_gs(iota_kernel, nseg, s, sperm.as<int32_t>(), (int64_t)nseg));
     AZ_TRY(stable_sort_pairs(skey.as<uint32_t>(), sperm.as<int32_t>(), nseg, bits_for(h->nrows - 1), s));
-    AZ_TRY(L.seg_slot.alloc(sizeof(int32_t) * nseg));
     AZ_TRY(launch_gs(scatter_slots_kernel, nseg, s, sperm.as<int32_t>(), nseg, L.seg_slot.as<int32_t>()));
-    AZ_TRY(rcnt.alloc(sizeof(int32_t) * h->nrows));
-    AZ_CUDA(cudaMemsetAsync(rcnt.p, 0, sizeof(int32_t) * h->nrows, s));
-    AZ_TRY(launch_gs(count_keys_kernel, nseg, s, seg_row.as<int32_t>(), (int64_t)nseg, rcnt.as<int32_t>()));
-    AZ_TRY(L.row_slot_ptr.alloc(sizeof(int32_t) * (h->nrows + 1)));
-    AZ_TRY(exclusive_scan_i32(rcnt.as<int32_t>(), L.row_slot_ptr.as<int32_t>(), h->nrows, s));
+    AZ_TRY(launch_gs(key_ptr_kernel<uint32_t>, (int64_t)h->nrows + 1, s, skey.as<uint32_t>(), (int64_t)nseg,
+                     (int64_t)h->nrows, L.row_slot_ptr.as<int32_t>()));
 
     // Work items: a tile whose entries would not fit, twice, beside two stages of four frame
     // planes in shared memory is cut at segment boundaries (about 11.5 bytes of shared memory
@@ -1425,11 +1463,11 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
         }
     }
     const int kItemEntries = (int)std::max<int64_t>(1024, std::min<int64_t>(60000, budget * 2 / 23) & ~7);
-    DevBuf icnt, ioff, chunks, mx;
+    TmpBuf icnt, ioff, chunks, mx;
     AZ_TRY(icnt.alloc(sizeof(int32_t) * ntiles));
     AZ_TRY(ioff.alloc(sizeof(int32_t) * (ntiles + 1)));
     AZ_TRY(mx.alloc(sizeof(int32_t) * 5));
-    AZ_TRY(launch_gs(chunk_kernel, ntiles, s, L.tile_seg_ptr.as<int32_t>(), L.seg_ent_ptr.as<int32_t>(),
+    AZ_TRY(launch_gs(chunk_kernel, 32 * (int64_t)ntiles, s, L.tile_seg_ptr.as<int32_t>(), L.seg_ent_ptr.as<int32_t>(),
                      L.seg_ent_ptr.as<int32_t>() + nseg, ntiles, kItemEntries, 0, icnt.as<int32_t>(),
                      (const int32_t *)nullptr, (int32_t *)nullptr));
     AZ_TRY(exclusive_scan_i32(icnt.as<int32_t>(), ioff.as<int32_t>(), ntiles, s));
@@ -1437,30 +1475,22 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     AZ_CUDA(cudaMemcpyAsync(&n_items, ioff.as<int32_t>() + ntiles, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     AZ_CUDA(cudaStreamSynchronize(s));
     AZ_TRY(chunks.alloc(sizeof(int32_t) * 3 * (size_t)std::max(n_items, 1)));
-    AZ_TRY(launch_gs(chunk_kernel, ntiles, s, L.tile_seg_ptr.as<int32_t>(), L.seg_ent_ptr.as<int32_t>(),
+    AZ_TRY(launch_gs(chunk_kernel, 32 * (int64_t)ntiles, s, L.tile_seg_ptr.as<int32_t>(), L.seg_ent_ptr.as<int32_t>(),
                      L.seg_ent_ptr.as<int32_t>() + nseg, ntiles, kItemEntries, 1, icnt.as<int32_t>(),
                      (const int32_t *)ioff.as<int32_t>(), chunks.as<int32_t>()));
 
     // per-item records and descriptors, and the largest item
-    DevBuf rwords, roff, ient, iseg;
+    TmpBuf rwords, roff;
     AZ_TRY(rwords.alloc(sizeof(int32_t) * std::max(n_items, 1)));
     AZ_TRY(roff.alloc(sizeof(int32_t) * (n_items + 1)));
-    AZ_TRY(ient.alloc(sizeof(int32_t) * std::max(n_items, 1)));
-    AZ_TRY(iseg.alloc(sizeof(int32_t) * std::max(n_items, 1)));
+    AZ_CUDA(cudaMemsetAsync(mx.p, 0, sizeof(int32_t) * 5, s));
     AZ_TRY(launch_gs(rec_words_kernel, n_items, s, chunks.as<int32_t>(), n_items, rwords.as<int32_t>()));
     AZ_TRY(exclusive_scan_i32(rwords.as<int32_t>(), roff.as<int32_t>(), n_items, s));
     int32_t rec_total = 0;
     AZ_CUDA(cudaMemcpyAsync(&rec_total, roff.as<int32_t>() + n_items, sizeof(int32_t),
                             cudaMemcpyDeviceToHost, s));
-    AZ_CUDA(cudaStreamSynchronize(s));
-    AZ_TRY(L.tile_rec.alloc(sizeof(int32_t) * std::max(rec_total, 4)));
-    AZ_TRY(L.tile_desc.alloc(sizeof(int32_t) * 8 * (size_t)std::max(n_items, 1)));
-    AZ_TRY(launch_gs(rec_fill_kernel, n_items, s, chunks.as<int32_t>(), n_items,
-                     L.seg_ent_ptr.as<int32_t>(), L.seg_ent_ptr.as<int32_t>() + nseg,
-                     L.seg_slot.as<int32_t>(), roff.as<int32_t>(), L.tile_rec.as<int32_t>(),
-                     L.tile_desc.as<int32_t>(), ient.as<int32_t>(), iseg.as<int32_t>()));
     // the same items in units for the frames kernel
-    DevBuf usteps, uwords, uoff, uroff;
+    TmpBuf usteps, uwords, uoff, uroff;
     int32_t f_steps = 0, f_words = 0;
     if (fslots) {
         TileGeom Tf = T;
@@ -1472,25 +1502,33 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
         AZ_TRY(uroff.alloc(sizeof(int32_t) * (n_items + 1)));
         AZ_TRY(launch_gs(unit_steps_kernel, 32 * (int64_t)n_items, s, chunks.as<int32_t>(), n_items,
                          L.seg_ent_ptr.as<int32_t>(), L.seg_ent_ptr.as<int32_t>() + nseg, usteps.as<int32_t>(),
-                         uwords.as<int32_t>()));
+                         uwords.as<int32_t>(), mx.as<int32_t>() + 3));
         AZ_TRY(exclusive_scan_i32(usteps.as<int32_t>(), uoff.as<int32_t>(), n_items, s));
         AZ_TRY(exclusive_scan_i32(uwords.as<int32_t>(), uroff.as<int32_t>(), n_items, s));
         AZ_CUDA(cudaMemcpyAsync(&f_steps, uoff.as<int32_t>() + n_items, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
         AZ_CUDA(cudaMemcpyAsync(&f_words, uroff.as<int32_t>() + n_items, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        AZ_CUDA(cudaStreamSynchronize(s));
+    }
+    AZ_CUDA(cudaStreamSynchronize(s));
+    if (fslots) {
         if ((int64_t)f_steps * 32 > INT32_MAX) fslots = 0;
     }
     L.f_entries = fslots ? 32 * (int64_t)f_steps : 0;
-    L.f_desc.release(); L.f_rec.release(); L.f_loc.release(); L.f_w32.release(); L.f_pix.release();
-    L.f_loc1.release(); L.f_w64.release();
+    const size_t ni = (size_t)std::max(n_items, 1), nf = (size_t)L.f_entries, fi = fslots ? 8 * ni : 0;
+    AZ_TRY(alloc_parts(L.slab_items, {{&L.tile_rec, sizeof(int32_t) * (size_t)std::max(rec_total, 4)},
+                                      {&L.tile_desc, sizeof(int32_t) * 8 * ni},
+                                      {&L.active_tiles, sizeof(int32_t) * ni},
+                                      {&L.f_desc, sizeof(int32_t) * fi},
+                                      {&L.f_rec, sizeof(int32_t) * (size_t)f_words},
+                                      {&L.f_loc, sizeof(uint16_t) * nf},
+                                      {&L.f_loc1, sizeof(uint16_t) * nf},
+                                      {&L.f_w32, sizeof(float) * nf},
+                                      {&L.f_w64, sizeof(double) * nf},
+                                      {&L.f_pix, sizeof(int32_t) * nf}}));
+    AZ_TRY(launch_gs(rec_fill_kernel, 32 * (int64_t)n_items, s, chunks.as<int32_t>(), n_items,
+                     L.seg_ent_ptr.as<int32_t>(), L.seg_ent_ptr.as<int32_t>() + nseg,
+                     L.seg_slot.as<int32_t>(), roff.as<int32_t>(), L.tile_rec.as<int32_t>(),
+                     L.tile_desc.as<int32_t>(), mx.as<int32_t>()));
     if (fslots) {
-        AZ_TRY(L.f_desc.alloc(sizeof(int32_t) * 8 * (size_t)std::max(n_items, 1)));
-        AZ_TRY(L.f_rec.alloc(sizeof(int32_t) * (size_t)std::max(f_words, 4)));
-        AZ_TRY(L.f_loc.alloc(sizeof(uint16_t) * (size_t)L.f_entries));
-        AZ_TRY(L.f_w32.alloc(sizeof(float) * (size_t)L.f_entries));
-        AZ_TRY(L.f_pix.alloc(sizeof(int32_t) * (size_t)L.f_entries));
-        AZ_TRY(L.f_loc1.alloc(sizeof(uint16_t) * (size_t)L.f_entries));
-        AZ_TRY(L.f_w64.alloc(sizeof(double) * (size_t)L.f_entries));
         UnitFillArgs U;
         U.Tf = T; U.Tf.srow = srow_f; U.Tf.ss = fslots * fslot_words;
         U.chunks = chunks.as<int32_t>(); U.seg_start = L.seg_ent_ptr.as<int32_t>();
@@ -1501,18 +1539,8 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
         U.loc1 = L.f_loc1.as<uint16_t>(); U.w64 = L.f_w64.as<double>(); U.w64_in = L.ent_w64.as<double>();
         U.cut = (fslots - 1) * fslot_words;
         U.n_items = n_items;
-        AZ_TRY(launch_gs(unit_fill_kernel, 32 * (int64_t)n_items, s, U));
-        max_kernel<<<1, 1024, 0, s>>>(usteps.as<int32_t>(), n_items, mx.as<int32_t>() + 3);
-        AZ_CUDA(cudaGetLastError());
-        max_kernel<<<1, 1024, 0, s>>>(uwords.as<int32_t>(), n_items, mx.as<int32_t>() + 4);
-        AZ_CUDA(cudaGetLastError());
+        AZ_TRY(launch_gs(unit_fill_kernel, 128 * (int64_t)n_items, s, U));
     }
-    max_kernel<<<1, 1024, 0, s>>>(ient.as<int32_t>(), n_items, mx.as<int32_t>());
-    AZ_CUDA(cudaGetLastError());
-    max_kernel<<<1, 1024, 0, s>>>(iseg.as<int32_t>(), n_items, mx.as<int32_t>() + 1);
-    AZ_CUDA(cudaGetLastError());
-    max_kernel<<<1, 1024, 0, s>>>(rwords.as<int32_t>(), n_items, mx.as<int32_t>() + 2);
-    AZ_CUDA(cudaGetLastError());
     int32_t maxes[5] = {};
     AZ_CUDA(cudaMemcpyAsync(maxes, mx.p, sizeof(maxes), cudaMemcpyDeviceToHost, s));
     AZ_CUDA(cudaStreamSynchronize(s));
@@ -1520,7 +1548,6 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
         return fail(AZ_EUNSUPPORTED, "a %dx%d tile item holds %d matrix entries (limit 65535): use smaller tiles",
                     th, tw, maxes[0]);
     // tile of every item (kept for accounting)
-    AZ_TRY(L.active_tiles.alloc(sizeof(int32_t) * std::max(n_items, 1)));
     if (n_items > 0)
         AZ_CUDA(cudaMemcpy2DAsync(L.active_tiles.p, sizeof(int32_t), chunks.p, 3 * sizeof(int32_t),
                                   sizeof(int32_t), (size_t)n_items, cudaMemcpyDeviceToDevice, s));

