@@ -486,9 +486,10 @@ int az_profile_read(az_integrator *h, az_profile *out);
  * one class are 16 * width bytes apart, which meets the tensor-map stride rule for any
  * width); it applies to tiles up to 236 pixels wide, wider tiles use AZ_COPY_ASYNC.
  * AZ_COPY_ASYNC issues 16-byte cp.async copies spread over the producer warps.  Results are
- * identical; only speed differs.  Defaults: 8 x 120 pixel tiles, 16 x 64 for dense 1D matrices (2.1
- * entries per pixel and more) and 48 x 40 for 2D integrators (larger ones where the segments
- * would otherwise pass az_integrate_noalloc's limit); 8 frames per pass. */
+ * identical; only speed differs.  Default tiles follow the matrix's entries per pixel: 8 x 120
+ * pixels below 2.1 (1D) or 48 x 40 below 2.4 (2D), then 16 x 64, 16 x 40 from 5, 16 x 24 from 10
+ * and 8 x 24 from 20 (larger ones where the segments would otherwise pass az_integrate_noalloc's
+ * limit); 8 frames per pass. */
 int az_set_copy_engine(az_integrator *h, int engine);
 
 /* Thread-local message of the last failing call on this thread ("" if none). */

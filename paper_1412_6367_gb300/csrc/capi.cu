@@ -48,12 +48,17 @@ int finish_build(az_integrator *h, cudaStream_t s) {
     // entries per pixel), 273 and 244 us (37 frames of 2167 x 2070, 2.6), 45 and 40 us (24 variances
     // of 1043 x 981, 2.8).  2D: 48 x 40 (500 x 360 bins of 2048 x 2048 pixels, 16 frames and one:
     // 91 and 29 us; 32 x 64, where only four frames fit a stage: 109 and 28 us; 24 x 56: 80 and 37).
-    int th = 48, tw = 40;
-    if (h->npt_azim == 0) {
-        const bool dense = (double)h->nnz >= 2.1 * (double)h->n_unmasked;
-        th = dense ? 16 : 8;
-        tw = dense ? 64 : 120;
-    }
+    // Denser matrices get smaller tiles, so that the stages of the FP64 single-frame kernel (14
+    // bytes an entry) still fit and no tile is cut: 962 x 972 pixels with 7.1 entries per pixel,
+    // 16 x 40 against 16 x 64: FP64 frame 80 and 260 us, 16 frames 134 and 173 us; with 4.0 entries
+    // 48 and 59, 92 and 89 us.
+    const double density = (double)h->nnz / (double)std::max(h->n_unmasked, 1);
+    int th = 8, tw = 24;
+    if (density < 20.0) { th = 16; tw = 24; }
+    if (density < 10.0) { th = 16; tw = 40; }
+    if (density < 5.0) { th = 16; tw = 64; }
+    if (h->npt_azim == 0 && density < 2.1) { th = 8; tw = 120; }
+    if (h->npt_azim > 0 && density < 2.4) { th = 48; tw = 40; }
     if (build_tiled_layout(h, th, tw, s) != AZ_OK) {  // a denser matrix: smaller tiles
         th = 8;
         tw = 64;

@@ -62,3 +62,11 @@ def test_phases_and_frames_per_pass(off, fpp):
 @pytest.mark.parametrize("npt,azim", [(1, 0), (3, 0), (20, 90)])
 def test_long_rows_and_heavy_tiles(npt, azim):
     _check(Case(small_workload(130, 140, split=2, npt=npt, npt_azim=azim, seed=9)), (48, 40), (1, 4, 11))
+
+
+# entries per pixel from about 1.5 to 25: every default tile
+@pytest.mark.parametrize("npt,azim", [(60, 0), (200, 0), (600, 0), (1300, 0), (3500, 0), (20, 30), (150, 300)])
+def test_default_tiles_by_density(npt, azim):
+    c = Case(small_workload(97, 110, split=1, npt=npt, npt_azim=azim, seed=10))
+    i = c.gpu_from_oracle_positions().info
+    _check(c, (i["tile_h"], i["tile_w"]), (1, 3, 9))
