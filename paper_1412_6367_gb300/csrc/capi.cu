@@ -69,11 +69,16 @@ int finish_build(az_integrator *h, cudaStream_t s) {
     // tiles if they bring it below.
     const int64_t most = (int64_t)AZ_NOALLOC_SCRATCH_BYTES / (3 * (int64_t)sizeof(double));
     if (h->tl.nseg > most) {
-        const int bh = h->npt_azim > 0 ? 32 : 8, bw = h->npt_azim > 0 ? 64 : 224;
-        int64_t runs = 0;
-        AZ_TRY(count_runs(h, bh, bw, s, &runs));
-        if (runs >= 0 && (runs <= most || (h->tl.nseg > 2 * most && runs <= 2 * most)))
-            AZ_TRY(build_tiled_layout(h, bh, bw, s));
+        const int larger[2][2][2] = {{{16, 64}, {8, 224}}, {{32, 64}, {32, 64}}};
+        for (int k = 0; k < 2; ++k) {
+            const int *t = larger[h->npt_azim > 0][k];
+            int64_t runs = 0;
+            AZ_TRY(count_runs(h, t[0], t[1], s, &runs));
+            if (runs >= 0 && (runs <= most || (h->tl.nseg > 2 * most && runs <= 2 * most))) {
+                AZ_TRY(build_tiled_layout(h, t[0], t[1], s));
+                break;
+            }
+        }
     }
     h->frames_per_pass = 8;
     h->rows_per_warp = 32 / h->frames_per_pass;

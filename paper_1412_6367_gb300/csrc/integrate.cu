@@ -714,21 +714,20 @@ phase1_kernel(const __grid_constant__ Inst single, const Inst *__restrict__ mult
 // issues every copy (bulk and tensor TMA); 15 consumer warps reduce.
 //
 // What bounds it (64 frames of 2527 x 2463 pixels, 9.63 M entries): staging alone runs at the
-// copy peak (246 us a launch), the consumers alone take 320 us, both together 340 us; the kernel
-// before this one took 468 us.  The consumers are held by shared memory (38 wavefronts per 256
-// products, half of them bank conflicts of the gathers) and by the FP32 pipe, which a packed
-// f32x2 instruction occupies for two cycles (1.45 us of pipe time per frame).  Why this form:
+// copy peak (246 us a launch), with the consumers it takes 343 us; the kernel before this one took
+// 468 us.  The consumers are held by shared memory (77% of its throughput; 43% of the wavefronts
+// are bank conflicts of the gathers) and by the FP32 pipe, which a packed f32x2 instruction
+// occupies for two cycles.  Why this form:
 //   - a lane sums one accumulator of one segment for all frames of a stage, so a unit of eight
 //     segments reads each entry once for eight frames: 7 words of metadata and 16 gathers per 256
-//     products.  One lane per (segment, frame) read 40 bytes of metadata per quad and frame group
-//     (18 wavefronts per 128 products); four frames per lane measured 12% slower than eight.
+//     products.  One lane per (segment, frame) read 40 bytes of metadata per quad and frame group;
+//     four frames per lane measured 7% slower than eight, two 28%.
 //   - a box of depth D moves one row class of D frames: four copies per 8-frame stage instead of
 //     sixteen, which takes the issue of the copies off the critical path.
 //   - consumers take units from one counter across stages and items instead of passing every
 //     stage together, so nobody waits for the slowest warp of a stage (11 to 15 consumer warps
-//     are within 2%, 23 are 5% slower).
-//   - f32x2 has no subtraction: sub.rn.f32x2 costs two more instructions, a multiply-add by -1
-//     does not.
+//     are within 3%, 19 are 4% slower).
+//   - sub.rn.f32x2 takes extra instructions, a multiply-add by -1 does not.
 constexpr int kFrConsumers = 15;
 constexpr int kFrThreads = 32 * (1 + kFrConsumers);
 constexpr int kFrMaxStages = 16;
