@@ -622,13 +622,6 @@ __global__ void i64_to_i32_kernel(const int64_t *in, int32_t *out, int64_t n) {
         out[k] = (int32_t)in[k];
 }
 
-__global__ void count_keys_kernel(const int32_t *__restrict__ key, int64_t n,
-                                  int32_t *__restrict__ cnt) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-         k += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&cnt[key[k]], 1);
-}
-
 // ptr[r] = first position of the ascending keys with key >= r, r = 0 .. nkeys.  (Counting the
 // keys with atomics and a scan took 35 us for 2.6 M keys of 1000 values.)
 template <class K>
