@@ -1009,7 +1009,11 @@ __global__ void unit_fill_kernel(UnitFillArgs A) {
                 const int p = 4 * q < len ? A.pix_in[e0 + 4 * q + j] : -1;
                 A.pix[o] = p;
                 A.w[o] = p >= 0 ? A.w_in[e0 + 4 * q + j] : 0.f;
-                A.w64[o] = p >= 0 ? A.w64_in[e0 + 4 * q + j] : -0.0;
+                // -0 is what marks the places past a segment's end: a matrix's own -0 (an imported
+                // one may hold it) becomes +0, whose products change no sum, and is NaN at an
+                // infinite pixel as any zero weight is
+                const double w = p >= 0 ? A.w64_in[e0 + 4 * q + j] : -0.0;
+                A.w64[o] = p >= 0 && w == 0.0 ? 0.0 : w;
                 const int l = p >= 0 ? (int)tile_loc(A.Tf, p) : last;
                 A.loc[o] = (uint16_t)l;
                 A.loc1[o] = (uint16_t)(l - l / A.Tf.ss * A.cut);

@@ -1388,8 +1388,9 @@ __device__ __forceinline__ void sg_unit(const SgInst &d, const SgGeom &sg, const
             double2 v;
             if (N) v = reinterpret_cast<const double2 *>(xn)[o];
             else v = make_double2(xn[o], 0.0);
-            // past the segment's end (weight -0): the value may be infinite
-            if (__double2hiint(w) == (int)0x80000000) v = make_double2(0.0, 0.0);
+            // past the segment's end (weight -0, all its bits: the upper half alone is also that
+            // of negative subnormal weights): the value may be infinite
+            if (__double_as_longlong(w) == (long long)(1ull << 63)) v = make_double2(0.0, 0.0);
             if (X) S = __fma_rn(w, v.x, S);
             if (N) M = __fma_rn(w, v.y, M);
         }
