@@ -394,7 +394,9 @@ int az_autotune(az_integrator *h, int n_trial_frames, az_stream_t stream, double
 
 /* Set the tuning by hand (0 keeps the current value).  tile_w must be a multiple of 4;
  * frames_per_pass is 1, 2, 4, 8, 16 or 32 and rows_per_warp = 32 / frames_per_pass (either
- * may be given; both must agree). */
+ * may be given; both must agree).  If the layout of the new tiles cannot be built (AZ_ENOMEM,
+ * AZ_EUNSUPPORTED), the one there was is built again; if that fails too, the calls that need a
+ * tiled layout return AZ_EINVAL until az_set_tuning or az_autotune has made one. */
 int az_set_tuning(az_integrator *h, int tile_h, int tile_w, int rows_per_warp,
                   int frames_per_pass);
 
@@ -458,6 +460,13 @@ int az_set_layout(az_integrator *h, int layout);
  * or a bound outside the range, before any launch.
  */
 int az_selftest_wait(int arrive, int64_t limit_cycles, int *out_status, az_stream_t stream);
+
+/*
+ * Allocation failures on request, for tests of the error paths: of the calling thread's next
+ * device allocations by this library, `after` succeed and the `count` after them fail as a full
+ * device makes them fail (AZ_ENOMEM).  count == 0 ends it.  Host-only.
+ */
+int az_selftest_alloc(int64_t after, int64_t count);
 
 /* ---- kernel timing --------------------------------------------------------------------- */
 

@@ -473,6 +473,12 @@ def selftest_wait(arrive=False, limit_cycles=2_000_000, device=None):
     return st.value
 
 
+def selftest_alloc(after=0, count=0):
+    """Of this thread's next device allocations by the library, `after` succeed and the `count`
+    after them fail with AZ_ENOMEM (az_selftest_alloc; count 0 ends it)."""
+    check(L.load().az_selftest_alloc(int(after), int(count)))
+
+
 class MultiPlan:
     """Several integrators of uneven shape in one persistent launch (az_multi_create)."""
 

@@ -40,6 +40,25 @@ int alloc_scratch(az_integrator *h, cudaStream_t s) {
     return count_layout(h, s);
 }
 
+// The layout of th x tw tiles with the scratch that goes with it.
+int set_tiles(az_integrator *h, int th, int tw, cudaStream_t s) {
+    AZ_TRY(build_tiled_layout(h, th, tw, s));  // (clears layout_ok once it changes anything)
+    AZ_TRY(alloc_scratch(h, s));
+    h->layout_ok = true;
+    return AZ_OK;
+}
+
+// After a failed set_tiles: back to the tiles there were.  The error text stays the failure's; if
+// these do not fit any more either, the integrator stays without a layout.
+void restore_tiles(az_integrator *h, int th, int tw, cudaStream_t s) {
+    if (h->layout_ok) return;
+    char text[sizeof(g_err)];
+    memcpy(text, g_err, sizeof(text));
+    cudaStreamSynchronize(s);
+    (void)set_tiles(h, th, tw, s);
+    memcpy(g_err, text, sizeof(text));
+}
+
 int finish_build(az_integrator *h, cudaStream_t s) {
     // Default tiles; az_autotune refines them per matrix.  1D: 8 x 120, or 16 x 64 from 2.1 entries
     // per pixel on -- taller tiles make fewer, longer segments, which pays where the entries set
@@ -83,6 +102,7 @@ int finish_build(az_integrator *h, cudaStream_t s) {
     h->frames_per_pass = 8;
     h->rows_per_warp = 32 / h->frames_per_pass;
     AZ_TRY(alloc_scratch(h, s));
+    h->layout_ok = true;
     AZ_TRY(h->status.alloc(sizeof(int)));
     AZ_CUDA(cudaMemsetAsync(h->status.p, 0, sizeof(int), s));
     AZ_CUDA(cudaStreamSynchronize(s));
@@ -119,6 +139,12 @@ int build_common(int ny, int nx, const double *rad, const double *chi, int npt_r
 }
 
 }  // namespace
+
+int check_layout(const az_integrator *h, const char *who) {
+    if (h->layout_ok) return AZ_OK;
+    return fail(AZ_EINVAL, "%s: the integrator has no tiled layout since a failed az_set_tuning or az_autotune: "
+                           "call az_set_tuning again", who);
+}
 
 int check_forward(const az_integrator *h, const void *image, int dtype, const float *dark,
                   const float *flat, const float *sa, const float *pol, const char *who) {
@@ -330,6 +356,7 @@ static int integrate_common(const az_integrator *h, const void *image, int dtype
     const_cast<az_integrator *>(h)->last_stream = (cudaStream_t)stream;
     if (h->layout == AZ_LAYOUT_LUT)
         return lut_forward(h, image, dtype, dark, flat, sa, pol, precision, oI, oS, oN, oC, (cudaStream_t)stream);
+    AZ_TRY(check_layout(h, who));
     return forward_single(h, image, dtype, dark, flat, sa, pol, precision, oI, oS, oN, oC,
                           (cudaStream_t)stream);
 }
@@ -365,6 +392,7 @@ extern "C" int az_integrate_batch(az_integrator *h, const void *frames_dev, int 
     static const uint32_t no_frames = 0;
     AZ_TRY(check_forward(h, n_frames == 0 ? &no_frames : frames_dev, image_dtype, dark, flat,
                          solid_angle, polarization, "az_integrate_batch"));
+    AZ_TRY(check_layout(h, "az_integrate_batch"));
     h->last_stream = (cudaStream_t)stream;
     if (n_frames == 0 && !out_sum_norm && !out_count) return AZ_OK;
     return forward_batch(h, frames_dev, n_frames, image_dtype, dark, flat, solid_angle,
@@ -379,6 +407,7 @@ extern "C" int az_set_corrections(az_integrator *h, const float *dark, const flo
     static const uint32_t no_frames = 0;
     AZ_TRY(check_forward(h, &no_frames, AZ_DTYPE_F32, dark, flat, solid_angle, polarization,
                          "az_set_corrections"));
+    AZ_TRY(check_layout(h, "az_set_corrections"));
     h->last_stream = (cudaStream_t)stream;
     return bind_corrections(h, dark, flat, solid_angle, polarization, (cudaStream_t)stream);
 }
@@ -391,6 +420,7 @@ extern "C" int az_integrate_batch_bound(az_integrator *h, const void *frames_dev
     static const uint32_t no_frames = 0;
     AZ_TRY(check_forward(h, n_frames == 0 ? &no_frames : frames_dev, image_dtype, nullptr, nullptr,
                          nullptr, nullptr, "az_integrate_batch_bound"));
+    AZ_TRY(check_layout(h, "az_integrate_batch_bound"));
     h->last_stream = (cudaStream_t)stream;
     return forward_batch_bound(h, frames_dev, n_frames, image_dtype, out_I, out_sum_signal, out_sum_norm,
                                out_count, (cudaStream_t)stream);
@@ -406,6 +436,7 @@ extern "C" int az_integrate_batch_pixelnorm(az_integrator *h, const void *frames
     static const uint32_t no_frames = 0;
     AZ_TRY(check_forward(h, n_frames == 0 ? &no_frames : frames_dev, image_dtype, dark, flat,
                          solid_angle, polarization, "az_integrate_batch_pixelnorm"));
+    AZ_TRY(check_layout(h, "az_integrate_batch_pixelnorm"));
     h->last_stream = (cudaStream_t)stream;
     return batch_pixelnorm(h, frames_dev, n_frames, image_dtype, dark, flat, solid_angle, polarization,
                            out_I, out_sum_corrected, out_count, (cudaStream_t)stream);
@@ -419,6 +450,7 @@ extern "C" int az_integrate_variance(az_integrator *h, const void *frames_dev, i
     AZ_TRY(check_forward(h, frames_dev, image_dtype, nullptr, nullptr, nullptr, nullptr,
                          "az_integrate_variance"));
     if (!out_sum_variance) return fail(AZ_EINVAL, "az_integrate_variance: NULL output");
+    AZ_TRY(check_layout(h, "az_integrate_variance"));
     h->last_stream = (cudaStream_t)stream;
     return batch_variance(h, frames_dev, n_frames, image_dtype, out_sum_variance, (cudaStream_t)stream);
 }
@@ -433,6 +465,7 @@ extern "C" int az_integrate_batch_host(az_integrator *h, const void *frames_host
                          "az_integrate_batch_host"));
     if (n_frames < 0) return fail(AZ_ESHAPE, "az_integrate_batch_host: n_frames < 0");
     if (n_frames == 0) return AZ_OK;
+    AZ_TRY(check_layout(h, "az_integrate_batch_host"));
     cudaStream_t s = (cudaStream_t)stream;
     const size_t fbytes = (size_t)h->ny * h->nx * 4u;
     const size_t obytes = (size_t)h->nrows * sizeof(float);
@@ -506,6 +539,7 @@ extern "C" int az_integrate_backward(const az_integrator *h, const void *grad_I,
     if (precision != AZ_PREC_FP64 && precision != AZ_PREC_FP32_COMP)
         return fail(AZ_EINVAL, "az_integrate_backward: bad precision %d", precision);
     if (!out_grad_image && !out_grad_flat) return AZ_OK;
+    AZ_TRY(check_layout(h, "az_integrate_backward"));  // (its scratch)
     const_cast<az_integrator *>(h)->last_stream = (cudaStream_t)stream;
     return backward(h, grad_I, I, sum_norm, solid_angle, polarization, precision, out_grad_image,
                     out_grad_flat, (cudaStream_t)stream);
@@ -527,6 +561,7 @@ extern "C" int az_multi_create(az_integrator *const *handles, int n, const void 
         AZ_TRY(check_forward(handles[k], images[k], image_dtype, darks ? darks[k] : nullptr,
                              flats ? flats[k] : nullptr, solid_angles ? solid_angles[k] : nullptr,
                              polarizations ? polarizations[k] : nullptr, "az_multi_create"));
+        AZ_TRY(check_layout(handles[k], "az_multi_create"));
     }
     az_multi *m = new (std::nothrow) az_multi;
     if (!m) return fail(AZ_ENOMEM, "az_multi_create: out of host memory");
@@ -604,12 +639,17 @@ extern "C" int az_set_tuning(az_integrator *h, int tile_h, int tile_w, int rows_
     if (rows_per_warp && frames_per_pass && rows_per_warp * frames_per_pass != 32)
         return fail(AZ_EINVAL, "az_set_tuning: rows_per_warp * frames_per_pass must be 32");
     const int th = tile_h ? tile_h : h->tl.th, tw = tile_w ? tile_w : h->tl.tw;
-    if (th != h->tl.th || tw != h->tl.tw) {
+    if (th != h->tl.th || tw != h->tl.tw || !h->layout_ok) {
         if ((int64_t)th * (tw + 8) > 65535 || th < 1 || tw < 4)
             return fail(AZ_EINVAL, "az_set_tuning: tile %dx%d out of range", th, tw);
+        const int th0 = h->tl.th, tw0 = h->tl.tw;
         cudaDeviceSynchronize();
-        AZ_TRY(build_tiled_layout(h, th, tw, nullptr));
-        AZ_TRY(alloc_scratch(h, nullptr));
+        const int rc = set_tiles(h, th, tw, nullptr);
+        if (rc != AZ_OK) {
+            restore_tiles(h, th0, tw0, nullptr);
+            cudaDeviceSynchronize();
+            return rc;
+        }
         AZ_CUDA(cudaDeviceSynchronize());
     }
     if (rows_per_warp) h->frames_per_pass = 32 / rows_per_warp;
@@ -697,7 +737,7 @@ extern "C" int az_autotune(az_integrator *h, int n_trial_frames, az_stream_t str
     AZ_CUDA(cudaMemsetAsync(dark.p, 0, sizeof(float) * npix, s));
     fill_frames_kernel<<<num_sms() * 8, 256, 0, s>>>(frames.as<uint32_t>(), npix * n_trial_frames, 12345u);
     AZ_CUDA(cudaGetLastError());
-    AZ_TRY(batch_norm(h, nullptr, nullptr, nullptr, nullptr, nullptr, s));
+    const int th0 = h->tl.th, tw0 = h->tl.tw, fpp0 = h->frames_per_pass, engine0 = h->copy_engine;
     cudaEvent_t e0, e1;
     AZ_CUDA(cudaEventCreate(&e0));
     AZ_CUDA(cudaEventCreate(&e1));
@@ -708,9 +748,11 @@ extern "C" int az_autotune(az_integrator *h, int n_trial_frames, az_stream_t str
     int bt = -1, bf = h->frames_per_pass, be = h->copy_engine;
     const int tile_count = (int)(sizeof(tiles) / sizeof(tiles[0]));
     for (int ti = 0; ti < tile_count; ++ti) {
-        if (build_tiled_layout(h, tiles[ti][0], tiles[ti][1], s) != AZ_OK) { clear_error(); continue; }
-        AZ_TRY(alloc_scratch(h, s));
-        AZ_TRY(batch_norm(h, nullptr, nullptr, nullptr, nullptr, nullptr, s));
+        if (set_tiles(h, tiles[ti][0], tiles[ti][1], s) != AZ_OK ||
+            batch_norm(h, nullptr, nullptr, nullptr, nullptr, nullptr, s) != AZ_OK) {
+            clear_error();
+            continue;
+        }
         for (int eg : engines)
             for (int f : fpps) {
                 h->frames_per_pass = f;
@@ -736,10 +778,16 @@ extern "C" int az_autotune(az_integrator *h, int n_trial_frames, az_stream_t str
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (best >= 1e30) return fail(AZ_EUNSUPPORTED, "az_autotune: no configuration ran");
-    if (bt < 0) return fail(AZ_EUNSUPPORTED, "az_autotune: no configuration ran");
-    AZ_TRY(build_tiled_layout(h, tiles[bt][0], tiles[bt][1], s));
-    AZ_TRY(alloc_scratch(h, s));
+    const int rc = bt < 0 ? fail(AZ_EUNSUPPORTED, "az_autotune: no configuration ran")
+                          : set_tiles(h, tiles[bt][0], tiles[bt][1], s);
+    if (rc != AZ_OK) {  // as it was
+        h->frames_per_pass = fpp0;
+        h->copy_engine = engine0;
+        if (h->tl.th != th0 || h->tl.tw != tw0) h->layout_ok = false;
+        restore_tiles(h, th0, tw0, s);
+        cudaStreamSynchronize(s);
+        return rc;
+    }
     h->frames_per_pass = bf;
     h->rows_per_warp = 32 / bf;
     h->copy_engine = be;

@@ -35,6 +35,22 @@ void clear_error();
         if (rc_ != AZ_OK) return rc_;                                                      \
     } while (0)
 
+// Allocation failures on request (az_selftest_alloc): of this thread's next device allocations,
+// `after` succeed and the `count` after them fail.
+struct AllocFault {
+    int64_t after = 0, count = 0;
+    static AllocFault &mine() {
+        static thread_local AllocFault f;
+        return f;
+    }
+    bool due() { return count > 0 && (after > 0 ? (--after, false) : (--count, true)); }
+};
+inline cudaError_t device_alloc(void **p, size_t n) {
+    const cudaError_t e = AllocFault::mine().due() ? cudaErrorMemoryAllocation : cudaMalloc(p, n);
+    if (e != cudaSuccess) (void)cudaGetLastError();  // reported here, not by the next launch's check
+    return e;
+}
+
 // Device memory of the library: an allocation of its own (freed in the destructor) or a part of
 // another one (view).
 struct DevBuf {
@@ -54,7 +70,7 @@ struct DevBuf {
     int alloc(size_t n) {
         release();
         if (n == 0) n = 16;
-        cudaError_t e = cudaMalloc(&p, n);
+        cudaError_t e = device_alloc(&p, n);
         if (e != cudaSuccess) {
             p = nullptr;
             return fail(AZ_ENOMEM, "cudaMalloc(%zu) failed: %s", n, cudaGetErrorString(e));
@@ -143,7 +159,7 @@ struct ScratchScope {
             if (c->n_chunks == Pool::kChunks) return fail(AZ_ENOMEM, "build scratch: more than %d chunks", Pool::kChunks);
             void *p = nullptr;
             const size_t want = std::max(n, room);
-            cudaError_t e = cudaMalloc(&p, want);
+            cudaError_t e = device_alloc(&p, want);
             if (e != cudaSuccess) return fail(AZ_ENOMEM, "cudaMalloc(%zu) failed: %s", want, cudaGetErrorString(e));
             c->chunks[c->n_chunks++] = {static_cast<char *>(p), want};
             c->off = 0;
@@ -288,6 +304,9 @@ struct az_integrator {
     // pixel-major CSC (columns = pixels) for the adjoint
     azint::DevBuf csc_ptr, csc_row, csc_w64, csc_w32;
     azint::TiledLayout tl;
+    // Set while tl and the scratch below belong together: a rebuild that fails part way leaves
+    // buffers of two layouts (or none), and calls that read them are refused (check_layout).
+    bool layout_ok = false;
     // tuning
     int rows_per_warp = 4, frames_per_pass = 8, copy_engine = AZ_COPY_TMA;
     // scratch: per-segment partial sums and per-row frame-independent sums
@@ -359,6 +378,7 @@ int batch_pixelnorm(az_integrator *h, const void *frames, int n, int dtype, cons
                     const float *flat, const float *sa, const float *pol, float *oI, float *oU,
                     float *oC, cudaStream_t s);
 // argument checks shared by the forward entry points (NULL, dtype, 4-byte alignment)
+int check_layout(const az_integrator *h, const char *who);
 int check_forward(const az_integrator *h, const void *image, int dtype, const float *dark,
                   const float *flat, const float *sa, const float *pol, const char *who);
 int lut_build(az_integrator *h, int precision, cudaStream_t s);

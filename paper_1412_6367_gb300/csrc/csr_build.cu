@@ -1280,7 +1280,6 @@ int count_runs(const az_integrator *h, int th, int tw, cudaStream_t s, int64_t *
 int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     ScratchScope scope;
     TiledLayout &L = h->tl;
-    h->corr_bound = false;   // bound corrections are per layout too (entry order, sums)
     const int64_t nnz = h->nnz;
     if (th < 4 || (th % 4) != 0 || tw < 4 || (tw % 4) != 0)
         return fail(AZ_EINVAL, "tile %dx%d: both sides must be positive multiples of 4", th, tw);
@@ -1290,8 +1289,10 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     T.ntx = (h->nx + tw - 1) / tw;
     const int nty = (h->ny + th - 1) / th;
     const int ntiles = T.ntx * nty;
-    AZ_TRY(ScratchScope::reserve(66 * (size_t)nnz + ((size_t)2 << 20)));
     if ((int64_t)4 * T.ss + 32 > 65535) return fail(AZ_EINVAL, "tile %dx%d too large", th, tw);
+    h->layout_ok = false;   // until the caller has made the scratch of this layout too
+    h->corr_bound = false;  // bound corrections are per layout (entry order, sums)
+    AZ_TRY(ScratchScope::reserve(66 * (size_t)nnz + ((size_t)2 << 20)));
 
     // row of each CSR entry, tile key of each CSR entry, stable sort by tile
     int32_t nseg = 0;

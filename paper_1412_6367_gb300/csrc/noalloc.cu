@@ -69,6 +69,7 @@ extern "C" int az_integrate_noalloc(const az_integrator *h, const void *image_de
         if (p && !aligned4(p)) return fail(AZ_EINVAL, "%s: arrays must be 4-byte aligned", who);
     if (precision != AZ_PREC_FP64 && precision != AZ_PREC_FP32_COMP)
         return fail(AZ_EINVAL, "%s: bad precision %d", who, precision);
+    AZ_TRY(check_layout(h, who));
     const size_t value_bytes = precision == AZ_PREC_FP64 ? sizeof(double) : sizeof(float);
     const size_t need = 3 * (size_t)h->tl.nseg * value_bytes;
     if (need > (size_t)AZ_NOALLOC_SCRATCH_BYTES)

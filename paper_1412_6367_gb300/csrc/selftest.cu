@@ -1,7 +1,7 @@
-// Self-test of the bounded device-side wait that every staged kernel of the library uses
-// (see az_selftest_wait in azint.h): a one-warp kernel waits on a shared-memory barrier that
-// nothing completes (or that its first thread completes, as a control) and reports, instead
-// of hanging, that the wait gave up.
+// Self-tests: allocation failures on request (az_selftest_alloc in azint.h), and the bounded
+// device-side wait that every staged kernel of the library uses (az_selftest_wait): a one-warp
+// kernel waits on a shared-memory barrier that nothing completes (or that its first thread
+// completes, as a control) and reports, instead of hanging, that the wait gave up.
 #include "common.cuh"
 
 using namespace azint;
@@ -23,6 +23,13 @@ __global__ void wait_selftest_kernel(int arrive, long long limit, int *status) {
 }
 
 }  // namespace
+
+extern "C" int az_selftest_alloc(int64_t after, int64_t count) {
+    clear_error();
+    if (after < 0 || count < 0) return fail(AZ_EINVAL, "az_selftest_alloc: negative argument");
+    AllocFault::mine() = AllocFault{after, count};
+    return AZ_OK;
+}
 
 extern "C" int az_selftest_wait(int arrive, int64_t limit_cycles, int *out_status, az_stream_t stream) {
     clear_error();
