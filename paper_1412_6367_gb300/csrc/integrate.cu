@@ -1084,7 +1084,7 @@ frames_kernel(const __grid_constant__ FrArgs a, FrGeom fg, const __grid_constant
                 if (j >= (uint32_t)S) {
                     bool ok = mbar_wait_bounded(&pempty[s], turn ^ 1u);
                     ok = __all_sync(0xffffffffu, ok);
-                    if (!ok || *abort_flag != 0) {
+                    if (__any_sync(0xffffffffu, !ok || *abort_flag != 0)) {  // warp-uniform decision
                         stop = true;
                         if (!ok && lane == 0) atomicExch(a.status, AZ_ETIMEOUT);
                         break;
@@ -1503,7 +1503,7 @@ single_kernel(const __grid_constant__ SgInst one, const SgInst *__restrict__ mul
             if (k >= S) {
                 bool ok = mbar_wait_bounded(&empty[s], turn ^ 1u);
                 ok = __all_sync(0xffffffffu, ok);
-                if (!ok || *abort_flag != 0) {
+                if (__any_sync(0xffffffffu, !ok || *abort_flag != 0)) {  // warp-uniform decision
                     if (lane == 0) {
                         if (!ok) atomicExch(status, AZ_ETIMEOUT);
                         *abort_flag = 1;
