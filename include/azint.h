@@ -365,7 +365,8 @@ int az_integrate_backward(const az_integrator *h, const void *grad_I, const void
  * out_sum_norm[k] / out_count[k] (device float[nrows_k]; the pointer arrays may be NULL).
  * The plan flattens every (instance, tile) pair into one work list processed by one
  * persistent FP32-compensated launch, followed by one finalising launch.  The pointer
- * arrays are copied; the integrators must outlive the plan.
+ * arrays are copied; the integrators must outlive the plan.  az_set_tuning and az_autotune free
+ * the layout a plan was made on: after other tiles az_multi_launch returns AZ_EINVAL.
  */
 int az_multi_create(az_integrator *const *handles, int n, const void *const *images,
                     int image_dtype, const float *const *darks, const float *const *flats,

@@ -307,6 +307,7 @@ struct az_integrator {
     // Set while tl and the scratch below belong together: a rebuild that fails part way leaves
     // buffers of two layouts (or none), and calls that read them are refused (check_layout).
     bool layout_ok = false;
+    int64_t layout_no = 0;  // counts the layouts: a plan holds pointers into the one it was made on
     // tuning
     int rows_per_warp = 4, frames_per_pass = 8, copy_engine = AZ_COPY_TMA;
     // scratch: per-segment partial sums and per-row frame-independent sums

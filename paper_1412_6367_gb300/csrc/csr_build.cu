@@ -1290,6 +1290,7 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     const int nty = (h->ny + th - 1) / th;
     const int ntiles = T.ntx * nty;
     if ((int64_t)4 * T.ss + 32 > 65535) return fail(AZ_EINVAL, "tile %dx%d too large", th, tw);
+    ++h->layout_no;
     h->layout_ok = false;   // until the caller has made the scratch of this layout too
     h->corr_bound = false;  // bound corrections are per layout (entry order, sums)
     AZ_TRY(ScratchScope::reserve(66 * (size_t)nnz + ((size_t)2 << 20)));

@@ -2778,6 +2778,7 @@ struct MultiPlan {
     SgGeom sgeo{};
     SgInst first{};
     DevBuf sg_dev;       // SgInst [n]
+    std::vector<std::pair<const az_integrator *, int64_t>> layouts;  // integrators and their layouts
     cudaGraphExec_t exec = nullptr;
     cudaGraph_t graph = nullptr;
 };
@@ -2864,6 +2865,7 @@ int multi_create(az_integrator *const *hs, int n, const void *const *images, int
     int stage_e = 0;
     P->sg = choose_stage(pw, planes, ecap, 4, rw, stage_e);
     for (auto &d : P->host) d.stage_entries = stage_e;
+    for (int k = 0; k < n; ++k) P->layouts.emplace_back(hs[k], hs[k]->layout_no);
     P->n_items = items;
     P->n_rows = rows;
     int rc = P->dev.alloc(sizeof(Inst) * (size_t)n);
@@ -2902,6 +2904,10 @@ int multi_enqueue(void *plan, cudaStream_t s) {
 
 int multi_launch(void *plan, int use_graph, cudaStream_t s) {
     MultiPlan *P = static_cast<MultiPlan *>(plan);
+    for (size_t k = 0; k < P->layouts.size(); ++k)
+        if (P->layouts[k].first->layout_no != P->layouts[k].second)
+            return fail(AZ_EINVAL, "az_multi_launch: integrator %d got other tiles (az_set_tuning, az_autotune) since "
+                                   "the plan was made: make a new plan", (int)k);
     if (!use_graph) return multi_enqueue(plan, s);
     if (!P->exec) {
         // Run once eagerly (this call's results; it also configures the kernels), then

@@ -139,3 +139,21 @@ def test_failed_autotune_keeps_the_tiles():
         g.set_tuning(20, 28)
         assert _equal(_all(c, g), ref)
     assert g.status() == 0
+
+
+def test_a_plan_of_former_tiles_is_refused():
+    c, g = _case(0)
+    c2, h = _case(24)
+    imgs = [c.image_dev(), c2.image_dev()]
+    plan = api().MultiPlan([g, h], imgs)
+    ref = [t.cpu().clone() for r in plan.launch(use_graph=True) for t in r]
+    h.set_tuning(frames_per_pass=4)  # no other tiles
+    assert _equal([t.cpu() for r in plan.launch(use_graph=True) for t in r], ref)
+    h.set_tuning(8, 40)
+    for graph in (False, True):
+        with pytest.raises(api().AzError) as e:
+            plan.launch(use_graph=graph)
+        assert e.value.code == EINVAL and "integrator 1" in str(e.value)
+    out = api().MultiPlan([g, h], imgs).launch(use_graph=True)
+    assert _equal([t.cpu() for t in out[0]], ref[:4])
+    assert g.status() == 0 and h.status() == 0
