@@ -29,6 +29,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <vector>
 
@@ -2779,6 +2780,8 @@ struct MultiPlan {
     SgInst first{};
     DevBuf sg_dev;       // SgInst [n]
     std::vector<std::pair<const az_integrator *, int64_t>> layouts;  // integrators and their layouts
+    // partial sums of an integrator's second and further instances (the first has its own)
+    std::vector<std::unique_ptr<DevBuf>> partials;
     cudaGraphExec_t exec = nullptr;
     cudaGraph_t graph = nullptr;
 };
@@ -2868,6 +2871,17 @@ int multi_create(az_integrator *const *hs, int n, const void *const *images, int
     for (int k = 0; k < n; ++k) P->layouts.emplace_back(hs[k], hs[k]->layout_no);
     P->n_items = items;
     P->n_rows = rows;
+    for (int k = 0; k < n; ++k) {
+        if (std::find(hs, hs + k, hs[k]) == hs + k) continue;
+        P->partials.emplace_back(new DevBuf);
+        const int rp = P->partials.back()->alloc(3 * sizeof(float) * (size_t)std::max(hs[k]->tl.nseg, 1));
+        if (rp != AZ_OK) {
+            delete P;
+            return rp;
+        }
+        P->host[(size_t)k].partial = P->partials.back()->p;
+        if (P->single) sgi[(size_t)k].partial = P->partials.back()->p;
+    }
     int rc = P->dev.alloc(sizeof(Inst) * (size_t)n);
     if (rc == AZ_OK) {
         cudaError_t e = cudaMemcpy(P->dev.p, P->host.data(), sizeof(Inst) * (size_t)n, cudaMemcpyHostToDevice);
