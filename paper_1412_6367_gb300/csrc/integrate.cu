@@ -2362,10 +2362,11 @@ int count_layout(az_integrator *h, cudaStream_t s) {
 // One frame through single_kernel; AZ_EUNSUPPORTED (without error text) where it does not fit.
 template <class AT>
 int forward_one(const az_integrator *h, const void *const arrs[5], int dtype, void *oI, void *oS, void *oN, void *oC,
-                cudaStream_t s) {
+                void *partial, Profiler *prof, cudaStream_t s) {
     constexpr bool fp64 = sizeof(AT) == 8;
     if (engine_for(h) != AZ_COPY_TMA || h->tl.fslots < 1) return AZ_EUNSUPPORTED;
-    const SgInst one = sg_inst(h, fp64, arrs);
+    SgInst one = sg_inst(h, fp64, arrs);
+    one.partial = partial;
     const bool norm = (one.present & 28) != 0;
     SgNeed need;
     need.add(h, one.present);
@@ -2373,11 +2374,12 @@ int forward_one(const az_integrator *h, const void *const arrs[5], int dtype, vo
     if (!sg_geom(need, fp64, norm, sg)) return AZ_EUNSUPPORTED;
     TmaSet tm;
     AZ_TRY(sg_maps(h, arrs, tm));
-    AZ_TRY((sg_launch_dt<AT>(dtype, norm, one, nullptr, 1, one.n_items, sg, tm, s, &h->prof)));
+    AZ_TRY((sg_launch_dt<AT>(dtype, norm, one, nullptr, 1, one.n_items, sg, tm, s, prof)));
     Inst d = make_inst(h, fp64);
+    d.partial = partial;
     d.oI = oI; d.oS = oS; d.oN = oN; d.oC = oC;
     d.single_nc = norm ? 1 : 2;
-    return run_phase2<AT, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s, &h->prof);
+    return run_phase2<AT, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s, prof);
 }
 
 // One FP32 frame with tiles whose six planes and entries do not fit twice: the corrected frame
@@ -2412,40 +2414,47 @@ int forward_planes(az_integrator *h, const void *image, int dtype, const float *
     return run_phase2<float, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s, &h->prof);
 }
 
+// One frame through phase1_kernel (tiles or engines the kernels above do not take).
+int forward_general(const az_integrator *h, const void *const arrs[5], int dtype, int precision, void *oI, void *oS,
+                    void *oN, void *oC, void *partial, Profiler *prof, cudaStream_t s) {
+    const bool fp64 = precision == AZ_PREC_FP64;
+    const float *const c[4] = {static_cast<const float *>(arrs[1]), static_cast<const float *>(arrs[2]),
+                               static_cast<const float *>(arrs[3]), static_cast<const float *>(arrs[4])};
+    Inst d = make_inst(h, fp64);
+    d.partial = partial;
+    d.img = static_cast<const char *>(arrs[0]);
+    d.dark = c[0]; d.flat = c[1]; d.sa = c[2]; d.pol = c[3];
+    d.oI = oI; d.oS = oS; d.oN = oN; d.oC = oC;
+    const int planes = 1 + (c[0] != nullptr) + (c[1] != nullptr) + (c[2] != nullptr) + (c[3] != nullptr);
+    StageGeom sg = choose_stage(plane_words_of(h), planes, (uint32_t)h->tl.max_tile_entries,
+                                fp64 ? 8 : 4, rec_words_of(h), d.stage_entries);
+    const int eng = engine_for(h);
+    TmaSet tm;
+    AZ_TRY(make_maps(h, eng, arrs[0], h->ny, c[0], c[1], c[2], c[3], tm));
+    if (fp64) {
+        AZ_TRY((run_phase1_dt<double, double, MODE_SINGLE, 1>(dtype, eng, d, nullptr, 1, d.n_items, sg, tm, s, prof)));
+        return run_phase2<double, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s, prof);
+    }
+    AZ_TRY((run_phase1_dt<float, float, MODE_SINGLE, 1>(dtype, eng, d, nullptr, 1, d.n_items, sg, tm, s, prof)));
+    return run_phase2<float, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s, prof);
+}
+
 int forward_single(const az_integrator *h, const void *image, int dtype, const float *dark,
                    const float *flat, const float *sa, const float *pol, int precision, void *oI,
                    void *oS, void *oN, void *oC, cudaStream_t s) {
     const bool fp64 = precision == AZ_PREC_FP64;
     const void *const arrs[5] = {image, dark, flat, sa, pol};
-    const int rc = fp64 ? forward_one<double>(h, arrs, dtype, oI, oS, oN, oC, s)
-                        : forward_one<float>(h, arrs, dtype, oI, oS, oN, oC, s);
+    Profiler *prof = &h->prof;
+    const int rc = fp64 ? forward_one<double>(h, arrs, dtype, oI, oS, oN, oC, h->partial.p, prof, s)
+                        : forward_one<float>(h, arrs, dtype, oI, oS, oN, oC, h->partial.p, prof, s);
     if (rc != AZ_EUNSUPPORTED) return rc;
     if (!fp64) {
         const int rp = forward_planes(const_cast<az_integrator *>(h), image, dtype, dark, flat, sa, pol, oI, oS, oN, oC, s);
         if (rp != AZ_EUNSUPPORTED) return rp;
     }
-    Inst d = make_inst(h, fp64);
-    d.img = static_cast<const char *>(image);
-    d.dark = dark; d.flat = flat; d.sa = sa; d.pol = pol;
-    d.oI = oI; d.oS = oS; d.oN = oN; d.oC = oC;
-    const int planes = 1 + (dark != nullptr) + (flat != nullptr) + (sa != nullptr) + (pol != nullptr);
-    StageGeom sg = choose_stage(plane_words_of(h), planes, (uint32_t)h->tl.max_tile_entries,
-                                fp64 ? 8 : 4, rec_words_of(h), d.stage_entries);
-    const int eng = engine_for(h);
-    TmaSet tm;
-    AZ_TRY(make_maps(h, eng, image, h->ny, dark, flat, sa, pol, tm));
-    if (fp64) {
-        AZ_TRY((run_phase1_dt<double, double, MODE_SINGLE, 1>(dtype, eng, d, nullptr, 1, d.n_items, sg, tm, s, &h->prof)));
-        AZ_TRY((run_phase2<double, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s, &h->prof)));
-    } else {
-        AZ_TRY((run_phase1_dt<float, float, MODE_SINGLE, 1>(dtype, eng, d, nullptr, 1, d.n_items, sg, tm, s, &h->prof)));
-        AZ_TRY((run_phase2<float, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s, &h->prof)));
-    }
-    return AZ_OK;
+    return forward_general(h, arrs, dtype, precision, oI, oS, oN, oC, h->partial.p, prof, s);
 }
 
-// forward_single with the per-segment partial sums in a buffer the caller supplies (at least
-// 3 * nseg values of the accumulation type) instead of the integrator's own; no profiling.
 // Loads, without launching them, the kernels forward_single_into can launch (both
 // precisions, every image type, both copy engines, and phase 2).  Under the CUDA runtime's
 // lazy loading a kernel's code is otherwise loaded, and may take device memory, at its first
@@ -2456,6 +2465,8 @@ template <class K> int preload_kernel(K k) {
     return AZ_OK;
 }
 template <class AT, int DT> int preload_single_dt() {
+    AZ_TRY((preload_kernel(single_kernel<AT, DT, true, true>)));
+    AZ_TRY((preload_kernel(single_kernel<AT, DT, true, false>)));
     AZ_TRY(preload_kernel(phase1_kernel<AT, AT, MODE_SINGLE, 1, DT, true>));
     return preload_kernel(phase1_kernel<AT, AT, MODE_SINGLE, 1, DT, false>);
 }
@@ -2472,29 +2483,18 @@ int preload_single_pass() {
     return preload_kernel(phase2_thread_kernel<float, MODE_SINGLE>);
 }
 
+// One frame with the per-segment partial sums in a buffer the caller supplies (at least
+// 3 * nseg values of the accumulation type) instead of the integrator's own; no profiling and no
+// allocation.  (On the default tiles phase1_kernel, which took every such call before, needs 151 us
+// for a 2527 x 2463 FP32 frame with four corrections, 91 us on tiles of 8 x 224; single_kernel 76.)
 int forward_single_into(const az_integrator *h, const void *image, int dtype, const float *dark,
                         const float *flat, const float *sa, const float *pol, int precision,
                         void *oI, void *oS, void *oN, void *oC, void *partial, cudaStream_t s) {
-    const bool fp64 = precision == AZ_PREC_FP64;
-    Inst d = make_inst(h, fp64);
-    d.partial = partial;
-    d.img = static_cast<const char *>(image);
-    d.dark = dark; d.flat = flat; d.sa = sa; d.pol = pol;
-    d.oI = oI; d.oS = oS; d.oN = oN; d.oC = oC;
-    const int planes = 1 + (dark != nullptr) + (flat != nullptr) + (sa != nullptr) + (pol != nullptr);
-    StageGeom sg = choose_stage(plane_words_of(h), planes, (uint32_t)h->tl.max_tile_entries,
-                                fp64 ? 8 : 4, rec_words_of(h), d.stage_entries);
-    const int eng = engine_for(h);
-    TmaSet tm;
-    AZ_TRY(make_maps(h, eng, image, h->ny, dark, flat, sa, pol, tm));
-    if (fp64) {
-        AZ_TRY((run_phase1_dt<double, double, MODE_SINGLE, 1>(dtype, eng, d, nullptr, 1, d.n_items, sg, tm, s)));
-        AZ_TRY((run_phase2<double, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s)));
-    } else {
-        AZ_TRY((run_phase1_dt<float, float, MODE_SINGLE, 1>(dtype, eng, d, nullptr, 1, d.n_items, sg, tm, s)));
-        AZ_TRY((run_phase2<float, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s)));
-    }
-    return AZ_OK;
+    const void *const arrs[5] = {image, dark, flat, sa, pol};
+    const int rc = precision == AZ_PREC_FP64 ? forward_one<double>(h, arrs, dtype, oI, oS, oN, oC, partial, nullptr, s)
+                                             : forward_one<float>(h, arrs, dtype, oI, oS, oN, oC, partial, nullptr, s);
+    if (rc != AZ_EUNSUPPORTED) return rc;
+    return forward_general(h, arrs, dtype, precision, oI, oS, oN, oC, partial, nullptr, s);
 }
 
 int batch_norm(az_integrator *h, const float *flat, const float *sa, const float *pol, float *oN,

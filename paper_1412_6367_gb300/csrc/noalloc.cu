@@ -1,7 +1,8 @@
 // Single-frame forward whose scratch lives in a fixed array compiled into this library, for
 // callers that must not allocate device memory while they run (see az_integrate_noalloc in
-// azint.h).  The kernels are the ones az_integrate1d / az_integrate2d launch; only the
-// buffer that holds the per-segment partial sums between the two phases differs.
+// azint.h).  The kernels are the ones az_integrate1d / az_integrate2d launch (single_kernel, or
+// phase1_kernel where that does not fit); only the buffer that holds the per-segment partial sums
+// between the two phases differs.
 #include <mutex>
 
 #include "common.cuh"
