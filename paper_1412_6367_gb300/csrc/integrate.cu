@@ -136,6 +136,15 @@ __device__ __forceinline__ TileDesc load_desc(const Inst &d, int64_t local) {
     return TileDesc{x.x, x.y, x.z, x.w, y.x, y.y};
 }
 
+// Descriptors of a CTA's items, 32 at a time: lane l holds the one of item 32 b + l of the CTA, and
+// the next 32 are read while these are used.  (Read one or two items ahead, each item waited for
+// its descriptor's trip to memory: about 1 us an item where an item has few stages.)
+__device__ __forceinline__ TileDesc shfl_desc(const TileDesc &d, int l) {
+    return TileDesc{__shfl_sync(0xffffffffu, d.t, l), __shfl_sync(0xffffffffu, d.rec_off, l),
+                    __shfl_sync(0xffffffffu, d.rec_words, l), __shfl_sync(0xffffffffu, d.e_off, l),
+                    __shfl_sync(0xffffffffu, d.ne, l), __shfl_sync(0xffffffffu, d.ns, l)};
+}
+
 // Words between two staged planes: four 128-byte aligned row-class slots and a band of 32
 // words that holds zeros (the padding entries of the matrix point there: their weight is 0
 // and the value they read is 0, whatever the image holds).  Planes are spread over the
@@ -276,23 +285,23 @@ __device__ void produce(const Inst &d, const TmaSet &tm, int64_t local, const Ti
         }
     }
     if (!TMA) {
-        // the same words as the tensor copies: for every (plane, class, row in class) a run of
-        // boxw / 4 16-byte pieces from column c0 - off_k; eight lanes per run
+        // the same words as the tensor copies: for every (plane, tile row) a run of boxw / 4
+        // 16-byte pieces from column c0 - off_k; eight lanes per run.  Tile row ly is row ly / 4
+        // of slot ly mod 4.
         const int sub = lane >> 3, l8 = lane & 7;
-        const int runs = np * 4 * rows4;
         const int nchunk = boxw >> 2;
-        for (int r = pwarp * 4 + sub; r < runs; r += 4 * kProducers) {
-            const int pl = r / (4 * rows4);
-            const int rem = r - pl * 4 * rows4;
-            const int k = rem / rows4, jj = rem - k * rows4;
+        int pl = 0, ly = pwarp * 4 + sub;
+        for (;; ly += 4 * kProducers) {
+            while (ly >= d.th) { ly -= d.th; ++pl; }
+            if (pl >= np) break;
             const char *arr;
             int64_t g0, rows_total;
             int kind;
             plane_geo(pl, arr, g0, rows_total, kind);
             const int beta = (int)((reinterpret_cast<uintptr_t>(arr) >> 2) & 3u);
             const int phi_row = (int)(g0 & 3);
-            const int sl = (k - phi_row) & 3;
-            const int64_t g = g0 + sl + 4 * (int64_t)jj;  // global row of this run
+            const int sl = ly & 3, k = (sl + phi_row) & 3, jj = ly >> 2;
+            const int64_t g = g0 + ly;  // global row of this run
             if (g >= rows_total) continue;
             const int phi = (beta + nu * phi_row) & 3;
             const int offk = (beta + k * nu) & 3;
@@ -320,11 +329,15 @@ __device__ void produce(const Inst &d, const TmaSet &tm, int64_t local, const Ti
         for (int pl = 0; pl < np; ++pl) planes[(size_t)pl * pw + pw - kZeroBand + lane] = 0u;
         __syncwarp();
     }
-    if (pwarp == 0 && lane == 0) {
+    if (pwarp == 0) {
         int *h = reinterpret_cast<int *>(stage);
-        h[0] = td.ns; h[1] = group; h[2] = nimg; h[3] = h[4] = h[5] = h[6] = -1;
-        h[7] = t; h[8] = td.e_off;
-        for (int pl = 0; pl < np; ++pl) {
+        if (lane == 0) {
+            h[0] = td.ns; h[1] = group; h[2] = nimg; h[3] = h[4] = h[5] = h[6] = -1;
+            h[7] = t; h[8] = td.e_off;
+            *ctr = 0;  // segment claim counter of this stage
+        }
+        __syncwarp();
+        for (int pl = lane; pl < np; pl += 32) {  // a lane per plane
             const char *arr;
             int64_t g0, rows_total;
             int kind;
@@ -334,8 +347,8 @@ __device__ void produce(const Inst &d, const TmaSet &tm, int64_t local, const Ti
             const int o = (int)(pl * pw + phi + 4 * (pl & 3));
             if (kind == 0) h[16 + pl] = o; else h[2 + kind] = o;
         }
-        *ctr = 0;          // segment claim counter of this stage
-        mbar_arrive(bar);  // publishes the header and the counter
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar);  // publishes the header and the counter
     }
 }
 
@@ -643,20 +656,37 @@ phase1_kernel(const __grid_constant__ Inst single, const Inst *__restrict__ mult
             if (!multi || (it >= hint->item_begin && it < hint->item_begin + hint->n_items)) return hint;
             return &inst_of(single, multi, n_inst, it);
         };
-        TileDesc td{};
-        if (item < n_items) {
-            if (multi) dc = dn = &inst_of(single, multi, n_inst, item);
+        // One instance: descriptors of the CTA's items 32 at a time, lane l the one of item 32 b + l
+        // (as in frames_kernel; read one item ahead, an item waits for the trip to memory).
+        // Several: the next item's while this one is staged.
+        auto read = [&](int b) {
+            const int64_t it = (int64_t)blockIdx.x + (int64_t)(32 * b + lane) * gridDim.x;
+            return it < n_items ? load_desc(single, it) : TileDesc{};
+        };
+        TileDesc td{}, cur{}, nxt{};
+        if (!multi) {
+            cur = read(0);
+            nxt = read(1);
+        } else if (item < n_items) {
+            dc = dn = &inst_of(single, multi, n_inst, item);
             td = load_desc(*dc, item - dc->item_begin);
         }
         for (; item < n_items; item += gridDim.x, ++k) {
             const int s = k % S, n = k / S;
-            // prefetch the next item's descriptor while this one is staged
-            const int64_t next = item + gridDim.x;
             TileDesc tn{};
-            dc = dn;
-            if (next < n_items) {
-                dn = find(next, dc);
-                tn = load_desc(*dn, next - dn->item_begin);
+            if (!multi) {
+                if (k > 0 && (k & 31) == 0) {
+                    cur = nxt;
+                    nxt = read((k >> 5) + 1);
+                }
+                td = shfl_desc(cur, k & 31);
+            } else {
+                const int64_t next = item + gridDim.x;
+                dc = dn;
+                if (next < n_items) {
+                    dn = find(next, dc);
+                    tn = load_desc(*dn, next - dn->item_begin);
+                }
             }
             bool ok = true;
             if (n > 0) ok = mbar_wait_bounded(&empty[s], (uint32_t)((n - 1) & 1));
@@ -777,15 +807,6 @@ __device__ __forceinline__ TileDesc fr_desc(const FrArgs &a, int item) {
     const int4 *p = reinterpret_cast<const int4 *>(a.desc) + 2 * (size_t)item;
     const int4 x = __ldg(p), y = __ldg(p + 1);
     return TileDesc{x.x, x.y, x.z, x.w, y.x, y.y};
-}
-
-// Descriptors of a CTA's items, 32 at a time: lane l holds the one of item 32 b + l of the CTA, and
-// the next 32 are read while these are used.  (Read one or two items ahead, each item waited for
-// its descriptor's trip to memory: about 1 us an item where an item has few stages.)
-__device__ __forceinline__ TileDesc shfl_desc(const TileDesc &d, int l) {
-    return TileDesc{__shfl_sync(0xffffffffu, d.t, l), __shfl_sync(0xffffffffu, d.rec_off, l),
-                    __shfl_sync(0xffffffffu, d.rec_words, l), __shfl_sync(0xffffffffu, d.e_off, l),
-                    __shfl_sync(0xffffffffu, d.ne, l), __shfl_sync(0xffffffffu, d.ns, l)};
 }
 
 // One thread: the tile's record, entry locations, weights and darks into entry buffer `eb`.
