@@ -66,7 +66,6 @@ struct Inst {
     float *norm;         // [2][nrows] N, C (FP32 batched path)
     void *oI, *oS, *oN, *oC;
     int frame_out0;      // first output frame of this launch
-    int norm_rows;       // norm pass: 2 = partials hold N and C, 1 = N only
     int64_t item_begin, row_begin;
     int n_items;
     int stage_entries;
@@ -74,9 +73,8 @@ struct Inst {
     const int32_t *tile_desc, *tile_rec;  // per active tile: descriptor [8] and record
     const float *ent_dark;                // frames pass: dark of each entry's pixel (or NULL)
     const CUtensorMap *maps;              // many-instance launch: this instance's [5][4] maps
-    int single_nc;  // single-frame phase 2: 0 S, N, C from the partials; 1 C from the layout's
-                    // count; 2 N and C from it (N == C)
-    const void *count;  // [nrows] in the accumulation type
+    int norm_is_count;  // single-frame phase 2: N is the count too, not the partials' second row
+    const void *count;  // [nrows] in the accumulation type: the layout's C
 };
 
 struct StageGeom {
@@ -432,11 +430,50 @@ template <> struct W4<double> {
     }
 };
 
-// One lane per (segment, quantity).  A warp takes 32 / Q segments at a time from the stage's
-// claim counter; the Q lanes of a segment share its entry stream (broadcast reads) and each
-// sums one quantity over all of the segment's entries:
-//   frames pass: quantity q = frame q of the item, value = cast(image) - dark;
-//   norm pass:   q = 0: flat * solid angle * polarisation, q = 1: 1 (the count).
+// Two FP32 values in one 64-bit register, operated on by the packed f32x2 instructions
+// (round to nearest, no flush): each half gives exactly the scalar result.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 f2_pack(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void f2_unpack(f32x2 x, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x));
+}
+__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// a - b as b (-1) + a: the same single rounding of the same exact value.
+__device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b) {
+    return f2_fma(b, 0xbf800000bf800000ull, a);
+}
+// Two Kahan accumulators stepped together: the same operations as kahan_add on each half.
+__device__ __forceinline__ void kahan2_add(f32x2 &s, f32x2 &nc, f32x2 w, f32x2 v) {
+    const f32x2 y = f2_fma(w, v, nc);
+    const f32x2 t = f2_add(s, y);
+    nc = f2_sub(y, f2_sub(t, s));
+    s = t;
+}
+// ... and merged: kahan_merge on each half.
+__device__ __forceinline__ void kahan2_merge(f32x2 &as, f32x2 &an, f32x2 bs, f32x2 bn) {
+    const f32x2 t = f2_add(as, bs);
+    const f32x2 z = f2_sub(t, as);
+    const f32x2 e = f2_add(f2_sub(as, f2_sub(t, z)), f2_sub(bs, z));
+    an = f2_add(f2_add(an, bn), e);
+    as = t;
+}
+
+// Frames pass: one lane per (segment, frame).  A warp takes 32 / Q segments at a time from the
+// stage's claim counter; the Q lanes of a segment share its entry stream (broadcast reads) and
+// lane q sums cast(image) - dark of frame q of the item over all of the segment's entries.
 // Segments start on a multiple of 4 entries and hold whole quads (the layout pads them with
 // entries of weight 0 that read the plane's zero band).  Entries are read four at a time (one
 // 8-byte read of the locations, 16-byte reads of the weights and per-entry darks); entry e
@@ -446,15 +483,14 @@ template <> struct W4<double> {
 template <int Q, class AT, class WT, int MODE, int DT, bool SE>
 __device__ void consume_serial(const ConsumerParams &cp, const unsigned char *stage,
                                const StageGeom &sg, int *ctr) {
-    static_assert(MODE != MODE_SINGLE, "the single pass has its own consumer");
+    static_assert(MODE == MODE_FRAMES, "the single and norm passes have their own consumer");
     constexpr int R = 32 / Q;
     const int lane = threadIdx.x & 31;
     const int sub = lane / Q, q = lane % Q;
     const int *h = reinterpret_cast<const int *>(stage);
     const int ns = h[0], group = h[1], nimg = h[2];
-    const int odark = h[3], oflat = h[4], osa = h[5], opol = h[6];
-    const int oimg = h[16 + (MODE == MODE_FRAMES ? q : 0)];
-    const bool active = MODE == MODE_FRAMES ? q < nimg : true;
+    const int oimg = h[16 + q];
+    const bool active = q < nimg;
     const int *slots = reinterpret_cast<const int *>(stage + kHeaderBytes) + 4;
     const uint16_t *starts = reinterpret_cast<const uint16_t *>(slots + ns);
     const uint32_t *planes = reinterpret_cast<const uint32_t *>(stage + kHeaderBytes + sg.rec_cap);
@@ -471,11 +507,8 @@ __device__ void consume_serial(const ConsumerParams &cp, const unsigned char *st
         W = static_cast<const WT *>(cp.ent_w) + h[8];
         DK = cp.ent_dark ? cp.ent_dark + h[8] : nullptr;
     }
-    const bool has_dk = MODE == MODE_FRAMES && sg.ent_dk;
-    size_t orow;
-    if (MODE == MODE_FRAMES) orow = (size_t)(group * cp.fpi + q) * cp.nseg;
-    else orow = (size_t)q * cp.nseg;
-    AT *out = static_cast<AT *>(cp.partial) + orow;
+    const bool has_dk = sg.ent_dk;
+    AT *out = static_cast<AT *>(cp.partial) + (size_t)(group * cp.fpi + q) * cp.nseg;
     while (true) {
         int b = 0;
         if (lane == 0) b = atomicAdd(ctr, R);
@@ -505,21 +538,9 @@ __device__ void consume_serial(const ConsumerParams &cp, const unsigned char *st
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                AT x;
-                if (MODE == MODE_FRAMES) {
-                    float v = img_f32<DT>(planes[oimg + loc[j]]);
-                    if (has_dk) v = __fsub_rn(v, dk[j]);
-                    x = (AT)v;
-                } else {
-                    AT n = AT(1);
-                    if (q == 0) {
-                        if (oflat >= 0) n = n * (AT)__uint_as_float(planes[oflat + loc[j]]);
-                        if (osa >= 0) n = n * (AT)__uint_as_float(planes[osa + loc[j]]);
-                        if (opol >= 0) n = n * (AT)__uint_as_float(planes[opol + loc[j]]);
-                    }
-                    x = n;
-                }
-                acc[j].add((AT)w[j], x);
+                float v = img_f32<DT>(planes[oimg + loc[j]]);
+                if (has_dk) v = __fsub_rn(v, dk[j]);
+                acc[j].add((AT)w[j], (AT)v);
             }
         }
         acc[0].merge(acc[1]);
@@ -529,24 +550,25 @@ __device__ void consume_serial(const ConsumerParams &cp, const unsigned char *st
     }
 }
 
-// Single-frame mode, four lanes per segment: lane j of a segment keeps accumulator j of each
-// of the three sums (the entries e = j mod 4, in order), with per entry x = image - dark,
-// n = ((1 flat) solid angle) polarisation and 1, each added with its weight (FP32:
-// compensated; FP64: fused multiply-adds); the four lanes are merged by shuffles as
+// Single-frame and norm modes, four lanes per segment: lane j of a segment keeps accumulator j of
+// the sums (the entries e = j mod 4, in order), with per entry x = image - dark and n = ((1 flat)
+// solid angle) polarisation, each added with its weight (FP32: compensated, the two sums stepped
+// as a packed pair; FP64: fused multiply-adds); the four lanes are merged by shuffles as
 // ((a0 + a1) + (a2 + a3)), the order every other reduction of the library uses, so a frame's
 // FP32 sums have the bits of the frames kernel's.  A quarter of the chain per lane, every
-// lane busy, eight segments per claim.  Without flat, solid angle and polarisation n = 1 for
-// every entry, so N is C and is not formed twice.
-template <class AT, class WT, int DT, bool SE>
-__device__ void consume_single_split(const ConsumerParams &cp, const unsigned char *stage,
-                                     const StageGeom &sg, int *ctr) {
+// lane busy, eight segments per claim.  The norm mode sums n only (X false).  C = sum w is the
+// layout's (count_layout), and without flat, solid angle and polarisation so is N.
+// (Summing C too, and n unpacked, a 2527 x 2463 frame on the cp.async engine took 150 us in place of
+// 142 in FP32 with four corrections, 88 in place of 81 without, and 291 in place of 258 in FP64.)
+template <class AT, class WT, int DT, bool SE, bool X>
+__device__ void consume_split(const ConsumerParams &cp, const unsigned char *stage, const StageGeom &sg, int *ctr) {
     const int lane = threadIdx.x & 31;
     const int j = lane & 3, sub = lane >> 2;
     const int *h = reinterpret_cast<const int *>(stage);
     const int ns = h[0];
     const int odark = h[3], oflat = h[4], osa = h[5], opol = h[6];
     const int oimg = h[16];
-    const bool norm1 = oflat < 0 && osa < 0 && opol < 0;
+    const bool norm = oflat >= 0 || osa >= 0 || opol >= 0;
     const int *slots = reinterpret_cast<const int *>(stage + kHeaderBytes) + 4;
     const uint16_t *starts = reinterpret_cast<const uint16_t *>(slots + ns);
     const uint32_t *planes = reinterpret_cast<const uint32_t *>(stage + kHeaderBytes + sg.rec_cap);
@@ -561,6 +583,23 @@ __device__ void consume_single_split(const ConsumerParams &cp, const unsigned ch
         W = static_cast<const WT *>(cp.ent_w) + h[8];
     }
     AT *out = static_cast<AT *>(cp.partial);
+    auto image = [&](int loc) -> AT {
+        if (sizeof(AT) == 8) {
+            AT x = (AT)img_f64<DT>(planes[oimg + loc]);
+            if (odark >= 0) x = x - (AT)__uint_as_float(planes[odark + loc]);
+            return x;
+        }
+        float v = img_f32<DT>(planes[oimg + loc]);
+        if (odark >= 0) v = __fsub_rn(v, __uint_as_float(planes[odark + loc]));
+        return (AT)v;
+    };
+    auto normal = [&](int loc) -> AT {
+        AT n = AT(1);
+        if (oflat >= 0) n = n * (AT)__uint_as_float(planes[oflat + loc]);
+        if (osa >= 0) n = n * (AT)__uint_as_float(planes[osa + loc]);
+        if (opol >= 0) n = n * (AT)__uint_as_float(planes[opol + loc]);
+        return n;
+    };
     while (true) {
         int b = 0;
         if (lane == 0) b = atomicAdd(ctr, 8);
@@ -569,35 +608,37 @@ __device__ void consume_single_split(const ConsumerParams &cp, const unsigned ch
         const int sl = b + sub;
         const bool live = sl < ns;
         const int e0 = live ? starts[sl] : 0, e1 = live ? starts[sl + 1] : 0, slot = live ? slots[sl] : 0;
-        Acc<AT> aS, aN, aC;
-        aS.zero(); aN.zero(); aC.zero();
-        for (int e = e0 + j; e < e1; e += 4) {
-            const int loc = L[e];
-            const AT w = (AT)W[e];
-            AT x, n = AT(1);
-            if (sizeof(AT) == 8) {
-                x = (AT)img_f64<DT>(planes[oimg + loc]);
-                if (odark >= 0) x = x - (AT)__uint_as_float(planes[odark + loc]);
+        Acc<AT> a0, a1;  // the first quantity's sum (X: x, else n), and n's
+        a0.zero();
+        a1.zero();
+        if (X && norm) {
+            if constexpr (sizeof(AT) == 4) {
+                f32x2 s = 0ull, c = 0ull;
+                for (int e = e0 + j; e < e1; e += 4) {
+                    const int loc = L[e];
+                    const float w = W[e];
+                    kahan2_add(s, c, f2_pack(w, w), f2_pack(image(loc), normal(loc)));
+                }
+                f2_unpack(s, a0.k.s, a1.k.s);
+                f2_unpack(c, a0.k.nc, a1.k.nc);
             } else {
-                float v = img_f32<DT>(planes[oimg + loc]);
-                if (odark >= 0) v = __fsub_rn(v, __uint_as_float(planes[odark + loc]));
-                x = (AT)v;
+                for (int e = e0 + j; e < e1; e += 4) {
+                    const int loc = L[e];
+                    const AT w = (AT)W[e];
+                    a0.add(w, image(loc));
+                    a1.add(w, normal(loc));
+                }
             }
-            if (oflat >= 0) n = n * (AT)__uint_as_float(planes[oflat + loc]);
-            if (osa >= 0) n = n * (AT)__uint_as_float(planes[osa + loc]);
-            if (opol >= 0) n = n * (AT)__uint_as_float(planes[opol + loc]);
-            aS.add(w, x);
-            if (!norm1) aN.add(w, n);
-            aC.add(w, AT(1));
+        } else {
+            for (int e = e0 + j; e < e1; e += 4) a0.add((AT)W[e], X ? image(L[e]) : normal(L[e]));
         }
         // lanes 0 and 2 form a0 + a1 and a2 + a3 (lower lane on the left); lane 0 adds them
-        aS.merge_lower_left(1); aC.merge_lower_left(1);
-        aS.merge_lower_left(2); aC.merge_lower_left(2);
-        if (!norm1) { aN.merge_lower_left(1); aN.merge_lower_left(2); }
+        a0.merge_lower_left(1);
+        a0.merge_lower_left(2);
+        if (X && norm) { a1.merge_lower_left(1); a1.merge_lower_left(2); }
         if (live && j == 0) {
-            out[slot] = aS.value();
-            out[(size_t)cp.nseg + slot] = norm1 ? aC.value() : aN.value();
-            out[2 * (size_t)cp.nseg + slot] = aC.value();
+            out[slot] = a0.value();
+            if (X && norm) out[(size_t)cp.nseg + slot] = a1.value();
         }
     }
 }
@@ -605,13 +646,12 @@ __device__ void consume_single_split(const ConsumerParams &cp, const unsigned ch
 template <class AT, class WT, int MODE, int NIMG, int DT>
 __device__ __forceinline__ void consume_dispatch(const ConsumerParams &cp, const unsigned char *stage,
                                                  const StageGeom &sg, int *ctr) {
-    if constexpr (MODE == MODE_SINGLE) {
-        if (cp.stage_entries) consume_single_split<AT, WT, DT, true>(cp, stage, sg, ctr);
-        else consume_single_split<AT, WT, DT, false>(cp, stage, sg, ctr);
+    if constexpr (MODE != MODE_FRAMES) {
+        if (cp.stage_entries) consume_split<AT, WT, DT, true, MODE == MODE_SINGLE>(cp, stage, sg, ctr);
+        else consume_split<AT, WT, DT, false, MODE == MODE_SINGLE>(cp, stage, sg, ctr);
     } else {
-        constexpr int Q = MODE == MODE_FRAMES ? NIMG : 2;
-        if (cp.stage_entries) consume_serial<Q, AT, WT, MODE, DT, true>(cp, stage, sg, ctr);
-        else consume_serial<Q, AT, WT, MODE, DT, false>(cp, stage, sg, ctr);
+        if (cp.stage_entries) consume_serial<NIMG, AT, WT, MODE, DT, true>(cp, stage, sg, ctr);
+        else consume_serial<NIMG, AT, WT, MODE, DT, false>(cp, stage, sg, ctr);
     }
 }
 
@@ -865,47 +905,6 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
     uint32_t v;
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
     return v;
-}
-
-// Two FP32 values in one 64-bit register, operated on by the packed f32x2 instructions
-// (round to nearest, no flush): each half gives exactly the scalar result.
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 f2_pack(float lo, float hi) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void f2_unpack(f32x2 x, float &lo, float &hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x));
-}
-__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-// a - b as b (-1) + a: the same single rounding of the same exact value.
-__device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b) {
-    return f2_fma(b, 0xbf800000bf800000ull, a);
-}
-// Two Kahan accumulators stepped together: the same operations as kahan_add on each half.
-__device__ __forceinline__ void kahan2_add(f32x2 &s, f32x2 &nc, f32x2 w, f32x2 v) {
-    const f32x2 y = f2_fma(w, v, nc);
-    const f32x2 t = f2_add(s, y);
-    nc = f2_sub(y, f2_sub(t, s));
-    s = t;
-}
-// ... and merged: kahan_merge on each half.
-__device__ __forceinline__ void kahan2_merge(f32x2 &as, f32x2 &an, f32x2 bs, f32x2 bn) {
-    const f32x2 t = f2_add(as, bs);
-    const f32x2 z = f2_sub(t, as);
-    const f32x2 e = f2_add(f2_sub(as, f2_sub(t, z)), f2_sub(bs, z));
-    an = f2_add(f2_add(an, bn), e);
-    as = t;
 }
 
 // One unit of work of a consumer warp: eight segments of the tile for the G frames of a stage.
@@ -1749,8 +1748,8 @@ __global__ void __launch_bounds__(256, 4) phase2_thread_kernel(const __grid_cons
         }
     } else if (MODE == MODE_SINGLE) {
         const AT S = row_sum_thread<AT>(P, a, b);
-        const AT N = d.single_nc == 2 ? static_cast<const AT *>(d.count)[r] : row_sum_thread<AT>(P + d.nseg, a, b);
-        const AT C = d.single_nc ? static_cast<const AT *>(d.count)[r] : row_sum_thread<AT>(P + 2 * (size_t)d.nseg, a, b);
+        const AT N = d.norm_is_count ? static_cast<const AT *>(d.count)[r] : row_sum_thread<AT>(P + d.nseg, a, b);
+        const AT C = static_cast<const AT *>(d.count)[r];
         if (d.oI) static_cast<AT *>(d.oI)[r] = N != AT(0) ? S / N : AT(0);
         if (d.oS) static_cast<AT *>(d.oS)[r] = S;
         if (d.oN) static_cast<AT *>(d.oN)[r] = N;
@@ -1759,11 +1758,6 @@ __global__ void __launch_bounds__(256, 4) phase2_thread_kernel(const __grid_cons
         const AT N = row_sum_thread<AT>(P, a, b);
         d.norm[r] = (float)N;
         if (d.oN) static_cast<float *>(d.oN)[r] = (float)N;
-        if (d.norm_rows == 2) {
-            const AT C = row_sum_thread<AT>(P + d.nseg, a, b);
-            d.norm[d.nrows + r] = (float)C;
-            if (d.oC) static_cast<float *>(d.oC)[r] = (float)C;
-        }
     }
 }
 
@@ -1793,8 +1787,8 @@ __global__ void phase2_kernel(const __grid_constant__ Inst single, const Inst *_
             const AT *P = static_cast<const AT *>(d.partial);
             if (MODE == MODE_SINGLE) {
                 const AT S = row_sum<AT>(P, a, b);
-                const AT N = d.single_nc == 2 ? static_cast<const AT *>(d.count)[r] : row_sum<AT>(P + d.nseg, a, b);
-                const AT C = d.single_nc ? static_cast<const AT *>(d.count)[r] : row_sum<AT>(P + 2 * (size_t)d.nseg, a, b);
+                const AT N = d.norm_is_count ? static_cast<const AT *>(d.count)[r] : row_sum<AT>(P + d.nseg, a, b);
+                const AT C = static_cast<const AT *>(d.count)[r];
                 if (lane == 0) {
                     const AT I = N != AT(0) ? S / N : AT(0);
                     if (d.oI) static_cast<AT *>(d.oI)[r] = I;
@@ -1804,14 +1798,9 @@ __global__ void phase2_kernel(const __grid_constant__ Inst single, const Inst *_
                 }
             } else {
                 const AT N = row_sum<AT>(P, a, b);
-                const AT C = d.norm_rows == 2 ? row_sum<AT>(P + d.nseg, a, b) : AT(0);
                 if (lane == 0) {
                     d.norm[r] = (float)N;
                     if (d.oN) static_cast<float *>(d.oN)[r] = (float)N;
-                    if (d.norm_rows == 2) {
-                        d.norm[d.nrows + r] = (float)C;
-                        if (d.oC) static_cast<float *>(d.oC)[r] = (float)C;
-                    }
                 }
             }
         }
@@ -1876,7 +1865,6 @@ Inst make_inst(const az_integrator *h, bool fp64) {
     d.rpw = 32 / h->frames_per_pass; d.nseg = L.nseg; d.nrows = h->nrows;
     d.npix = (int64_t)h->ny * h->nx;
     d.n_frames = 1; d.fpi = 1; d.n_groups = 1;
-    d.norm_rows = 2;
     d.partial = h->partial.p;
     d.norm = h->norm.as<float>();
     d.count = fp64 ? (const void *)h->count64.p : (const void *)(h->norm.as<float>() + h->nrows);
@@ -2366,14 +2354,14 @@ int count_layout(az_integrator *h, cudaStream_t s) {
                                                   L.nseg, h->partial.as<float>());
             AZ_CUDA(cudaGetLastError());
             d.oS = h->norm.as<float>() + h->nrows;
-            d.single_nc = 2;  // (S only)
+            d.norm_is_count = 1;  // (S only)
             AZ_TRY((run_phase2<float, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s)));
         } else {
             count_kernel<double><<<g, 256, 0, s>>>(start, start + L.nseg, L.seg_slot.as<int32_t>(), L.ent_w64.as<double>(),
                                                    L.nseg, h->partial.as<double>());
             AZ_CUDA(cudaGetLastError());
             d.oS = h->count64.p;
-            d.single_nc = 2;
+            d.norm_is_count = 1;
             AZ_TRY((run_phase2<double, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s)));
         }
     }
@@ -2399,7 +2387,7 @@ int forward_one(const az_integrator *h, const void *const arrs[5], int dtype, vo
     Inst d = make_inst(h, fp64);
     d.partial = partial;
     d.oI = oI; d.oS = oS; d.oN = oN; d.oC = oC;
-    d.single_nc = norm ? 1 : 2;
+    d.norm_is_count = !norm;
     return run_phase2<AT, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s, prof);
 }
 
@@ -2431,7 +2419,7 @@ int forward_planes(az_integrator *h, const void *image, int dtype, const float *
     if (rc != AZ_OK) return rc;
     Inst d = make_inst(h, false);
     d.oI = oI; d.oS = oS; d.oN = oN; d.oC = oC;
-    d.single_nc = corr ? 1 : 2;
+    d.norm_is_count = !corr;
     return run_phase2<float, MODE_SINGLE>(d, nullptr, 1, h->nrows, 1, s, &h->prof);
 }
 
@@ -2446,6 +2434,7 @@ int forward_general(const az_integrator *h, const void *const arrs[5], int dtype
     d.img = static_cast<const char *>(arrs[0]);
     d.dark = c[0]; d.flat = c[1]; d.sa = c[2]; d.pol = c[3];
     d.oI = oI; d.oS = oS; d.oN = oN; d.oC = oC;
+    d.norm_is_count = !(c[1] || c[2] || c[3]);
     const int planes = 1 + (c[0] != nullptr) + (c[1] != nullptr) + (c[2] != nullptr) + (c[3] != nullptr);
     StageGeom sg = choose_stage(plane_words_of(h), planes, (uint32_t)h->tl.max_tile_entries,
                                 fp64 ? 8 : 4, rec_words_of(h), d.stage_entries);
@@ -2531,7 +2520,6 @@ int batch_norm(az_integrator *h, const float *flat, const float *sa, const float
     Inst d = make_inst(h, false);
     d.flat = flat; d.sa = sa; d.pol = pol;
     d.oN = oN;
-    d.norm_rows = 1;
     if (engine_for(h) == AZ_COPY_TMA && h->tl.fslots >= 1) {
         // flat * solid angle * polarisation formed per pixel in the tiles of single_kernel: each
         // weight meets the same value as in the norm mode below, through the same accumulation.
@@ -2874,7 +2862,7 @@ int multi_create(az_integrator *const *hs, int n, const void *const *images, int
         d.oN = oN ? oN[k] : nullptr;
         d.oC = oC ? oC[k] : nullptr;
         if (P->engine == AZ_COPY_TMA) d.maps = &P->maps.as<TmaSet>()[k].m[0][0];
-        if (P->single) d.single_nc = P->norm ? 1 : 2;
+        d.norm_is_count = P->single ? !P->norm : !(d.flat || d.sa || d.pol);
         d.item_begin = items;
         d.row_begin = rows;
         items += d.n_items;
