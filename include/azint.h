@@ -497,7 +497,7 @@ int az_profile_read(az_integrator *h, az_profile *out);
  * width); it applies to tiles up to 236 pixels wide, wider tiles use AZ_COPY_ASYNC.
  * AZ_COPY_ASYNC issues 16-byte cp.async copies spread over the producer warps.  Results are
  * identical; only speed differs.  Default tiles follow the matrix's entries per pixel: 8 x 120
- * pixels below 2.1 (1D) or 48 x 40 below 2.4 (2D), then 16 x 64, 16 x 40 from 5, 16 x 24 from 10
+ * pixels below 2.1 (1D; 8 x 152 below 1.75 on large detectors) or 48 x 40 below 2.4 (2D), then 16 x 64, 16 x 40 from 5, 16 x 24 from 10
  * and 8 x 24 from 20 (larger ones where the segments would otherwise pass az_integrate_noalloc's
  * limit); 8 frames per pass. */
 int az_set_copy_engine(az_integrator *h, int engine);

@@ -65,7 +65,15 @@ int finish_build(az_integrator *h, cudaStream_t s) {
     // the time, wider rows make fewer pieces of a copy, which pays where the pixels do.  Frames
     // kernel, 8 x 120 against 16 x 64: 683 and 777 us (128 frames of 2527 x 2463 pixels, 1.7
     // entries per pixel), 273 and 244 us (37 frames of 2167 x 2070, 2.6), 45 and 40 us (24 variances
-    // of 1043 x 981, 2.8).  2D: 48 x 40 (500 x 360 bins of 2048 x 2048 pixels, 16 frames and one:
+    // of 1043 x 981, 2.8).
+    // Below 1.75 on large detectors, 8 x 152: a launch of few frames spends about 1.5 us an item, and
+    // has a fifth fewer of them (2527 x 2463: one to four frames against bound corrections 73 to 94
+    // us on 8 x 120, 64 to 82 here, twenty 205 and 179, 64 380 and 383; an FP64 frame 144 and 139;
+    // nine matrices of 2.9 to 6.2 Mpixel with 1.0 to 1.89 entries per pixel: 8 to 20% for up to 20
+    // frames, 1 to 10% for 48).  Above, three stages of the FP64 single-frame kernel no longer
+    // fit (2540 x 1800, 1.90: 119 and 173 us), as they do not with 8 x 168 (1.7: 144 and 200 us); with
+    // fewer than twelve tiles per SM (1043 x 981) the two are equal within 5%.
+    // 2D: 48 x 40 (500 x 360 bins of 2048 x 2048 pixels, 16 frames and one:
     // 91 and 29 us; 32 x 64, where only four frames fit a stage: 109 and 28 us; 24 x 56: 80 and 37).
     // Denser matrices get smaller tiles, so that the stages of the FP64 single-frame kernel (14
     // bytes an entry) still fit and no tile is cut: 962 x 972 pixels with 7.1 entries per pixel,
@@ -77,6 +85,8 @@ int finish_build(az_integrator *h, cudaStream_t s) {
     if (density < 10.0) { th = 16; tw = 40; }
     if (density < 5.0) { th = 16; tw = 64; }
     if (h->npt_azim == 0 && density < 2.1) { th = 8; tw = 120; }
+    const int64_t wide = (int64_t)((h->ny + 7) / 8) * ((h->nx + 151) / 152);
+    if (h->npt_azim == 0 && density < 1.75 && wide >= 12 * (int64_t)num_sms()) tw = 152;
     if (h->npt_azim > 0 && density < 2.4) { th = 48; tw = 40; }
     if (build_tiled_layout(h, th, tw, s) != AZ_OK) {  // a denser matrix: smaller tiles
         th = 8;
