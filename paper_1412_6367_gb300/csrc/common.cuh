@@ -393,7 +393,7 @@ int batch_norm(az_integrator *h, const float *flat, const float *sa, const float
                float *oC, cudaStream_t s);
 int batch_frames(az_integrator *h, const void *frames, int n, int dtype, const float *dark,
                  float *oI, float *oS, int frame_out0, cudaStream_t s,
-                 bool bound_dark = false, const float *norm = nullptr);
+                 bool bound_dark = false, const float *norm = nullptr, float *oN = nullptr, float *oC = nullptr);
 int bind_corrections(az_integrator *h, const float *dark, const float *flat, const float *sa,
                      const float *pol, cudaStream_t s);
 int forward_batch_bound(az_integrator *h, const void *frames, int n, int dtype, float *oI, float *oS,

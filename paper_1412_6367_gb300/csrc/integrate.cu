@@ -1721,6 +1721,12 @@ __device__ __forceinline__ AT row_sum_thread(const AT *p, int a, int b) {
     return row_tree<AT, 1>(p + a, b - a, 0).value();
 }
 
+// The frame-independent outputs of a batch, where asked for (a copy launch each cost 2 to 4 us).
+__device__ __forceinline__ void put_nc(const Inst &d, int r, float N) {
+    if (d.oN) static_cast<float *>(d.oN)[r] = N;
+    if (d.oC) static_cast<float *>(d.oC)[r] = static_cast<const float *>(d.count)[r];
+}
+
 // Phase 2 for rows of few slots (2D patterns have one or two): a thread per row, which in
 // frames mode takes kThreadFrames frames (blockIdx.y) so that the row's slot range and N are read
 // once for them and the frames' loads are independent.  Bound by memory traffic: a slot's sum is
@@ -1750,6 +1756,7 @@ __global__ void __launch_bounds__(256, 4) phase2_thread_kernel(const __grid_cons
             if (d.oS) static_cast<float *>(d.oS)[o] = S;
             if (d.oI) static_cast<float *>(d.oI)[o] = N != 0.f ? __fdiv_rn(S, N) : 0.f;
         }
+        if (f0 == 0) put_nc(d, r, N);
     } else if (MODE == MODE_SINGLE) {
         const AT S = row_sum_thread<AT>(P, a, b);
         const AT N = d.norm_is_count ? static_cast<const AT *>(d.count)[r] : row_sum_thread<AT>(P + d.nseg, a, b);
@@ -1761,7 +1768,7 @@ __global__ void __launch_bounds__(256, 4) phase2_thread_kernel(const __grid_cons
     } else {
         const AT N = row_sum_thread<AT>(P, a, b);
         d.norm[r] = (float)N;
-        if (d.oN) static_cast<float *>(d.oN)[r] = (float)N;
+        put_nc(d, r, (float)N);
     }
 }
 
@@ -1783,6 +1790,7 @@ __global__ void phase2_kernel(const __grid_constant__ Inst single, const Inst *_
                 const size_t o = (size_t)(d.frame_out0 + f) * d.nrows + r;
                 if (d.oS) static_cast<float *>(d.oS)[o] = (float)S;
                 if (d.oI) static_cast<float *>(d.oI)[o] = N != 0.f ? __fdiv_rn((float)S, N) : 0.f;
+                if (f == 0) put_nc(d, r, N);
             }
         } else {
             const Inst &d = inst_of_row(single, multi, n_inst, job);
@@ -1804,7 +1812,7 @@ __global__ void phase2_kernel(const __grid_constant__ Inst single, const Inst *_
                 const AT N = row_sum<AT>(P, a, b);
                 if (lane == 0) {
                     d.norm[r] = (float)N;
-                    if (d.oN) static_cast<float *>(d.oN)[r] = (float)N;
+                    put_nc(d, r, (float)N);
                 }
             }
         }
@@ -2515,15 +2523,15 @@ int batch_norm(az_integrator *h, const float *flat, const float *sa, const float
                float *oC, cudaStream_t s) {
     const int nrows = h->nrows;
     float *Cdev = h->norm.as<float>() + nrows;
-    if (oC) AZ_CUDA(cudaMemcpyAsync(oC, Cdev, sizeof(float) * nrows, cudaMemcpyDeviceToDevice, s));
     if (!flat && !sa && !pol) {  // N = C
+        if (oC) AZ_CUDA(cudaMemcpyAsync(oC, Cdev, sizeof(float) * nrows, cudaMemcpyDeviceToDevice, s));
         AZ_CUDA(cudaMemcpyAsync(h->norm.as<float>(), Cdev, sizeof(float) * nrows, cudaMemcpyDeviceToDevice, s));
         if (oN) AZ_CUDA(cudaMemcpyAsync(oN, Cdev, sizeof(float) * nrows, cudaMemcpyDeviceToDevice, s));
         return AZ_OK;
     }
     Inst d = make_inst(h, false);
     d.flat = flat; d.sa = sa; d.pol = pol;
-    d.oN = oN;
+    d.oN = oN; d.oC = oC;
     if (engine_for(h) == AZ_COPY_TMA && h->tl.fslots >= 1) {
         // flat * solid angle * polarisation formed per pixel in the tiles of single_kernel: each
         // weight meets the same value as in the norm mode below, through the same accumulation.
@@ -2585,7 +2593,8 @@ int gather_darks(az_integrator *h, const float *dark, bool f, DevBuf &out, cudaS
 }
 
 int batch_frames(az_integrator *h, const void *frames, int n, int dtype, const float *dark,
-                 float *oI, float *oS, int frame_out0, cudaStream_t s, bool bound_dark, const float *norm) {
+                 float *oI, float *oS, int frame_out0, cudaStream_t s, bool bound_dark, const float *norm,
+                 float *oN, float *oC) {
     // the dark of every entry, in entry order, so that the frames pass reads it with the
     // weights instead of staging a dark plane with every group of frames (bound_dark: gathered
     // once by az_set_corrections)
@@ -2611,6 +2620,7 @@ int batch_frames(az_integrator *h, const void *frames, int n, int dtype, const f
                 if (norm) d.norm = const_cast<float *>(norm);
                 d.n_frames = nf;
                 d.oI = oI; d.oS = oS; d.frame_out0 = frame_out0 + f0;
+                if (f0 == 0) { d.oN = oN; d.oC = oC; }
                 AZ_TRY((run_phase2<float, MODE_FRAMES>(d, nullptr, 1, (int64_t)nf * h->nrows, nf, s, &h->prof)));
             }
             return AZ_OK;
@@ -2644,6 +2654,7 @@ int batch_frames(az_integrator *h, const void *frames, int n, int dtype, const f
         d.ent_dark = ent_dk ? ent_dark : nullptr;
         if (norm) d.norm = const_cast<float *>(norm);
         d.oI = oI; d.oS = oS; d.frame_out0 = frame_out0 + f0;
+        if (f0 == 0) { d.oN = oN; d.oC = oC; }
         d.stage_entries = stage_e;
         d.n_items = h->tl.n_active * d.n_groups;
         TmaSet tm;
@@ -2674,8 +2685,10 @@ int batch_pixelnorm(az_integrator *h, const void *frames, int n, int dtype, cons
     const int nrows = h->nrows;
     // C of the current layout
     const float *Cdev = h->norm.as<float>() + nrows;
-    if (oC) AZ_CUDA(cudaMemcpyAsync(oC, Cdev, sizeof(float) * nrows, cudaMemcpyDeviceToDevice, s));
-    if (n == 0) return AZ_OK;
+    if (n == 0) {
+        if (oC) AZ_CUDA(cudaMemcpyAsync(oC, Cdev, sizeof(float) * nrows, cudaMemcpyDeviceToDevice, s));
+        return AZ_OK;
+    }
     // per-pixel normalisation, per-entry corrected weights and darks
     const int64_t pblocks = std::min<int64_t>((npix + 255) / 256, (int64_t)num_sms() * 8);
     const int64_t eblocks = std::max<int64_t>(1, std::min<int64_t>((L.f_entries + 255) / 256, (int64_t)num_sms() * 8));
@@ -2708,6 +2721,7 @@ int batch_pixelnorm(az_integrator *h, const void *frames, int n, int dtype, cons
         d.n_frames = nf;
         d.norm = const_cast<float *>(Cdev);  // I = U / C
         d.oI = oI; d.oS = oU; d.frame_out0 = f0;
+        if (f0 == 0) d.oC = oC;
         AZ_TRY((run_phase2<float, MODE_FRAMES>(d, nullptr, 1, (int64_t)nf * nrows, nf, s, &h->prof)));
     }
     return AZ_OK;
@@ -2738,8 +2752,11 @@ int batch_variance(az_integrator *h, const void *frames, int n, int dtype, float
 int forward_batch(az_integrator *h, const void *frames, int n, int dtype, const float *dark,
                   const float *flat, const float *sa, const float *pol, float *oI, float *oS,
                   float *oN, float *oC, cudaStream_t s) {
-    AZ_TRY(batch_norm(h, flat, sa, pol, oN, oC, s));
-    return batch_frames(h, frames, n, dtype, dark, oI, oS, 0, s);
+    if (n == 0) return batch_norm(h, flat, sa, pol, oN, oC, s);
+    const bool corr = flat || sa || pol;
+    if (corr) AZ_TRY(batch_norm(h, flat, sa, pol, nullptr, nullptr, s));
+    const float *norm = corr ? nullptr : h->norm.as<float>() + h->nrows;  // N = C
+    return batch_frames(h, frames, n, dtype, dark, oI, oS, 0, s, false, norm, oN, oC);
 }
 
 // az_set_corrections: the frame-independent work of a batch formed once -- each entry's dark
@@ -2771,10 +2788,12 @@ int forward_batch_bound(az_integrator *h, const void *frames, int n, int dtype, 
                                "or the tiled layout changed since they were");
     const float *bN = h->bound_norm.as<float>();
     const size_t rb = sizeof(float) * (size_t)h->nrows;
-    if (oN) AZ_CUDA(cudaMemcpyAsync(oN, bN, rb, cudaMemcpyDeviceToDevice, s));
-    if (oC) AZ_CUDA(cudaMemcpyAsync(oC, bN + h->nrows, rb, cudaMemcpyDeviceToDevice, s));
-    if (n == 0) return AZ_OK;
-    return batch_frames(h, frames, n, dtype, nullptr, oI, oS, 0, s, h->corr_dark, bN);
+    if (n == 0) {
+        if (oN) AZ_CUDA(cudaMemcpyAsync(oN, bN, rb, cudaMemcpyDeviceToDevice, s));
+        if (oC) AZ_CUDA(cudaMemcpyAsync(oC, bN + h->nrows, rb, cudaMemcpyDeviceToDevice, s));
+        return AZ_OK;
+    }
+    return batch_frames(h, frames, n, dtype, nullptr, oI, oS, 0, s, h->corr_dark, bN, oN, oC);
 }
 
 // ------------------------------------------------------------------------------------
