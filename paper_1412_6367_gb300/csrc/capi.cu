@@ -305,7 +305,7 @@ extern "C" int az_integrator_info(const az_integrator *h, az_info *out) {
                             &h->partial, &h->norm, &h->adj, &h->status, &h->host_stage,
                             &h->tl.tile_desc, &h->tl.tile_rec, &h->tl.ent_pix, &h->tl.ent_dark,
                             &h->tl.norm_frames, &h->tl.ent_wnorm, &h->lut32, &h->lut64,
-                            &h->lut_vals, &h->lut_part, &h->one_planes, &h->bound_ent_dark, &h->bound_dark_f,
+                            &h->lut_vals, &h->lut_part, &h->one_planes, &h->bound_dark[0], &h->bound_dark[1],
                             &h->bound_norm};
     int64_t tot = 0;
     for (const DevBuf *b : bufs) tot += (int64_t)b->bytes;
@@ -631,8 +631,11 @@ extern "C" int az_set_copy_engine(az_integrator *h, int engine) {
     if (!h) return fail(AZ_EINVAL, "az_set_copy_engine: NULL integrator");
     if (engine != AZ_COPY_TMA && engine != AZ_COPY_ASYNC)
         return fail(AZ_EINVAL, "az_set_copy_engine: bad engine %d", engine);
+    const int before = h->copy_engine;
     h->copy_engine = engine;
-    return AZ_OK;
+    const int rc = convert_bound_darks(h, h->last_stream);
+    if (rc != AZ_OK) h->copy_engine = before;
+    return rc;
 }
 
 extern "C" int az_set_tuning(az_integrator *h, int tile_h, int tile_w, int rows_per_warp,

@@ -326,8 +326,10 @@ struct az_integrator {
     int layout = AZ_LAYOUT_TILED;  // what az_integrate1d/2d use
     // corrections bound by az_set_corrections: per-entry darks, N and C of the current layout
     bool corr_bound = false, corr_dark = false;
-    azint::DevBuf bound_ent_dark;  // float [padded_nnz], entry order of the general kernel
-    azint::DevBuf bound_dark_f;    // float [f_entries], of the frames kernel
+    // ... the darks in the entry order of the kernel a batch takes, in the other one only after a
+    // change of the copy engine ([0] general kernel: float [padded_nnz]; [1] frames kernel: [f_entries])
+    azint::DevBuf bound_dark[2];
+    bool bound_dark_ok[2] = {false, false};
     azint::DevBuf bound_norm;      // float [2][nrows]: N, C
     // host copies for the end-to-end path
     azint::DevBuf host_stage;  // device frames buffer for az_integrate_batch_host
@@ -394,6 +396,8 @@ int batch_norm(az_integrator *h, const float *flat, const float *sa, const float
 int batch_frames(az_integrator *h, const void *frames, int n, int dtype, const float *dark,
                  float *oI, float *oS, int frame_out0, cudaStream_t s,
                  bool bound_dark = false, const float *norm = nullptr, float *oN = nullptr, float *oC = nullptr);
+// the bound darks in the order that the current copy engine's kernel reads
+int convert_bound_darks(az_integrator *h, cudaStream_t s);
 int bind_corrections(az_integrator *h, const float *dark, const float *flat, const float *sa,
                      const float *pol, cudaStream_t s);
 int forward_batch_bound(az_integrator *h, const void *frames, int n, int dtype, float *oI, float *oS,

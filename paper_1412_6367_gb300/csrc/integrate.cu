@@ -2608,7 +2608,7 @@ int batch_frames(az_integrator *h, const void *frames, int n, int dtype, const f
         int G = 0;
         if (n > 0 && fr_plan(h, std::min(chunk, n), ent_dk, fa, fgeo, G)) {
             if (dark && !bound_dark) AZ_TRY(gather_darks(h, dark, true, h->tl.ent_dark, s));
-            const float *ent_dark = !ent_dk ? nullptr : (bound_dark ? h->bound_dark_f : h->tl.ent_dark).as<float>();
+            const float *ent_dark = !ent_dk ? nullptr : (bound_dark ? h->bound_dark[1] : h->tl.ent_dark).as<float>();
             for (int f0 = 0; f0 < n; f0 += chunk) {
                 const int nf = std::min(chunk, n - f0);
                 Inst d = make_inst(h, false);
@@ -2627,7 +2627,7 @@ int batch_frames(az_integrator *h, const void *frames, int n, int dtype, const f
         }
     }
     if (dark && !bound_dark) AZ_TRY(gather_darks(h, dark, false, h->tl.ent_dark, s));
-    const float *ent_dark = (bound_dark ? h->bound_ent_dark : h->tl.ent_dark).as<float>();
+    const float *ent_dark = (bound_dark ? h->bound_dark[0] : h->tl.ent_dark).as<float>();
     // frames per pass as tuned, halved while two stages of that many frame planes do not fit,
     // or while the tile's entries would not fit beside them (down to 4 frames per pass)
     int fpi = h->frames_per_pass;
@@ -2759,6 +2759,41 @@ int forward_batch(az_integrator *h, const void *frames, int n, int dtype, const 
     return batch_frames(h, frames, n, dtype, dark, oI, oS, 0, s, false, norm, oN, oC);
 }
 
+// Whether a batch with darks goes through the frames kernel.  (If one frame fits, any number does:
+// fr_plan comes down to the same stages.)
+bool takes_frames_kernel(const az_integrator *h) {
+    FrArgs a{};
+    FrGeom fg;
+    int G = 0;
+    return fr_plan(h, 1, 1, a, fg, G);
+}
+
+__global__ void scatter_dark_kernel(const int32_t *__restrict__ pix, const float *__restrict__ ent, int64_t n,
+                                    float *__restrict__ dark) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
+         e += (int64_t)gridDim.x * blockDim.x)
+        if (pix[e] >= 0) dark[pix[e]] = ent[e];  // (equal values for the entries of a pixel)
+}
+
+// The caller's dark is not at hand any more: its pixels from the entries of one order, then the
+// entries of the other.
+int convert_bound_darks(az_integrator *h, cudaStream_t s) {
+    const bool f = takes_frames_kernel(h);
+    if (!h->corr_bound || !h->corr_dark || h->bound_dark_ok[f]) return AZ_OK;
+    ScratchScope scope;
+    TmpBuf plane;
+    AZ_TRY(plane.alloc(sizeof(float) * (size_t)h->ny * (size_t)h->nx));
+    const int64_t n = f ? h->tl.padded_nnz : h->tl.f_entries;
+    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)num_sms() * 8));
+    scatter_dark_kernel<<<(unsigned)blocks, 256, 0, s>>>((f ? h->tl.ent_pix : h->tl.f_pix).as<int32_t>(),
+                                                         h->bound_dark[!f].as<float>(), n, plane.as<float>());
+    AZ_CUDA(cudaGetLastError());
+    AZ_TRY(gather_darks(h, plane.as<float>(), f, h->bound_dark[f], s));
+    AZ_CUDA(cudaStreamSynchronize(s));
+    h->bound_dark_ok[f] = true;
+    return AZ_OK;
+}
+
 // az_set_corrections: the frame-independent work of a batch formed once -- each entry's dark
 // (gathered from `dark`) and N, C per row -- into buffers of their own, which later calls of
 // az_integrate_batch do not touch.  The caller's arrays are not read again.
@@ -2766,10 +2801,11 @@ int bind_corrections(az_integrator *h, const float *dark, const float *flat, con
                      const float *pol, cudaStream_t s) {
     h->corr_bound = false;
     h->corr_dark = dark != nullptr;
+    h->bound_dark_ok[0] = h->bound_dark_ok[1] = false;
     if (dark) {
-        // for both kernels: which one a batch takes depends on the copy engine of the time
-        AZ_TRY(gather_darks(h, dark, false, h->bound_ent_dark, s));
-        if (h->tl.fslots) AZ_TRY(gather_darks(h, dark, true, h->bound_dark_f, s));
+        const bool f = takes_frames_kernel(h);
+        AZ_TRY(gather_darks(h, dark, f, h->bound_dark[f], s));
+        h->bound_dark_ok[f] = true;
     }
     if (h->bound_norm.bytes < 2 * sizeof(float) * (size_t)h->nrows)
         AZ_TRY(h->bound_norm.alloc(2 * sizeof(float) * (size_t)h->nrows));
