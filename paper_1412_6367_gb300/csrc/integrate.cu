@@ -1302,7 +1302,7 @@ __device__ __forceinline__ double to_double(uint32_t b) {
     return __hiloint2double((int)(sign | (((uint32_t)(1054 - lz) << 20) + ((m & 0x7fffffffu) >> 11))), (int)(m << 21));
 }
 
-template <class AT, int DT, bool X, bool N>
+template <class AT, int DT, bool X, bool N, bool V>
 __device__ __forceinline__ void sg_correct(const SgInst &d, const SgGeom &sg, unsigned char *stage, int part) {
     const int lane = threadIdx.x & 31;
     const int words = 4 * d.slot;
@@ -1358,6 +1358,7 @@ __device__ __forceinline__ void sg_correct(const SgInst &d, const SgGeom &sg, un
                 if (X) {
                     const uint4 u = *reinterpret_cast<const uint4 *>(img + p);
                     float4 v = make_float4(img_f32<DT>(u.x), img_f32<DT>(u.y), img_f32<DT>(u.z), img_f32<DT>(u.w));
+                    if (V) v = make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
                     if (dark) {
                         const float4 k = *reinterpret_cast<const float4 *>(dark + p);
                         v = make_float4(__fsub_rn(v.x, k.x), __fsub_rn(v.y, k.y), __fsub_rn(v.z, k.z), __fsub_rn(v.w, k.w));
@@ -1380,6 +1381,7 @@ __device__ __forceinline__ void sg_correct(const SgInst &d, const SgGeom &sg, un
             for (int p = p0 + lane; p < p1; p += 32) {
                 if (X) {
                     float v = img_f32<DT>(img[p]);
+                    if (V) v = fmaxf(v, 0.f);
                     if (dark) v = __fsub_rn(v, dark[p + sh]);
                     x[p] = v;
                 }
@@ -1394,7 +1396,7 @@ __device__ __forceinline__ void sg_correct(const SgInst &d, const SgGeom &sg, un
     }
 }
 
-template <class AT, bool X, bool N>
+template <class AT, bool X, bool N, bool V>
 __device__ __forceinline__ void sg_unit(const SgInst &d, const SgGeom &sg, const unsigned char *stage, int u) {
     const int lane = threadIdx.x & 31, j = lane & 3;
     const int *unit = reinterpret_cast<const int *>(stage) + kUnitWords * u;
@@ -1455,8 +1457,11 @@ __device__ __forceinline__ void sg_unit(const SgInst &d, const SgGeom &sg, const
             const uint32_t pv = X ? px : pn;
             Kahan k{0.f, 0.f};
 #pragma unroll 4
-            for (int t = 0; t < n; ++t)
-                kahan_add(k, W[32 * t], __uint_as_float(lds_u32(pv + ((uint32_t)L[32 * t] << 2))));
+            for (int t = 0; t < n; ++t) {
+                float w = W[32 * t];
+                if (V) w = __fmul_rn(w, w);
+                kahan_add(k, w, __uint_as_float(lds_u32(pv + ((uint32_t)L[32 * t] << 2))));
+            }
             kahan_merge(k, shfl_xor(k, 1));
             kahan_merge(k, shfl_xor(k, 2));
             if (slot >= 0 && j == 0) out[slot] = kahan_value(k);
@@ -1464,8 +1469,9 @@ __device__ __forceinline__ void sg_unit(const SgInst &d, const SgGeom &sg, const
     }
 }
 
-// X: the signal sums S; N: the normalisation sums (with X: after S).
-template <class AT, int DT, bool X, bool N>
+// X: the signal sums S; N: the normalisation sums (with X: after S); V (FP32, the image alone): the
+// propagated variance sum w^2 max(img, 0) in place of S.
+template <class AT, int DT, bool X, bool N, bool V = false>
 __global__ void __launch_bounds__(kSgThreads, 1)
 single_kernel(const __grid_constant__ SgInst one, const SgInst *__restrict__ multi, int n_inst, int n_items,
               SgGeom sg, const __grid_constant__ TmaSet tm) {
@@ -1644,12 +1650,12 @@ single_kernel(const __grid_constant__ SgInst one, const SgInst *__restrict__ mul
         const int x = u - first;
         if (x < nc) {
             if (!wait(k + 1, &full[s1], t1)) return;
-            sg_correct<AT, DT, X, N>(*d1, sg, smem + (size_t)s1 * sg.stage_bytes, x);
+            sg_correct<AT, DT, X, N, V>(*d1, sg, smem + (size_t)s1 * sg.stage_bytes, x);
             __syncwarp();
             if (lane == 0) mbar_arrive(&conv[s1]);
         } else {
             if (!wait(k, &conv[s0], t0)) return;
-            sg_unit<AT, X, N>(*d0, sg, smem + (size_t)s0 * sg.stage_bytes, x - nc);
+            sg_unit<AT, X, N, V>(*d0, sg, smem + (size_t)s0 * sg.stage_bytes, x - nc);
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[s0]);
         }
@@ -2254,12 +2260,12 @@ int sg_maps(const az_integrator *h, const void *const arrs[5], TmaSet &tm) {
     return AZ_OK;
 }
 
-template <class AT, int DT, bool X, bool N>
+template <class AT, int DT, bool X, bool N, bool V = false>
 int sg_launch(const SgInst &one, const SgInst *multi, int n_inst, int n_items, const SgGeom &sg, const TmaSet &tm,
               cudaStream_t s, Profiler *prof, int kind) {
     if (n_items <= 0) return AZ_OK;
     const uint32_t smem = (uint32_t)sg.nstages * sg.stage_bytes + kSgFixedBytes;
-    auto kern = single_kernel<AT, DT, X, N>;
+    auto kern = single_kernel<AT, DT, X, N, V>;
     AZ_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     ProfScope ps(prof, kind, s);
     kern<<<std::min(n_items, num_sms()), kSgThreads, smem, s>>>(one, multi, n_inst, n_items, sg, tm);
@@ -2727,6 +2733,25 @@ int batch_pixelnorm(az_integrator *h, const void *frames, int n, int dtype, cons
     return AZ_OK;
 }
 
+// One frame's variance sums through single_kernel; AZ_EUNSUPPORTED (without error text) where its
+// stages do not fit.
+int variance_one(const az_integrator *h, const void *img, int dtype, cudaStream_t s) {
+    if (engine_for(h) != AZ_COPY_TMA || h->tl.fslots < 1) return AZ_EUNSUPPORTED;
+    const void *const arrs[5] = {img, nullptr, nullptr, nullptr, nullptr};
+    const SgInst one = sg_inst(h, false, arrs);
+    SgNeed need;
+    need.add(h, one.present);
+    SgGeom sg;
+    if (!sg_geom(need, false, false, sg)) return AZ_EUNSUPPORTED;
+    TmaSet tm;
+    AZ_TRY(sg_maps(h, arrs, tm));
+    switch (dtype) {
+        case AZ_DTYPE_F32: return sg_launch<float, AZ_DTYPE_F32, true, false, true>(one, nullptr, 1, one.n_items, sg, tm, s, &h->prof, 0);
+        case AZ_DTYPE_U32: return sg_launch<float, AZ_DTYPE_U32, true, false, true>(one, nullptr, 1, one.n_items, sg, tm, s, &h->prof, 0);
+        default: return sg_launch<float, AZ_DTYPE_I32, true, false, true>(one, nullptr, 1, one.n_items, sg, tm, s, &h->prof, 0);
+    }
+}
+
 // Propagated variance of the signal sums, V = sum w^2 max(img, 0), for n frames through the
 // frames kernel (chunks of up to kMaxFramesPerLaunch frames), written to oV [n][nrows].
 int batch_variance(az_integrator *h, const void *frames, int n, int dtype, float *oV, cudaStream_t s) {
@@ -2738,7 +2763,8 @@ int batch_variance(az_integrator *h, const void *frames, int n, int dtype, float
         const int nf = std::min(chunk, n - f0);
         Inst d = make_inst(h, false);
         d.img = static_cast<const char *>(frames) + (size_t)f0 * (size_t)d.npix * 4u;
-        const int rc = frames_v3(h, d.img, nf, dtype, nullptr, 0, s, true);
+        int rc = nf == 1 ? variance_one(h, d.img, dtype, s) : AZ_EUNSUPPORTED;
+        if (rc == AZ_EUNSUPPORTED) rc = frames_v3(h, d.img, nf, dtype, nullptr, 0, s, true);
         if (rc == AZ_EUNSUPPORTED)
             return fail(AZ_EUNSUPPORTED, "az_integrate_variance: the tiles do not fit in shared memory");
         AZ_TRY(rc);
