@@ -2304,13 +2304,16 @@ __global__ void norm_pixels_kernel(const float *__restrict__ flat, const float *
 }
 
 // Weight of each entry divided by its pixel's flat * solid angle * polarisation (0 for
-// padding entries): the weights of the per-pixel-corrected form.
+// padding entries): the weights of the per-pixel-corrected form; and, with a dark, its pixel's dark.
+// (In two passes, each reading the entries' pixels, a call with one 2527 x 2463 frame took 137 us.)
 __global__ void gather_wnorm_kernel(const int32_t *__restrict__ pix, const float *__restrict__ w,
-                                    const float *__restrict__ npx, int64_t n, float *__restrict__ out) {
+                                    const float *__restrict__ npx, const float *__restrict__ dark, int64_t n,
+                                    float *__restrict__ out, float *__restrict__ out_dark) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
          e += (int64_t)gridDim.x * blockDim.x) {
         const int32_t p = pix[e];
         out[e] = p >= 0 ? __fdiv_rn(w[e], npx[p]) : 0.f;
+        if (dark) out_dark[e] = p >= 0 ? dark[p] : 0.f;
     }
 }
 
@@ -2701,18 +2704,16 @@ int batch_pixelnorm(az_integrator *h, const void *frames, int n, int dtype, cons
     if (L.norm_frames.bytes < sizeof(float) * (size_t)npix) AZ_TRY(L.norm_frames.alloc(sizeof(float) * (size_t)npix));
     if (L.ent_wnorm.bytes < sizeof(float) * (size_t)L.f_entries)
         AZ_TRY(L.ent_wnorm.alloc(sizeof(float) * (size_t)L.f_entries));
+    if (dark && L.ent_dark.bytes < sizeof(float) * (size_t)L.f_entries)
+        AZ_TRY(L.ent_dark.alloc(sizeof(float) * (size_t)L.f_entries));
+    const float *ent_dk = dark ? L.ent_dark.as<float>() : nullptr;
     {
         ProfScope ps(&h->prof, 4, s);
         norm_pixels_kernel<<<(unsigned)pblocks, 256, 0, s>>>(flat, sa, pol, npix, L.norm_frames.as<float>());
         gather_wnorm_kernel<<<(unsigned)eblocks, 256, 0, s>>>(L.f_pix.as<int32_t>(), L.f_w32.as<float>(),
-                                                              L.norm_frames.as<float>(), L.f_entries,
-                                                              L.ent_wnorm.as<float>());
+                                                              L.norm_frames.as<float>(), dark, L.f_entries,
+                                                              L.ent_wnorm.as<float>(), L.ent_dark.as<float>());
         AZ_CUDA(cudaGetLastError());
-    }
-    const float *ent_dk = nullptr;
-    if (dark) {
-        AZ_TRY(gather_darks(h, dark, true, L.ent_dark, s));
-        ent_dk = L.ent_dark.as<float>();
     }
     const int64_t cap = (int64_t)(h->partial_bytes / (sizeof(float) * (size_t)std::max(L.nseg, 1)));
     const int chunk = (int)std::max<int64_t>(1, std::min<int64_t>(cap, kMaxFramesPerLaunch));
