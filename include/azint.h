@@ -393,6 +393,12 @@ void az_multi_destroy(az_multi *plan);
  */
 int az_autotune(az_integrator *h, int n_trial_frames, az_stream_t stream, double *best_ms);
 
+/* The pixel tiles az_autotune would time for this integrator: (height, width) pairs, up to
+ * `capacity` of them, into tiles (host int32[2 * capacity]; may be NULL with 0), their number into
+ * *n_tiles.  The integrator's present tile comes first, so that tuning does not leave it with a
+ * slower batch than it had.  Host-only. */
+int az_autotune_tiles(const az_integrator *h, int32_t *tiles, int capacity, int *n_tiles);
+
 /* Set the tuning by hand (0 keeps the current value).  tile_w must be a multiple of 4;
  * frames_per_pass is 1, 2, 4, 8, 16 or 32 and rows_per_warp = 32 / frames_per_pass (either
  * may be given; both must agree).  If the layout of the new tiles cannot be built (AZ_ENOMEM,

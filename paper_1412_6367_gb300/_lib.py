@@ -84,6 +84,7 @@ SIGNATURES = {
     "az_multi_launch": ([vp, i32, vp], i32),
     "az_multi_destroy": ([vp], None),
     "az_autotune": ([vp, i32, vp, ctypes.POINTER(ctypes.c_double)], i32),
+    "az_autotune_tiles": ([vp, vp, i32, ctypes.POINTER(i32)], i32),
     "az_set_tuning": ([vp, i32, i32, i32, i32], i32),
     "az_lut_build": ([vp, i32, vp], i32),
     "az_lut_export": ([vp, vp, vp, vp, vp], i32),

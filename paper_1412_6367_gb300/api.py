@@ -405,6 +405,13 @@ class Integrator:
         self.refresh_info()
         return best.value
 
+    def autotune_tiles(self):
+        """The (height, width) pixel tiles that autotune() times, the present one first."""
+        n = ctypes.c_int(0)
+        t = (ctypes.c_int32 * 64)()
+        check(self._lib.az_autotune_tiles(self._h, ctypes.cast(t, ctypes.c_void_p), 32, ctypes.byref(n)))
+        return [(t[2 * k], t[2 * k + 1]) for k in range(n.value)]
+
     def set_copy_engine(self, engine):
         """"tma" (one bulk copy per tile row) or "async" (16-byte cp.async copies)."""
         code = {"tma": 0, "async": 1}[engine] if isinstance(engine, str) else int(engine)

@@ -59,8 +59,9 @@ void restore_tiles(az_integrator *h, int th, int tw, cudaStream_t s) {
     memcpy(g_err, text, sizeof(text));
 }
 
-int finish_build(az_integrator *h, cudaStream_t s) {
-    // Default tiles; az_autotune refines them per matrix.  1D: 8 x 120, or 16 x 64 from 2.1 entries
+// Default tiles.
+void default_tile(const az_integrator *h, int &th, int &tw) {
+    // az_autotune refines them per matrix.  1D: 8 x 120, or 16 x 64 from 2.1 entries
     // per pixel on -- taller tiles make fewer, longer segments, which pays where the entries set
     // the time, wider rows make fewer pieces of a copy, which pays where the pixels do.  Frames
     // kernel, 8 x 120 against 16 x 64: 683 and 777 us (128 frames of 2527 x 2463 pixels, 1.7
@@ -80,7 +81,7 @@ int finish_build(az_integrator *h, cudaStream_t s) {
     // 16 x 40 against 16 x 64: FP64 frame 80 and 260 us, 16 frames 134 and 173 us; with 4.0 entries
     // 48 and 59, 92 and 89 us.
     const double density = (double)h->nnz / (double)std::max(h->n_unmasked, 1);
-    int th = 8, tw = 24;
+    th = 8; tw = 24;
     if (density < 20.0) { th = 16; tw = 24; }
     if (density < 10.0) { th = 16; tw = 40; }
     if (density < 5.0) { th = 16; tw = 64; }
@@ -88,6 +89,11 @@ int finish_build(az_integrator *h, cudaStream_t s) {
     const int64_t wide = (int64_t)((h->ny + 7) / 8) * ((h->nx + 151) / 152);
     if (h->npt_azim == 0 && density < 1.75 && wide >= 12 * (int64_t)num_sms()) tw = 152;
     if (h->npt_azim > 0 && density < 2.4) { th = 48; tw = 40; }
+}
+
+int finish_build(az_integrator *h, cudaStream_t s) {
+    int th = 0, tw = 0;
+    default_tile(h, th, tw);
     if (build_tiled_layout(h, th, tw, s) != AZ_OK) {  // a denser matrix: smaller tiles
         th = 8;
         tw = 64;
@@ -735,6 +741,36 @@ static int tune_layout(az_integrator *h, const void *frame, const float *dark, c
     return AZ_OK;
 }
 
+// The tiles az_autotune times: the integrator's own first, the default of its matrix, and others:
+// small ones where the entries are many (16 x 40 with 7.1 entries per pixel: a batch of 16 frames 121
+// us, 16 x 64 173; an FP64 frame 77 and 260).
+static std::vector<std::pair<int, int>> trial_tiles(const az_integrator *h) {
+    std::vector<std::pair<int, int>> out{{h->tl.th, h->tl.tw}};
+    int th = 0, tw = 0;
+    default_tile(h, th, tw);
+    out.emplace_back(th, tw);
+    for (const auto &t : {std::pair<int, int>{8, 120}, {16, 64}, {16, 96}, {16, 56}, {32, 64}}) out.push_back(t);
+    if ((double)h->nnz < 4.0 * (double)std::max(h->n_unmasked, 1))
+        for (const auto &t : {std::pair<int, int>{8, 224}, {8, 152}, {48, 40}, {24, 56}}) out.push_back(t);
+    else
+        for (const auto &t : {std::pair<int, int>{8, 64}, {16, 40}, {16, 24}, {8, 24}}) out.push_back(t);
+    for (size_t k = 0; k < out.size(); ++k)
+        out.erase(std::remove(out.begin() + k + 1, out.end(), out[k]), out.end());
+    return out;
+}
+
+extern "C" int az_autotune_tiles(const az_integrator *h, int32_t *tiles, int capacity, int *n_tiles) {
+    clear_error();
+    if (!h || !n_tiles || capacity < 0 || (capacity > 0 && !tiles)) return fail(AZ_EINVAL, "az_autotune_tiles: bad argument");
+    const auto t = trial_tiles(h);
+    *n_tiles = (int)t.size();
+    for (int k = 0; k < std::min(capacity, *n_tiles); ++k) {
+        tiles[2 * k] = t[(size_t)k].first;
+        tiles[2 * k + 1] = t[(size_t)k].second;
+    }
+    return AZ_OK;
+}
+
 extern "C" int az_autotune(az_integrator *h, int n_trial_frames, az_stream_t stream,
                            double *best_ms) {
     clear_error();
@@ -754,20 +790,20 @@ extern "C" int az_autotune(az_integrator *h, int n_trial_frames, az_stream_t str
     cudaEvent_t e0, e1;
     AZ_CUDA(cudaEventCreate(&e0));
     AZ_CUDA(cudaEventCreate(&e1));
-    const int tiles[][2] = {{8, 224}, {8, 120}, {16, 64}, {16, 96}, {16, 56}, {48, 40}, {32, 64}, {24, 56}};
+    const auto tiles = trial_tiles(h);
     const int fpps[] = {4, 8, 16};
     const int engines[] = {AZ_COPY_TMA, AZ_COPY_ASYNC};
     double best = 1e30;
     int bt = -1, bf = h->frames_per_pass, be = h->copy_engine;
-    const int tile_count = (int)(sizeof(tiles) / sizeof(tiles[0]));
-    for (int ti = 0; ti < tile_count; ++ti) {
-        if (set_tiles(h, tiles[ti][0], tiles[ti][1], s) != AZ_OK ||
+    for (int ti = 0; ti < (int)tiles.size(); ++ti) {
+        if (set_tiles(h, tiles[(size_t)ti].first, tiles[(size_t)ti].second, s) != AZ_OK ||
             batch_norm(h, nullptr, nullptr, nullptr, nullptr, nullptr, s) != AZ_OK) {
             clear_error();
             continue;
         }
         for (int eg : engines)
             for (int f : fpps) {
+                if (eg == AZ_COPY_TMA && f > 8) continue;  // the frames kernel takes eight at most
                 h->frames_per_pass = f;
                 h->copy_engine = eg;
                 float best_t = 1e30f;
@@ -792,7 +828,7 @@ extern "C" int az_autotune(az_integrator *h, int n_trial_frames, az_stream_t str
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     const int rc = bt < 0 ? fail(AZ_EUNSUPPORTED, "az_autotune: no configuration ran")
-                          : set_tiles(h, tiles[bt][0], tiles[bt][1], s);
+                          : set_tiles(h, tiles[(size_t)bt].first, tiles[(size_t)bt].second, s);
     if (rc != AZ_OK) {  // as it was
         h->frames_per_pass = fpp0;
         h->copy_engine = engine0;
