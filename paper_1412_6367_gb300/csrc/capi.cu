@@ -95,25 +95,29 @@ int finish_build(az_integrator *h, cudaStream_t s) {
     int th = 0, tw = 0;
     default_tile(h, th, tw);
     if (build_tiled_layout(h, th, tw, s) != AZ_OK) {  // a denser matrix: smaller tiles
+        clear_error();
         th = 8;
         tw = 64;
         AZ_TRY(build_tiled_layout(h, th, tw, s));
     }
     // The allocation-free entry point takes integrators whose FP64 partial sums fit its fixed
     // array, or whose FP32 ones do (twice the segments).  A matrix past either limit gets larger
-    // tiles if they bring it below.
+    // tiles if they bring it below -- and if there is the memory for that: else its own stay.
     const int64_t most = (int64_t)AZ_NOALLOC_SCRATCH_BYTES / (3 * (int64_t)sizeof(double));
     if (h->tl.nseg > most) {
-        const int larger[2][2][2] = {{{16, 64}, {8, 224}}, {{32, 64}, {32, 64}}};
-        for (int k = 0; k < 2; ++k) {
-            const int *t = larger[h->npt_azim > 0][k];
+        const std::vector<std::pair<int, int>> larger =
+            h->npt_azim > 0 ? std::vector<std::pair<int, int>>{{32, 64}}
+                            : std::vector<std::pair<int, int>>{{16, 64}, {8, 224}};
+        const int64_t nseg = h->tl.nseg;
+        for (const auto &t : larger) {
             int64_t runs = 0;
-            AZ_TRY(count_runs(h, t[0], t[1], s, &runs));
-            if (runs >= 0 && (runs <= most || (h->tl.nseg > 2 * most && runs <= 2 * most))) {
-                AZ_TRY(build_tiled_layout(h, t[0], t[1], s));
+            if (count_runs(h, t.first, t.second, s, &runs) != AZ_OK) break;
+            if (runs <= most || (nseg > 2 * most && runs <= 2 * most)) {
+                if (build_tiled_layout(h, t.first, t.second, s) != AZ_OK) AZ_TRY(build_tiled_layout(h, th, tw, s));
                 break;
             }
         }
+        clear_error();
     }
     h->frames_per_pass = 8;
     h->rows_per_warp = 32 / h->frames_per_pass;

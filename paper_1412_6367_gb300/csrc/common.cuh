@@ -351,7 +351,7 @@ int build_integrator(int ny, int nx, const double *rad, const double *chi, int n
                      int npt_azim, int unit, int split, const uint8_t *mask, cudaStream_t s,
                      az_integrator *h);
 int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s);
-// (tile, row) pairs that hold entries under th x tw tiles; -1 if not counted (too much scratch)
+// (tile, row) pairs that hold entries under th x tw tiles
 int count_runs(const az_integrator *h, int th, int tw, cudaStream_t s, int64_t *out);
 int import_csr(az_integrator *h, const int32_t *indptr, const int32_t *indices, const double *data,
                cudaStream_t s);

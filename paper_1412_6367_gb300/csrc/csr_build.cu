@@ -870,7 +870,7 @@ __global__ void scatter_slots_kernel(const int32_t *__restrict__ perm, int nseg,
         slot[perm[s]] = (int32_t)s;
 }
 
-// One bit per (row, tile) that has entries, and their number.
+// One bit per (row, tile) that has entries, for the rows of ptr, and their number.
 __global__ void mark_runs_kernel(TileGeom T, const int32_t *__restrict__ ptr, const int32_t *__restrict__ idx,
                                  int nrows, int64_t words, uint32_t *__restrict__ bits,
                                  unsigned long long *__restrict__ count) {
@@ -1255,21 +1255,25 @@ int import_csr(az_integrator *h, const int32_t *indptr, const int32_t *indices, 
 
 int count_runs(const az_integrator *h, int th, int tw, cudaStream_t s, int64_t *out) {
     ScratchScope scope;
-    *out = -1;
+    *out = 0;
     TileGeom T{};
     T.nx = h->nx; T.th = th; T.tw = tw; T.ntx = (h->nx + tw - 1) / tw;
     const int64_t words = ((int64_t)T.ntx * ((h->ny + th - 1) / th) + 31) / 32;
-    const size_t bytes = sizeof(uint32_t) * (size_t)words * (size_t)h->nrows;
-    if (bytes > ((size_t)1 << 30)) return AZ_OK;
+    // some rows at a time: up to 1 GiB of bits
+    const int step = (int)std::max<int64_t>(1, std::min<int64_t>(h->nrows, ((int64_t)1 << 28) / words));
+    const size_t bytes = sizeof(uint32_t) * (size_t)words * (size_t)step;
     TmpBuf bits, count;
     AZ_TRY(bits.alloc(bytes));
     AZ_TRY(count.alloc(sizeof(unsigned long long)));
-    AZ_CUDA(cudaMemsetAsync(bits.p, 0, bytes, s));
     AZ_CUDA(cudaMemsetAsync(count.p, 0, sizeof(unsigned long long), s));
-    mark_runs_kernel<<<std::min(h->nrows, num_sms() * 16), 256, 0, s>>>(T, h->csr_ptr.as<int32_t>(), h->csr_idx.as<int32_t>(),
-                                                                      h->nrows, words, bits.as<uint32_t>(),
-                                                                      count.as<unsigned long long>());
-    AZ_CUDA(cudaGetLastError());
+    for (int r0 = 0; r0 < h->nrows; r0 += step) {
+        const int nr = std::min(step, h->nrows - r0);
+        AZ_CUDA(cudaMemsetAsync(bits.p, 0, bytes, s));
+        mark_runs_kernel<<<std::min(nr, num_sms() * 16), 256, 0, s>>>(T, h->csr_ptr.as<int32_t>() + r0,
+                                                                    h->csr_idx.as<int32_t>(), nr, words,
+                                                                    bits.as<uint32_t>(), count.as<unsigned long long>());
+        AZ_CUDA(cudaGetLastError());
+    }
     unsigned long long n = 0;
     AZ_CUDA(cudaMemcpyAsync(&n, count.p, sizeof(n), cudaMemcpyDeviceToHost, s));
     AZ_CUDA(cudaStreamSynchronize(s));
