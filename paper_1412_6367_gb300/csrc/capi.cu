@@ -217,7 +217,7 @@ extern "C" int az_csr_build(const az_geometry *geom, int ny, int nx, int npt_rad
     const int64_t npos = corners ? (int64_t)(ny + 1) * (nx + 1) : (int64_t)ny * nx;
     // scratch of the whole build; at first positions, bin coordinates, counts and their sums
     ScratchScope scope;
-    AZ_TRY(ScratchScope::reserve((size_t)npos * 8 * (need_chi ? 3 : 2) + (size_t)ny * nx * 16 + ((size_t)2 << 20)));
+    ScratchScope::reserve((size_t)npos * 8 * (need_chi ? 3 : 2) + (size_t)ny * nx * 16 + ((size_t)2 << 20));
     TmpBuf rad, chi;
     AZ_TRY(rad.alloc(sizeof(double) * npos));
     if (need_chi) AZ_TRY(chi.alloc(sizeof(double) * npos));

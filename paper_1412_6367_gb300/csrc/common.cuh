@@ -116,7 +116,7 @@ inline int alloc_parts(DevBuf &slab, std::initializer_list<Part> parts) {
 // not share chunks.
 struct ScratchScope {
     struct Pool {
-        static constexpr int kChunks = 64;
+        static constexpr int kChunks = 128;
         struct Chunk { char *p; size_t n; } chunks[kChunks] = {};
         int n_chunks = 0, chunk = 0;
         size_t off = 0;
@@ -158,8 +158,9 @@ struct ScratchScope {
         if (c->chunk == c->n_chunks) {
             if (c->n_chunks == Pool::kChunks) return fail(AZ_ENOMEM, "build scratch: more than %d chunks", Pool::kChunks);
             void *p = nullptr;
-            const size_t want = std::max(n, room);
+            size_t want = std::max(n, room);
             cudaError_t e = device_alloc(&p, want);
+            if (e != cudaSuccess && want > n) e = device_alloc(&p, want = n);
             if (e != cudaSuccess) return fail(AZ_ENOMEM, "cudaMalloc(%zu) failed: %s", want, cudaGetErrorString(e));
             c->chunks[c->n_chunks++] = {static_cast<char *>(p), want};
             c->off = 0;
@@ -168,12 +169,12 @@ struct ScratchScope {
         c->off += n;
         return AZ_OK;
     }
-    // Room for `n` more bytes in one chunk, ahead of several pieces.
-    static int reserve(size_t n) {
+    // Room for `n` more bytes in one chunk, ahead of several pieces.  It saves allocations and is
+    // not needed: without it (a device nearly full) the pieces are allocated as they are taken.
+    static void reserve(size_t n) {
         void *p = nullptr;
-        const int rc = take(n, &p, n);
-        if (rc == AZ_OK) current()->off -= (std::max<size_t>(n, 16) + 255) & ~(size_t)255;
-        return rc;
+        if (take(n, &p, n) == AZ_OK) current()->off -= (std::max<size_t>(n, 16) + 255) & ~(size_t)255;
+        else clear_error();
     }
 };
 

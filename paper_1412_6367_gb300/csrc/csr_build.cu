@@ -1197,8 +1197,8 @@ int build_integrator(int ny, int nx, const double *rad, const double *chi, int n
 
     // 4. pixel-major fill (the "scatter" view, kept as the CSC for the adjoint)
     AZ_TRY(alloc_matrix(h));
-    // the rest of the build takes about 60 bytes of scratch per entry
-    AZ_TRY(ScratchScope::reserve(72 * (size_t)nnz + ((size_t)4 << 20)));
+    // the rest of the build takes about 46 bytes of scratch per entry (the tiled layout; 20 here)
+    ScratchScope::reserve(46 * (size_t)nnz + ((size_t)4 << 20));
     TmpBuf pix;
     AZ_TRY(pix.alloc(sizeof(int32_t) * nnz));
     AZ_TRY(launch_gs(fill_kernel, npix, s, P, ptr64.as<int64_t>(), h->csc_row.as<int32_t>(),
@@ -1297,7 +1297,7 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     ++h->layout_no;
     h->layout_ok = false;   // until the caller has made the scratch of this layout too
     h->corr_bound = false;  // bound corrections are per layout (entry order, sums)
-    AZ_TRY(ScratchScope::reserve(66 * (size_t)nnz + ((size_t)2 << 20)));
+    ScratchScope::reserve(46 * (size_t)nnz + ((size_t)2 << 20));
 
     // row of each CSR entry, tile key of each CSR entry, stable sort by tile
     int32_t nseg = 0;
@@ -1306,6 +1306,7 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
     AZ_TRY(csr_row.alloc(sizeof(int32_t) * nnz));
     AZ_TRY(tkey.alloc(sizeof(uint32_t) * nnz));
     AZ_TRY(perm.alloc(sizeof(int32_t) * nnz));
+    AZ_TRY(seg_of.alloc(sizeof(int32_t) * nnz));
     AZ_TRY(launch_gs(csr_rows_kernel, nnz, s, h->csr_ptr.as<int32_t>(), h->nrows, nnz,
                      csr_row.as<int32_t>()));
     AZ_TRY(launch_gs(tile_keys_kernel, nnz, s, T, h->csr_idx.as<int32_t>(), nnz, tkey.as<uint32_t>()));
@@ -1320,11 +1321,11 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
         // up to 59 quads in a 16 x 64 tile of the 6-Mpixel detector, 15 on average); where that
         // makes more than kSegFew segments the pieces are made longer, because the partial sums
         // of a frame (24 bytes a segment in FP64) have to fit the allocation-free entry point.
+        ScratchScope inner;
         TmpBuf f0, id0, seg0, first0, key2;
         AZ_TRY(f0.alloc(sizeof(int32_t) * nnz));
         AZ_TRY(id0.alloc(sizeof(int32_t) * (nnz + 1)));
         AZ_TRY(seg0.alloc(sizeof(int32_t) * nnz));
-        AZ_TRY(seg_of.alloc(sizeof(int32_t) * nnz));
         AZ_TRY(launch_gs(seg_flags_kernel, nnz, s, tkey.as<uint32_t>(), perm.as<int32_t>(),
                          csr_row.as<int32_t>(), nnz, f0.as<int32_t>()));
         AZ_TRY(first0.alloc(sizeof(int32_t) * (nnz + 1)));

@@ -157,3 +157,24 @@ def test_a_plan_of_former_tiles_is_refused():
     out = api().MultiPlan([g, h], imgs).launch(use_graph=True)
     assert _equal([t.cpu() for t in out[0]], ref[:4])
     assert g.status() == 0 and h.status() == 0
+
+
+def test_builds_without_room_for_a_reservation():
+    """A build's scratch is reserved in one piece; where that piece does not fit, smaller ones do."""
+    c, g = _case(0)
+    ref = _all(c, g)
+    built = 0
+    for after in range(16):
+        api().selftest_alloc(after, 1)
+        try:
+            h = c.gpu_from_oracle_positions()
+            built += 1
+        except api().AzError as e:
+            assert e.code == ENOMEM
+            continue
+        finally:
+            api().selftest_alloc()
+        assert (h.info["tile_h"], h.info["tile_w"]) in ((g.info["tile_h"], g.info["tile_w"]), (8, 64))
+        if h.info["tile_w"] == g.info["tile_w"]:
+            assert _equal(_all(c, h), ref), after
+    assert built >= 3  # the two reservations, and more failures allowed than allocations made
