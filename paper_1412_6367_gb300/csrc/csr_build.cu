@@ -1326,8 +1326,6 @@ int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s) {
         AZ_TRY(f0.alloc(sizeof(int32_t) * nnz));
         AZ_TRY(id0.alloc(sizeof(int32_t) * (nnz + 1)));
         AZ_TRY(seg0.alloc(sizeof(int32_t) * nnz));
-        AZ_TRY(launch_gs(seg_flags_kernel, nnz, s, tkey.as<uint32_t>(), perm.as<int32_t>(),
-                         csr_row.as<int32_t>(), nnz, f0.as<int32_t>()));
         AZ_TRY(first0.alloc(sizeof(int32_t) * (nnz + 1)));
         auto number = [&]() -> int {  // segments of the flags: their ids and firsts
             AZ_TRY(exclusive_scan_i32(f0.as<int32_t>(), id0.as<int32_t>(), nnz, s));

@@ -51,11 +51,10 @@ enum Mode { MODE_SINGLE = 0, MODE_NORM = 1, MODE_FRAMES = 2 };
 // Everything phase 1 and phase 2 need about one integrator and its inputs.
 struct Inst {
     // tiled layout
-    const int32_t *tile_seg_ptr, *tile_ent_ptr, *active_tiles;
-    const int32_t *seg_start, *seg_end, *seg_slot, *row_slot_ptr;
+    const int32_t *row_slot_ptr;
     const uint16_t *ent_loc;
     const void *ent_w;
-    int ny, nx, th, tw, srow, ss, ntx, rpw, nseg, nrows;
+    int ny, nx, th, tw, srow, ss, ntx, nseg, nrows;
     int64_t npix;
     // inputs
     const char *img;  // first frame of this launch
@@ -1870,17 +1869,11 @@ StageGeom choose_stage(uint32_t plane_words, int planes, uint32_t max_entries, i
 Inst make_inst(const az_integrator *h, bool fp64) {
     Inst d{};
     const TiledLayout &L = h->tl;
-    d.tile_seg_ptr = L.tile_seg_ptr.as<int32_t>();
-    d.tile_ent_ptr = L.tile_ent_ptr.as<int32_t>();
-    d.active_tiles = L.active_tiles.as<int32_t>();
-    d.seg_start = L.seg_ent_ptr.as<int32_t>();
-    d.seg_end = L.seg_ent_ptr.as<int32_t>() + L.nseg;
-    d.seg_slot = L.seg_slot.as<int32_t>();
     d.row_slot_ptr = L.row_slot_ptr.as<int32_t>();
     d.ent_loc = L.ent_loc.as<uint16_t>();
     d.ent_w = fp64 ? (const void *)L.ent_w64.p : (const void *)L.ent_w32.p;
     d.ny = h->ny; d.nx = h->nx; d.th = L.th; d.tw = L.tw; d.srow = L.srow; d.ss = L.ss; d.ntx = L.ntx;
-    d.rpw = 32 / h->frames_per_pass; d.nseg = L.nseg; d.nrows = h->nrows;
+    d.nseg = L.nseg; d.nrows = h->nrows;
     d.npix = (int64_t)h->ny * h->nx;
     d.n_frames = 1; d.fpi = 1; d.n_groups = 1;
     d.partial = h->partial.p;
@@ -2658,7 +2651,6 @@ int batch_frames(az_integrator *h, const void *frames, int n, int dtype, const f
         Inst d = make_inst(h, false);
         d.img = static_cast<const char *>(frames) + (size_t)f0 * (size_t)d.npix * 4u;
         d.n_frames = nf; d.fpi = fpi; d.n_groups = (nf + fpi - 1) / fpi;
-        d.rpw = 32 / fpi;
         d.dark = dark;
         d.ent_dark = ent_dk ? ent_dark : nullptr;
         if (norm) d.norm = const_cast<float *>(norm);
