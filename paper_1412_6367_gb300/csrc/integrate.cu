@@ -39,8 +39,11 @@ namespace azint {
 
 namespace {
 
-constexpr int kProducers = 4;                               // producer warps per CTA
-constexpr int kConsumers = 16;                              // consumer warps per CTA
+// phase1_kernel's warps.  With the cp.async engine the staging holds an FP32 frame up: 2167 x 2070
+// pixels with four corrections took 120 us with 4 + 16, 114 with 6 + 14, 108 with 8 + 12 and 119 with
+// 8 + 16 warps, a batch of 16 frames 437, 402, 374 and 407.
+constexpr int kProducers = 8;                               // producer warps per CTA
+constexpr int kConsumers = 12;                              // consumer warps per CTA
 constexpr int kThreads = 32 * (kProducers + kConsumers);
 constexpr uint32_t kFullCount = 32u * kProducers + 1u;       // arrivals completing a stage
 constexpr int kMaxPlanes = 12;
@@ -658,9 +661,9 @@ __device__ __forceinline__ void consume_dispatch(const ConsumerParams &cp, const
     }
 }
 
-// Warp-specialised persistent kernel.  Warp 0 produces: for each work item of this CTA
-// (static round robin) it waits until the stage is free (empty barrier), copies the item
-// into it and arms the full barrier.  Warps 1..kConsumers consume: they wait for the item's
+// Warp-specialised persistent kernel.  The first kProducers warps produce: for each work item of
+// this CTA (static round robin) they wait until the stage is free (empty barrier), copy the item
+// into it and arm the full barrier.  The kConsumers others consume: they wait for the item's
 // full barrier, claim and reduce its segments, and release the stage (empty barrier, one
 // arrival per consumer warp).  Every wait is bounded; a wait that gives up records
 // AZ_ETIMEOUT in the status word, raises the CTA's abort flag and leaves, the producer
