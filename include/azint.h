@@ -197,11 +197,9 @@ void az_integrator_destroy(az_integrator *h);
  *   N_b = sum_p A_bp flat_p solid_angle_p pol_p  (out_sum_norm)
  *   C_b = sum_p A_bp                             (out_count)
  *   I_b = S_b / N_b, 0 where N_b == 0            (out_I)
- * with no output zeroing (Sec. 6.4's "memset").  FP64: one fused pass, the cast of the image
- * (Sec. 6.4 "cast"), the corrections ("correction") and the reduction ("integrate") in one
- * kernel.  FP32: a pixel pass forms cast(img) - dark and flat * solid_angle * polarization,
- * which the batched kernel then reduces (the bits of that frame in any batch); C is kept per
- * layout.  With az_set_layout(AZ_LAYOUT_LUT) both go through the look-up table instead.
+ * with no output zeroing (Sec. 6.4's "memset").  One fused pass: the cast of the image (Sec. 6.4
+ * "cast"), the corrections ("correction") and the reduction ("integrate") in one kernel, in both
+ * precisions; in FP32 with the bits of that frame in any batch.  C is kept per layout.  With az_set_layout(AZ_LAYOUT_LUT) both go through the look-up table instead.
  * image_dev: device [ny][nx] of image_dtype.  dark/flat/solid_angle/polarization: device
  * float [ny][nx], each may be NULL (dark = 0, the others = 1).  precision AZ_PREC_FP64:
  * FP64 weights and accumulation, outputs are device double[nrows]; AZ_PREC_FP32_COMP:
@@ -365,7 +363,8 @@ int az_integrate_backward(const az_integrator *h, const void *grad_I, const void
  * out_sum_norm[k] / out_count[k] (device float[nrows_k]; the pointer arrays may be NULL).
  * The plan flattens every (instance, tile) pair into one work list processed by one
  * persistent FP32-compensated launch, followed by one finalising launch.  The pointer
- * arrays are copied; the integrators must outlive the plan.  az_set_tuning and az_autotune free
+ * arrays are copied; the integrators must outlive the plan; one may be listed several times (each
+ * instance then has partial sums of its own).  az_set_tuning and az_autotune free
  * the layout a plan was made on: after other tiles az_multi_launch returns AZ_EINVAL.
  */
 int az_multi_create(az_integrator *const *handles, int n, const void *const *images,
@@ -478,7 +477,7 @@ int az_selftest_alloc(int64_t after, int64_t count);
 /* ---- kernel timing --------------------------------------------------------------------- */
 
 /* Per-kernel totals recorded while profiling is enabled.  Kinds: 0 = phase-1 frames kernel
- * (az_integrate_batch*), 1 = phase-1 kernel of the frame-independent sums N and C,
+ * (az_integrate_batch*, az_integrate_variance), 1 = phase-1 kernel of the frame-independent sum N,
  * 2 = phase-1 single-frame kernel (az_integrate1d/2d; with the look-up table, its gather),
  * 3 = phase-2 (finalise) kernel (with the look-up table, the chunk combination),
  * 4 = per-call preparation (per-entry dark gather, per-pixel flat * solid angle *
@@ -502,10 +501,13 @@ int az_profile_read(az_integrator *h, az_profile *out);
  * one class are 16 * width bytes apart, which meets the tensor-map stride rule for any
  * width); it applies to tiles up to 236 pixels wide, wider tiles use AZ_COPY_ASYNC.
  * AZ_COPY_ASYNC issues 16-byte cp.async copies spread over the producer warps.  Results are
- * identical; only speed differs.  Default tiles follow the matrix's entries per pixel: 8 x 120
- * pixels below 2.1 (1D; 8 x 152 below 1.75 on large detectors) or 48 x 40 below 2.4 (2D), then 16 x 64, 16 x 40 from 5, 16 x 24 from 10
- * and 8 x 24 from 20 (larger ones where the segments would otherwise pass az_integrate_noalloc's
- * limit); 8 frames per pass. */
+ * identical; only speed differs.  With corrections bound (az_set_corrections) the other engine may
+ * read the darks in another order: the call then forms it, synchronises their stream, and
+ * leaves the engine as it was if there is no memory for it (AZ_ENOMEM).
+ * Default tiles follow the matrix's entries per pixel: 8 x 120 pixels below 2.1 (1D; 8 x 152 below
+ * 1.75 on large detectors) or 48 x 40 below 2.4 (2D), then 16 x 64, 16 x 40 from 5, 16 x 24 from
+ * 10 and 8 x 24 from 20 (larger ones where the segments would otherwise pass
+ * az_integrate_noalloc's limit); 8 frames per pass. */
 int az_set_copy_engine(az_integrator *h, int engine);
 
 /* Thread-local message of the last failing call on this thread ("" if none). */

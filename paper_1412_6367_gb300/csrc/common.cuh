@@ -193,22 +193,23 @@ struct GeomParams {
 };
 
 // Pixel-tiled layout of the matrix used by the forward kernels.  Entries are grouped by
-// (tile, row, pixel); a "segment" is the run of one matrix row inside one tile.  Each
-// tile's entries start on a multiple of 8 entries so that they can be bulk-copied.
+// (tile, row, pixel); a "segment" is the run of one matrix row inside one tile, or a piece of a
+// long run.  phase1_kernel reads the padded entries ent_*, the other kernels the units f_*
+// (2 + 2 + 4 + 8 + 4 bytes a unit entry beside 18 a padded entry).  Each tile's entries start on a multiple of 8 entries so that they can be bulk-copied.
 struct TiledLayout {
-    int th = 0, tw = 0, srow = 0;      // tile rows/cols, shared-memory row pitch (tw + 4 words)
+    int th = 0, tw = 0, srow = 0;      // tile rows/cols, phase1_kernel's staged row (tw + 20 words)
     int ss = 0;                        // words per row-class slot (tile rows of equal index mod 4)
     int ntx = 0, nty = 0, ntiles = 0;  // tile grid
-    int n_active = 0;                  // tiles with at least one entry
+    int n_active = 0;                  // work items: tiles with entries, heavy ones in pieces
     int nseg = 0;
-    int max_tile_entries = 0;          // padded entry count of the largest tile
+    int max_tile_entries = 0;          // padded entry count of the largest item
     int max_tile_segments = 0;
     int64_t padded_nnz = 0;
     DevBuf slab_tiles, slab_entries, slab_items;  // hold the buffers below
     DevBuf tile_seg_ptr;    // int32 [ntiles + 1]
     DevBuf tile_ent_ptr;    // int32 [ntiles + 1]  (padded start of each tile's entries)
-    DevBuf active_tiles;    // int32 [n_active]
-    DevBuf seg_ent_ptr;     // int32 [nseg + 1]    (absolute, in the padded entry arrays)
+    DevBuf active_tiles;    // int32 [n_active]    (tile of the item)
+    DevBuf seg_ent_ptr;     // int32 [2][nseg]     (starts, ends, in the padded entry arrays)
     DevBuf seg_slot;        // int32 [nseg]        (position of the segment in row order)
     DevBuf row_slot_ptr;    // int32 [nrows + 1]
     DevBuf ent_loc;         // uint16 [padded_nnz] (shared-memory word offset in the tile)
@@ -235,7 +236,7 @@ struct TiledLayout {
                             // kernel that reads it
     DevBuf norm_frames;     // float  [ny][nx]: flat * solid angle * polarisation
     DevBuf ent_wnorm;       // float  [f_entries]: weight / (flat * solid angle * polarisation)
-    // Per active tile: a 32-byte descriptor {tile, record offset (words), record words,
+    // Per work item: a 32-byte descriptor {tile, record offset (words), record words,
     // entry offset, padded entry count, segment count, 0, 0} and a 16-byte aligned record
     // {tile, ns, entry offset, entry count, slot[ns], uint16 start[ns + 1]} that the forward
     // copies into shared memory with the tile.

@@ -1,29 +1,31 @@
 // Fused correction + sparse matrix-vector product (Sec. 5.2, Sec. 6.4) on the pixel-tiled
-// layout.  Every form ends with the same deterministic phase 2; phase 1 comes in two kernels:
+// layout.  Every form ends with the same deterministic phase 2; phase 1 comes in three kernels,
+// all persistent, one CTA per SM, their stages filled by bulk, tensor (or cp.async) copies that
+// mbarriers track, every wait bounded:
 //
-//   frames_kernel (persistent, one CTA per SM): a work item is a pixel tile (or a piece of
-//     a heavy one) for every frame of the launch.  One producer warp copies the item's
-//     units and entries (location, weight, per-entry dark) once into a ring of entry
-//     buffers and streams the tile's pixels, G frames at a time, into a ring of plane stages
-//     (bulk and tensor TMA, mbarrier-tracked, every wait bounded); 15 consumer warps take
-//     units of eight segments, four lanes a segment and G frames a lane, and write one partial
-//     sum per (segment, frame).  It serves
-//     batches, the frame-independent sums N and C, the propagated variance, the per-pixel-
-//     corrected form and single FP32 frames (after single_planes_kernel forms the corrected
-//     frame and its normalisation per pixel).
-//   phase1_kernel (persistent): one item per tile with all planes of one frame (image, dark,
-//     flat, solid angle, polarisation) and the tile's entries in a ring of stages; four
-//     lanes per segment form S, N and C.  It serves FP64 frames, the many-instance launch,
-//     the allocation-free entry point and the cp.async copy engine.
-//   phase 2: per (row, frame), the row's segment partials summed in a fixed order; then
-//     S, N, C and I = S / N.
+//   frames_kernel: a work item is a pixel tile (or a piece of a heavy one) for every frame of
+//     the launch.  One producer warp copies the item's units and entries (location, weight,
+//     per-entry dark) once into a ring of entry buffers and streams the tile's pixels, G frames
+//     at a time, into a ring of plane stages; 15 consumer warps take units of eight segments,
+//     four lanes a segment and G frames a lane, and write one partial sum per (segment, frame).
+//     Batches, the propagated variance of two frames or more, the per-pixel-corrected form.
+//   single_kernel: a stage holds an item's units, entries and the planes given (image, dark, flat,
+//     solid angle, polarisation) of one frame; 15 consumer warps correct the tile's pixels in
+//     shared memory, then reduce the units.  Single frames in both precisions (also without
+//     allocation), the many-detector plan, the normalisation sums N, the variance of one frame.
+//   phase1_kernel: one item per tile with the planes of one frame, or of fpi frames, and the
+//     tile's entries in a ring of stages.  The cp.async copy engine, and what does not fit the
+//     other two (FP32 single frames of large tiles go through single_planes_kernel, which
+//     writes the corrected frame and its normalisation, and frames_kernel).
+//   phase 2: per (row, frame), the row's segment partials summed in a fixed order; then S, N, C
+//     and I = S / N.  C = sum w is the layout's (count_layout).
 //
-// Where a segment is one matrix row's entries inside one tile.  The image cast, the dark
-// and flat * solid angle * polarisation are applied inside these kernels or in one per-pixel
-// pass (the paper runs separate cast / correction / memset / integrate kernels).  FP32 sums
-// are Kahan-compensated (Sec. 5.2.2); FP64 sums are plain.  No atomics touch the sums, so
-// results are bit-reproducible run to run, and a frame gives the same bits alone or in any
-// batch.
+// Where a segment is one matrix row's entries inside one tile, long runs cut in pieces of 96
+// entries.  The image cast, the dark and flat * solid angle * polarisation are applied inside these
+// kernels or in one per-pixel pass (the paper runs separate cast / correction / memset / integrate
+// kernels).  FP32 sums are Kahan-compensated (Sec. 5.2.2); FP64 sums are plain.  No atomics touch
+// the sums, so results are bit-reproducible run to run, and a frame gives the same bits alone or
+// in any batch.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -1240,11 +1242,13 @@ frames_kernel(const __grid_constant__ FrArgs a, FrGeom fg, const __grid_constant
 // FP64 (one 2527 x 2463 frame, four corrections): the FP64 pipe, whose instructions take 64 cycles a
 // warp, conversions to double included, needs about 66 us: per pixel one subtraction and two
 // products (the conversions are done with integer instructions, exactly), per entry two multiply-
-// adds.  The pass takes 140 us; correcting every entry and forming C each time took 351 us.
-// FP32 (the same frame): one launch of 66 us in place of a pass that wrote two planes to memory
-// (28 us) and the frames kernel over them (40 us).  Copies alone take 60 us, the entries and the
-// queue without planes 25 us: five arrays are twenty small copies an item.  16 detectors without
-// corrections: 278 us in place of 562 us.
+// adds.  A call takes 134 us with tiles of 8 x 152 (140 with 8 x 120); correcting every entry and
+// forming C each time took 351 us.
+// FP32 (the same frame): 70 us a call (80 with 8 x 120), where a pass that wrote two planes to memory
+// (28 us) and the frames kernel over them (40 us) took 78 with tiles of 8 x 224.  Of the 66 us of
+// the launch with 8 x 120 the copies alone take 60, the entries and the queue without planes 25:
+// five arrays are twenty small copies an item.  16 detectors without corrections: 309 us a call,
+// 609 through phase1_kernel.
 constexpr int kSgWarps = 15;
 constexpr int kSgThreads = 32 * (1 + kSgWarps);
 constexpr int kSgMaxStages = 8;
@@ -2512,8 +2516,9 @@ int preload_single_pass() {
 
 // One frame with the per-segment partial sums in a buffer the caller supplies (at least
 // 3 * nseg values of the accumulation type) instead of the integrator's own; no profiling and no
-// allocation.  (On the default tiles phase1_kernel, which took every such call before, needs 151 us
-// for a 2527 x 2463 FP32 frame with four corrections, 91 us on tiles of 8 x 224; single_kernel 76.)
+// allocation.  (phase1_kernel, which took every such call before, needed 151 us for a 2527 x 2463
+// FP32 frame with four corrections on 8 x 120 tiles and 94 on 8 x 224; this takes 80 and 62, and
+// 70 on the default 8 x 152.)
 int forward_single_into(const az_integrator *h, const void *image, int dtype, const float *dark,
                         const float *flat, const float *sa, const float *pol, int precision,
                         void *oI, void *oS, void *oN, void *oC, void *partial, cudaStream_t s) {
