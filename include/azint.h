@@ -502,10 +502,10 @@ int az_profile_read(az_integrator *h, az_profile *out);
  * width); it applies to tiles up to 236 pixels wide, wider tiles use AZ_COPY_ASYNC.
  * AZ_COPY_ASYNC issues 16-byte cp.async copies spread over the producer warps.  Results are
  * identical; only speed differs.  With corrections bound (az_set_corrections) the other engine may
- * read the darks in another order: the call then forms it, synchronises their stream, and
+ * read the darks in another order: the call then waits for the device and forms it, and
  * leaves the engine as it was if there is no memory for it (AZ_ENOMEM).
  * Default tiles follow the matrix's entries per pixel: 8 x 120 pixels below 2.1 (1D; 8 x 152 below
- * 1.75 on large detectors) or 48 x 40 below 2.4 (2D), then 16 x 64, 16 x 40 from 5, 16 x 24 from
+ * 1.75 on large detectors whose heaviest tile leaves room for it) or 48 x 40 below 2.4 (2D), then 16 x 64, 16 x 40 from 5, 16 x 24 from
  * 10 and 8 x 24 from 20 (larger ones where the segments would otherwise pass
  * az_integrate_noalloc's limit); 8 frames per pass. */
 int az_set_copy_engine(az_integrator *h, int engine);

@@ -67,13 +67,6 @@ void default_tile(const az_integrator *h, int &th, int &tw) {
     // kernel, 8 x 120 against 16 x 64: 683 and 777 us (128 frames of 2527 x 2463 pixels, 1.7
     // entries per pixel), 273 and 244 us (37 frames of 2167 x 2070, 2.6), 45 and 40 us (24 variances
     // of 1043 x 981, 2.8).
-    // Below 1.75 on large detectors, 8 x 152: a launch of few frames spends about 1.5 us an item, and
-    // has a fifth fewer of them (2527 x 2463: one to four frames against bound corrections 73 to 94
-    // us on 8 x 120, 64 to 82 here, twenty 205 and 179, 64 380 and 383; an FP64 frame 144 and 139;
-    // nine matrices of 2.9 to 6.2 Mpixel with 1.0 to 1.89 entries per pixel: 8 to 20% for up to 20
-    // frames, 1 to 10% for 48).  Above, three stages of the FP64 single-frame kernel no longer
-    // fit (2540 x 1800, 1.90: 119 and 173 us), as they do not with 8 x 168 (1.7: 144 and 200 us); with
-    // fewer than twelve tiles per SM (1043 x 981) the two are equal within 5%.
     // 2D: 48 x 40 (500 x 360 bins of 2048 x 2048 pixels, 16 frames and one:
     // 91 and 29 us; 32 x 64, where only four frames fit a stage: 109 and 28 us; 24 x 56: 80 and 37).
     // Denser matrices get smaller tiles, so that the stages of the FP64 single-frame kernel (14
@@ -86,15 +79,41 @@ void default_tile(const az_integrator *h, int &th, int &tw) {
     if (density < 10.0) { th = 16; tw = 40; }
     if (density < 5.0) { th = 16; tw = 64; }
     if (h->npt_azim == 0 && density < 2.1) { th = 8; tw = 120; }
-    const int64_t wide = (int64_t)((h->ny + 7) / 8) * ((h->nx + 151) / 152);
-    if (h->npt_azim == 0 && density < 1.75 && wide >= 12 * (int64_t)num_sms()) tw = 152;
     if (h->npt_azim > 0 && density < 2.4) { th = 48; tw = 40; }
+}
+
+// Whether 8 x 152 tiles may take the place of the default 8 x 120 (1D, below 1.75 entries per pixel,
+// large detectors): a launch of few frames spends about 1.5 us an item, and has a fifth fewer of
+// them.  2527 x 2463, full split: one to four frames against bound corrections 73 to 94 us on 8 x
+// 120, 64 to 82 here, twenty 205 and 179, 64 380 and 383; an FP64 frame 144 and 139.  Nine matrices of
+// 2.9 to 6.2 Mpixel with 1.0 to 1.89 entries per pixel: 8 to 20% for up to 20 frames, 1 to 10% for
+// 48.  But the rings are sized for the heaviest tile: where four stages of the frames kernel or
+// three of the FP64 single-frame kernel no longer fit, the narrow tiles are faster (2880 x 2880,
+// bounding boxes, 1.55: 32 frames 321 and 511 us, an FP64 frame 134 and 185; 2540 x 1800, 1.90: an
+// FP64 frame 119 and 173), which wide_tiles_fit says once they are built.  With fewer than twelve
+// tiles per SM (1043 x 981) the two are equal within 5%.
+int try_wide_tiles(az_integrator *h, cudaStream_t s, bool *kept) {
+    *kept = false;
+    const int64_t tiles = (int64_t)((h->ny + 7) / 8) * ((h->nx + 151) / 152);
+    if (h->npt_azim > 0 || (double)h->nnz >= 1.75 * (double)std::max(h->n_unmasked, 1) || tiles < 12 * (int64_t)num_sms())
+        return AZ_OK;
+    // the heaviest tile's entries, 10 bytes each and a tenth of padding, twice beside four blocks of
+    // planes: if that is too much, the layout is not built to find out
+    int64_t most = 0;
+    AZ_TRY(heaviest_tile(h, 8, 152, s, &most));
+    if (2 * 11 * most + 4 * 16 * 8 * 320 > max_smem_per_block()) return AZ_OK;
+    AZ_TRY(build_tiled_layout(h, 8, 152, s));
+    *kept = wide_tiles_fit(h);
+    return AZ_OK;
 }
 
 int finish_build(az_integrator *h, cudaStream_t s) {
     int th = 0, tw = 0;
     default_tile(h, th, tw);
-    if (build_tiled_layout(h, th, tw, s) != AZ_OK) {  // a denser matrix: smaller tiles
+    bool wide = false;
+    if (try_wide_tiles(h, s, &wide) != AZ_OK) clear_error();
+    if (wide) tw = 152;
+    else if (build_tiled_layout(h, th, tw, s) != AZ_OK) {  // a denser matrix: smaller tiles
         clear_error();
         th = 8;
         tw = 64;
@@ -643,7 +662,7 @@ extern "C" int az_set_copy_engine(az_integrator *h, int engine) {
         return fail(AZ_EINVAL, "az_set_copy_engine: bad engine %d", engine);
     const int before = h->copy_engine;
     h->copy_engine = engine;
-    const int rc = convert_bound_darks(h, h->last_stream);
+    const int rc = convert_bound_darks(h);
     if (rc != AZ_OK) h->copy_engine = before;
     return rc;
 }

@@ -353,6 +353,11 @@ int build_integrator(int ny, int nx, const double *rad, const double *chi, int n
                      int npt_azim, int unit, int split, const uint8_t *mask, cudaStream_t s,
                      az_integrator *h);
 int build_tiled_layout(az_integrator *h, int th, int tw, cudaStream_t s);
+// entries of the heaviest th x tw tile
+int heaviest_tile(const az_integrator *h, int th, int tw, cudaStream_t s, int64_t *out);
+// the current layout leaves room for four stages of eight frames in the frames kernel and three of
+// the FP64 single-frame kernel, with all corrections
+bool wide_tiles_fit(const az_integrator *h);
 // (tile, row) pairs that hold entries under th x tw tiles
 int count_runs(const az_integrator *h, int th, int tw, cudaStream_t s, int64_t *out);
 int import_csr(az_integrator *h, const int32_t *indptr, const int32_t *indices, const double *data,
@@ -399,7 +404,7 @@ int batch_frames(az_integrator *h, const void *frames, int n, int dtype, const f
                  float *oI, float *oS, int frame_out0, cudaStream_t s,
                  bool bound_dark = false, const float *norm = nullptr, float *oN = nullptr, float *oC = nullptr);
 // the bound darks in the order that the current copy engine's kernel reads
-int convert_bound_darks(az_integrator *h, cudaStream_t s);
+int convert_bound_darks(az_integrator *h);
 int bind_corrections(az_integrator *h, const float *dark, const float *flat, const float *sa,
                      const float *pol, cudaStream_t s);
 int forward_batch_bound(az_integrator *h, const void *frames, int n, int dtype, float *oI, float *oS,

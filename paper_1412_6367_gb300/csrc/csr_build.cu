@@ -870,6 +870,20 @@ __global__ void scatter_slots_kernel(const int32_t *__restrict__ perm, int nseg,
         slot[perm[s]] = (int32_t)s;
 }
 
+// Largest number of entries in a tile, a thread per tile: the pixels of a tile row are neighbours in
+// the pixel-major matrix.
+__global__ void tile_entries_kernel(const int32_t *__restrict__ csc_ptr, int ny, int nx, int th, int tw, int ntx,
+                                    int64_t ntiles, int32_t *__restrict__ most) {
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < ntiles;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const int r0 = (int)(t / ntx) * th, c0 = (int)(t % ntx) * tw, c1 = min(nx, c0 + tw);
+        int n = 0;
+        for (int r = r0; r < min(ny, r0 + th); ++r)
+            n += csc_ptr[(int64_t)r * nx + c1] - csc_ptr[(int64_t)r * nx + c0];
+        atomicMax(most, n);
+    }
+}
+
 // One bit per (row, tile) that has entries, for the rows of ptr, and their number.
 __global__ void mark_runs_kernel(TileGeom T, const int32_t *__restrict__ ptr, const int32_t *__restrict__ idx,
                                  int nrows, int64_t words, uint32_t *__restrict__ bits,
@@ -1250,6 +1264,21 @@ int import_csr(az_integrator *h, const int32_t *indptr, const int32_t *indices, 
     AZ_CUDA(cudaMemcpyAsync(&n_unmasked, nonempty.p, sizeof(int), cudaMemcpyDeviceToHost, s));
     AZ_CUDA(cudaStreamSynchronize(s));
     h->n_unmasked = n_unmasked;
+    return AZ_OK;
+}
+
+int heaviest_tile(const az_integrator *h, int th, int tw, cudaStream_t s, int64_t *out) {
+    ScratchScope scope;
+    TmpBuf most;
+    AZ_TRY(most.alloc(sizeof(int32_t)));
+    AZ_CUDA(cudaMemsetAsync(most.p, 0, sizeof(int32_t), s));
+    const int ntx = (h->nx + tw - 1) / tw, nty = (h->ny + th - 1) / th;
+    AZ_TRY(launch_gs(tile_entries_kernel, (int64_t)ntx * nty, s, h->csc_ptr.as<int32_t>(), h->ny, h->nx, th, tw, ntx,
+                     (int64_t)ntx * nty, most.as<int32_t>()));
+    int32_t n = 0;
+    AZ_CUDA(cudaMemcpyAsync(&n, most.p, sizeof(n), cudaMemcpyDeviceToHost, s));
+    AZ_CUDA(cudaStreamSynchronize(s));
+    *out = n;
     return AZ_OK;
 }
 

@@ -1240,9 +1240,9 @@ frames_kernel(const __grid_constant__ FrArgs a, FrGeom fg, const __grid_constant
 // waits for pixels that are still being corrected.  C = sum w is kept per layout.
 //
 // FP64 (one 2527 x 2463 frame, four corrections): the FP64 pipe, whose instructions take 64 cycles a
-// warp, conversions to double included, needs about 66 us: per pixel one subtraction and two
-// products (the conversions are done with integer instructions, exactly), per entry two multiply-
-// adds.  A call takes 134 us with tiles of 8 x 152 (140 with 8 x 120); correcting every entry and
+// warp, conversions to double included, is busy for 82 us of a launch of 122 (67%; shared memory 25%,
+// DRAM 24%): per pixel one subtraction and two products (the conversions are done with integer
+// instructions, exactly), per entry two multiply-adds.  A call takes 134 us with tiles of 8 x 152 (140 with 8 x 120); correcting every entry and
 // forming C each time took 351 us.
 // FP32 (the same frame): 70 us a call (80 with 8 x 120), where a pass that wrote two planes to memory
 // (28 us) and the frames kernel over them (40 us) took 78 with tiles of 8 x 224.  Of the 66 us of
@@ -2362,6 +2362,14 @@ int max_smem_per_block() {
     return g_max_smem;
 }
 
+bool wide_tiles_fit(const az_integrator *h) {
+    FrGeom fg;
+    SgNeed need;
+    need.add(h, 31);
+    SgGeom sg;
+    return fr_geom(h, 8, 1, kMaxFramesPerLaunch / 8, fg) && fg.nstages >= 4 && sg_geom(need, true, true, sg) && sg.nstages >= 3;
+}
+
 // C = sum w per row of the current layout, in both precisions (it does not depend on the
 // inputs): formed when the layout is built.
 int count_layout(az_integrator *h, cudaStream_t s) {
@@ -2803,10 +2811,12 @@ __global__ void scatter_dark_kernel(const int32_t *__restrict__ pix, const float
 }
 
 // The caller's dark is not at hand any more: its pixels from the entries of one order, then the
-// entries of the other.
-int convert_bound_darks(az_integrator *h, cudaStream_t s) {
+// entries of the other.  No stream is given: the device is waited for before and after.
+int convert_bound_darks(az_integrator *h) {
     const bool f = takes_frames_kernel(h);
     if (!h->corr_bound || !h->corr_dark || h->bound_dark_ok[f]) return AZ_OK;
+    const cudaStream_t s = nullptr;
+    AZ_CUDA(cudaDeviceSynchronize());
     ScratchScope scope;
     TmpBuf plane;
     AZ_TRY(plane.alloc(sizeof(float) * (size_t)h->ny * (size_t)h->nx));

@@ -46,3 +46,18 @@ def test_default_tile(ny, nx, npt, azim, split, dist, density, tile):
         tol = 1e-12 if k < 4 else 1e-5
         assert per <= tol and norm <= tol, k
     assert g.status() == 0
+
+
+@pytest.mark.parametrize("ny,nx,npt,tile", [(2880, 2880, 1000, (8, 120)), (2048, 2048, 600, (8, 152))])
+def test_wide_tiles_need_room_for_the_heaviest(ny, nx, npt, tile):
+    """Both below 1.75 entries per pixel; around the beam centre of the first a wide tile holds so many
+    entries that the kernels' rings would lose stages."""
+    geo = api().Geometry(0.1, 0.5 * ny * 100e-6, 0.5 * nx * 100e-6, 0.0, 0.0, 0.0, 100e-6, 100e-6)
+    g = api().Integrator.build(geo, (ny, nx), npt, 0, "q_nm^-1", "bbox")
+    assert 1.2 < g.info["nnz"] / g.info["n_unmasked"] < 1.75
+    assert (g.info["tile_h"], g.info["tile_w"]) == tile
+    img = torch.ones((ny, nx), dtype=torch.int32, device="cuda")
+    for prec in ("fp64", "fp32"):  # a flat image: S is C in every bin
+        r = g.integrate(img, precision=prec)
+        assert torch.equal(r.sum_signal, r.count) and torch.equal(r.sum_norm, r.count)
+    assert g.status() == 0
